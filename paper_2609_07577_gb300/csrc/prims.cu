@@ -1,9 +1,11 @@
 // Device-wide primitives: scratch arena, prefix scans and a stable LSD radix
 // sort. Everything here is deterministic (no atomics on values whose order
-// matters, no spin waits): reduce-then-scan for scans, and for the sort a
+// matters, no spin waits): the scans of scan.cuh, and for the sort a
 // per-tile digit histogram, a scan of the digit-major histogram table and a
-// stable scatter whose in-tile ranks come from warp match_any groups.
+// stable scatter whose in-tile ranks come from warp match_any groups; short
+// sorts run all their passes in one launch of one thread block cluster.
 #include "common.cuh"
+#include "scan.cuh"
 
 #include <atomic>
 #include <climits>
@@ -201,194 +203,70 @@ Status iota_i32(int32_t* p, int64_t n, cudaStream_t s)
 }
 
 // ---------------------------------------------------------------------------
-// Scans
+// Scans of plain arrays (scan.cuh)
 
-constexpr int SC_THREADS = 256;
-constexpr int SC_ITEMS = 8;
-constexpr int SC_TILE = SC_THREADS * SC_ITEMS;
+namespace {
 
-template <typename T>
-struct OpSum {
-    __device__ static T id() { return (T)0; }
-    __device__ T operator()(T a, T b) const { return a + b; }
+// running maximum as a "sum"
+struct Max32 {
+    int32_t v;
+    __device__ Max32() : v(INT_MIN) {}
+    __device__ explicit Max32(int32_t x) : v(x) {}
+    __device__ Max32 operator+(const Max32& o) const { return Max32(v > o.v ? v : o.v); }
+};
+__device__ __forceinline__ Max32 scan_shfl_up(Max32 x, int o)
+{
+    return Max32(__shfl_up_sync(FULL, x.v, o));
+}
+__device__ __forceinline__ Max32 scan_shfl(Max32 x, int src)
+{
+    return Max32(__shfl_sync(FULL, x.v, src));
+}
+struct Max32Store {
+    int32_t* p;
+    __device__ void operator()(int64_t i, Max32 ex, Max32 x) const { p[i] = (ex + x).v; }
 };
 
-template <typename T>
-struct OpMax {
-    __device__ static T id() { return sizeof(T) == 8 ? (T)LLONG_MIN : (T)INT_MIN; }
-    __device__ T operator()(T a, T b) const { return a > b ? a : b; }
-};
-
-template <typename T, typename Op>
-__device__ T block_reduce(T v, T* sh)
+template <typename Tin, typename T, bool INCL>
+Status scan_plain(const Tin* in, T* out, int64_t n, T* total, Arena& ar, cudaStream_t s)
 {
-    Op op;
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(FULL, v, o));
-    if (lane == 0) sh[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        v = lane < SC_THREADS / 32 ? sh[lane] : Op::id();
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(FULL, v, o));
-    }
-    return v;
+    return scan_run<T>(ScanLoad<Tin, T>{in}, ScanStore<T, INCL>{out}, n, total, ar, s);
 }
 
-// exclusive scan of one value per thread across the block; sh holds >= 64 T
-template <typename T, typename Op>
-__device__ T block_exclusive(T v, T* sh)
-{
-    Op op;
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    T inc = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        T t = __shfl_up_sync(FULL, inc, o);
-        if (lane >= o) inc = op(t, inc);
-    }
-    if (lane == 31) sh[warp] = inc;
-    __syncthreads();
-    if (warp == 0) {
-        T wi = lane < SC_THREADS / 32 ? sh[lane] : Op::id();
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            T t = __shfl_up_sync(FULL, wi, o);
-            if (lane >= o) wi = op(t, wi);
-        }
-        T ex = __shfl_up_sync(FULL, wi, 1);
-        if (lane == 0) ex = Op::id();
-        if (lane < SC_THREADS / 32) sh[32 + lane] = ex;
-    }
-    __syncthreads();
-    T warp_ex = sh[32 + warp];
-    T exl = __shfl_up_sync(FULL, inc, 1);
-    if (lane == 0) exl = Op::id();
-    T r = op(warp_ex, exl);
-    __syncthreads();
-    return r;
-}
-
-template <typename Tin, typename T, typename Op>
-__global__ void __launch_bounds__(SC_THREADS) k_scan_reduce(const Tin* in, int64_t n, T* bsum)
-{
-    __shared__ T sh[SC_THREADS / 32];
-    Op op;
-    T acc = Op::id();
-    int64_t base = (int64_t)blockIdx.x * SC_TILE;
-    for (int i = threadIdx.x; i < SC_TILE; i += SC_THREADS) {
-        int64_t j = base + i;
-        if (j < n) acc = op(acc, (T)in[j]);
-    }
-    acc = block_reduce<T, Op>(acc, sh);
-    if (threadIdx.x == 0) bsum[blockIdx.x] = acc;
-}
-
-template <typename Tin, typename T, typename Op, bool INCL>
-__global__ void __launch_bounds__(SC_THREADS)
-    k_scan_tile(const Tin* in, int64_t n, T* out, const T* boff, T* total)
-{
-    __shared__ T tile[SC_TILE];
-    __shared__ T sh[64];
-    Op op;
-    int64_t base = (int64_t)blockIdx.x * SC_TILE;
-    for (int i = threadIdx.x; i < SC_TILE; i += SC_THREADS) {
-        int64_t j = base + i;
-        tile[i] = j < n ? (T)in[j] : Op::id();
-    }
-    __syncthreads();
-    T v[SC_ITEMS];
-    T run = Op::id();
-#pragma unroll
-    for (int k = 0; k < SC_ITEMS; k++) {
-        v[k] = tile[threadIdx.x * SC_ITEMS + k];
-        run = op(run, v[k]);
-    }
-    T ex = block_exclusive<T, Op>(run, sh);
-    T acc = op(boff ? boff[blockIdx.x] : Op::id(), ex);
-#pragma unroll
-    for (int k = 0; k < SC_ITEMS; k++) {
-        if (INCL) {
-            acc = op(acc, v[k]);
-            tile[threadIdx.x * SC_ITEMS + k] = acc;
-        } else {
-            tile[threadIdx.x * SC_ITEMS + k] = acc;
-            acc = op(acc, v[k]);
-        }
-    }
-    if (total && blockIdx.x == gridDim.x - 1 && threadIdx.x == SC_THREADS - 1) *total = acc;
-    __syncthreads();
-    for (int i = threadIdx.x; i < SC_TILE; i += SC_THREADS) {
-        int64_t j = base + i;
-        if (j < n) out[j] = tile[i];
-    }
-}
-
-template <typename T, typename Op>
-__global__ void k_set_identity(T* p)
-{
-    *p = Op::id();
-}
-
-template <typename Tin, typename T, typename Op, bool INCL>
-static Status scan_impl(const Tin* in, T* out, int64_t n, T* total, Arena& ar, cudaStream_t s)
-{
-    if (n <= 0) {
-        if (total) {
-            SNN_L k_set_identity<T, Op><<<1, 1, 0, s>>>(total);
-            SNN_CUDA(cudaGetLastError());
-        }
-        return Status{};
-    }
-    int64_t nb = ceil_div(n, SC_TILE);
-    if (nb == 1) {
-        SNN_L k_scan_tile<Tin, T, Op, INCL><<<1, SC_THREADS, 0, s>>>(in, n, out, nullptr, total);
-        SNN_CUDA(cudaGetLastError());
-        return Status{};
-    }
-    T* bsum = nullptr;
-    SNN_TRY(ar.alloc(&bsum, nb));
-    SNN_L k_scan_reduce<Tin, T, Op><<<(unsigned)nb, SC_THREADS, 0, s>>>(in, n, bsum);
-    SNN_CUDA(cudaGetLastError());
-    SNN_TRY((scan_impl<T, T, Op, false>(bsum, bsum, nb, nullptr, ar, s)));
-    SNN_L k_scan_tile<Tin, T, Op, INCL><<<(unsigned)nb, SC_THREADS, 0, s>>>(in, n, out, bsum, total);
-    SNN_CUDA(cudaGetLastError());
-    return Status{};
-}
+}  // namespace
 
 Status scan_exclusive_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* total,
                                  Arena& ar, cudaStream_t s)
 {
-    return scan_impl<int32_t, int64_t, OpSum<int64_t>, false>(in, out, n, total, ar, s);
+    return scan_plain<int32_t, int64_t, false>(in, out, n, total, ar, s);
 }
 
 Status scan_exclusive_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* total, Arena& ar,
                           cudaStream_t s)
 {
-    return scan_impl<int64_t, int64_t, OpSum<int64_t>, false>(in, out, n, total, ar, s);
+    return scan_plain<int64_t, int64_t, false>(in, out, n, total, ar, s);
 }
 
 Status scan_exclusive_i32(const int32_t* in, int32_t* out, int64_t n, int32_t* total, Arena& ar,
                           cudaStream_t s)
 {
-    return scan_impl<int32_t, int32_t, OpSum<int32_t>, false>(in, out, n, total, ar, s);
+    return scan_plain<int32_t, int32_t, false>(in, out, n, total, ar, s);
 }
 
 Status scan_inclusive_i64(const int64_t* in, int64_t* out, int64_t n, Arena& ar, cudaStream_t s)
 {
-    return scan_impl<int64_t, int64_t, OpSum<int64_t>, true>(in, out, n, nullptr, ar, s);
+    return scan_plain<int64_t, int64_t, true>(in, out, n, (int64_t*)nullptr, ar, s);
 }
 
 Status scan_inclusive_i32(const int32_t* in, int32_t* out, int64_t n, Arena& ar, cudaStream_t s)
 {
-    return scan_impl<int32_t, int32_t, OpSum<int32_t>, true>(in, out, n, nullptr, ar, s);
+    return scan_plain<int32_t, int32_t, true>(in, out, n, (int32_t*)nullptr, ar, s);
 }
 
 Status scan_inclusive_max_i32(const int32_t* in, int32_t* out, int64_t n, Arena& ar,
                               cudaStream_t s)
 {
-    return scan_impl<int32_t, int32_t, OpMax<int32_t>, true>(in, out, n, nullptr, ar, s);
+    return scan_run<Max32>(ScanLoad<int32_t, Max32>{in}, Max32Store{out}, n, (Max32*)nullptr, ar, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -469,24 +347,212 @@ __global__ void __launch_bounds__(RS_THREADS)
     }
 }
 
+// The whole sort in one launch for short inputs: one cluster of 8 blocks
+// runs every pass, with the cluster's hardware barrier between the phases
+// and the blocks' digit counts read through distributed shared memory. A
+// short sort is bound by its launches and by the latency of a pass, not by
+// bytes: in the form above a pass of a few thousand keys is an upsweep, one
+// to three scan kernels and a downsweep by one or a few blocks.
+// Passes in which every key has the same digit move nothing and are skipped.
+constexpr int RSC_CTAS = 8;
+constexpr int RSC_THREADS = 1024;
+constexpr int RSC_WARPS = RSC_THREADS / 32;
+constexpr int RSC_ROUNDS = 12;
+constexpr int64_t RSC_MAX = (int64_t)RSC_CTAS * RSC_THREADS * RSC_ROUNDS;   // 98,304
+
+__global__ void __cluster_dims__(RSC_CTAS, 1, 1) __launch_bounds__(RSC_THREADS)
+    k_rs_cluster(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t* vals_alt, int32_t n,
+                 int passes)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ uint32_t wcnt[RSC_WARPS][256];
+    __shared__ uint32_t hist[256];
+    __shared__ uint32_t goff[256];
+    __shared__ uint32_t tmp[RSC_WARPS][32];
+    __shared__ uint32_t wsum[8];
+    __shared__ int same;
+    const int rank = (int)cl.block_rank();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned lt = lanemask_lt();
+    const int rounds = (n + RSC_CTAS * RSC_THREADS - 1) / (RSC_CTAS * RSC_THREADS);
+    const int w0 = (rank * RSC_THREADS + warp * 32) * rounds;
+    uint64_t *ki = keys, *ko = keys_alt;
+    uint32_t *vi = vals, *vo = vals_alt;
+    for (int p = 0; p < passes; p++) {
+        const int shift = 8 * p;
+        for (int i = threadIdx.x; i < RSC_WARPS * 256; i += RSC_THREADS) (&wcnt[0][0])[i] = 0;
+        if (threadIdx.x == 0) same = 0;
+        uint64_t k[RSC_ROUNDS];
+        uint32_t rk[RSC_ROUNDS];
+        // keys written by the other blocks in the pass before: read past L1
+#pragma unroll
+        for (int r = 0; r < RSC_ROUNDS; r++) {
+            int j = w0 + r * 32 + lane;
+            k[r] = r < rounds && j < n ? __ldcg((unsigned long long*)&ki[j]) : 0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < RSC_ROUNDS; r++) {
+            if (r >= rounds) continue;   // the same for the whole cluster
+            bool valid = w0 + r * 32 + lane < n;
+            uint32_t d = valid ? (uint32_t)((k[r] >> shift) & 255) : 256u;
+            unsigned peers = __match_any_sync(FULL, d);
+            int leader = __ffs(peers) - 1;
+            if (lane == leader && valid) {
+                uint32_t c = wcnt[warp][d];
+                tmp[warp][lane] = c;
+                wcnt[warp][d] = c + __popc(peers);
+            }
+            __syncwarp();
+            rk[r] = valid ? tmp[warp][leader] + __popc(peers & lt) : 0;
+            __syncwarp();
+        }
+        __syncthreads();
+        if (threadIdx.x < 256) {
+            uint32_t acc = 0;
+#pragma unroll 8
+            for (int w = 0; w < RSC_WARPS; w++) {
+                uint32_t c = wcnt[w][threadIdx.x];
+                wcnt[w][threadIdx.x] = acc;
+                acc += c;
+            }
+            hist[threadIdx.x] = acc;
+        }
+        cl.sync();
+        uint32_t before = 0, tot = 0, inc = 0;
+        if (threadIdx.x < 256) {
+#pragma unroll
+            for (int b = 0; b < RSC_CTAS; b++) {
+                uint32_t c = cl.map_shared_rank(hist, b)[threadIdx.x];
+                if (b < rank) before += c;
+                tot += c;
+            }
+            if (tot == (uint32_t)n) same = 1;
+            inc = warp_inclusive(tot);
+            if (lane == 31) wsum[warp] = inc;
+        }
+        __syncthreads();
+        if (threadIdx.x < 256) {
+            uint32_t acc = inc - tot + before;
+            for (int w = 0; w < warp; w++) acc += wsum[w];
+            goff[threadIdx.x] = acc;
+        }
+        __syncthreads();
+        if (!same) {   // the same in every block: all saw the same totals
+#pragma unroll
+            for (int r = 0; r < RSC_ROUNDS; r++) {
+                int j = w0 + r * 32 + lane;
+                if (r < rounds && j < n) {
+                    uint32_t d = (uint32_t)((k[r] >> shift) & 255);
+                    uint32_t pos = goff[d] + wcnt[warp][d] + rk[r];
+                    __stcg((unsigned long long*)&ko[pos], (unsigned long long)k[r]);
+                    __stcg(&vo[pos], __ldcg(&vi[j]));
+                }
+            }
+            uint64_t* tk = ki; ki = ko; ko = tk;
+            uint32_t* tv = vi; vi = vo; vo = tv;
+            __threadfence();
+        }
+        // the pass is complete, and hist may be written again
+        cl.sync();
+    }
+    if (ki != keys) {
+#pragma unroll
+        for (int r = 0; r < RSC_ROUNDS; r++) {
+            int j = w0 + r * 32 + lane;
+            if (r < rounds && j < n) {
+                keys[j] = __ldcg((unsigned long long*)&ki[j]);
+                vals[j] = __ldcg(&vi[j]);
+            }
+        }
+    }
+}
+
+// Up to SB_MAX items one block sorts in shared memory: a bitonic network over
+// the words key << ibits | position, whose order is the stable order of the
+// keys. A refinement round sorts its moves and its events, mostly a few
+// hundred to a few thousand of each, and there even one launch of the radix
+// passes is a chain of barriers: 1,000 keys of 20 bits take 24 us in the
+// cluster form.
+constexpr int SB_MAX = 4096;
+constexpr int SB_THREADS = 1024;
+
+__global__ void __launch_bounds__(SB_THREADS)
+    k_sort_block(uint64_t* keys, uint32_t* vals, int32_t n, int N, int ibits)
+{
+    __shared__ uint64_t w[SB_MAX];
+    uint32_t v[SB_MAX / SB_THREADS];
+    const uint64_t imask = (1ull << ibits) - 1;
+    for (int i = threadIdx.x; i < N; i += SB_THREADS)
+        w[i] = i < n ? (keys[i] << ibits) | (uint64_t)i : ~0ull;
+    __syncthreads();
+    // a warp's 32 pairs of a step with stride <= 32 lie in one aligned run of
+    // 64 words, so only longer strides need the whole block
+    for (int k = 2; k <= N; k <<= 1) {
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int t = threadIdx.x; t < N / 2; t += SB_THREADS) {
+                int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
+                uint64_t a = w[i], b = w[i + j];
+                if ((a > b) == ((i & k) == 0)) {
+                    w[i] = b;
+                    w[i + j] = a;
+                }
+            }
+            // the next step's stride is j / 2, or k after the last of these
+            if (j > 32 || (j == 1 && k > 32)) __syncthreads();
+            else __syncwarp();
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < SB_MAX / SB_THREADS; r++) {
+        int i = r * SB_THREADS + threadIdx.x;
+        if (i < n) v[r] = vals[w[i] & imask];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < SB_MAX / SB_THREADS; r++) {
+        int i = r * SB_THREADS + threadIdx.x;
+        if (i < n) {
+            keys[i] = w[i] >> ibits;
+            vals[i] = v[r];
+        }
+    }
+}
+
 Status radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t* vals_alt,
                         int64_t n, int end_bit, Arena& ar, cudaStream_t s)
 {
     if (n <= 1 || end_bit <= 0) return Status{};
     if (n >= ((int64_t)1 << 32)) return Status{1, "radix sort: too many items"};
+    int passes = (end_bit + 7) / 8;
+    if (n <= SB_MAX) {
+        int N = 64, ib = bits_for((uint64_t)(n - 1));
+        while (N < n) N <<= 1;
+        if (end_bit + ib < 64) {   // the padding stays above every word
+            SNN_L k_sort_block<<<1, SB_THREADS, 0, s>>>(keys, vals, (int32_t)n, N, ib);
+            SNN_CUDA(cudaGetLastError());
+            return Status{};
+        }
+    }
+    if (n <= RSC_MAX) {
+        SNN_L k_rs_cluster<<<RSC_CTAS, RSC_THREADS, 0, s>>>(keys, vals, keys_alt, vals_alt, (int32_t)n,
+                                                            passes);
+        SNN_CUDA(cudaGetLastError());
+        return Status{};
+    }
     int nblk = (int)ceil_div(n, RS_TILE);
     uint32_t* counts = nullptr;
     SNN_TRY(ar.alloc(&counts, (int64_t)256 * nblk));
-    int passes = (end_bit + 7) / 8;
     uint64_t *ki = keys, *ko = keys_alt;
     uint32_t *vi = vals, *vo = vals_alt;
     for (int p = 0; p < passes; p++) {
         int shift = 8 * p;
         SNN_L k_rs_upsweep<<<nblk, RS_THREADS, 0, s>>>(ki, n, shift, counts, nblk);
         SNN_CUDA(cudaGetLastError());
-        SNN_TRY((scan_impl<uint32_t, uint32_t, OpSum<uint32_t>, false>(counts, counts,
-                                                                      (int64_t)256 * nblk,
-                                                                      nullptr, ar, s)));
+        SNN_TRY((scan_plain<uint32_t, uint32_t, false>(counts, counts, (int64_t)256 * nblk,
+                                                       (uint32_t*)nullptr, ar, s)));
         SNN_L k_rs_downsweep<<<nblk, RS_THREADS, 0, s>>>(ki, vi, ko, vo, n, shift, counts, nblk);
         SNN_CUDA(cudaGetLastError());
         uint64_t* tk = ki; ki = ko; ko = tk;
