@@ -439,7 +439,14 @@ __global__ void k_ac_prep(int32_t V, const int32_t* __restrict__ cid,
     }
 }
 
-// per hyperedge: its number of new super-nodes; work[0] += (|a| - cnt) cnt.
+// per hyperedge: its number of new super-nodes; work[0] += (|a| - cnt) cnt,
+// the carried vertices' visits of the lists, and work[1] += |a| cnt, what
+// the new super-nodes' full histograms visit (MERGED vertices mostly keep
+// the new super-node their candidate merged into (k_ac_check), so they are
+// left out of the estimate). Summing the latter over hyperedges instead of
+// over the new super-nodes' incidence lists needs no pass of its own: a
+// warp walking the list of a super-node that is in most hyperedges took
+// 390 us a level (60,052-neuron layered network, 45,039 hyperedges).
 // A group of G lanes per hyperedge; each warp takes 32 / G consecutive
 // hyperedges per step, so the group sums run with the whole warp.
 template <int G>
@@ -451,7 +458,7 @@ __global__ void __launch_bounds__(256)
     int grp = (threadIdx.x & 31) / G;
     int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    int64_t acc = 0;
+    int64_t acc = 0, full = 0;
     for (int64_t base = warp * PER; base < L.E; base += nwarp * PER) {
         int64_t a = base + grp;
         int c = 0;
@@ -466,9 +473,15 @@ __global__ void __launch_bounds__(256)
         if (lane == 0 && a < L.E) {
             lcnt[a] = c;
             acc += (len - c) * (int64_t)c;
+            full += len * (int64_t)c;
         }
     }
-    if (lane == 0 && acc) atomicAdd((unsigned long long*)work, (unsigned long long)acc);
+    acc = warp_sum(acc);
+    full = warp_sum(full);
+    if ((threadIdx.x & 31) == 0 && full) {
+        atomicAdd((unsigned long long*)work, (unsigned long long)acc);
+        atomicAdd((unsigned long long*)work + 1, (unsigned long long)full);
+    }
 }
 
 // the lists: new super-nodes of each hyperedge in pin order, bit 31 set for
@@ -496,33 +509,6 @@ __global__ void __launch_bounds__(256)
             o += __popc(mk);
         }
     }
-}
-
-// work[0] += incidence segment lengths of the NEW vertices (what their full
-// histograms cost); MERGED vertices mostly keep the new super-node their
-// candidate merged into (k_ac_check), so they are left out of the estimate
-__global__ void __launch_bounds__(256)
-    k_ac_fullwork(Level L, const uint8_t* __restrict__ kind, int64_t* work)
-{
-    int lane = threadIdx.x & 31;
-    int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    int64_t acc = 0;
-    for (int64_t base = gw * 32; base < L.V; base += nw * 32) {
-        int64_t n = base + lane;
-        unsigned mem = __ballot_sync(FULL, n < L.V && kind[n] == AK_NEW);
-        while (mem) {
-            int src = __ffs(mem) - 1;
-            mem &= mem - 1;
-            int32_t m = (int32_t)__shfl_sync(FULL, (int32_t)n, src);
-            for (int64_t i = L.voff[m] + lane; i < L.voff[m + 1]; i += 32) {
-                int32_t a = (int32_t)((uint32_t)L.vinc[i] & ~SRC_BIT);
-                acc += L.hoff[a + 1] - L.hoff[a];
-            }
-        }
-    }
-    acc = warp_sum(acc);
-    if (lane == 0 && acc) atomicAdd((unsigned long long*)work, (unsigned long long)acc);
 }
 
 // MERGED vertices whose best valid new super-node is not w = cand (full
@@ -746,7 +732,6 @@ static Status affinity_carried(snnmap_hgraph* h, Level& L, bool* done)
     SNN_CUDA(cudaMemsetAsync(work, 0, 4 * sizeof(int64_t), s));
     SNN_L k_level_min<<<grid_for(L.V, 256), 256, 0, s>>>(L, vmin);
     if (E > 0) SNN_HEDGE_LAUNCH(hedge_lanes(L.P, E), k_ac_count, E, s, L, C.kind, lcnt, work);
-    SNN_L k_ac_fullwork<<<grid_for(L.V, 256), 256, 0, s>>>(L, C.kind, work + 1);
     SNN_CUDA(cudaGetLastError());
     SNN_TRY(scan_exclusive_i32_to_i64(lcnt, loff, E, loff + E, ar, s));
     int64_t hv[3];
