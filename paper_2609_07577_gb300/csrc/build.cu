@@ -160,87 +160,70 @@ void level_release(snnmap_hgraph* h, Level& L)
 // ---------------------------------------------------------------------------
 // size buckets
 
-__device__ __forceinline__ int seg_bucket(int64_t len)
-{
-    return len <= SEG_T_CAP ? SEG_BT
-         : len <= 32 ? SEG_BB0 : (len <= SEG_B1_CAP ? SEG_BB1 : (len <= SEG_B2_CAP ? SEG_BB2 : SEG_BB3));
-}
+struct SegStart {
+    int32_t at[SEG_NB], n[SEG_NB];
+};
 
-// bucket flags packed two per int64 (pa: T, B0; pb: B1, B2; pc: B3)
-__global__ void k_seg_flags(const int64_t* __restrict__ hoff, int32_t E, int64_t* pa, int64_t* pb,
-                            int64_t* pc, int64_t* w2)
+// One tile of 1024 hyperedges per block and step: the block counts its tile
+// per bucket, reserves a run of each bucket with one atomic, and writes its
+// ids in id order.
+__global__ void __launch_bounds__(1024)
+    k_seg_lists(const int64_t* __restrict__ hoff, int32_t E, SegStart st, int32_t* cursor,
+                int32_t* meta, int32_t* list)
 {
-    int64_t acc = 0;
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < E;
-         a += (int64_t)gridDim.x * blockDim.x) {
-        int64_t len = hoff[a + 1] - hoff[a];
-        int b = seg_bucket(len);
-        pa[a] = (int64_t)(b == SEG_BT) | ((int64_t)(b == SEG_BB0) << 32);
-        pb[a] = (int64_t)(b == SEG_BB1) | ((int64_t)(b == SEG_BB2) << 32);
-        pc[a] = (int64_t)(b == SEG_BB3);
-        acc += len * (len - 1);
+    __shared__ int32_t wc[SEG_NB][32];
+    __shared__ int32_t base[SEG_NB];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned lt = lanemask_lt();
+    if (blockIdx.x == 0 && threadIdx.x < SEG_NB) {
+        meta[threadIdx.x] = st.at[threadIdx.x];
+        meta[SEG_NB + threadIdx.x] = st.n[threadIdx.x];
     }
-    acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0 && acc) atomicAdd((unsigned long long*)w2, (unsigned long long)acc);
-}
-
-__global__ void k_seg_meta(const int64_t* tot, int32_t* meta)
-{
-    int32_t c[SEG_NB] = {(int32_t)(tot[0] & 0xffffffff), (int32_t)(tot[0] >> 32),
-                         (int32_t)(tot[1] & 0xffffffff), (int32_t)(tot[1] >> 32),
-                         (int32_t)(tot[2] & 0xffffffff)};
-    int32_t run = 0;
-    for (int b = 0; b < SEG_NB; b++) {
-        meta[b] = run;
-        meta[SEG_NB + b] = c[b];
-        run += c[b];
-    }
-}
-
-__global__ void k_seg_scatter(const int64_t* __restrict__ hoff, int32_t E,
-                              const int64_t* __restrict__ pa, const int64_t* __restrict__ pb,
-                              const int64_t* __restrict__ pc, const int32_t* __restrict__ meta,
-                              int32_t* list)
-{
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < E;
-         a += (int64_t)gridDim.x * blockDim.x) {
-        int b = seg_bucket(hoff[a + 1] - hoff[a]);
-        int64_t pos = b == SEG_BT ? (pa[a] & 0xffffffff)
-                    : b == SEG_BB0 ? (pa[a] >> 32)
-                    : b == SEG_BB1 ? (pb[a] & 0xffffffff)
-                    : b == SEG_BB2 ? (pb[a] >> 32)
-                                   : (pc[a] & 0xffffffff);
-        list[meta[b] + pos] = (int32_t)a;
+    for (int64_t t0 = (int64_t)blockIdx.x * 1024; t0 < E; t0 += (int64_t)gridDim.x * 1024) {
+        int64_t a = t0 + threadIdx.x;
+        int b = a < E ? seg_bucket(hoff[a + 1] - hoff[a]) : -1;
+        int rank = 0;
+#pragma unroll
+        for (int i = 0; i < SEG_NB; i++) {
+            unsigned m = __ballot_sync(FULL, b == i);
+            if (b == i) rank = __popc(m & lt);
+            if (lane == 0) wc[i][warp] = __popc(m);
+        }
+        __syncthreads();
+        if (warp < SEG_NB) {
+            int32_t c = wc[warp][lane], inc = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                int32_t x = __shfl_up_sync(FULL, inc, o);
+                if (lane >= o) inc += x;
+            }
+            wc[warp][lane] = inc - c;
+            if (lane == 31) base[warp] = st.at[warp] + (inc ? atomicAdd(&cursor[warp], inc) : 0);
+        }
+        __syncthreads();
+        if (b >= 0) list[base[b] + wc[b][warp] + rank] = (int32_t)a;
+        __syncthreads();
     }
 }
 
-Status seg_classify(const int64_t* hoff, int32_t E, int32_t maxlen, SegBuckets& b, Arena& ar,
-                    cudaStream_t s, int64_t* w2)
+Status seg_lists(const int64_t* hoff, int32_t E, int32_t maxlen, SegBuckets& b, int32_t* cursor,
+                 cudaStream_t s)
 {
-    int64_t *pa, *pb, *pc, *tot;
-    SNN_TRY(ar.alloc(&pa, E));
-    SNN_TRY(ar.alloc(&pb, E));
-    SNN_TRY(ar.alloc(&pc, E));
-    SNN_TRY(ar.alloc(&tot, 3));
     b.b3_cap = 0;
     if (maxlen > SEG_B2_CAP) {
         int64_t c = SEG_B2_CAP;
         while (c < maxlen) c <<= 1;
         b.b3_cap = c;
     }
-    if (E > 0) {
-        SNN_L k_seg_flags<<<grid_for(E, 256), 256, 0, s>>>(hoff, E, pa, pb, pc, w2);
-        SNN_CUDA(cudaGetLastError());
+    SegStart st;
+    int32_t run = 0;
+    for (int i = 0; i < SEG_NB; i++) {
+        st.at[i] = run;
+        st.n[i] = b.n[i];
+        run += b.n[i];
     }
-    SNN_TRY(scan_exclusive_i64(pa, pa, E, tot, ar, s));
-    SNN_TRY(scan_exclusive_i64(pb, pb, E, tot + 1, ar, s));
-    SNN_TRY(scan_exclusive_i64(pc, pc, E, tot + 2, ar, s));
-    SNN_L k_seg_meta<<<1, 1, 0, s>>>(tot, b.meta);
+    SNN_L k_seg_lists<<<grid_for(E, 1024, 152 * 2), 1024, 0, s>>>(hoff, E, st, cursor, b.meta, b.list);
     SNN_CUDA(cudaGetLastError());
-    if (E > 0) {
-        SNN_L k_seg_scatter<<<grid_for(E, 256), 256, 0, s>>>(hoff, E, pa, pb, pc, b.meta, b.list);
-        SNN_CUDA(cudaGetLastError());
-    }
     return Status{};
 }
 
@@ -313,6 +296,7 @@ Status build_incidence(snnmap_hgraph* h, Level& L)
 __global__ void k_in_hedges(const int64_t* __restrict__ off, const int32_t* __restrict__ w,
                             int32_t E, int32_t* kept, int64_t* klen, int64_t* scal)
 {
+    SegTally tally;
     int32_t bad = 0;
     int64_t mx = 0, wsum = 0;
     int32_t zero = 0;
@@ -324,6 +308,7 @@ __global__ void k_in_hedges(const int64_t* __restrict__ off, const int32_t* __re
         if (k && w[a] == 0) zero = 1;
         kept[a] = k;
         klen[a] = k ? len : 0;
+        if (k) tally.add(len);
         if (len > mx) mx = len;
         wsum += w[a] > 0 ? w[a] : 0;
     }
@@ -341,6 +326,7 @@ __global__ void k_in_hedges(const int64_t* __restrict__ off, const int32_t* __re
         atomicMax((unsigned long long*)&scal[SC_C], (unsigned long long)mx);
         atomicAdd((unsigned long long*)&scal[SC_D], (unsigned long long)wsum);
     }
+    tally.flush(scal + SC_SEG, scal + SC_W2);
 }
 
 __global__ void k_in_pins(const int32_t* __restrict__ pins, int64_t P, int32_t V, int64_t* scal)
@@ -463,7 +449,7 @@ Status build_level0(snnmap_hgraph* h, int32_t V, int32_t E, const int64_t* d_off
     SNN_TRY(ar.alloc(&klen, E));
     SNN_TRY(ar.alloc(&newoff, E));
     if (E > 0) {
-        SNN_L k_in_hedges<<<grid_for(E, 256), 256, 0, s>>>(d_off, d_w, E, kept, klen, h->d_scal);
+        SNN_L k_in_hedges<<<grid_for(E, 256, 152 * 8), 256, 0, s>>>(d_off, d_w, E, kept, klen, h->d_scal);
         SNN_CUDA(cudaGetLastError());
     }
     if (Pin > 0) {
@@ -481,6 +467,7 @@ Status build_level0(snnmap_hgraph* h, int32_t V, int32_t E, const int64_t* d_off
     h->wide = (uint64_t)h->h_scal[SC_D] >= 0xffffffffull;
     h->wsum = h->h_scal[SC_D];
     h->wzero = h->h_scal[SC_E] != 0;
+    int64_t terms = h->h_scal[SC_W2];
 
     h->levels.emplace_back();
     h->extra.emplace_back();
@@ -495,7 +482,12 @@ Status build_level0(snnmap_hgraph* h, int32_t V, int32_t E, const int64_t* d_off
     }
     SNN_L k_set_last_off<<<1, 1, 0, s>>>(L.hoff, E0, h->d_scal + SC_B);
     SNN_CUDA(cudaGetLastError());
-    SNN_TRY(seg_classify(L.hoff, E0, maxlen, X.seg, ar, s, h->d_scal + SC_W2));
+    X.pair_terms = terms;
+    for (int i = 0; i < SEG_NB; i++) X.seg.n[i] = (int32_t)h->h_scal[SC_SEG + i];
+    int32_t* cursor;
+    SNN_TRY(ar.alloc(&cursor, SEG_NB));
+    SNN_CUDA(cudaMemsetAsync(cursor, 0, SEG_NB * sizeof(int32_t), s));
+    SNN_TRY(seg_lists(L.hoff, E0, maxlen, X.seg, cursor, s));
     BuildCheckJob job{L.hoff, L.hpins, h->d_scal};
     {
         ProfScope prof(h, PS_BUILD);
@@ -512,7 +504,6 @@ Status build_level0(snnmap_hgraph* h, int32_t V, int32_t E, const int64_t* d_off
     }
     SNN_TRY(build_incidence(h, L));
     SNN_TRY(read_scalars(h));
-    X.pair_terms = h->h_scal[SC_W2];
     h->scratch.reset();
     if (h->h_scal[SC_STATUS] & ST_INVALID)
         return Status{SNNMAP_ERR_INVALID, "repeated destination or source listed as a destination"};

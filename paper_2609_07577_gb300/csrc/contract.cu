@@ -14,30 +14,35 @@
 //    through cid, sorted, made unique; s' among them sets selfdst and is
 //    removed. A hyperedge left with no destination is dropped and its
 //    multiplicity k moves into the source super-node's internal count.
-// 4. Duplicate hyperedges (same s', selfdst, destination list) merge: a
-//    stable radix sort on (s', 32-bit content hash) brings candidates
-//    together, an exact comparison of the contents decides, and the first
-//    of each equal group becomes the coarse hyperedge; omega and k add up.
-// 5. Compaction into the next level's arrays, then its incidence lists.
+// 4. Duplicate hyperedges (same s', selfdst, destination list) merge: every
+//    remaining hyperedge enters a hash table under a 64-bit content hash, the
+//    lowest id of an entry represents it, an exact comparison with the
+//    representative decides, and omega and k add up. Different contents
+//    under one hash go through the table again, by themselves, until each
+//    has its own representative.
+// 5. Compaction (in id order) into the next level's arrays, its size
+//    buckets, then its incidence lists.
 //
 // The same routine (build_coarse) materializes any level l from a resident
 // level j < l through the composed map cid_{l-1} o ... o cid_j: the image of
 // an axon does not depend on the order of the merges, so a level whose
 // arrays were released to save memory is rebuilt exactly.
 #include "internal.cuh"
+#include "scan.cuh"
 
 #include <memory>
 
 namespace snn {
 
-__global__ void k_rep_flags(int32_t V, const int32_t* __restrict__ match, int32_t* isrep)
-{
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
-         n += (int64_t)gridDim.x * blockDim.x) {
+// a vertex stands for its pair when it is unmatched or the lower id
+struct RepFlag {
+    const int32_t* match;
+    __device__ int32_t operator()(int64_t n) const
+    {
         int32_t m = match[n];
-        isrep[n] = (m < 0 || (int32_t)n < m) ? 1 : 0;
+        return m < 0 || (int32_t)n < m ? 1 : 0;
     }
-}
+};
 
 struct NextState {
     int32_t *size, *inpins, *inint;
@@ -50,6 +55,37 @@ __global__ void k_cid_map(int32_t V, const int32_t* __restrict__ match,
          n += (int64_t)gridDim.x * blockDim.x) {
         int32_t m = match[n];
         cid[n] = repidx[(m < 0 || (int32_t)n < m) ? (int32_t)n : m];
+    }
+}
+
+// State of the next level's vertices from a matching, one thread per pair
+// (the representative adds up both members, so no atomics and nothing to
+// clear); dropped: the multiplicities of the hyperedges that vanished inside
+// a super-node. in_count: an unmatched vertex keeps its count; a pair has
+// in_count(n) + in_count(m) - shared(n, m), the shared count being the
+// candidate overlap of the member whose candidate is the other (pairs are
+// matched along candidate arcs).
+__global__ void k_next_state(Level S, const int32_t* __restrict__ map,
+                             const int32_t* __restrict__ match, const int32_t* __restrict__ cand,
+                             const int32_t* __restrict__ cov, const int32_t* __restrict__ dropped,
+                             Level N)
+{
+    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < S.V;
+         n += (int64_t)gridDim.x * blockDim.x) {
+        int32_t m = match[n];
+        if (m >= 0 && m < (int32_t)n) continue;
+        int32_t u = map[n];
+        int32_t sz = S.vsize[n], ip = S.vinpins[n], ii = S.vinint[n], ic = S.vincnt[n];
+        if (m >= 0) {
+            sz += S.vsize[m];
+            ip += S.vinpins[m];
+            ii += S.vinint[m];
+            ic += S.vincnt[m] - (cand[n] == m ? cov[n] : cov[m]);
+        }
+        N.vsize[u] = sz;
+        N.vinpins[u] = ip;
+        N.vinint[u] = ii + dropped[u];
+        N.vincnt[u] = ic;
     }
 }
 
@@ -80,26 +116,6 @@ __global__ void k_in_count(Level N)
     }
 }
 
-// in_count of the next level straight from a matching: an unmatched vertex
-// keeps its count; a pair's super-node has in_count(n) + in_count(m) -
-// shared(n, m), the shared count being the candidate overlap of the member
-// whose candidate is the other (pairs are matched along candidate arcs)
-__global__ void k_in_count_pairs(Level S, const int32_t* __restrict__ map,
-                                 const int32_t* __restrict__ match, const int32_t* __restrict__ cand,
-                                 const int32_t* __restrict__ cov, int32_t* incnt_next)
-{
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < S.V;
-         n += (int64_t)gridDim.x * blockDim.x) {
-        int32_t m = match[n];
-        if (m < 0) {
-            incnt_next[map[n]] = S.vincnt[n];
-        } else if ((int32_t)n < m) {
-            int32_t ov = cand[n] == m ? cov[n] : cov[m];
-            incnt_next[map[n]] = S.vincnt[n] + S.vincnt[m] - ov;
-        }
-    }
-}
-
 __global__ void k_compose(int64_t n, int32_t* c, const int32_t* __restrict__ next)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -118,10 +134,14 @@ struct ContractJob {
     int32_t* tpins;
     int32_t* tlen;
     uint8_t* tsd;
-    uint32_t* thash;
+    uint64_t* thash;         // content hash (destinations, selfdst)
     int32_t* inint_next;     // may be null (nothing recorded for dropped hyperedges)
     bool discard_self = false;   // G_P: a destination in the source's part is discarded
                                  // without marking selfdst
+    static __device__ uint64_t content_hash(uint64_t hsum, int sd, int cnt)
+    {
+        return hsum + mix64(0x5bd1e995ull + (uint64_t)sd) + mix64((uint64_t)cnt << 1);
+    }
     __device__ int len(int32_t a) const { return (int)(hoff[a + 1] - hoff[a] - 1); }
     __device__ uint32_t load(int32_t a, int i) const
     {
@@ -160,8 +180,7 @@ struct ContractJob {
             } else {
                 tlen[a] = 1 + cnt;
                 tsd[a] = (uint8_t)sd;
-                uint64_t hh = hsum + mix64(0x5bd1e995ull + (uint64_t)sd) + mix64((uint64_t)cnt << 1);
-                thash[a] = (uint32_t)(hh ^ (hh >> 32));
+                thash[a] = content_hash(hsum, sd, cnt);
             }
         }
     }
@@ -188,21 +207,21 @@ struct ContractJob {
         } else {
             tlen[a] = 1 + cnt;
             tsd[a] = (uint8_t)sd;
-            uint64_t hh = hsum + mix64(0x5bd1e995ull + (uint64_t)sd) + mix64((uint64_t)cnt << 1);
-            thash[a] = (uint32_t)(hh ^ (hh >> 32));
+            thash[a] = content_hash(hsum, sd, cnt);
         }
     }
 };
 
 __global__ void k_dedup_keys(int32_t E, const int32_t* __restrict__ tlen,
                              const int64_t* __restrict__ hoff, const int32_t* __restrict__ tpins,
-                             const uint32_t* __restrict__ thash, uint64_t dropped_hi,
+                             const uint64_t* __restrict__ thash, uint64_t dropped_hi,
                              uint64_t* keys, uint32_t* vals)
 {
     for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < E;
          a += (int64_t)gridDim.x * blockDim.x) {
         uint64_t hi = tlen[a] > 0 ? (uint64_t)(uint32_t)tpins[hoff[a]] : dropped_hi;
-        keys[a] = (hi << 32) | (tlen[a] > 0 ? thash[a] : 0u);
+        uint64_t hh = thash[a];
+        keys[a] = (hi << 32) | (tlen[a] > 0 ? (uint32_t)(hh ^ (hh >> 32)) : 0u);
         vals[a] = (uint32_t)a;
     }
 }
@@ -225,6 +244,113 @@ __device__ __forceinline__ bool same_content(int32_t a, int32_t b, const int64_t
         if (pa[i] != pb[i]) return false;
     return true;
 }
+
+// ---------------------------------------------------------------------------
+// Duplicate hyperedges of a contracted level, by a hash table of at least
+// twice as many slots as hyperedges: key = the 64-bit hash of (source,
+// content), low = complement of the lowest id under it (so a cleared table
+// is all zeros). A stable radix sort of (source, 32-bit hash) stood here
+// before; its six passes over keys and values were most of a tail level's
+// contraction (conv network of 65,536 neurons: 57,344 hyperedges a level,
+// 0.18 of 0.50 ms a level) and the order it gave is not part of a level.
+
+constexpr int32_t REP_NONE = -1;      // dropped
+constexpr int32_t REP_PENDING = -2;   // another content under the same hash
+
+struct DedupTable {
+    unsigned long long* key;
+    uint32_t* low;
+    uint32_t* slot;    // per hyperedge
+    int32_t* rep;      // per hyperedge: representative, REP_NONE or REP_PENDING
+    uint32_t mask;
+};
+
+// round 0: every remaining hyperedge (tw/tk start as its own omega and k);
+// later rounds: the pending ones
+__global__ void k_dedup_insert(int32_t E, const int32_t* __restrict__ tlen,
+                               const int64_t* __restrict__ hoff, const int32_t* __restrict__ tpins,
+                               const uint64_t* __restrict__ thash, const int64_t* __restrict__ hw,
+                               const int32_t* __restrict__ hk, int64_t* tw, int32_t* tk,
+                               DedupTable t, int round)
+{
+    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < E;
+         a += (int64_t)gridDim.x * blockDim.x) {
+        if (round > 0 && t.rep[a] != REP_PENDING) continue;
+        if (tlen[a] == 0) continue;
+        if (round == 0) {
+            tw[a] = hw[a];
+            tk[a] = hk[a];
+        }
+        // the source under a salt: it must not look like one more destination
+        unsigned long long h = mix64(thash[a] + mix64((1ull << 40) + (uint32_t)tpins[hoff[a]]));
+        if (h == 0) h = 1;
+        uint32_t sl = (uint32_t)(h >> 32) & t.mask;
+        for (;;) {   // at most half the slots are ever taken
+            unsigned long long prev = atomicCAS(&t.key[sl], 0ull, h);
+            if (prev == 0 || prev == h) break;
+            sl = (sl + 1) & t.mask;
+        }
+        atomicMax(&t.low[sl], ~(uint32_t)a);
+        t.slot[a] = sl;
+    }
+}
+
+// Representatives; merged hyperedges add their omega and k to theirs. The
+// level's size buckets and pair terms are counted here, so that they reach
+// the host together with its sizes.
+__global__ void __launch_bounds__(256)
+    k_dedup_resolve(int32_t E, const int32_t* __restrict__ tlen, const int64_t* __restrict__ hoff,
+                    const int32_t* __restrict__ tpins, const uint8_t* __restrict__ tsd,
+                    const int64_t* __restrict__ hw, const int32_t* __restrict__ hk, int64_t* tw,
+                    int32_t* tk, DedupTable t, int round, int64_t* scal)
+{
+    SegTally tally;
+    int pending = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < E;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        int32_t a = (int32_t)i;
+        if (tlen[a] == 0) {
+            t.rep[a] = REP_NONE;
+            continue;
+        }
+        if (round > 0 && t.rep[a] != REP_PENDING) continue;
+        int32_t r = (int32_t)~t.low[t.slot[a]];
+        if (r == a) {
+            t.rep[a] = a;
+            tally.add(tlen[a]);
+        } else if (tpins[hoff[r]] == tpins[hoff[a]] && same_content(r, a, hoff, tpins, tlen, tsd)) {
+            t.rep[a] = r;
+            atomicAdd((unsigned long long*)&tw[r], (unsigned long long)hw[a]);
+            atomicAdd(&tk[r], hk[a]);
+        } else {
+            t.rep[a] = REP_PENDING;
+            pending++;
+        }
+    }
+    tally.flush(scal + SC_SEG, scal + SC_W2);
+    pending = warp_sum(pending);
+    if ((threadIdx.x & 31) == 0 && pending)
+        atomicAdd((unsigned long long*)&scal[SC_D], (unsigned long long)pending);
+}
+
+// (representatives, their pins) before each hyperedge
+struct RepSizes {
+    const int32_t *rep, *tlen;
+    __device__ Sum2 operator()(int64_t a) const
+    {
+        bool r = rep[a] == (int32_t)a;
+        return Sum2(r ? 1 : 0, r ? tlen[a] : 0);
+    }
+};
+struct RepPlaces {
+    int32_t* gid;
+    int64_t* off;
+    __device__ void operator()(int64_t a, Sum2 ex, Sum2) const
+    {
+        gid[a] = (int32_t)ex.a;
+        off[a] = ex.b;
+    }
+};
 
 // rep[i] = first position j of i's run (equal keys) whose content equals i's
 __global__ void k_dedup_rep(int32_t E, const uint64_t* __restrict__ keys,
@@ -298,92 +424,106 @@ __global__ void k_dedup_emit(int32_t E, const uint32_t* __restrict__ vals,
     }
 }
 
+// the same from representatives in id order
+template <int G>
+__global__ void k_level_emit(int32_t E, const int32_t* __restrict__ rep,
+                             const int32_t* __restrict__ gid, const int64_t* __restrict__ hoff,
+                             const int32_t* __restrict__ tpins, const int32_t* __restrict__ tlen,
+                             const uint8_t* __restrict__ tsd, const int64_t* __restrict__ tw,
+                             const int32_t* __restrict__ tk, const int64_t* __restrict__ newoff,
+                             Level N)
+{
+    int lane = threadIdx.x & (G - 1);
+    int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
+    int64_t nw = ((int64_t)gridDim.x * blockDim.x) / G;
+    if (gw == 0 && lane == 0) N.hoff[N.E] = N.P;
+    for (int64_t a = gw; a < E; a += nw) {
+        if (rep[a] != (int32_t)a) continue;
+        int32_t g = gid[a];
+        int64_t dst = newoff[a], src = hoff[a];
+        int32_t len = tlen[a];
+        for (int32_t j = lane; j < len; j += G) N.hpins[dst + j] = tpins[src + j];
+        if (lane == 0) {
+            N.hoff[g] = dst;
+            N.hsd[g] = tsd[a];
+            N.hw[g] = tw[a];
+            N.hk[g] = tk[a];
+        }
+    }
+}
+
 __global__ void k_set_off_end(int64_t* hoff, int32_t E, int64_t P) { hoff[E] = P; }
 
 // Materializes levels[dst] from the resident levels[src] through `map`
-// (int32[V(src)] into the new level's ids); *d_V2 (device) is its vertex
-// count. If levels[dst] already records sizes (a released level being
-// rebuilt), the rebuilt sizes must match them.
-Status build_coarse(snnmap_hgraph* h, int32_t src, const int32_t* map, const int64_t* d_V2,
-                    int32_t dst, const int32_t* match, const int32_t* cand, const int32_t* cov)
+// (int32[V(src)] into the new level's ids). The new level's vertex count is
+// V2, or the scalar SC_A when V2 < 0. If levels[dst] already records sizes (a
+// released level being rebuilt), the rebuilt sizes must match them.
+Status build_coarse(snnmap_hgraph* h, int32_t src, const int32_t* map, int32_t V2, int32_t dst,
+                    const int32_t* match, const int32_t* cand, const int32_t* cov)
 {
     cudaStream_t s = h->stream;
     Arena& ar = h->scratch;
     Level& L = h->levels[src];
     LevelExtra& X = h->extra[src];
     int32_t V = L.V, E = L.E;
-    SNN_TRY(zero_scalars(h));
     std::unique_ptr<ProfScope> prof(new ProfScope(h, PS_CONTRACT));
-    NextState ns;
-    SNN_TRY(ar.alloc(&ns.size, V));
-    SNN_TRY(ar.alloc(&ns.inpins, V));
-    SNN_TRY(ar.alloc(&ns.inint, V));
-    if (V > 0) {
-        SNN_CUDA(cudaMemsetAsync(ns.size, 0, (size_t)V * 4, s));
-        SNN_CUDA(cudaMemsetAsync(ns.inpins, 0, (size_t)V * 4, s));
-        SNN_CUDA(cudaMemsetAsync(ns.inint, 0, (size_t)V * 4, s));
-        SNN_L k_sum_state<<<grid_for(V, 256), 256, 0, s>>>(L, map, ns);
-        SNN_CUDA(cudaGetLastError());
-    }
-    SNN_CUDA(cudaMemcpyAsync(h->d_scal + SC_A, d_V2, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+
+    // everything that starts cleared, in one run of memory
+    DedupTable dt;
+    int64_t cap = 64;
+    while (cap < 2 * (int64_t)E) cap <<= 1;
+    dt.mask = (uint32_t)(cap - 1);
+    int32_t *dropped, *cursor;
+    Carver zc;
+    zc.add(&dt.key, cap);
+    zc.add(&dt.low, cap);
+    zc.add(&dropped, V);
+    zc.add(&cursor, SEG_NB);
+    char* zbase;
+    SNN_TRY(ar.alloc(&zbase, (int64_t)zc.total));
+    zc.assign(zbase);
+    SNN_CUDA(cudaMemsetAsync(zbase, 0, zc.total, s));
 
     // per-hyperedge remap, sort, unique
-    int32_t *tpins, *tlen;
+    int32_t *tpins, *tlen, *gid, *tk;
     uint8_t* tsd;
-    uint32_t* thash;
+    uint64_t* thash;
+    int64_t *tw, *newoff;
     SNN_TRY(ar.alloc(&tpins, L.P));
     SNN_TRY(ar.alloc(&tlen, E));
     SNN_TRY(ar.alloc(&tsd, E));
     SNN_TRY(ar.alloc(&thash, E));
-    ContractJob job{L.hoff, L.hpins, L.hsd, L.hk, map, tpins, tlen, tsd, thash, ns.inint};
+    SNN_TRY(ar.alloc(&dt.slot, E));
+    SNN_TRY(ar.alloc(&dt.rep, E));
+    SNN_TRY(ar.alloc(&gid, E));
+    SNN_TRY(ar.alloc(&newoff, E));
+    SNN_TRY(ar.alloc(&tk, E));
+    SNN_TRY(ar.alloc(&tw, E));
+    ContractJob job{L.hoff, L.hpins, L.hsd, L.hk, map, tpins, tlen, tsd, thash, dropped};
     SNN_TRY(seg_run(job, X.seg, E, ar, s));
 
     // duplicate hyperedges
-    uint64_t *keys, *keys2;
-    uint32_t *vals, *vals2;
-    int32_t *headpos, *runstart, *rep, *head, *gidh, *gid, *tk;
-    int64_t *tw, *newlen, *newoff;
-    SNN_TRY(ar.alloc(&keys, E));
-    SNN_TRY(ar.alloc(&keys2, E));
-    SNN_TRY(ar.alloc(&vals, E));
-    SNN_TRY(ar.alloc(&vals2, E));
-    SNN_TRY(ar.alloc(&headpos, E));
-    SNN_TRY(ar.alloc(&runstart, E));
-    SNN_TRY(ar.alloc(&rep, E));
-    SNN_TRY(ar.alloc(&head, E));
-    SNN_TRY(ar.alloc(&gidh, E));
-    SNN_TRY(ar.alloc(&gid, E));
-    SNN_TRY(ar.alloc(&tk, E));
-    SNN_TRY(ar.alloc(&tw, E));
-    SNN_TRY(ar.alloc(&newlen, E));
-    SNN_TRY(ar.alloc(&newoff, E));
     int ge = grid_for(E, 256);
-    int hibits = bits_for((uint64_t)V);
-    if (E > 0) {
-        SNN_L k_dedup_keys<<<ge, 256, 0, s>>>(E, tlen, L.hoff, tpins, thash, (uint64_t)V, keys, vals);
-        SNN_CUDA(cudaGetLastError());
-        SNN_TRY(radix_sort_pairs(keys, vals, keys2, vals2, E, 32 + hibits, ar, s));
-        SNN_L k_run_heads<<<ge, 256, 0, s>>>(E, keys, headpos);
-        SNN_CUDA(cudaGetLastError());
+    for (int round = 0;; round++) {
+        if (E > 0) {
+            SNN_L k_dedup_insert<<<ge, 256, 0, s>>>(E, tlen, L.hoff, tpins, thash, L.hw, L.hk, tw, tk,
+                                                    dt, round);
+            SNN_L k_dedup_resolve<<<grid_for(E, 256, 152 * 8), 256, 0, s>>>(E, tlen, L.hoff, tpins, tsd, L.hw, L.hk, tw, tk, dt,
+                                                     round, h->d_scal);
+            SNN_CUDA(cudaGetLastError());
+        }
+        SNN_TRY(scan_run<Sum2>(RepSizes{dt.rep, tlen}, RepPlaces{gid, newoff}, E,
+                               (Sum2*)(h->d_scal + SC_B), ar, s));
+        prof.reset();
+        SNN_TRY(read_scalars(h));
+        // a pending class loses at least its representative every round
+        if (h->h_scal[SC_D] == 0) break;
+        SNN_CUDA(cudaMemsetAsync(h->d_scal + SC_D, 0, sizeof(int64_t), s));
+        SNN_CUDA(cudaMemsetAsync(dt.key, 0, (size_t)cap * sizeof(*dt.key), s));
+        SNN_CUDA(cudaMemsetAsync(dt.low, 0, (size_t)cap * sizeof(*dt.low), s));
     }
-    SNN_TRY(scan_inclusive_max_i32(headpos, runstart, E, ar, s));
-    if (E > 0) {
-        SNN_L k_dedup_rep<<<ge, 256, 0, s>>>(E, keys, vals, runstart, L.hoff, tpins, tlen, tsd, rep, head);
-        SNN_CUDA(cudaGetLastError());
-    }
-    SNN_TRY(scan_exclusive_i32(head, gidh, E, (int32_t*)(h->d_scal + SC_B), ar, s));
-    if (E > 0) {
-        SNN_CUDA(cudaMemsetAsync(tw, 0, (size_t)E * sizeof(int64_t), s));
-        SNN_CUDA(cudaMemsetAsync(tk, 0, (size_t)E * sizeof(int32_t), s));
-        SNN_CUDA(cudaMemsetAsync(newlen, 0, (size_t)E * sizeof(int64_t), s));
-        SNN_L k_dedup_accum<<<ge, 256, 0, s>>>(E, vals, rep, gidh, tlen, L.hw, L.hk, tw, tk, newlen, gid);
-        SNN_CUDA(cudaGetLastError());
-    }
-    SNN_TRY(scan_exclusive_i64(newlen, newoff, E, h->d_scal + SC_C, ar, s));
-    prof.reset();
-    SNN_TRY(read_scalars(h));
-    int32_t V2 = (int32_t)h->h_scal[SC_A];
-    int32_t E2 = (int32_t)(h->h_scal[SC_B] & 0xffffffff);
+    if (V2 < 0) V2 = (int32_t)h->h_scal[SC_A];
+    int32_t E2 = (int32_t)h->h_scal[SC_B];
     int64_t P2 = h->h_scal[SC_C];
 
     Level& N = h->levels[dst];
@@ -394,35 +534,31 @@ Status build_coarse(snnmap_hgraph* h, int32_t src, const int32_t* map, const int
     }
     SNN_TRY(level_alloc(h, N, NX, V2, E2, P2));
     N.maxlen = L.maxlen;
+    NX.pair_terms = h->h_scal[SC_W2];
+    for (int i = 0; i < SEG_NB; i++) NX.seg.n[i] = (int32_t)h->h_scal[SC_SEG + i];
     prof.reset(new ProfScope(h, PS_CONTRACT));
-    if (V2 > 0) {
-        SNN_CUDA(cudaMemcpyAsync(N.vsize, ns.size, (size_t)V2 * 4, cudaMemcpyDeviceToDevice, s));
-        SNN_CUDA(cudaMemcpyAsync(N.vinpins, ns.inpins, (size_t)V2 * 4, cudaMemcpyDeviceToDevice, s));
-        SNN_CUDA(cudaMemcpyAsync(N.vinint, ns.inint, (size_t)V2 * 4, cudaMemcpyDeviceToDevice, s));
-        if (!match)
-            SNN_CUDA(cudaMemcpyAsync(N.vincnt, ns.inint, (size_t)V2 * 4, cudaMemcpyDeviceToDevice, s));
-    }
     if (match && V > 0) {
-        SNN_L k_in_count_pairs<<<grid_for(V, 256), 256, 0, s>>>(L, map, match, cand, cov, N.vincnt);
+        SNN_L k_next_state<<<grid_for(V, 256), 256, 0, s>>>(L, map, match, cand, cov, dropped, N);
         SNN_CUDA(cudaGetLastError());
-    }
-    if (E > 0) {
-        SNN_HEDGE_LAUNCH(hedge_lanes(L.P, L.E), k_dedup_emit, E, s, E, vals, rep, gid, L.hoff, tpins,
-                         tlen, tsd, tw, tk, newoff, N);
+    } else if (V2 > 0) {
+        SNN_CUDA(cudaMemsetAsync(N.vsize, 0, (size_t)V2 * 4, s));
+        SNN_CUDA(cudaMemsetAsync(N.vinpins, 0, (size_t)V2 * 4, s));
+        SNN_CUDA(cudaMemcpyAsync(N.vinint, dropped, (size_t)V2 * 4, cudaMemcpyDeviceToDevice, s));
+        SNN_L k_sum_state<<<grid_for(V, 256), 256, 0, s>>>(L, map, NextState{N.vsize, N.vinpins, N.vinint});
         SNN_CUDA(cudaGetLastError());
+        SNN_CUDA(cudaMemcpyAsync(N.vincnt, N.vinint, (size_t)V2 * 4, cudaMemcpyDeviceToDevice, s));
     }
-    SNN_L k_set_off_end<<<1, 1, 0, s>>>(N.hoff, E2, P2);
+    // at least one group runs, which closes the offsets
+    SNN_HEDGE_LAUNCH(hedge_lanes(L.P, L.E), k_level_emit, E, s, E, dt.rep, gid, L.hoff, tpins, tlen, tsd,
+                     tw, tk, newoff, N);
     SNN_CUDA(cudaGetLastError());
     if (E2 > 0 && !match) {
         SNN_L k_in_count<<<grid_for((int64_t)E2 * 32, 256), 256, 0, s>>>(N);
         SNN_CUDA(cudaGetLastError());
     }
+    SNN_TRY(seg_lists(N.hoff, E2, N.maxlen, NX.seg, cursor, s));
     prof.reset();
     SNN_TRY(build_incidence(h, N));
-    SNN_CUDA(cudaMemsetAsync(h->d_scal + SC_W2, 0, sizeof(int64_t), s));
-    SNN_TRY(seg_classify(N.hoff, E2, N.maxlen, NX.seg, ar, s, h->d_scal + SC_W2));
-    SNN_TRY(read_scalars(h));
-    NX.pair_terms = h->h_scal[SC_W2];
     ar.reset();
     return Status{};
 }
@@ -435,23 +571,19 @@ Status contract_level(snnmap_hgraph* h)
     int32_t src = (int32_t)h->levels.size() - 1;
     Level& L = h->levels[src];
     int32_t V = L.V;
-    int32_t *isrep, *repidx;
-    int64_t* d_V2;
-    SNN_TRY(ar.alloc(&isrep, V));
+    int32_t* repidx;
     SNN_TRY(ar.alloc(&repidx, V));
-    SNN_TRY(ar.alloc(&d_V2, 1));
-    SNN_CUDA(cudaMemsetAsync(d_V2, 0, sizeof(int64_t), s));
+    SNN_TRY(zero_scalars(h));
     {
         ProfScope prof(h, PS_CONTRACT);
-        SNN_L k_rep_flags<<<grid_for(V, 256), 256, 0, s>>>(V, h->match, isrep);
-        SNN_CUDA(cudaGetLastError());
-        SNN_TRY(scan_exclusive_i32(isrep, repidx, V, (int32_t*)d_V2, ar, s));
+        SNN_TRY(scan_run<int32_t>(RepFlag{h->match}, ScanStore<int32_t, false>{repidx}, V,
+                                  (int32_t*)(h->d_scal + SC_A), ar, s));
         SNN_L k_cid_map<<<grid_for(V, 256), 256, 0, s>>>(V, h->match, repidx, L.cid);
         SNN_CUDA(cudaGetLastError());
     }
     h->levels.emplace_back();
     h->extra.emplace_back();
-    SNN_TRY(build_coarse(h, src, h->levels[src].cid, d_V2, src + 1, h->match, h->cand, h->cov));
+    SNN_TRY(build_coarse(h, src, h->levels[src].cid, -1, src + 1, h->match, h->cand, h->cov));
     h->have_matching = false;
     ProfScope prof(h, PS_AFFINITY);
     if (h->mat.level == src) SNN_TRY(mat_descend(h, src));
@@ -498,7 +630,7 @@ Status emit_gp(snnmap_hgraph* h, int32_t K, const int32_t* rho)
     SNN_TRY(zero_scalars(h));
     int32_t *tpins, *tlen;
     uint8_t* tsd;
-    uint32_t* thash;
+    uint64_t* thash;
     SNN_TRY(ar.alloc(&tpins, L.P));
     SNN_TRY(ar.alloc(&tlen, E));
     SNN_TRY(ar.alloc(&tsd, E));
@@ -609,19 +741,15 @@ Status ensure_resident(snnmap_hgraph* h, int32_t l)
     Arena& ar = h->scratch;
     const Level& S = h->levels[j];
     int32_t* c;
-    int64_t* d_V2;
     SNN_TRY(ar.alloc(&c, S.V));
-    SNN_TRY(ar.alloc(&d_V2, 1));
     if (S.V > 0)
         SNN_CUDA(cudaMemcpyAsync(c, S.cid, (size_t)S.V * 4, cudaMemcpyDeviceToDevice, s));
     for (int32_t m = j + 1; m < l; m++) {
         SNN_L k_compose<<<grid_for(S.V, 256), 256, 0, s>>>(S.V, c, h->levels[m].cid);
         SNN_CUDA(cudaGetLastError());
     }
-    int64_t v2 = h->levels[l].V;
-    SNN_CUDA(cudaMemcpyAsync(d_V2, &v2, sizeof(int64_t), cudaMemcpyHostToDevice, s));
-    SNN_CUDA(cudaStreamSynchronize(s));
-    return build_coarse(h, j, c, d_V2, l);
+    SNN_TRY(zero_scalars(h));
+    return build_coarse(h, j, c, h->levels[l].V, l);
 }
 
 }  // namespace snn

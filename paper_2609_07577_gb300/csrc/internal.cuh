@@ -13,7 +13,8 @@ namespace snn {
 enum Scalar : int {
     SC_STATUS = 0,   // int32 status bits live in the low word of this slot
     SC_A, SC_B, SC_C, SC_D, SC_E, SC_F, SC_G,
-    SC_W2 = 9,       // pair terms of the level being classified
+    SC_W2 = 9,       // pair terms of the level being built
+    SC_SEG = 10,     // and its hyperedges per size bucket (SEG_NB slots)
     SC_COUNT = 16,
 };
 
@@ -224,11 +225,12 @@ Status contract_level(snnmap_hgraph* h);
 // after a contraction of `src`: candidates of src carried to src + 1
 Status aff_carry(snnmap_hgraph* h, int32_t src);
 void aff_carry_free(snnmap_hgraph* h);
-// materializes levels[dst] from resident levels[src] through map (V(src) ids);
+// materializes levels[dst] (V2 vertices; V2 < 0: the scalar SC_A holds their
+// number) from resident levels[src] through map (V(src) ids), scalars cleared;
 // with the matching that produced map (match, and the candidates and their
 // overlaps), in_count comes from the pairs instead of a pass over the pins
-Status build_coarse(snnmap_hgraph* h, int32_t src, const int32_t* map, const int64_t* d_V2,
-                    int32_t dst, const int32_t* match = nullptr, const int32_t* cand = nullptr,
+Status build_coarse(snnmap_hgraph* h, int32_t src, const int32_t* map, int32_t V2, int32_t dst,
+                    const int32_t* match = nullptr, const int32_t* cand = nullptr,
                     const int32_t* cov = nullptr);
 // rebuilds a released level from the nearest resident level below it
 Status ensure_resident(snnmap_hgraph* h, int32_t level);

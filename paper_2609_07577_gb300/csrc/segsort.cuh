@@ -1,9 +1,9 @@
 // Segmented sort of small uint32 key lists, one list per hyperedge, followed
 // by a per-hyperedge epilogue. Hyperedges are split into size buckets once
 // per level (by pin count L):
-//   T:  L <= 16      one thread, keys in a local array (insertion sort)
+//   T:  L <= 16      one thread, keys in registers
 //   B0: L <= 32      one warp, keys in registers (shuffle bitonic network)
-//   B1: L <= 256     one warp, keys in a per-warp shared-memory slice
+//   B1: L <= 256     one warp, 2, 4 or 8 keys a lane in registers
 //   B2: L <= 16384   one block of 512 threads, keys in dynamic shared memory
 //   B3: larger       one block of 1024 threads, keys in a global scratch slice
 // Each kernel walks its bucket's list with a grid-stride loop whose bound is
@@ -34,10 +34,14 @@ constexpr uint32_t KEY_PAD = 0xffffffffu;
 // Per-level bucket lists of hyperedge ids: one array of E ids holding the
 // buckets (T, B0, B1, B2, B3) back to back; meta (device int32[10]) =
 // start[5], count[5].
+// n: the counts on the host, or -1 while they are not known there; a filtered
+// copy of the lists keeps its level's counts as upper bounds (seg_run sizes
+// its launches by them and leaves out empty buckets).
 struct SegBuckets {
     int32_t* list = nullptr;
     int32_t* meta = nullptr;
     int64_t b3_cap = 0;        // power of two >= longest hyperedge if any is in B3
+    int32_t n[5] = {-1, -1, -1, -1, -1};
 };
 
 __device__ __forceinline__ uint32_t warp_bitonic32(uint32_t v)
@@ -64,28 +68,6 @@ __device__ __forceinline__ int pow2_at_least(int n, int lo)
     return p;
 }
 
-// bitonic sort of s[0..N) (N a power of two) by one warp
-__device__ __forceinline__ void warp_bitonic_smem(uint32_t* s, int N)
-{
-    int lane = threadIdx.x & 31;
-    for (int k = 2; k <= N; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = lane; i < N; i += 32) {
-                int ixj = i ^ j;
-                if (ixj > i) {
-                    uint32_t a = s[i], b = s[ixj];
-                    bool asc = (i & k) == 0;
-                    if ((a > b) == asc) {
-                        s[i] = b;
-                        s[ixj] = a;
-                    }
-                }
-            }
-            __syncwarp();
-        }
-    }
-}
-
 // bitonic sort of s[0..N) by the whole block (s in shared or global memory)
 __device__ __forceinline__ void block_bitonic(uint32_t* s, int N)
 {
@@ -109,18 +91,65 @@ __device__ __forceinline__ void block_bitonic(uint32_t* s, int N)
 
 enum : int { SEG_BT = 0, SEG_BB0 = 1, SEG_BB1 = 2, SEG_BB2 = 3, SEG_BB3 = 4, SEG_NB = 5 };
 
-// One thread per list of at most SEG_T_CAP keys: the keys are sorted in
+// Ascending sort of the 32 R keys a warp holds in registers, key r of lane l
+// at position l R + r: a bitonic network whose strides below R stay inside a
+// lane and whose longer strides are one shuffle per key.
+template <int R>
+__device__ __forceinline__ void warp_bitonic_regs(uint32_t (&k)[R])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int w = 2; w <= 32 * R; w <<= 1) {
+#pragma unroll
+        for (int j = w >> 1; j > 0; j >>= 1) {
+            if (j >= R) {
+                const bool lower = (lane & (j / R)) == 0;
+#pragma unroll
+                for (int r = 0; r < R; r++) {
+                    uint32_t o = __shfl_xor_sync(FULL, k[r], j / R);
+                    bool up = ((lane * R + r) & w) == 0;
+                    k[r] = (lower == up) ? min(k[r], o) : max(k[r], o);
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; r++) {
+                    if ((r & j) != 0) continue;
+                    bool up = ((lane * R + r) & w) == 0;
+                    uint32_t x = k[r], y = k[r | j];
+                    k[r] = up ? min(x, y) : max(x, y);
+                    k[r | j] = up ? max(x, y) : min(x, y);
+                }
+            }
+        }
+    }
+}
+
+// keys of hyperedge a (L <= 32 R) sorted into s by one warp
+template <int R, class Job>
+__device__ __forceinline__ void warp_sort_list(const Job& job, int32_t a, int L, uint32_t* s)
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t k[R];
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+        int i = r * 32 + lane;
+        k[r] = i < L ? job.load(a, i) : KEY_PAD;
+    }
+    warp_bitonic_regs<R>(k);
+#pragma unroll
+    for (int r = 0; r < R; r++) s[lane * R + r] = k[r];
+    __syncwarp();
+}
+
+// T: one thread per list of at most SEG_T_CAP keys: the keys are sorted in
 // registers by a fully unrolled bitonic network (padding sorts last) and
 // handed to the epilogue through shared memory, slot i of thread t at
 // i * blockDim + t so that a warp's lanes touch consecutive banks.
 template <class Job>
-__global__ void __launch_bounds__(256) k_seg_t(Job job, const int32_t* __restrict__ lists,
-                                               const int32_t* __restrict__ meta)
+__device__ __forceinline__ void seg_thread_lists(const Job& job, const int32_t* __restrict__ list,
+                                                 int n, int block, int nblocks, uint32_t* sk)
 {
-    __shared__ uint32_t sk[SEG_T_CAP * 256];
-    const int32_t* list = lists + meta[SEG_BT];
-    int n = meta[SEG_NB + SEG_BT];
-    for (int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
+    for (int base = block * 256; base < n; base += nblocks * 256) {
         int idx = base + threadIdx.x;
         if (idx >= n) continue;
         int32_t a = list[idx];
@@ -152,44 +181,50 @@ __global__ void __launch_bounds__(256) k_seg_t(Job job, const int32_t* __restric
     }
 }
 
+// The three small buckets in one launch: blocks [0, gt) take T, the next gb0
+// blocks B0 and the rest B1, so a level pays one launch and one tail for
+// them (three launches of mostly few blocks before).
+//
+// B0 and B1 sort in registers. B1 held its keys in shared memory, one
+// compare-exchange a load pair, a store pair and a warp barrier: the
+// partition hypergraph of the 1,048,576-neuron conv network (917,504 lists
+// of 77 keys) took 2.14 ms there; see the measured figure at seg_run.
 template <class Job>
-__global__ void __launch_bounds__(256) k_seg_b0(Job job, const int32_t* __restrict__ lists,
-                                                const int32_t* __restrict__ meta)
+__global__ void __launch_bounds__(256) k_seg_small(Job job, const int32_t* __restrict__ lists,
+                                                   const int32_t* __restrict__ meta, int gt, int gb0)
 {
-    __shared__ uint32_t buf[8][32];
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int32_t* list = lists + meta[SEG_BB0];
-    int n = meta[SEG_NB + SEG_BB0];
-    for (int idx = blockIdx.x * 8 + warp; idx < n; idx += gridDim.x * 8) {
-        int32_t a = list[idx];
-        int L = job.len(a);
-        uint32_t v = lane < L ? job.load(a, lane) : KEY_PAD;
-        v = warp_bitonic32(v);
-        buf[warp][lane] = v;
-        __syncwarp();
-        job.finish(a, buf[warp], L);
-        __syncwarp();
-    }
-}
-
-template <class Job>
-__global__ void __launch_bounds__(256) k_seg_b1(Job job, const int32_t* __restrict__ lists,
-                                                const int32_t* __restrict__ meta)
-{
-    __shared__ uint32_t buf[8][SEG_B1_CAP];
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int32_t* list = lists + meta[SEG_BB1];
-    int n = meta[SEG_NB + SEG_BB1];
-    uint32_t* s = buf[warp];
-    for (int idx = blockIdx.x * 8 + warp; idx < n; idx += gridDim.x * 8) {
-        int32_t a = list[idx];
-        int L = job.len(a);
-        int N = pow2_at_least(L, 32);
-        for (int i = lane; i < N; i += 32) s[i] = i < L ? job.load(a, i) : KEY_PAD;
-        __syncwarp();
-        warp_bitonic_smem(s, N);
-        job.finish(a, s, L);
-        __syncwarp();
+    __shared__ __align__(16) uint32_t buf[SEG_T_CAP * 256];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int blk = blockIdx.x;
+    if (blk < gt) {
+        seg_thread_lists(job, lists + meta[SEG_BT], meta[SEG_NB + SEG_BT], blk, gt, buf);
+    } else if (blk < gt + gb0) {
+        const int32_t* list = lists + meta[SEG_BB0];
+        int n = meta[SEG_NB + SEG_BB0];
+        uint32_t* s = buf + warp * 32;
+        for (int idx = (blk - gt) * 8 + warp; idx < n; idx += gb0 * 8) {
+            int32_t a = list[idx];
+            int L = job.len(a);
+            uint32_t v = lane < L ? job.load(a, lane) : KEY_PAD;
+            s[lane] = warp_bitonic32(v);
+            __syncwarp();
+            job.finish(a, s, L);
+            __syncwarp();
+        }
+    } else {
+        const int32_t* list = lists + meta[SEG_BB1];
+        int n = meta[SEG_NB + SEG_BB1];
+        const int g = gridDim.x - gt - gb0;
+        uint32_t* s = buf + warp * SEG_B1_CAP;
+        for (int idx = (blk - gt - gb0) * 8 + warp; idx < n; idx += g * 8) {
+            int32_t a = list[idx];
+            int L = job.len(a);
+            if (L <= 64) warp_sort_list<2>(job, a, L, s);
+            else if (L <= 128) warp_sort_list<4>(job, a, L, s);
+            else warp_sort_list<8>(job, a, L, s);
+            job.finish(a, s, L);
+            __syncwarp();
+        }
     }
 }
 
@@ -215,35 +250,75 @@ __global__ void k_seg_big(Job job, const int32_t* __restrict__ lists,
     }
 }
 
-// Builds the bucket lists of a level (device-only; list holds E ids, meta 8
-// ints, both caller-allocated).
-// Also adds sum |e|(|e|-1) over the level's hyperedges to *w2 (device).
-Status seg_classify(const int64_t* hoff, int32_t E, int32_t maxlen, SegBuckets& b, Arena& ar,
-                    cudaStream_t s, int64_t* w2);
+__device__ __forceinline__ int seg_bucket(int64_t len)
+{
+    return len <= SEG_T_CAP ? SEG_BT
+         : len <= 32 ? SEG_BB0 : (len <= SEG_B1_CAP ? SEG_BB1 : (len <= SEG_B2_CAP ? SEG_BB2 : SEG_BB3));
+}
 
-// Grid sizes for the four bucket kernels.
-inline int seg_grid_small(int32_t E) { return grid_for((int64_t)E * 32, 256, 152 * 16); }
+// Per-thread bucket counts and pair terms, added to device words by whole
+// blocks (every thread of the block calls flush).
+struct SegTally {
+    int32_t c[SEG_NB] = {0, 0, 0, 0, 0};
+    int64_t terms = 0;
+    __device__ void add(int64_t len)
+    {
+        int b = seg_bucket(len);
+#pragma unroll
+        for (int i = 0; i < SEG_NB; i++) c[i] += b == i;
+        terms += len * (len - 1);
+    }
+    __device__ void flush(int64_t* counts, int64_t* w2)
+    {
+        __shared__ int32_t sc[SEG_NB];
+        __shared__ unsigned long long st;
+        if (threadIdx.x < SEG_NB) sc[threadIdx.x] = 0;
+        if (threadIdx.x == 0) st = 0;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < SEG_NB; i++) {
+            int32_t t = warp_sum(c[i]);
+            if ((threadIdx.x & 31) == 0 && t) atomicAdd(&sc[i], t);
+        }
+        int64_t t = warp_sum(terms);
+        if ((threadIdx.x & 31) == 0 && t) atomicAdd(&st, (unsigned long long)t);
+        __syncthreads();
+        if (threadIdx.x < SEG_NB && sc[threadIdx.x])
+            atomicAdd((unsigned long long*)&counts[threadIdx.x], (unsigned long long)sc[threadIdx.x]);
+        if (threadIdx.x == 0 && st) atomicAdd((unsigned long long*)w2, st);
+    }
+};
+
+// Builds the bucket lists of a level from the counts known on the host
+// (b.n); cursor: SEG_NB device words, zero on entry. The order within a
+// bucket follows the hyperedge ids up to the order in which blocks arrive
+// (no result depends on it).
+Status seg_lists(const int64_t* hoff, int32_t E, int32_t maxlen, SegBuckets& b, int32_t* cursor,
+                 cudaStream_t s);
+
 inline int seg_grid_big(int32_t E) { return grid_for(E, 1, 152 * 2); }
 
 template <class Job>
 Status seg_run(const Job& job, const SegBuckets& b, int32_t E, Arena& ar, cudaStream_t s)
 {
     if (E <= 0) return Status{};
-    SNN_L k_seg_t<Job><<<grid_for(E, 256, 152 * 16), 256, 0, s>>>(job, b.list, b.meta);
-    SNN_CUDA(cudaGetLastError());
-    SNN_L k_seg_b0<Job><<<seg_grid_small(E), 256, 0, s>>>(job, b.list, b.meta);
-    SNN_CUDA(cudaGetLastError());
-    SNN_L k_seg_b1<Job><<<seg_grid_small(E), 256, 0, s>>>(job, b.list, b.meta);
-    SNN_CUDA(cudaGetLastError());
-    {
+    auto count = [&](int k) { return b.n[k] >= 0 ? b.n[k] : E; };
+    int gt = count(SEG_BT) > 0 ? grid_for(count(SEG_BT), 256, 152 * 16) : 0;
+    int gb0 = count(SEG_BB0) > 0 ? grid_for(count(SEG_BB0), 8, 152 * 16) : 0;
+    int gb1 = count(SEG_BB1) > 0 ? grid_for(count(SEG_BB1), 8, 152 * 16) : 0;
+    if (gt + gb0 + gb1 > 0) {
+        SNN_L k_seg_small<Job><<<gt + gb0 + gb1, 256, 0, s>>>(job, b.list, b.meta, gt, gb0);
+        SNN_CUDA(cudaGetLastError());
+    }
+    if (count(SEG_BB2) > 0) {
         size_t smem = SEG_B2_CAP * sizeof(uint32_t);
         SNN_CUDA(cudaFuncSetAttribute(k_seg_big<Job>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)smem));
-        SNN_L k_seg_big<Job><<<seg_grid_big(E), SEG_B2_THREADS, smem, s>>>(job, b.list, b.meta,
-                                                                            SEG_BB2, nullptr, 0);
+        SNN_L k_seg_big<Job><<<seg_grid_big(count(SEG_BB2)), SEG_B2_THREADS, smem, s>>>(
+            job, b.list, b.meta, SEG_BB2, nullptr, 0);
         SNN_CUDA(cudaGetLastError());
     }
-    if (b.b3_cap > 0) {
+    if (b.b3_cap > 0 && count(SEG_BB3) > 0) {
         uint32_t* g = nullptr;
         SNN_TRY(ar.alloc(&g, (int64_t)SEG_B3_BLOCKS * b.b3_cap));
         SNN_L k_seg_big<Job><<<SEG_B3_BLOCKS, SEG_B3_THREADS, 0, s>>>(job, b.list, b.meta, SEG_BB3,
