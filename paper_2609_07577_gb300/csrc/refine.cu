@@ -102,6 +102,9 @@ __global__ void k_cost_slots(const int64_t* __restrict__ slots, int64_t* out)
     if ((threadIdx.x & 31) == 0 && v) atomicAdd((unsigned long long*)out, (unsigned long long)v);
 }
 
+// most partitions whose inbound sums a block keeps in shared memory (32 KB)
+constexpr int32_t PC_SMEM_K = 8192;
+
 struct PinCountJob {
     const int64_t* hoff;
     const int32_t* hpins;
@@ -112,6 +115,25 @@ struct PinCountJob {
     PinCounts pc;
     int64_t* pincnt;
     int64_t* cost;     // COST_SLOTS partial sums of Conn
+    // inbound axons per partition summed per block first (a sum never passes
+    // the number of input hyperedges, so 32 bits hold it): a level adds one
+    // term per partition a hyperedge reaches, all on the K words of pincnt.
+    // 45,039 hyperedges on 111 partitions: 67 us a level without.
+    static constexpr bool kShared = true;
+    int32_t K = 0;     // words kept per block; 0: add to pincnt directly
+    uint32_t* acc = nullptr;
+    __host__ __device__ int shared_words() const { return K; }
+    __device__ void attach(uint32_t* w) { acc = K > 0 ? w : nullptr; }
+    __device__ void flush() const
+    {
+        for (int32_t p = threadIdx.x; p < K; p += blockDim.x)
+            if (acc[p]) atomicAdd((unsigned long long*)&pincnt[p], (unsigned long long)acc[p]);
+    }
+    __device__ __forceinline__ void add_inbound(int32_t p, int32_t k) const
+    {
+        if (acc) atomicAdd(&acc[p], (uint32_t)k);
+        else atomicAdd((unsigned long long*)&pincnt[p], (unsigned long long)k);
+    }
     __device__ int len(int32_t a) const { return (int)(hoff[a + 1] - hoff[a]); }
     __device__ uint32_t load(int32_t a, int i) const
     {
@@ -159,7 +181,7 @@ struct PinCountJob {
                 int dc = dsx >= 0 ? nx - dsx : 0;
                 pc.cnt[base + r] = nx - st;
                 pc.dcnt[base + r] = dc;
-                if (dc > 0) atomicAdd((unsigned long long*)&pincnt[pc.p[base + r]], (unsigned long long)hk[a]);
+                if (dc > 0) add_inbound(pc.p[base + r], hk[a]);
             }
             __syncwarp();
         }
@@ -178,7 +200,7 @@ struct PinCountJob {
                 pc.p[base + R] = (int32_t)(s[(i - 1) * st] >> 1);
                 pc.cnt[base + R] = c;
                 pc.dcnt[base + R] = d;
-                if (d > 0) atomicAdd((unsigned long long*)&pincnt[s[(i - 1) * st] >> 1], (unsigned long long)hk[a]);
+                if (d > 0) add_inbound((int32_t)(s[(i - 1) * st] >> 1), hk[a]);
                 R++;
                 c = 0;
                 d = 0;
@@ -190,7 +212,7 @@ struct PinCountJob {
             pc.p[base + R] = (int32_t)(s[(n - 1) * st] >> 1);
             pc.cnt[base + R] = c;
             pc.dcnt[base + R] = d;
-            if (d > 0) atomicAdd((unsigned long long*)&pincnt[s[(n - 1) * st] >> 1], (unsigned long long)hk[a]);
+            if (d > 0) add_inbound((int32_t)(s[(n - 1) * st] >> 1), hk[a]);
             R++;
         }
         pc.lam[a] = R;
@@ -267,6 +289,42 @@ __global__ void __launch_bounds__(256)
             lookup_count(pc, b, lam, rho[x], c, d);
             if (c == 1) atomicAdd((unsigned long long*)&savev[x], w);
         }
+    }
+}
+
+// The same with both sums kept per block in shared memory, for levels with
+// few vertices: there a heavy super-node's two words take an atomic from most
+// hyperedges. 32-bit sums (W and save are at most the summed omega).
+constexpr int SAVE_SMEM_V = 24 * 1024;   // 192 KB
+constexpr int SAVE_THREADS = 1024;
+
+template <int G>
+__global__ void __launch_bounds__(SAVE_THREADS)
+    k_save_smem(Level L, PinCounts pc, const int32_t* __restrict__ rho, int64_t* savev, int64_t* Wv)
+{
+    extern __shared__ uint32_t ssum[];   // W, then save
+    uint32_t *sW = ssum, *sS = ssum + L.V;
+    for (int32_t v = threadIdx.x; v < 2 * L.V; v += SAVE_THREADS) ssum[v] = 0;
+    __syncthreads();
+    int lane = threadIdx.x & (G - 1);
+    int64_t a1 = (int64_t)L.E * (blockIdx.x + 1) / gridDim.x;
+    for (int64_t a = (int64_t)L.E * blockIdx.x / gridDim.x + threadIdx.x / G; a < a1;
+         a += SAVE_THREADS / G) {
+        int64_t b = L.hoff[a], e = L.hoff[a + 1];
+        int32_t lam = pc.lam[a];
+        uint32_t w = (uint32_t)L.hw[a];
+        for (int64_t j = b + lane; j < e; j += G) {
+            int32_t x = L.hpins[j];
+            atomicAdd(&sW[x], w);
+            int32_t c, d;
+            lookup_count(pc, b, lam, rho[x], c, d);
+            if (c == 1) atomicAdd(&sS[x], w);
+        }
+    }
+    __syncthreads();
+    for (int32_t v = threadIdx.x; v < L.V; v += SAVE_THREADS) {
+        if (sW[v]) atomicAdd((unsigned long long*)&Wv[v], (unsigned long long)sW[v]);
+        if (sS[v]) atomicAdd((unsigned long long*)&savev[v], (unsigned long long)sS[v]);
     }
 }
 
@@ -1593,6 +1651,7 @@ static Status pin_counts_into(snnmap_hgraph* h, Level& L, LevelExtra& X, int32_t
     SNN_TRY(ar.alloc(&slots, COST_SLOTS));
     SNN_CUDA(cudaMemsetAsync(slots, 0, COST_SLOTS * sizeof(int64_t), s));
     PinCountJob job{L.hoff, L.hpins, L.hsd, L.hk, L.hw, rho, pc, ps.pincnt, slots};
+    if (K <= PC_SMEM_K && L.E >= 16 * (int64_t)K) job.K = K;
     SNN_TRY(seg_run(job, X.seg, L.E, ar, s));
     SNN_L k_cost_slots<<<1, 256, 0, s>>>(slots, cost);
     SNN_CUDA(cudaGetLastError());
@@ -1815,7 +1874,22 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
         prof.reset(new ProfScope(h, PS_SAVE));
         SNN_CUDA(cudaMemsetAsync(savev, 0, (size_t)(V > 0 ? V : 1) * 8, s));
         SNN_CUDA(cudaMemsetAsync(Wv, 0, (size_t)(V > 0 ? V : 1) * 8, s));
-        if (L.E > 0) {
+        if (L.E > 0 && !h->wide && V <= SAVE_SMEM_V) {
+            auto launch = [&](auto kern) -> Status {
+                SNN_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              SAVE_SMEM_V * 8));
+                SNN_L kern<<<grid_for(L.P, 4096, 152), SAVE_THREADS, (size_t)V * 8, s>>>(L, pc, rho,
+                                                                                        savev, Wv);
+                return Status{};
+            };
+            switch (hedge_lanes(L.P, L.E)) {
+            case 4: SNN_TRY(launch(k_save_smem<4>)); break;
+            case 8: SNN_TRY(launch(k_save_smem<8>)); break;
+            case 16: SNN_TRY(launch(k_save_smem<16>)); break;
+            default: SNN_TRY(launch(k_save_smem<32>));
+            }
+            SNN_CUDA(cudaGetLastError());
+        } else if (L.E > 0) {
             SNN_HEDGE_LAUNCH(hedge_lanes(L.P, L.E), k_save, L.E, s, L, pc, rho, savev, Wv);
             SNN_CUDA(cudaGetLastError());
         }

@@ -18,8 +18,15 @@
 //   __device__ void finish_thread(int32_t a, const uint32_t* s, int n, int st)
 //                                                   (key i at s[i * st])
 //        the same, run by a single thread
+// and optionally kShared = true with
+//   int shared_words() const                     32-bit words of shared memory a block keeps
+//                                                for it (0: none), zero on entry
+//   __device__ void attach(uint32_t* words)      that memory, before any finish
+//   __device__ void flush() const                run by the whole block after its lists
 #pragma once
 #include "common.cuh"
+
+#include <type_traits>
 
 namespace snn {
 
@@ -189,10 +196,21 @@ __device__ __forceinline__ void seg_thread_lists(const Job& job, const int32_t* 
 // compare-exchange a load pair, a store pair and a warp barrier: the
 // partition hypergraph of the 1,048,576-neuron conv network (917,504 lists
 // of 77 keys) took 2.14 ms there; see the measured figure at seg_run.
+template <class J, class = void>
+struct seg_shared : std::false_type {};
+template <class J>
+struct seg_shared<J, std::enable_if_t<J::kShared>> : std::true_type {};
+
 template <class Job>
 __global__ void __launch_bounds__(256) k_seg_small(Job job, const int32_t* __restrict__ lists,
                                                    const int32_t* __restrict__ meta, int gt, int gb0)
 {
+    extern __shared__ uint32_t seg_dyn[];
+    if constexpr (seg_shared<Job>::value) {
+        for (int i = threadIdx.x; i < job.shared_words(); i += 256) seg_dyn[i] = 0;
+        job.attach(seg_dyn);
+        __syncthreads();
+    }
     __shared__ __align__(16) uint32_t buf[SEG_T_CAP * 256];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int blk = blockIdx.x;
@@ -225,6 +243,10 @@ __global__ void __launch_bounds__(256) k_seg_small(Job job, const int32_t* __res
             job.finish(a, s, L);
             __syncwarp();
         }
+    }
+    if constexpr (seg_shared<Job>::value) {
+        __syncthreads();
+        job.flush();
     }
 }
 
@@ -303,11 +325,21 @@ Status seg_run(const Job& job, const SegBuckets& b, int32_t E, Arena& ar, cudaSt
 {
     if (E <= 0) return Status{};
     auto count = [&](int k) { return b.n[k] >= 0 ? b.n[k] : E; };
-    int gt = count(SEG_BT) > 0 ? grid_for(count(SEG_BT), 256, 152 * 16) : 0;
-    int gb0 = count(SEG_BB0) > 0 ? grid_for(count(SEG_BB0), 8, 152 * 16) : 0;
-    int gb1 = count(SEG_BB1) > 0 ? grid_for(count(SEG_BB1), 8, 152 * 16) : 0;
+    size_t dyn = 0;
+    int cap = 152 * 16;
+    if constexpr (seg_shared<Job>::value) {
+        // every block clears and flushes its words: fewer, longer blocks
+        dyn = (size_t)job.shared_words() * sizeof(uint32_t);
+        if (dyn) cap = 152 * 4;
+    }
+    int gt = count(SEG_BT) > 0 ? grid_for(count(SEG_BT), 256, cap) : 0;
+    int gb0 = count(SEG_BB0) > 0 ? grid_for(count(SEG_BB0), 8, cap) : 0;
+    int gb1 = count(SEG_BB1) > 0 ? grid_for(count(SEG_BB1), 8, cap) : 0;
     if (gt + gb0 + gb1 > 0) {
-        SNN_L k_seg_small<Job><<<gt + gb0 + gb1, 256, 0, s>>>(job, b.list, b.meta, gt, gb0);
+        if (dyn)
+            SNN_CUDA(cudaFuncSetAttribute(k_seg_small<Job>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)dyn));
+        SNN_L k_seg_small<Job><<<gt + gb0 + gb1, 256, dyn, s>>>(job, b.list, b.meta, gt, gb0);
         SNN_CUDA(cudaGetLastError());
     }
     if (count(SEG_BB2) > 0) {
