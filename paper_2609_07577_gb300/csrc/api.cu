@@ -192,7 +192,7 @@ static int snnmap_build_hgraph_impl(const snnmap_params* params, int32_t n_verti
         else h->level_budget = (int64_t)1 << 34;
     }
     cudaError_t e = cudaMallocHost(&h->h_scal, snn::SC_COUNT * sizeof(int64_t));
-    if (e == cudaSuccess) e = cudaMallocHost(&h->h_tier, 2 * snn::TIER_SLOTS * sizeof(int64_t));
+    if (e == cudaSuccess) e = cudaMallocHost(&h->h_tier, (2 * snn::TIER_SLOTS + 8) * sizeof(int64_t));
     if (e == cudaSuccess) memset(h->h_tier, 0, 2 * snn::TIER_SLOTS * sizeof(int64_t));
     if (e == cudaSuccess) e = snn::dev_malloc(&h->d_scal, snn::SC_COUNT * sizeof(int64_t), h->stream);
     if (e == cudaSuccess) e = snn::dev_malloc(&h->cand, (size_t)cap * 4, h->stream);

@@ -27,9 +27,9 @@
 // with pointer jumping for chains longer than the walk.
 #include "histo.cuh"
 #include "internal.cuh"
+#include "scan.cuh"
 
 #include <algorithm>
-#include <memory>
 
 namespace snn {
 
@@ -57,7 +57,7 @@ struct AffPol {
     int32_t* cand;
     int64_t* cscore;
     int32_t* cov;
-    const int32_t* vmin;   // smallest size and inbound pins over the level's vertices
+    const uint32_t* vmin;  // complements of the level's smallest size and inbound pins
     bool prefilter;        // some pair can break Omega or Phi (else elem skips the test)
     const uint8_t* only = nullptr;   // if set, the vertices evaluated (others untouched)
     const int4* vst;       // (size, inbound pins, inbound axons) per vertex
@@ -66,7 +66,8 @@ struct AffPol {
     __device__ bool skip(int32_t n) const
     {
         if (only && !only[n]) return true;
-        return (int64_t)L.vsize[n] + vmin[0] > omega || (int64_t)L.vinpins[n] + vmin[1] > phi;
+        return (int64_t)L.vsize[n] + (int32_t)~vmin[0] > omega ||
+               (int64_t)L.vinpins[n] + (int32_t)~vmin[1] > phi;
     }
     __device__ int64_t vb(int32_t n) const { return L.voff[n]; }
     __device__ int64_t ve(int32_t n) const { return L.voff[n + 1]; }
@@ -117,11 +118,6 @@ struct AffPol {
     {
         return it.m < 0 || t.add(it.m, it.w, it.o);
     }
-    template <class Tb>
-    __device__ bool elem(int32_t n, const Seg<S>& g, int32_t off, const Tb& t, Acc& acc) const
-    {
-        return put(n, load(n, g, off), t, acc);
-    }
     __device__ void consider(int32_t n, int32_t m, int64_t s, uint32_t o, const Acc&, int64_t& bs,
                              int32_t& bk, uint32_t& bo) const
     {
@@ -155,88 +151,94 @@ __global__ void k_pack_state(Level L, int4* vst)
 // ---------------------------------------------------------------------------
 // matching
 
-__global__ void k_count_cand(int32_t V, const int32_t* __restrict__ cand, int64_t* scal)
+// Per vertex, over its children (the vertices whose candidate it is): the
+// best score and, below, the lowest id having it. Both arrays start cleared:
+// scores are never negative, and ids are kept complemented (0: no child).
+__global__ void __launch_bounds__(256)
+    k_child_best_score(int32_t V, const int32_t* __restrict__ cand,
+                       const int64_t* __restrict__ cscore, unsigned long long* bestsc, int64_t* scal)
 {
-    int c = 0;
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
-         n += (int64_t)gridDim.x * blockDim.x)
-        c += cand[n] >= 0;
-    c = warp_sum(c);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd((unsigned long long*)&scal[SC_A], (unsigned long long)c);
-}
-
-__global__ void k_child_best_score(int32_t V, const int32_t* __restrict__ cand,
-                                   const int64_t* __restrict__ cscore, int64_t* bestsc)
-{
+    int k = 0;
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
         int32_t c = cand[n];
-        if (c >= 0) atomicMax((long long*)&bestsc[c], (long long)cscore[n]);
+        if (c >= 0) atomicMax(&bestsc[c], (unsigned long long)cscore[n]);
+        k += c >= 0;
     }
+    block_add(k, &scal[SC_A]);
 }
 
 __global__ void k_child_best_id(int32_t V, const int32_t* __restrict__ cand,
                                 const int64_t* __restrict__ cscore,
-                                const int64_t* __restrict__ bestsc, int32_t* bc)
+                                const unsigned long long* __restrict__ bestsc, uint32_t* bc)
 {
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
         int32_t c = cand[n];
-        if (c >= 0 && cscore[n] == bestsc[c]) atomicMin(&bc[c], (int32_t)n);
+        if (c >= 0 && (unsigned long long)cscore[n] == bestsc[c]) atomicMax(&bc[c], ~(uint32_t)n);
     }
 }
 
-__device__ __forceinline__ bool is_root(const int32_t* cand, int32_t n)
+// n's parent when n is its best child and neither is a root, else -1
+__device__ __forceinline__ int32_t chain_link(const int32_t* __restrict__ cand,
+                                              const uint32_t* __restrict__ bc, int32_t n)
 {
     int32_t c = cand[n];
-    return c >= 0 && cand[c] == n;
+    if (c < 0) return -1;
+    int32_t cc = cand[c];
+    if (cc == n || (cc >= 0 && cand[cc] == c) || bc[c] != ~(uint32_t)n) return -1;
+    return c;
 }
 
-// link(n) = parent when n is its parent's best child and neither is a root
-__global__ void k_link(int32_t V, const int32_t* __restrict__ cand, const int32_t* __restrict__ bc,
-                       int32_t* link)
+// Eq. matching for a vertex at odd or even distance from its chain's top:
+// matched to the parent at odd distance (or in a root two-cycle), otherwise
+// to the best child if any
+__device__ __forceinline__ int32_t match_of(const int32_t* __restrict__ cand,
+                                            const uint32_t* __restrict__ bc, int32_t n, bool odd)
 {
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
-         n += (int64_t)gridDim.x * blockDim.x) {
-        int32_t c = cand[n];
-        int32_t lk = -1;
-        if (c >= 0 && cand[c] != (int32_t)n && !is_root(cand, c) && bc[c] == (int32_t)n) lk = c;
-        link[n] = lk;
-    }
+    int32_t c = cand[n];
+    if (c >= 0 && (odd || cand[c] == n)) return c;
+    return bc[n] ? (int32_t)~bc[n] : -1;
 }
 
-// parity of the distance to the chain top, by a walk of at most MATCH_WALK
-// links; longer chains are left to pointer jumping (par = 2)
-__global__ void k_walk(int32_t V, const int32_t* __restrict__ link, uint8_t* par, int64_t* scal)
+// The matching, each vertex finding its distance to the chain's top by a walk
+// of at most MATCH_WALK links (computed on the way: most walks end at once).
+// Longer chains are counted and left to pointer jumping.
+__global__ void __launch_bounds__(256)
+    k_match(int32_t V, const int32_t* __restrict__ cand, const uint32_t* __restrict__ bc,
+            int32_t* match, int64_t* scal)
 {
-    int c = 0;
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
-         n += (int64_t)gridDim.x * blockDim.x) {
-        int32_t x = (int32_t)n;
+    int longer = 0, pairs = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < V;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        int32_t n = (int32_t)i, x = chain_link(cand, bc, n);
         int d = 0;
-        while (d < MATCH_WALK && link[x] >= 0) {
-            x = link[x];
+        while (x >= 0 && d < MATCH_WALK) {
+            x = chain_link(cand, bc, x);
             d++;
         }
-        if (link[x] >= 0) {
-            par[n] = 2;
-            c++;
-        } else {
-            par[n] = (uint8_t)(d & 1);
+        if (x >= 0) {
+            longer++;
+            continue;
         }
+        int32_t m = match_of(cand, bc, n, d & 1);
+        match[n] = m;
+        pairs += m > n;
     }
-    c = warp_sum(c);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd((unsigned long long*)&scal[SC_B], (unsigned long long)c);
+    block_add(longer, &scal[SC_B]);
+    block_add(pairs, &scal[SC_C]);
 }
 
 // pointer jumping over all vertices (fallback): nxt/pj hold the current
 // jump target and the parity of the distance covered so far
-__global__ void k_jump_init(int32_t V, const int32_t* __restrict__ link, int32_t* nxt, uint8_t* pj)
+__global__ void k_jump_init(int32_t V, const int32_t* __restrict__ cand,
+                            const uint32_t* __restrict__ bc, int32_t* nxt, uint8_t* pj)
 {
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
-        nxt[n] = link[n];
-        pj[n] = link[n] >= 0 ? 1 : 0;
+        int32_t l = chain_link(cand, bc, (int32_t)n);
+        nxt[n] = l;
+        pj[n] = l >= 0 ? 1 : 0;
     }
 }
 
@@ -260,69 +262,60 @@ __global__ void k_jump(int32_t V, const int32_t* __restrict__ nxt, const uint8_t
     if ((threadIdx.x & 31) == 0 && c) atomicAdd((unsigned long long*)&scal[SC_B], (unsigned long long)c);
 }
 
-__global__ void k_jump_done(int32_t V, const uint8_t* __restrict__ pj, uint8_t* par)
+// the matching from the jumped parities
+__global__ void __launch_bounds__(256)
+    k_match_jumped(int32_t V, const int32_t* __restrict__ cand, const uint32_t* __restrict__ bc,
+                   const uint8_t* __restrict__ pj, int32_t* match, int64_t* scal)
 {
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
-         n += (int64_t)gridDim.x * blockDim.x)
-        if (par[n] == 2) par[n] = pj[n];
-}
-
-// Eq. matching: matched to the parent at odd distance (or in a root
-// two-cycle), otherwise to the best child if any
-__global__ void k_match_finish(int32_t V, const int32_t* __restrict__ cand,
-                               const int32_t* __restrict__ bc, const uint8_t* __restrict__ par,
-                               int32_t* match, int64_t* scal)
-{
-    int c = 0;
+    int pairs = 0;
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
-        int32_t cn = cand[n];
-        int32_t m = -1;
-        if (cn >= 0 && (cand[cn] == (int32_t)n || par[n] == 1)) m = cn;
-        else if (bc[n] != 0x7fffffff) m = bc[n];
+        int32_t m = match_of(cand, bc, (int32_t)n, pj[n] != 0);
         match[n] = m;
-        c += m > (int32_t)n;
+        pairs += m > (int32_t)n;
     }
-    c = warp_sum(c);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd((unsigned long long*)&scal[SC_C], (unsigned long long)c);
+    block_add(pairs, &scal[SC_C]);
 }
 
 // ---------------------------------------------------------------------------
 
-// vm[0], vm[1]: smallest size and inbound pins; vm[2], vm[3]: largest
-__global__ void k_level_min(Level L, int32_t* vm)
+// vm[0], vm[1]: complements of the smallest size and inbound pins; vm[2],
+// vm[3]: the largest (all start cleared)
+__global__ void __launch_bounds__(256) k_level_min(Level L, uint32_t* vm)
 {
-    int32_t ms = 0x7fffffff, mi = 0x7fffffff, xs = 0, xi = 0;
+    __shared__ uint32_t sv[4];
+    if (threadIdx.x < 4) sv[threadIdx.x] = 0;
+    __syncthreads();
+    uint32_t ms = 0, mi = 0, xs = 0, xi = 0;
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < L.V;
          n += (int64_t)gridDim.x * blockDim.x) {
-        ms = min(ms, L.vsize[n]);
-        mi = min(mi, L.vinpins[n]);
-        xs = max(xs, L.vsize[n]);
-        xi = max(xi, L.vinpins[n]);
+        uint32_t a = (uint32_t)L.vsize[n], b = (uint32_t)L.vinpins[n];
+        ms = max(ms, ~a);
+        mi = max(mi, ~b);
+        xs = max(xs, a);
+        xi = max(xi, b);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        ms = min(ms, __shfl_xor_sync(FULL, ms, o));
-        mi = min(mi, __shfl_xor_sync(FULL, mi, o));
-        xs = max(xs, __shfl_xor_sync(FULL, xs, o));
-        xi = max(xi, __shfl_xor_sync(FULL, xi, o));
-    }
+    ms = __reduce_max_sync(FULL, ms);
+    mi = __reduce_max_sync(FULL, mi);
+    xs = __reduce_max_sync(FULL, xs);
+    xi = __reduce_max_sync(FULL, xi);
     if ((threadIdx.x & 31) == 0) {
-        atomicMin(&vm[0], ms);
-        atomicMin(&vm[1], mi);
-        atomicMax(&vm[2], xs);
-        atomicMax(&vm[3], xi);
+        atomicMax(&sv[0], ms);
+        atomicMax(&sv[1], mi);
+        atomicMax(&sv[2], xs);
+        atomicMax(&sv[3], xi);
     }
+    __syncthreads();
+    if (threadIdx.x < 4) atomicMax(&vm[threadIdx.x], sv[threadIdx.x]);
 }
 
 template <typename S>
 static Status affinity(snnmap_hgraph* h, Level& L)
 {
-    int32_t* vmin;
+    uint32_t* vmin;
     SNN_TRY(h->scratch.alloc(&vmin, 4));
-    SNN_TRY(fill_i32(vmin, 0x7fffffff, 2, h->stream));
-    SNN_CUDA(cudaMemsetAsync(vmin + 2, 0, 2 * sizeof(int32_t), h->stream));
-    SNN_L k_level_min<<<grid_for(L.V, 256), 256, 0, h->stream>>>(L, vmin);
+    SNN_CUDA(cudaMemsetAsync(vmin, 0, 4 * sizeof(int32_t), h->stream));
+    SNN_L k_level_min<<<grid_for(L.V, 256, 152 * 4), 256, 0, h->stream>>>(L, vmin);
     SNN_CUDA(cudaGetLastError());
     int32_t vm[4];
     SNN_CUDA(cudaMemcpyAsync(vm, vmin, sizeof(vm), cudaMemcpyDeviceToHost, h->stream));
@@ -347,7 +340,8 @@ static Status affinity(snnmap_hgraph* h, Level& L)
     int64_t* cnt;
     SNN_TRY(h->scratch.alloc(&cnt, HT_NCNT));
     if (L.V <= 0) SNN_CUDA(cudaMemsetAsync(cnt, 0, HT_NCNT * sizeof(int64_t), h->stream));
-    SNN_TRY(run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->d_scal, h->tiers));
+    SNN_TRY(run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->d_scal, h->tiers, L.V,
+                          !h->wzero));
     // the counters reach the level record after the matching's synchronization
     SNN_CUDA(cudaMemcpyAsync(h->h_tier, cnt, HT_NCNT * sizeof(int64_t), cudaMemcpyDeviceToHost,
                              h->stream));
@@ -633,11 +627,6 @@ struct AffNewPol {
     {
         return it.m < 0 || t.add(it.m, it.w, it.o);
     }
-    template <class Tb>
-    __device__ bool elem(int32_t n, const Seg<S>& g, int32_t off, const Tb& t, Acc& acc) const
-    {
-        return put(n, load(n, g, off), t, acc);
-    }
     __device__ void consider(int32_t n, int32_t m, int64_t s, uint32_t o, const Acc&, int64_t& bs,
                              int32_t& bk, uint32_t& bo) const
     {
@@ -711,6 +700,17 @@ Status aff_carry(snnmap_hgraph* h, int32_t src)
     return Status{};
 }
 
+// exclusive list positions, closed by the end of the last list
+struct ListPlaces {
+    int64_t* off;
+    int64_t n;
+    __device__ void operator()(int64_t i, int64_t ex, int64_t v) const
+    {
+        off[i] = ex;
+        if (i == n - 1) off[n] = ex + v;
+    }
+};
+
 // S1 on a level whose candidates were carried: *done false when the full
 // histogram is expected to be cheaper (nothing written then)
 template <typename S>
@@ -721,25 +721,21 @@ static Status affinity_carried(snnmap_hgraph* h, Level& L, bool* done)
     Arena& ar = h->scratch;
     AffCarry& C = h->icar;
     int64_t E = L.E;
-    int32_t *vmin, *lcnt;
-    int64_t *work, *loff;
-    SNN_TRY(ar.alloc(&vmin, 4));
-    SNN_TRY(ar.alloc(&work, 4));
+    int32_t* lcnt;
+    int64_t *work, *loff;   // work: [0], [1] the two estimates, [2] list entries, [3..4] vmin
+    SNN_TRY(ar.alloc(&work, 5));
     SNN_TRY(ar.alloc(&lcnt, E));
     SNN_TRY(ar.alloc(&loff, E + 1));
-    SNN_TRY(fill_i32(vmin, 0x7fffffff, 2, s));
-    SNN_CUDA(cudaMemsetAsync(vmin + 2, 0, 2 * sizeof(int32_t), s));
-    SNN_CUDA(cudaMemsetAsync(work, 0, 4 * sizeof(int64_t), s));
-    SNN_L k_level_min<<<grid_for(L.V, 256), 256, 0, s>>>(L, vmin);
+    SNN_CUDA(cudaMemsetAsync(work, 0, 5 * sizeof(int64_t), s));
+    uint32_t* vmin = (uint32_t*)(work + 3);
+    SNN_L k_level_min<<<grid_for(L.V, 256, 152 * 4), 256, 0, s>>>(L, vmin);
     if (E > 0) SNN_HEDGE_LAUNCH(hedge_lanes(L.P, E), k_ac_count, E, s, L, C.kind, lcnt, work);
     SNN_CUDA(cudaGetLastError());
-    SNN_TRY(scan_exclusive_i32_to_i64(lcnt, loff, E, loff + E, ar, s));
-    int64_t hv[3];
-    int32_t vm[4];
-    SNN_CUDA(cudaMemcpyAsync(vm, vmin, sizeof(vm), cudaMemcpyDeviceToHost, s));
-    SNN_CUDA(cudaMemcpyAsync(hv, work, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    SNN_CUDA(cudaMemcpyAsync(hv + 2, loff + E, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    SNN_TRY(scan_run<int64_t>(ScanLoad<int32_t, int64_t>{lcnt}, ListPlaces{loff, E}, E, work + 2, ar, s));
+    int64_t* hv = h->h_tier + 2 * TIER_SLOTS;   // pinned
+    SNN_CUDA(cudaMemcpyAsync(hv, work, 5 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     SNN_CUDA(cudaStreamSynchronize(s));
+    const int32_t* vm = (const int32_t*)(hv + 3);
     // carried work: the new super-nodes' lists and the new super-nodes' full
     // histograms (plus those of the few MERGED vertices whose super-node no
     // longer suits them)
@@ -774,7 +770,7 @@ static Status affinity_carried(snnmap_hgraph* h, Level& L, bool* done)
         pol.cand = h->cand;
         pol.cscore = h->cscore;
         pol.cov = h->cov;
-        SNN_TRY(run_histogram(pol, ar, s, cnt, h->h_scal + 12, h->d_scal, h->tiers));
+        SNN_TRY(run_histogram(pol, ar, s, cnt, h->h_scal + 12, h->d_scal, h->tiers, L.V, !h->wzero));
         SNN_CUDA(cudaMemcpyAsync(h->h_tier, cnt, HT_NCNT * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     }
     SNN_L k_ac_check<<<grid_for(L.V, 256), 256, 0, s>>>(L, C, h->prm.omega, h->prm.delta,
@@ -795,7 +791,7 @@ static Status affinity_carried(snnmap_hgraph* h, Level& L, bool* done)
         pol.cand = h->cand;
         pol.cscore = h->cscore;
         pol.cov = h->cov;
-        SNN_TRY(run_histogram(pol, ar, s, cnt, h->h_scal + 12, h->d_scal, h->tiers));
+        SNN_TRY(run_histogram(pol, ar, s, cnt, h->h_scal + 12, h->d_scal, h->tiers, L.V, !h->wzero));
         SNN_CUDA(cudaMemcpyAsync(h->h_tier + TIER_SLOTS, cnt, HT_NCNT * sizeof(int64_t),
                                  cudaMemcpyDeviceToHost, s));
     }
@@ -803,6 +799,60 @@ static Status affinity_carried(snnmap_hgraph* h, Level& L, bool* done)
     h->tier_level = (int32_t)h->extra.size() - 1;
     h->tier_form = 2;
     *done = true;
+    return Status{};
+}
+
+// Candidates and pairs of the matching; d_scal (device, cleared but for the
+// status) and h_scal (host): SC_COUNT words. One wait, unless some chain is
+// longer than the walk.
+static Status match_into(int32_t V, const int32_t* cand, const int64_t* cscore, int32_t* match,
+                         int64_t* d_scal, int64_t* h_scal, Arena& ar, cudaStream_t s,
+                         int64_t* n_cand, int64_t* n_pairs)
+{
+    int g = grid_for(V, 256);
+    unsigned long long* bestsc;
+    uint32_t* bc;
+    Carver c;
+    c.add(&bestsc, V);
+    c.add(&bc, V);
+    char* base;
+    SNN_TRY(ar.alloc(&base, (int64_t)c.total));
+    c.assign(base);
+    SNN_CUDA(cudaMemsetAsync(base, 0, c.total, s));
+    SNN_L k_child_best_score<<<g, 256, 0, s>>>(V, cand, cscore, bestsc, d_scal);
+    SNN_L k_child_best_id<<<g, 256, 0, s>>>(V, cand, cscore, bestsc, bc);
+    SNN_L k_match<<<g, 256, 0, s>>>(V, cand, bc, match, d_scal);
+    SNN_CUDA(cudaGetLastError());
+    auto read = [&]() -> Status {
+        SNN_CUDA(cudaMemcpyAsync(h_scal, d_scal, SC_COUNT * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        SNN_CUDA(cudaStreamSynchronize(s));
+        return Status{};
+    };
+    SNN_TRY(read());
+    *n_cand = h_scal[SC_A];
+    if (h_scal[SC_B] > 0) {
+        int32_t *nxt, *nxt2;
+        uint8_t *pj, *pj2;
+        SNN_TRY(ar.alloc(&nxt, V));
+        SNN_TRY(ar.alloc(&nxt2, V));
+        SNN_TRY(ar.alloc(&pj, V));
+        SNN_TRY(ar.alloc(&pj2, V));
+        SNN_L k_jump_init<<<g, 256, 0, s>>>(V, cand, bc, nxt, pj);
+        SNN_CUDA(cudaGetLastError());
+        for (int it = 0; it < 40; it++) {
+            SNN_CUDA(cudaMemsetAsync(d_scal + SC_B, 0, 2 * sizeof(int64_t), s));
+            SNN_L k_jump<<<g, 256, 0, s>>>(V, nxt, pj, nxt2, pj2, d_scal);
+            SNN_CUDA(cudaGetLastError());
+            std::swap(nxt, nxt2);
+            std::swap(pj, pj2);
+            SNN_TRY(read());
+            if (h_scal[SC_B] == 0) break;
+        }
+        SNN_L k_match_jumped<<<g, 256, 0, s>>>(V, cand, bc, pj, match, d_scal);
+        SNN_CUDA(cudaGetLastError());
+        SNN_TRY(read());
+    }
+    *n_pairs = h_scal[SC_C];
     return Status{};
 }
 
@@ -833,55 +883,15 @@ Status coarsen_level(snnmap_hgraph* h, int32_t* n_cand, int32_t* n_pairs)
             SNN_TRY(affinity<uint32_t>(h, L));
         }
     }
-    int g = grid_for(V, 256);
-    std::unique_ptr<ProfScope> prof(new ProfScope(h, PS_MATCH));
-    SNN_L k_count_cand<<<g, 256, 0, s>>>(V, h->cand, h->d_scal);
-    SNN_CUDA(cudaGetLastError());
-    int64_t* bestsc;
-    int32_t *bc, *link, *nxt, *nxt2;
-    uint8_t *par, *pj, *pj2;
-    SNN_TRY(ar.alloc(&bestsc, V));
-    SNN_TRY(ar.alloc(&bc, V));
-    SNN_TRY(ar.alloc(&link, V));
-    SNN_TRY(ar.alloc(&par, V));
-    SNN_TRY(fill_i64(bestsc, INT64_MIN, V, s));
-    SNN_TRY(fill_i32(bc, 0x7fffffff, V, s));
-    SNN_L k_child_best_score<<<g, 256, 0, s>>>(V, h->cand, h->cscore, bestsc);
-    SNN_L k_child_best_id<<<g, 256, 0, s>>>(V, h->cand, h->cscore, bestsc, bc);
-    SNN_L k_link<<<g, 256, 0, s>>>(V, h->cand, bc, link);
-    SNN_L k_walk<<<g, 256, 0, s>>>(V, link, par, h->d_scal);
-    SNN_CUDA(cudaGetLastError());
-    prof.reset();
-    SNN_TRY(read_scalars(h));
-    *n_cand = (int32_t)h->h_scal[SC_A];
-    int64_t unresolved = h->h_scal[SC_B];
-    if (*n_cand == 0) return Status{};
-    if (unresolved > 0) {
-        SNN_TRY(ar.alloc(&nxt, V));
-        SNN_TRY(ar.alloc(&nxt2, V));
-        SNN_TRY(ar.alloc(&pj, V));
-        SNN_TRY(ar.alloc(&pj2, V));
-        SNN_L k_jump_init<<<g, 256, 0, s>>>(V, link, nxt, pj);
-        SNN_CUDA(cudaGetLastError());
-        for (int it = 0; it < 40; it++) {
-            SNN_TRY(zero_scalars(h));
-            SNN_L k_jump<<<g, 256, 0, s>>>(V, nxt, pj, nxt2, pj2, h->d_scal);
-            SNN_CUDA(cudaGetLastError());
-            std::swap(nxt, nxt2);
-            std::swap(pj, pj2);
-            SNN_TRY(read_scalars(h));
-            if (h->h_scal[SC_B] == 0) break;
-        }
-        SNN_L k_jump_done<<<g, 256, 0, s>>>(V, pj, par);
-        SNN_CUDA(cudaGetLastError());
+    int64_t np = 0;
+    {
+        ProfScope prof(h, PS_MATCH);
+        int64_t nc = 0;
+        SNN_TRY(match_into(V, h->cand, h->cscore, h->match, h->d_scal, h->h_scal, ar, s, &nc, &np));
+        *n_cand = (int32_t)nc;
     }
-    SNN_TRY(zero_scalars(h));
-    prof.reset(new ProfScope(h, PS_MATCH));
-    SNN_L k_match_finish<<<g, 256, 0, s>>>(V, h->cand, bc, par, h->match, h->d_scal);
-    SNN_CUDA(cudaGetLastError());
-    prof.reset();
-    SNN_TRY(read_scalars(h));
-    *n_pairs = (int32_t)h->h_scal[SC_C];
+    if (*n_cand == 0) return Status{};
+    *n_pairs = (int32_t)np;
     h->have_matching = true;
     h->last_pairs = *n_pairs;
     return Status{};
@@ -897,52 +907,9 @@ Status match_forest(int32_t V, const int32_t* cand, const int64_t* cscore, int32
 {
     *n_pairs = 0;
     if (V <= 0) return Status{};
-    int g = grid_for(V, 256);
-    int64_t h_scal[SC_COUNT];
-    int64_t* bestsc;
-    int32_t *bc, *link, *nxt, *nxt2;
-    uint8_t *par, *pj, *pj2;
-    SNN_TRY(ar.alloc(&bestsc, V));
-    SNN_TRY(ar.alloc(&bc, V));
-    SNN_TRY(ar.alloc(&link, V));
-    SNN_TRY(ar.alloc(&par, V));
+    int64_t h_scal[SC_COUNT], nc = 0;
     SNN_CUDA(cudaMemsetAsync(d_scal, 0, SC_COUNT * sizeof(int64_t), s));
-    SNN_TRY(fill_i64(bestsc, INT64_MIN, V, s));
-    SNN_TRY(fill_i32(bc, 0x7fffffff, V, s));
-    SNN_L k_child_best_score<<<g, 256, 0, s>>>(V, cand, cscore, bestsc);
-    SNN_L k_child_best_id<<<g, 256, 0, s>>>(V, cand, cscore, bestsc, bc);
-    SNN_L k_link<<<g, 256, 0, s>>>(V, cand, bc, link);
-    SNN_L k_walk<<<g, 256, 0, s>>>(V, link, par, d_scal);
-    SNN_CUDA(cudaGetLastError());
-    SNN_CUDA(cudaMemcpyAsync(h_scal, d_scal, sizeof(h_scal), cudaMemcpyDeviceToHost, s));
-    SNN_CUDA(cudaStreamSynchronize(s));
-    if (h_scal[SC_B] > 0) {
-        SNN_TRY(ar.alloc(&nxt, V));
-        SNN_TRY(ar.alloc(&nxt2, V));
-        SNN_TRY(ar.alloc(&pj, V));
-        SNN_TRY(ar.alloc(&pj2, V));
-        SNN_L k_jump_init<<<g, 256, 0, s>>>(V, link, nxt, pj);
-        SNN_CUDA(cudaGetLastError());
-        for (int it = 0; it < 40; it++) {
-            SNN_CUDA(cudaMemsetAsync(d_scal, 0, SC_COUNT * sizeof(int64_t), s));
-            SNN_L k_jump<<<g, 256, 0, s>>>(V, nxt, pj, nxt2, pj2, d_scal);
-            SNN_CUDA(cudaGetLastError());
-            std::swap(nxt, nxt2);
-            std::swap(pj, pj2);
-            SNN_CUDA(cudaMemcpyAsync(h_scal, d_scal, sizeof(h_scal), cudaMemcpyDeviceToHost, s));
-            SNN_CUDA(cudaStreamSynchronize(s));
-            if (h_scal[SC_B] == 0) break;
-        }
-        SNN_L k_jump_done<<<g, 256, 0, s>>>(V, pj, par);
-        SNN_CUDA(cudaGetLastError());
-    }
-    SNN_CUDA(cudaMemsetAsync(d_scal, 0, SC_COUNT * sizeof(int64_t), s));
-    SNN_L k_match_finish<<<g, 256, 0, s>>>(V, cand, bc, par, match, d_scal);
-    SNN_CUDA(cudaGetLastError());
-    SNN_CUDA(cudaMemcpyAsync(h_scal, d_scal, sizeof(h_scal), cudaMemcpyDeviceToHost, s));
-    SNN_CUDA(cudaStreamSynchronize(s));
-    *n_pairs = h_scal[SC_C];
-    return Status{};
+    return match_into(V, cand, cscore, match, d_scal, h_scal, ar, s, &nc, n_pairs);
 }
 
 }  // namespace snn

@@ -84,6 +84,20 @@ __device__ __forceinline__ T warp_sum(T v)
     return v;
 }
 
+// adds the block's sum of v to *out: one atomic per block and call (every
+// thread of the block takes part)
+__device__ __forceinline__ void block_add(int v, int64_t* out)
+{
+    __shared__ int s;
+    if (threadIdx.x == 0) s = 0;
+    __syncthreads();
+    v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0 && v) atomicAdd(&s, v);
+    __syncthreads();
+    if (threadIdx.x == 0 && s) atomicAdd((unsigned long long*)out, (unsigned long long)s);
+    __syncthreads();
+}
+
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 inline int bits_for(uint64_t maxval)

@@ -17,7 +17,9 @@
 //               one global-memory table per vertex sized to twice its bound
 //               of distinct keys (so it cannot overflow); one block per
 //               vertex then reduces the table.
-// Every tier visits a chunk of 32 incidences at a time with their segments
+// Key spaces of up to 24,576 keys take arrays instead of the tables of the
+// block tier (up to 4,096 keys) and of the big and split tiers (k_ht_dense).
+// The hash tiers visit a chunk of 32 incidences at a time with their segments
 // flattened into one range, so all 32 lanes load consecutive elements even
 // when segments are short.
 //
@@ -32,7 +34,9 @@
 //   __device__ int64_t seg_len(int64_t i)           segment length of incidence i
 //   __device__ int64_t vb(n), ve(n)                 incidence range of vertex n
 //   __device__ Seg<S> seg(int64_t i, Acc&)          segment of incidence i
-//   __device__ bool elem(n, const Seg<S>&, off, const Table<S>&, Acc&)
+//   struct Item, Item load(n, const Seg<S>&, off)   one element's reads; none() an empty Item
+//   __device__ bool put(n, const Item&, table, Acc&)  its table update
+//   (apart, so that several elements' loads are in flight per thread)
 //   __device__ void consider(n, key, int64 sc, uint32 ov, const Acc& total,
 //                            int64_t& best, int32_t& bkey, uint32_t& bov)
 //   __device__ void write(n, best, bkey, bov, const Acc& total)
@@ -157,7 +161,7 @@ __device__ bool warp_visit(const Pol& pol, int32_t n, int64_t i0, int64_t ve, in
             g.nd = __shfl_sync(FULL, sg.nd, lo);
             g.sd = __shfl_sync(FULL, sg.sd, lo);
             int32_t pt = __shfl_sync(FULL, pre, lo);
-            if (v < total && !pol.elem(n, g, v - pt, t, acc)) ok = false;
+            if (v < total && !pol.put(n, pol.load(n, g, v - pt), t, acc)) ok = false;
         }
     }
     return __all_sync(FULL, ok);
@@ -221,7 +225,8 @@ enum : int { HT_TIER_WARP = 0, HT_TIER_BLOCK = 1, HT_TIER_BIG = 2, HT_TIER_SPLIT
 // scheduling: a block takes the next vertex when it is done with one)
 enum : int {
     HT_CNT_WORK = HT_NTIER, HT_CNT_VERTS = HT_NTIER + 1, HT_CNT_NEXT = HT_NTIER + 2,
-    HT_NCNT = HT_NTIER + 2 + HT_NTIER
+    HT_CNT_TODO = HT_NTIER + 2 + HT_NTIER,   // vertices not skipped (k_ht_skip)
+    HT_NCNT = HT_CNT_TODO + 1
 };
 
 template <typename S>
@@ -244,7 +249,7 @@ __host__ __device__ inline int64_t pow2_ceil(int64_t x)
 // vertices pay a thread, not a warp, per skipped vertex, while full passes
 // keep a warp per vertex.
 template <class Pol>
-__global__ void __launch_bounds__(256) k_ht_skip(Pol pol, int64_t* work, int32_t* todo, int32_t* ntodo)
+__global__ void __launch_bounds__(256) k_ht_skip(Pol pol, int64_t* work, int32_t* todo, int64_t* ntodo)
 {
     int lane = threadIdx.x & 31;
     unsigned lt = lanemask_lt();
@@ -260,26 +265,53 @@ __global__ void __launch_bounds__(256) k_ht_skip(Pol pol, int64_t* work, int32_t
         if (!m) continue;
         int leader = __ffs(m) - 1;
         int32_t pos = 0;
-        if (lane == leader) pos = atomicAdd(ntodo, __popc(m));
+        if (lane == leader) pos = (int32_t)atomicAdd((unsigned long long*)ntodo, (unsigned long long)__popc(m));
         pos = __shfl_sync(FULL, pos, leader);
         if (count) todo[pos + __popc(m & lt)] = (int32_t)n;
     }
 }
 
+// (A vertex of more than HT_WORK_LONG incidences is summed by its whole
+// block: on a tail level one super-node may be in most hyperedges, and one
+// warp took 78 us for its 10,000 incidences.)
+constexpr int64_t HT_WORK_LONG = 1024;
+
 template <class Pol>
 __global__ void __launch_bounds__(256)
-    k_ht_work(Pol pol, int64_t* work, const int32_t* __restrict__ todo, const int32_t* __restrict__ ntodo)
+    k_ht_work(Pol pol, int64_t* work, const int32_t* __restrict__ todo, const int64_t* __restrict__ ntodo)
 {
-    int lane = threadIdx.x & 31;
-    int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    int32_t nt = *ntodo;
-    for (int64_t idx = gw; idx < nt; idx += nw) {
-        int32_t n = todo[idx];
-        int64_t w = 0;
-        for (int64_t i = pol.vb(n) + lane; i < pol.ve(n); i += 32) w += pol.seg_len(i);
-        w = warp_sum(w);
-        if (lane == 0) work[n] = w;
+    __shared__ unsigned long long part;
+    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int64_t nt = *ntodo;
+    for (int64_t base = (int64_t)blockIdx.x * 8; base < nt; base += (int64_t)gridDim.x * 8) {
+        bool longer = false;
+        if (base + warp < nt) {
+            int32_t n = todo[base + warp];
+            int64_t vb = pol.vb(n), ve = pol.ve(n);
+            longer = ve - vb > HT_WORK_LONG;
+            if (!longer) {
+                int64_t w = 0;
+#pragma unroll 4
+                for (int64_t i = vb + lane; i < ve; i += 32) w += pol.seg_len(i);
+                w = warp_sum(w);
+                if (lane == 0) work[n] = w;
+            }
+        }
+        if (!__syncthreads_or(longer)) continue;
+        for (int x = 0; x < 8 && base + x < nt; x++) {
+            int32_t n = todo[base + x];
+            int64_t vb = pol.vb(n), ve = pol.ve(n);
+            if (ve - vb <= HT_WORK_LONG) continue;
+            if (threadIdx.x == 0) part = 0;
+            __syncthreads();
+            int64_t w = 0;
+#pragma unroll 4
+            for (int64_t i = vb + threadIdx.x; i < ve; i += 256) w += pol.seg_len(i);
+            w = warp_sum(w);
+            if (lane == 0) atomicAdd(&part, (unsigned long long)w);
+            __syncthreads();
+            if (threadIdx.x == 0) work[n] = (int64_t)part;
+        }
     }
 }
 
@@ -300,7 +332,7 @@ __device__ __forceinline__ void ht_push(const Pol& pol, int tier, int32_t n, int
 template <class Pol>
 __global__ void __launch_bounds__(256)
     k_ht_classify(Pol pol, const int64_t* __restrict__ workv, int32_t* lists, int64_t* cnt,
-                  int64_t* scap, HtTiers tiers)
+                  int64_t* scap, HtTiers tiers, bool dense)
 {
     int lane = threadIdx.x & 31;
     unsigned lt = lanemask_lt();
@@ -320,7 +352,10 @@ __global__ void __launch_bounds__(256)
                 wsum += work;
                 vsum++;
                 int64_t bound = work < pol.keys ? work : pol.keys;
-                if (bound <= HT_WLOAD) tier = work <= tiers.wwork ? HT_TIER_WARP : HT_TIER_SPLIT;
+                // few keys but much work: many warps into one small table, or
+                // (dense) a block's arrays
+                if (bound <= HT_WLOAD && (work <= tiers.wwork || !dense))
+                    tier = work <= tiers.wwork ? HT_TIER_WARP : HT_TIER_SPLIT;
                 else if (Pol::kOptimistic && work <= tiers.wwork) tier = HT_TIER_WARP;
                 else if (work <= tiers.bwork) tier = HT_TIER_BLOCK;
                 else if (work <= tiers.gwork) tier = HT_TIER_BIG;
@@ -400,14 +435,6 @@ __global__ void __launch_bounds__(HT_WARPS * 32)
     }
 }
 
-// A policy may split elem into load (the element's global reads, giving an
-// Item) and put (the table update), declaring `struct Item`; the block tiers
-// then keep several elements' loads in flight per thread.
-template <class P, class = void>
-struct has_item : std::false_type {};
-template <class P>
-struct has_item<P, std::void_t<typename P::Item>> : std::true_type {};
-
 // the last index lo in [from, n) with spre[lo] <= v (spre non-decreasing,
 // spre[from] <= v): one probe while v stays in the same segment, a binary
 // search when it moved on
@@ -463,31 +490,21 @@ __device__ bool block_visit(const Pol& pol, int32_t n, int64_t vb, int64_t ve, c
         int32_t total = swarp[nw];
         __syncthreads();
         int32_t lo = 0;
-        if constexpr (has_item<Pol>::value) {
-            constexpr int U = 4;
-            for (int32_t v0 = threadIdx.x; v0 < total && ok; v0 += U * T) {
-                typename Pol::Item it[U];
+        constexpr int U = 4;   // elements in flight per thread
+        for (int32_t v0 = threadIdx.x; v0 < total && ok; v0 += U * T) {
+            typename Pol::Item it[U];
 #pragma unroll
-                for (int u = 0; u < U; u++) {
-                    int32_t v = v0 + u * T;
-                    if (v < total) {
-                        lo = seg_find(spre, T, lo, v);
-                        it[u] = pol.load(n, sseg[lo], v - spre[lo]);
-                    } else {
-                        it[u] = Pol::none();
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < U; u++) ok = pol.put(n, it[u], t, acc) && ok;
-            }
-        } else {
-            for (int32_t v = threadIdx.x; v < total; v += T) {
-                lo = seg_find(spre, T, lo, v);
-                if (!pol.elem(n, sseg[lo], v - spre[lo], t, acc)) {
-                    ok = false;
-                    break;
+            for (int u = 0; u < U; u++) {
+                int32_t v = v0 + u * T;
+                if (v < total) {
+                    lo = seg_find(spre, T, lo, v);
+                    it[u] = pol.load(n, sseg[lo], v - spre[lo]);
+                } else {
+                    it[u] = Pol::none();
                 }
             }
+#pragma unroll
+            for (int u = 0; u < U; u++) ok = pol.put(n, it[u], t, acc) && ok;
         }
         if (!ok) *sfail = 1;
         __syncthreads();
@@ -559,6 +576,149 @@ __global__ void __launch_bounds__(T)
         __syncthreads();
         if (threadIdx.x == 0) {
             for (int w = 1; w < nwarps; w++)
+                if (better(rs[w], rk[w], bs, bk)) {
+                    bs = rs[w];
+                    bk = rk[w];
+                    bo = ro[w];
+                }
+            pol.write(n, bs, bk, bo, tot);
+        }
+        __syncthreads();
+    }
+}
+
+// Dense tier: where the key space is small enough for one word pair per key
+// in shared memory, a block counts a vertex straight into arrays indexed by
+// key: no hashing, no probing, no table that can fill up, hence no vertex
+// handed on, no split tier and no wait for its sizes. Presence of a key is a
+// nonzero sum, so every weight has to be positive (the callers know).
+//
+// A group of G lanes takes an incidence (G: the mean segment, a power of
+// two) and loops over its segment, U incidences in flight per group, since a
+// block walking one heavy super-node's incidences is a chain of gathers
+// (incidence -> hyperedge -> pins); segments longer than HT_DENSE_LONG are
+// left to the whole block.
+//
+// Clearing, scanning and occupancy bound it from above: a vertex costs the
+// whole key range once, so vertices of little work stay on the hash tiers
+// unless the range itself is small (HT_DENSE_SMALL).
+constexpr int64_t HT_DENSE_KEYS = 24 * 1024;   // 192 KB of 32-bit sum pairs
+constexpr int64_t HT_DENSE_SMALL = 4 * 1024;   // 32 KB: several 256-thread blocks per SM
+constexpr int64_t HT_DENSE_BWORK = 8192;       // most elements a 256-thread block takes there
+constexpr int HT_DENSE_LONG = 1024;
+constexpr int HT_DENSE_NLONG = 256;
+
+template <typename S>
+struct DenseTable {
+    S* sc;
+    uint32_t* ov;
+    __device__ __forceinline__ bool add(int32_t m, S w, uint32_t o) const
+    {
+        atomicAdd(&sc[m], w);
+        if (o) atomicAdd(&ov[m], o);
+        return true;
+    }
+};
+
+template <class Pol, int T, int TIER>
+__global__ void __launch_bounds__(T)
+    k_ht_dense(Pol pol, const int32_t* __restrict__ lists, int64_t* cnt, int32_t keys, int glog)
+{
+    using S = typename Pol::S;
+    using Acc = typename Pol::Acc;
+    extern __shared__ __align__(16) unsigned char ht_dyn[];
+    __shared__ int64_t slong[HT_DENSE_NLONG];
+    __shared__ int32_t nlong;
+    __shared__ __align__(16) unsigned char wacc_raw[sizeof(Acc) * (T / 32)];
+    __shared__ int64_t rs[T / 32];
+    __shared__ int32_t rk[T / 32];
+    __shared__ uint32_t ro[T / 32];
+    __shared__ int64_t snext;
+    Acc* wacc = (Acc*)wacc_raw;
+    DenseTable<S> t{(S*)ht_dyn, (uint32_t*)(ht_dyn + (size_t)keys * sizeof(S))};
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int G = 1 << glog, gl = threadIdx.x & (G - 1), grp = threadIdx.x >> glog;
+    const int ngrp = T >> glog;
+    const unsigned gmask = G == 32 ? FULL : ((1u << G) - 1) << (lane & ~(G - 1));
+    constexpr int U = 4;
+    const int32_t* list = lists + (int64_t)TIER * pol.V;
+    const int64_t nl = cnt[TIER];
+    if (nl == 0) return;
+    for (int32_t k = threadIdx.x; k < keys; k += T) {
+        t.sc[k] = 0;
+        t.ov[k] = 0;
+    }
+    for (;;) {
+        if (threadIdx.x == 0) {
+            snext = (int64_t)atomicAdd((unsigned long long*)&cnt[HT_CNT_NEXT + TIER], 1ull);
+            nlong = 0;
+        }
+        __syncthreads();
+        const int64_t idx = snext;
+        if (idx >= nl) break;
+        const int32_t n = list[idx];
+        const int64_t vb = pol.vb(n), ve = pol.ve(n);
+        Acc acc, other;   // a segment's own terms count once, in its first lane
+        for (int64_t i0 = vb + grp; i0 < ve; i0 += (int64_t)U * ngrp) {
+            Seg<S> g[U];
+            typename Pol::Item it[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                int64_t i = i0 + (int64_t)u * ngrp;
+                g[u] = Seg<S>{0, 0, 0, 0, 0, 0};
+                if (i < ve) g[u] = pol.seg(i, gl == 0 ? acc : other);
+                if (g[u].len > HT_DENSE_LONG) {
+                    int32_t at = HT_DENSE_NLONG;
+                    if (gl == 0) at = atomicAdd(&nlong, 1);
+                    at = __shfl_sync(gmask, at, lane & ~(G - 1));
+                    if (at < HT_DENSE_NLONG) {
+                        if (gl == 0) slong[at] = i;
+                        g[u].len = 0;
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                it[u] = gl < g[u].len ? pol.load(n, g[u], gl) : Pol::none();
+#pragma unroll
+            for (int u = 0; u < U; u++) pol.put(n, it[u], t, acc);
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                for (int32_t off = gl + G; off < g[u].len; off += G)
+                    pol.put(n, pol.load(n, g[u], off), t, acc);
+        }
+        __syncthreads();
+        const int nlg = nlong < HT_DENSE_NLONG ? nlong : HT_DENSE_NLONG;
+        for (int x = 0; x < nlg; x++) {
+            Seg<S> g = pol.seg(slong[x], other);   // its own terms are in already
+            for (int32_t off = threadIdx.x; off < g.len; off += T)
+                pol.put(n, pol.load(n, g, off), t, acc);
+        }
+        Acc wa = Pol::warp_reduce(acc);
+        if (lane == 0) wacc[warp] = wa;
+        __syncthreads();
+        Acc tot = wacc[0];
+        for (int w = 1; w < T / 32; w++) tot.add(wacc[w]);
+        int64_t bs = 0;
+        int32_t bk = -1;
+        uint32_t bo = 0;
+        for (int32_t k = threadIdx.x; k < keys; k += T) {
+            S v = t.sc[k];
+            if (v == 0) continue;
+            uint32_t o = t.ov[k];
+            t.sc[k] = 0;
+            t.ov[k] = 0;
+            pol.consider(n, k, (int64_t)v, o, tot, bs, bk, bo);
+        }
+        warp_argmax(bs, bk, bo);
+        if (lane == 0) {
+            rs[warp] = bs;
+            rk[warp] = bk;
+            ro[warp] = bo;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < T / 32; w++)
                 if (better(rs[w], rk[w], bs, bk)) {
                     bs = rs[w];
                     bk = rk[w];
@@ -911,25 +1071,32 @@ Status split_cuts(const Pol& pol, Arena& ar, cudaStream_t s, const int32_t* sl, 
 // work, vertices histogrammed).
 template <class Pol>
 Status run_histogram(const Pol& pol, Arena& ar, cudaStream_t s, int64_t* d_cnt, int64_t* h_cnt,
-                     int64_t* status, const HtTiers& tiers = HtTiers{})
+                     int64_t* status, HtTiers tiers, int32_t key_space, bool positive)
 {
     using S = typename Pol::S;
     int32_t V = pol.V;
     if (V <= 0) return Status{};
+    // forms of the block and the big tier: arrays over the whole key space
+    // where they fit (see k_ht_dense), else hash tables
+    const bool dense_big = positive && sizeof(S) == 4 && key_space <= HT_DENSE_KEYS;
+    const bool dense_block = dense_big && key_space <= HT_DENSE_SMALL;
+    if (dense_block && tiers.bwork > HT_DENSE_BWORK && tiers.bwork < tiers.gwork)
+        tiers.bwork = HT_DENSE_BWORK;
+    // a vertex meets every pin of the level at most once
+    const bool split = !dense_big || tiers.gwork < pol.L.P;
     int32_t* lists;
     int64_t *scap, *workv;
     SNN_TRY(ar.alloc(&lists, (int64_t)HT_NTIER * V));
     SNN_TRY(ar.alloc(&scap, V));
     SNN_TRY(ar.alloc(&workv, V));
     SNN_CUDA(cudaMemsetAsync(d_cnt, 0, HT_NCNT * sizeof(int64_t), s));
-    int32_t *todo, *ntodo;
+    int32_t* todo;
+    int64_t* ntodo = d_cnt + HT_CNT_TODO;
     SNN_TRY(ar.alloc(&todo, V));
-    SNN_TRY(ar.alloc(&ntodo, 1));
-    SNN_CUDA(cudaMemsetAsync(ntodo, 0, sizeof(int32_t), s));
     SNN_L k_ht_skip<Pol><<<grid_for(V, 256), 256, 0, s>>>(pol, workv, todo, ntodo);
-    SNN_L k_ht_work<Pol><<<grid_for((int64_t)V * 32, 256), 256, 0, s>>>(pol, workv, todo, ntodo);
+    SNN_L k_ht_work<Pol><<<grid_for(V, 8), 256, 0, s>>>(pol, workv, todo, ntodo);
     SNN_CUDA(cudaGetLastError());
-    SNN_L k_ht_classify<Pol><<<grid_for(V, 256), 256, 0, s>>>(pol, workv, lists, d_cnt, scap, tiers);
+    SNN_L k_ht_classify<Pol><<<grid_for(V, 256), 256, 0, s>>>(pol, workv, lists, d_cnt, scap, tiers, dense_big);
     SNN_CUDA(cudaGetLastError());
     size_t wsm = (size_t)HT_WARPS * HT_WCAP * slot_bytes<S>();
     size_t bsm = (size_t)HT_BCAP * slot_bytes<S>();
@@ -939,15 +1106,32 @@ Status run_histogram(const Pol& pol, Arena& ar, cudaStream_t s, int64_t* d_cnt, 
     // set on every call: the attribute is per device, and handles on other
     // host threads may reach this point concurrently
     SNN_TRY(set_smem(k_ht_warp<Pol>, wsm));
-    SNN_TRY(set_smem(kb, bsm));
-    SNN_TRY(set_smem(kg, gsm));
     SNN_L k_ht_warp<Pol><<<(int)std::min<int64_t>(ceil_div(V, HT_WARPS), 152 * 8), HT_WARPS * 32, wsm,
                            s>>>(pol, lists, d_cnt, workv, scap);
     SNN_CUDA(cudaGetLastError());
-    SNN_L kb<<<(int)std::min<int64_t>(V, 152 * 8), HT_BTHREADS, bsm, s>>>(pol, lists, d_cnt, scap, workv);
+    const size_t dsm = (size_t)key_space * (sizeof(S) + sizeof(uint32_t));
+    int glog = 2;   // lanes per incidence: the level's mean hyperedge size
+    while (glog < 5 && (1 << glog) < hedge_lanes(pol.L.P, pol.L.E)) glog++;
+    if (dense_block) {
+        auto kd = k_ht_dense<Pol, HT_BTHREADS, HT_TIER_BLOCK>;
+        SNN_L kd<<<(int)std::min<int64_t>(V, 152 * 6), HT_BTHREADS, dsm, s>>>(pol, lists, d_cnt,
+                                                                              key_space, glog);
+    } else {
+        SNN_TRY(set_smem(kb, bsm));
+        SNN_L kb<<<(int)std::min<int64_t>(V, 152 * 8), HT_BTHREADS, bsm, s>>>(pol, lists, d_cnt, scap,
+                                                                              workv);
+    }
     SNN_CUDA(cudaGetLastError());
-    SNN_L kg<<<152, HT_GTHREADS, gsm, s>>>(pol, lists, d_cnt, scap, workv);
+    if (dense_big) {
+        auto kd = k_ht_dense<Pol, 1024, HT_TIER_BIG>;
+        SNN_TRY(set_smem(kd, (size_t)HT_DENSE_KEYS * (sizeof(S) + sizeof(uint32_t))));
+        SNN_L kd<<<(int)std::min<int64_t>(V, 152), 1024, dsm, s>>>(pol, lists, d_cnt, key_space, glog);
+    } else {
+        SNN_TRY(set_smem(kg, gsm));
+        SNN_L kg<<<152, HT_GTHREADS, gsm, s>>>(pol, lists, d_cnt, scap, workv);
+    }
     SNN_CUDA(cudaGetLastError());
+    if (!split) return Status{};
     SNN_CUDA(cudaMemcpyAsync(h_cnt, d_cnt + HT_TIER_SPLIT, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     SNN_CUDA(cudaStreamSynchronize(s));
     int64_t ns = h_cnt[0];

@@ -121,7 +121,8 @@ struct snnmap_hgraph {
     int64_t* h_scal = nullptr;   // pinned mirror
     // pinned: the counters of a level's neighbour histograms (two sets for the
     // carried form), copied without a wait and folded into the level's extra
-    // record once the stream has been synchronized (tier_fold)
+    // record once the stream has been synchronized (tier_fold); then 8 words
+    // for the carried form's estimates
     int64_t* h_tier = nullptr;
     int32_t tier_level = -1;     // level whose counters are in flight, else -1
     int32_t tier_form = 0;       // 1 full histogram, 2 carried form

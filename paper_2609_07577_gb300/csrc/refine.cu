@@ -392,19 +392,29 @@ struct GainPol {
         acc.W += L.hw[a];
         return g;
     }
-    template <class Tb>
-    __device__ bool elem(int32_t n, const Seg<S>& g, int32_t off, const Tb& t, Acc& acc) const
+    // one element: partition p (-1: nothing to add, -2: weight w to save)
+    struct Item {
+        int32_t p;
+        S w;
+        uint32_t o;
+    };
+    static __device__ Item none() { return Item{-1, 0, 0u}; }
+    __device__ Item load(int32_t n, const Seg<S>& g, int32_t off) const
     {
         int64_t e = g.b + off;
         int32_t p = pc.p[e];
-        if (p == rho[n]) {
-            if (pc.cnt[e] == 1) acc.save += (int64_t)g.w;
-            return true;
-        }
+        if (p == rho[n]) return Item{pc.cnt[e] == 1 ? -2 : -1, g.w, 0u};
         // a partition that cannot take n by size or inbound pins is never
         // the chosen move: leave it out of the table
-        if (ps.size[p] + L.vsize[n] > omega || ps.inpins[p] + L.vinpins[n] > phi) return true;
-        return t.add(p, g.w, (g.nd && pc.dcnt[e] > 0) ? g.k : 0u);
+        if (ps.size[p] + L.vsize[n] > omega || ps.inpins[p] + L.vinpins[n] > phi) return none();
+        return Item{p, g.w, (g.nd && pc.dcnt[e] > 0) ? g.k : 0u};
+    }
+    template <class Tb>
+    __device__ bool put(int32_t, const Item& it, const Tb& t, Acc& acc) const
+    {
+        if (it.p >= 0) return t.add(it.p, it.w, it.o);
+        if (it.p == -2) acc.save += (int64_t)it.w;
+        return true;
     }
     // gain = save - loss with loss = W - conn(p); feasible if p stays within
     // Omega, Phi, and Delta on its inbound set grown by n's axons not yet
@@ -502,11 +512,21 @@ struct RowPol {
         g.k = (uint32_t)L.hk[a];
         return g;
     }
-    template <class Tb>
-    __device__ bool elem(int32_t, const Seg<S>& g, int32_t off, const Tb& t, Acc&) const
+    struct Item {
+        int32_t p;
+        S w;
+        uint32_t o;
+    };
+    static __device__ Item none() { return Item{-1, 0, 0u}; }
+    __device__ Item load(int32_t, const Seg<S>& g, int32_t off) const
     {
         int64_t e = g.b + off;
-        return t.add(pc.p[e], g.w, (g.nd && pc.dcnt[e] > 0) ? g.k : 0u);
+        return Item{pc.p[e], g.w, (g.nd && pc.dcnt[e] > 0) ? g.k : 0u};
+    }
+    template <class Tb>
+    __device__ bool put(int32_t, const Item& it, const Tb& t, Acc&) const
+    {
+        return it.p < 0 || t.add(it.p, it.w, it.o);
     }
     // every key of the finished histogram lands in the row (stores, so a
     // vertex redone by a later tier overwrites its partial entries)
@@ -1520,7 +1540,8 @@ static Status gains(snnmap_hgraph* h, Level& L, const PinCounts& pc, const int32
     pol.pgain = pgain;
     int64_t* cnt;
     SNN_TRY(h->scratch.alloc(&cnt, HT_NCNT));
-    return run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->d_scal, h->tiers);
+    return run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->d_scal, h->tiers, K,
+                         !h->wzero);
 }
 
 // rows of the vertices flagged fresh, from the round's pin counts
@@ -1541,7 +1562,8 @@ static Status dense_fresh(snnmap_hgraph* h, Level& L, const PinCounts& pc)
     pol.cw = D.cw;
     int64_t* cnt;
     SNN_TRY(h->scratch.alloc(&cnt, HT_NCNT));
-    return run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->d_scal, h->tiers);
+    return run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->d_scal, h->tiers, D.K,
+                         !h->wzero);
 }
 
 int64_t dense_row_budget(const snnmap_hgraph* h)

@@ -61,13 +61,22 @@ struct ScorePol {
         g.k = (uint32_t)L.hk[a];
         return g;
     }
-    template <class Tb>
-    __device__ bool elem(int32_t n, const Seg<S>& g, int32_t off, const Tb& t, Acc&) const
+    struct Item {
+        int32_t m;
+        S w;
+        uint32_t o;
+    };
+    static __device__ Item none() { return Item{-1, 0, 0u}; }
+    __device__ Item load(int32_t n, const Seg<S>& g, int32_t off) const
     {
         int32_t m = L.hpins[g.b + off];
-        if (m == n) return true;
         int md = off != 0 || g.sd;   // pin 0 is the source
-        return t.add(m, g.w, (g.nd && md) ? g.k : 0u);
+        return Item{m == n ? -1 : m, g.w, (g.nd && md) ? g.k : 0u};
+    }
+    template <class Tb>
+    __device__ bool put(int32_t, const Item& it, const Tb& t, Acc&) const
+    {
+        return it.m < 0 || t.add(it.m, it.w, it.o);
     }
     // every neighbour lands in the row (stores: a vertex redone by a later
     // tier overwrites its partial entries)
@@ -81,30 +90,11 @@ struct ScorePol {
     __device__ void write(int32_t, int64_t, int32_t, uint32_t, const Acc&) const {}
 };
 
-__global__ void k_mat_min(Level L, int32_t* vmin)
-{
-    int32_t ms = 0x7fffffff, mi = 0x7fffffff;
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < L.V;
-         n += (int64_t)gridDim.x * blockDim.x) {
-        ms = min(ms, L.vsize[n]);
-        mi = min(mi, L.vinpins[n]);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        ms = min(ms, __shfl_xor_sync(FULL, ms, o));
-        mi = min(mi, __shfl_xor_sync(FULL, mi, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMin(&vmin[0], ms);
-        atomicMin(&vmin[1], mi);
-    }
-}
-
 // candidate of n: the valid neighbour with the largest score, ties to the
-// lower id (the rules of the histogram path, including its skip of vertices
-// that cannot merge even with the smallest vertex)
+// lower id (the rules of the histogram path; its skip of vertices that cannot
+// merge even with the smallest vertex finds nothing valid here either)
 __global__ void __launch_bounds__(256)
-    k_mat_best(Level L, const int32_t* __restrict__ vmin, const int32_t* __restrict__ Sm,
+    k_mat_best(Level L, const int32_t* __restrict__ Sm,
                const int32_t* __restrict__ OVm, int64_t Vs, int32_t omega, int32_t delta,
                int32_t phi, int32_t* cand, int64_t* cscore, int32_t* cov)
 {
@@ -116,7 +106,7 @@ __global__ void __launch_bounds__(256)
         int64_t r0 = n * Vs;
         int64_t bs = 0;
         int32_t bk = -1;
-        if (sz + vmin[0] <= omega && ip + vmin[1] <= phi) {
+        {
             const int4* row = reinterpret_cast<const int4*>(Sm + r0);
             for (int64_t q = lane; 4 * q < L.V; q += 32) {
                 int4 c4 = row[q];
@@ -165,36 +155,27 @@ __global__ void k_mat_reps(int32_t V, const int32_t* __restrict__ cid,
     }
 }
 
-// S2[i][j] = S[rep(i)][rep(j)] (one block per row)
+// S2[i][j] = S[rep(i)][rep(j)] (one block per row); rows of merged vertices
+// are cleared for their fresh sums
 __global__ void __launch_bounds__(256)
-    k_mat_gather(int32_t V2, const int32_t* __restrict__ repof, const int32_t* __restrict__ Sm,
+    k_mat_gather(int32_t V2, const int32_t* __restrict__ repof, const int32_t* __restrict__ fresh,
+                 const int32_t* __restrict__ Sm,
                  const int32_t* __restrict__ OVm, int64_t Vs, int32_t* S2, int32_t* OV2, int64_t Vs2)
 {
     for (int64_t i = blockIdx.x; i < V2; i += gridDim.x) {
         int64_t src = (int64_t)repof[i] * Vs;
         int64_t dst = i * Vs2;
+        if (fresh[i]) {
+            for (int64_t j = threadIdx.x; j < Vs2; j += blockDim.x) {
+                S2[dst + j] = 0;
+                OV2[dst + j] = 0;
+            }
+            continue;
+        }
         for (int64_t j = threadIdx.x; j < V2; j += blockDim.x) {
             int64_t c = repof[j];
             S2[dst + j] = Sm[src + c];
             OV2[dst + j] = OVm[src + c];
-        }
-    }
-}
-
-// rows of fresh vertices cleared (one warp per vertex)
-__global__ void k_mat_zero(int32_t V, const int32_t* __restrict__ fresh, int32_t* Sm, int32_t* OVm,
-                           int64_t Vs)
-{
-    int lane = threadIdx.x & 31;
-    int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t n = gw; n < V; n += nw) {
-        if (!fresh[n]) continue;
-        int4* s = reinterpret_cast<int4*>(Sm + n * Vs);
-        int4* o = reinterpret_cast<int4*>(OVm + n * Vs);
-        for (int64_t q = lane; q < Vs / 4; q += 32) {
-            s[q] = make_int4(0, 0, 0, 0);
-            o[q] = make_int4(0, 0, 0, 0);
         }
     }
 }
@@ -228,7 +209,8 @@ static Status mat_rows(snnmap_hgraph* h, const Level& L, const int32_t* fresh)
     pol.Vs = M.Vs;
     int64_t* cnt;
     SNN_TRY(h->scratch.alloc(&cnt, HT_NCNT));
-    return run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->d_scal, h->tiers);
+    return run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->d_scal, h->tiers, L.V,
+                         !h->wzero);
 }
 
 void mat_close(snnmap_hgraph* h)
@@ -280,13 +262,9 @@ Status mat_affinity(snnmap_hgraph* h, int32_t level, bool* done)
         SNN_TRY(mat_rows(h, L, nullptr));
         M.level = level;
     }
-    int32_t* vmin;
-    SNN_TRY(h->scratch.alloc(&vmin, 2));
-    SNN_TRY(fill_i32(vmin, 0x7fffffff, 2, s));
     if (L.V > 0) {
-        SNN_L k_mat_min<<<grid_for(L.V, 256), 256, 0, s>>>(L, vmin);
         SNN_L k_mat_best<<<grid_for((int64_t)L.V * 32, 256), 256, 0, s>>>(
-            L, vmin, M.S, M.OV, M.Vs, h->prm.omega, h->prm.delta, h->prm.phi, h->cand, h->cscore,
+            L, M.S, M.OV, M.Vs, h->prm.omega, h->prm.delta, h->prm.phi, h->cand, h->cscore,
             h->cov);
         SNN_CUDA(cudaGetLastError());
     }
@@ -321,15 +299,13 @@ Status mat_descend(snnmap_hgraph* h, int32_t src)
     }
     if (L.V > 0) {
         SNN_L k_mat_gather<<<(int)std::min<int64_t>(L.V, 152 * 16), 256, 0, s>>>(
-            L.V, repof, M.S, M.OV, M.Vs, M.S2, M.OV2, Vs2);
+            L.V, repof, fresh, M.S, M.OV, M.Vs, M.S2, M.OV2, Vs2);
         SNN_CUDA(cudaGetLastError());
     }
     std::swap(M.S, M.S2);
     std::swap(M.OV, M.OV2);
     M.Vs = Vs2;
     if (L.V > 0) {
-        SNN_L k_mat_zero<<<grid_for((int64_t)L.V * 32, 256), 256, 0, s>>>(L.V, fresh, M.S, M.OV, M.Vs);
-        SNN_CUDA(cudaGetLastError());
         SNN_TRY(mat_rows(h, L, fresh));
         SNN_L k_mat_mirror<<<grid_for((int64_t)L.V * 32, 256), 256, 0, s>>>(L.V, fresh, M.S, M.OV, M.Vs);
         SNN_CUDA(cudaGetLastError());
