@@ -475,9 +475,6 @@ __global__ void __cluster_dims__(RSC_CTAS, 1, 1) __launch_bounds__(RSC_THREADS)
 // hundred to a few thousand of each, and there even one launch of the radix
 // passes is a chain of barriers: 1,000 keys of 20 bits take 24 us in the
 // cluster form.
-constexpr int SB_MAX = 4096;
-constexpr int SB_THREADS = 1024;
-
 __global__ void __launch_bounds__(SB_THREADS)
     k_sort_block(uint64_t* keys, uint32_t* vals, int32_t n, int N, int ibits)
 {
@@ -487,24 +484,7 @@ __global__ void __launch_bounds__(SB_THREADS)
     for (int i = threadIdx.x; i < N; i += SB_THREADS)
         w[i] = i < n ? (keys[i] << ibits) | (uint64_t)i : ~0ull;
     __syncthreads();
-    // a warp's 32 pairs of a step with stride <= 32 lie in one aligned run of
-    // 64 words, so only longer strides need the whole block
-    for (int k = 2; k <= N; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int t = threadIdx.x; t < N / 2; t += SB_THREADS) {
-                int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
-                uint64_t a = w[i], b = w[i + j];
-                if ((a > b) == ((i & k) == 0)) {
-                    w[i] = b;
-                    w[i + j] = a;
-                }
-            }
-            // the next step's stride is j / 2, or k after the last of these
-            if (j > 32 || (j == 1 && k > 32)) __syncthreads();
-            else __syncwarp();
-        }
-    }
-    __syncthreads();
+    block_sort_words(w, N);
 #pragma unroll
     for (int r = 0; r < SB_MAX / SB_THREADS; r++) {
         int i = r * SB_THREADS + threadIdx.x;

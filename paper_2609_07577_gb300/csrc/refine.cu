@@ -30,6 +30,7 @@
 //      enacted.
 #include "histo.cuh"
 #include "internal.cuh"
+#include "scan.cuh"
 
 #include <algorithm>
 #include <climits>
@@ -38,16 +39,12 @@
 namespace snn {
 
 enum : int {
-    RS_M = SC_A,       // proposals
-    RS_MAXG = SC_B,    // largest proposed gain
     RS_BEST = SC_C,    // best valid prefix gain
     RS_ISTAR = SC_D,   // index of its last move
     RS_COST = SC_E,    // Conn at round start
     RS_NEV = SC_F,     // inbound events emitted
     RS_NHV = SC_G,     // hyperedges replayed by the block tier
-    RS_DEG = 8,        // incidences of proposing vertices
-    RS_ACT = 10,       // vertices evaluated
-    RS_MING = 11,      // smallest proposed gain (<= 0)
+    RS_NHL = 11,       // listed hyperedges (int32)
 };
 
 constexpr int REPLAY_WARP_MAX = 32;
@@ -114,13 +111,14 @@ struct PinCountJob {
     const int32_t* rho;
     PinCounts pc;
     int64_t* pincnt;
-    int64_t* cost;     // COST_SLOTS partial sums of Conn
+    int64_t* cost;     // partial sums of Conn, by hyperedge id & cost_mask
     // inbound axons per partition summed per block first (a sum never passes
     // the number of input hyperedges, so 32 bits hold it): a level adds one
     // term per partition a hyperedge reaches, all on the K words of pincnt.
     // 45,039 hyperedges on 111 partitions: 67 us a level without.
     static constexpr bool kShared = true;
     int32_t K = 0;     // words kept per block; 0: add to pincnt directly
+    int32_t cost_mask = COST_SLOTS - 1;
     uint32_t* acc = nullptr;
     __host__ __device__ int shared_words() const { return K; }
     __device__ void attach(uint32_t* w) { acc = K > 0 ? w : nullptr; }
@@ -187,7 +185,7 @@ struct PinCountJob {
         }
         if (lane == 0) {
             pc.lam[a] = R;
-            if (R > 1) atomicAdd((unsigned long long*)&cost[a & (COST_SLOTS - 1)], (unsigned long long)(hw[a] * (R - 1)));
+            if (R > 1) atomicAdd((unsigned long long*)&cost[a & cost_mask], (unsigned long long)(hw[a] * (R - 1)));
         }
     }
     __device__ void finish_thread(int32_t a, const uint32_t* s, int n, int st) const
@@ -216,7 +214,7 @@ struct PinCountJob {
             R++;
         }
         pc.lam[a] = R;
-        if (R > 1) atomicAdd((unsigned long long*)&cost[a & (COST_SLOTS - 1)], (unsigned long long)(hw[a] * (R - 1)));
+        if (R > 1) atomicAdd((unsigned long long*)&cost[a & cost_mask], (unsigned long long)(hw[a] * (R - 1)));
     }
 };
 
@@ -619,43 +617,31 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// Row updates for the enacted prefix: per hyperedge, the moves of its pins
-// with index <= i* give each touched partition's count after the prefix;
-// where cnt(p, e) crosses zero every pin's C[.][p] changes by omega(e), and
-// where dcnt(p, e) crosses zero every destination's O[.][p] by k(e). One
-// warp per hyperedge; buf (one word per pin) collects the enacted moves.
-__global__ void __launch_bounds__(256)
-    k_dense_cross(Level L, PinCounts pc, const int32_t* __restrict__ moveidx, Moves mv,
-                  const int64_t* __restrict__ scal, const int32_t* __restrict__ rowid, int32_t* C,
-                  int32_t* O, unsigned long long* M, int32_t cw, int64_t Kp, uint32_t* buf,
-                  HedgeList hl)
+struct RowsRef {
+    const int32_t* rowid;   // null: the level has no rows
+    int32_t *C, *O;
+    unsigned long long* M;
+    int32_t cw;
+    int64_t Kp;
+};
+
+// Row updates of hyperedge a for the enacted prefix (one warp): the moves of
+// its pins with index <= i* (buf[b .. b + m)) give each touched partition's
+// count after the prefix; where cnt(p, e) crosses zero every pin's C[.][p]
+// changes by omega(e), and where dcnt(p, e) crosses zero every
+// destination's O[.][p] by k(e).
+__device__ __forceinline__ void rows_cross(const Level& L, const PinCounts& pc, const Moves& mv,
+                                           const RowsRef& R, int32_t a, int64_t b, int64_t e, int sd,
+                                           int32_t lam, int64_t w, int32_t k, const uint32_t* buf,
+                                           int m)
 {
-    int64_t istar = scal[RS_BEST] > 0 ? scal[RS_ISTAR] : -1;
-    if (istar < 0) return;
-    int lane = threadIdx.x & 31;
-    unsigned lt = lanemask_lt();
-    int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    int32_t nh = *hl.n;
-    for (int64_t x = gw; x < nh; x += nw) {
-        int32_t a = hl.a[x];
-        int64_t b = L.hoff[a], e = L.hoff[a + 1];
-        int sd = L.hsd[a];
-        int m = 0;
-        for (int64_t cb = b; cb < e; cb += 32) {
-            int64_t j = cb + lane;
-            int32_t mi = -1;
-            if (j < e) mi = moveidx[L.hpins[j]];
-            bool ap = mi >= 0 && mi <= istar;
-            unsigned mk = __ballot_sync(FULL, ap);
-            if (ap) buf[b + m + __popc(mk & lt)] = ((uint32_t)mi << 1) | ((j != b || sd) ? 1u : 0u);
-            m += __popc(mk);
-        }
-        if (m == 0) continue;
-        __syncwarp();
-        int32_t lam = pc.lam[a];
-        int64_t w = L.hw[a];
-        int32_t k = L.hk[a];
+    const int lane = threadIdx.x & 31;
+    const int32_t* rowid = R.rowid;
+    int32_t *C = R.C, *O = R.O;
+    unsigned long long* M = R.M;
+    const int32_t cw = R.cw;
+    const int64_t Kp = R.Kp;
+    {
         for (int ib = 0; ib < m; ib += 32) {
             int ii = ib + lane;
             // up to two crossing records per lane: partition, C sign, O sign
@@ -1149,67 +1135,54 @@ __global__ void k_ps_reset(int32_t M, Moves mv, const int64_t* __restrict__ scal
 // ---------------------------------------------------------------------------
 // S8
 
-__global__ void k_prop_stats(Level L, const int32_t* __restrict__ pto,
-                             const int64_t* __restrict__ pgain,
-                             const int64_t* __restrict__ savev,
-                             const int32_t* __restrict__ dirty, int nonpos, int32_t* flag,
-                             int64_t* scal)
+// (proposals, their incidences, vertices evaluated) before each vertex: one
+// scan compacts the proposals in vertex order, keyed by bias - gain (gains
+// lie within the summed omega, so no pass is needed to find their range),
+// and counts what the round's buffers need
+struct PropSums {
+    int64_t m, deg, act;
+    __host__ __device__ PropSums() : m(0), deg(0), act(0) {}
+    __device__ PropSums(int64_t a, int64_t b, int64_t c) : m(a), deg(b), act(c) {}
+    __device__ PropSums operator+(const PropSums& o) const
+    {
+        return PropSums(m + o.m, deg + o.deg, act + o.act);
+    }
+};
+__device__ __forceinline__ PropSums scan_shfl_up(PropSums v, int o)
 {
-    int64_t mg = 0, ng = 0, deg = 0;
-    int act = 0;
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < L.V;
-         n += (int64_t)gridDim.x * blockDim.x) {
-        act += (nonpos || savev[n] > 0) && (!dirty || dirty[n]);
-        int f = pto[n] >= 0;
-        flag[n] = f;
-        if (f) {
-            mg = pgain[n] > mg ? pgain[n] : mg;
-            ng = pgain[n] < ng ? pgain[n] : ng;
-            deg += L.voff[n + 1] - L.voff[n];
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        int64_t m2 = __shfl_xor_sync(FULL, mg, o);
-        mg = m2 > mg ? m2 : mg;
-        int64_t n2 = __shfl_xor_sync(FULL, ng, o);
-        ng = n2 < ng ? n2 : ng;
-        deg += __shfl_xor_sync(FULL, deg, o);
-    }
-    act = warp_sum(act);
-    if ((threadIdx.x & 31) == 0) {
-        if (mg) atomicMax((unsigned long long*)&scal[RS_MAXG], (unsigned long long)mg);
-        if (deg) atomicAdd((unsigned long long*)&scal[RS_DEG], (unsigned long long)deg);
-        if (act) atomicAdd((unsigned long long*)&scal[RS_ACT], (unsigned long long)act);
-        if (ng < 0) atomicMin((long long*)&scal[RS_MING], (long long)ng);
-    }
+    return PropSums(__shfl_up_sync(FULL, v.m, o), __shfl_up_sync(FULL, v.deg, o),
+                    __shfl_up_sync(FULL, v.act, o));
 }
-
-__global__ void k_prop_keys(int32_t V, const int32_t* __restrict__ pto,
-                            const int64_t* __restrict__ pgain, const int32_t* __restrict__ pos,
-                            int64_t maxg, uint64_t* keys, uint32_t* vals)
+__device__ __forceinline__ PropSums scan_shfl(PropSums v, int src)
 {
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
-         n += (int64_t)gridDim.x * blockDim.x) {
-        if (pto[n] < 0) continue;
-        int32_t i = pos[n];
-        keys[i] = (uint64_t)(maxg - pgain[n]);
-        vals[i] = (uint32_t)n;
-    }
+    return PropSums(__shfl_sync(FULL, v.m, src), __shfl_sync(FULL, v.deg, src),
+                    __shfl_sync(FULL, v.act, src));
 }
-
-__global__ void k_moves(int32_t M, const uint32_t* __restrict__ vals, const int32_t* __restrict__ rho,
-                        const int32_t* __restrict__ pto, Moves mv, int32_t* moveidx)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < M;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t n = (int32_t)vals[i];
-        mv.n[i] = n;
-        mv.from[i] = rho[n];
-        mv.to[i] = pto[n];
-        moveidx[n] = (int32_t)i;
+struct PropIn {
+    const int32_t* pto;
+    const int64_t* savev;
+    const int32_t* dirty;
+    const int64_t* voff;
+    int nonpos;
+    __device__ PropSums operator()(int64_t n) const
+    {
+        bool f = pto[n] >= 0;
+        return PropSums(f, f ? voff[n + 1] - voff[n] : 0,
+                        (nonpos || savev[n] > 0) && (!dirty || dirty[n]));
     }
-}
+};
+struct PropOut {
+    const int64_t* pgain;
+    int64_t bias;
+    uint64_t* keys;
+    uint32_t* vals;
+    __device__ void operator()(int64_t n, PropSums ex, PropSums v) const
+    {
+        if (!v.m) return;
+        keys[ex.m] = (uint64_t)(bias - pgain[n]);
+        vals[ex.m] = (uint32_t)n;
+    }
+};
 
 // ---------------------------------------------------------------------------
 // The list of hyperedges holding a proposed move, from the proposers'
@@ -1230,17 +1203,6 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// the marks of the listed hyperedges back to zero for the next round
-__global__ void k_hedges_clear(HedgeList hl, int32_t* hmark, int32_t* hdirty)
-{
-    int32_t nh = *hl.n;
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < nh;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        hmark[hl.a[x]] = 0;
-        hdirty[hl.a[x]] = 0;
-    }
-}
-
 // ---------------------------------------------------------------------------
 // S9 / S10 events
 
@@ -1254,14 +1216,32 @@ struct Events {
     int ibits;
 };
 
-__global__ void k_size_events(int32_t M, Moves mv, Level L, Events ev)
+// the sorted moves: their arrays, cleared gains and violation changes, and
+// their size and inbound-pin events; and what the rounds keep per vertex (no
+// vertex flagged, the saves before the moves)
+__global__ void k_moves(int32_t M, const uint32_t* __restrict__ vals, const int32_t* __restrict__ rho,
+                        const int32_t* __restrict__ pto, Moves mv, int32_t* moveidx, Level L,
+                        Events ev, int64_t* gp, int32_t* dv, int32_t* dirty,
+                        const int64_t* __restrict__ savev, int64_t* save0)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < M;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t n = mv.n[i];
+    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t n = t0; n < L.V; n += step) {
+        dirty[n] = 0;
+        if (save0) save0[n] = savev[n];
+    }
+    for (int64_t i = t0; i < M; i += step) {
+        int32_t n = (int32_t)vals[i];
+        int32_t f = rho[n], t = pto[n];
+        mv.n[i] = n;
+        mv.from[i] = f;
+        mv.to[i] = t;
+        moveidx[n] = (int32_t)i;
+        gp[i] = 0;
+        dv[i] = 0;
         int64_t e0 = 2 * i, e1 = 2 * i + 1;
-        ev.key[e0] = ((uint64_t)mv.from[i] << ev.ibits) | (uint64_t)i;
-        ev.key[e1] = ((uint64_t)mv.to[i] << ev.ibits) | (uint64_t)i;
+        ev.key[e0] = ((uint64_t)f << ev.ibits) | (uint64_t)i;
+        ev.key[e1] = ((uint64_t)t << ev.ibits) | (uint64_t)i;
         ev.idx[e0] = (uint32_t)e0;
         ev.idx[e1] = (uint32_t)e1;
         ev.dsize[e0] = -L.vsize[n];
@@ -1504,17 +1484,160 @@ __global__ void k_best2(int32_t M, const int64_t* __restrict__ G, const int32_t*
         if (nviol[i] == 0 && G[i] == best) atomicMin((unsigned long long*)&scal[RS_ISTAR], (unsigned long long)i);
 }
 
-__global__ void k_apply(int32_t M, Moves mv, int32_t* rho, int32_t* moveidx, const int64_t* scal)
+// S10 and S11 in one block, for rounds whose events and moves fit its shared
+// memory: events sorted by (partition, move), each partition's limits after
+// each of its moves from a segmented scan, violation changes and gains
+// summed along the moves, and the best valid prefix. The event count stays
+// on the device, so a round takes no wait between replay and prefix; as
+// separate launches (sort, bounds, validity, two scans, two maxima, with the
+// wait before them) this was about 70 us of a round.
+struct Seg3 {
+    int64_t s, i, c;   // size, inbound pins, inbound axons
+    int head;          // the run started here
+};
+__device__ __forceinline__ Seg3 seg3_join(const Seg3& a, const Seg3& b)
 {
-    int64_t istar = scal[RS_BEST] > 0 ? scal[RS_ISTAR] : -1;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < M;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (i <= istar) rho[mv.n[i]] = mv.to[i];
-        moveidx[mv.n[i]] = -1;
+    if (b.head) return b;
+    return Seg3{a.s + b.s, a.i + b.i, a.c + b.c, a.head};
+}
+__device__ __forceinline__ Seg3 seg3_shfl_up(const Seg3& v, int o)
+{
+    return Seg3{__shfl_up_sync(FULL, v.s, o), __shfl_up_sync(FULL, v.i, o), __shfl_up_sync(FULL, v.c, o),
+                __shfl_up_sync(FULL, v.head, o)};
+}
+
+constexpr int TAIL_EVENTS = SB_MAX;
+constexpr int TAIL_PER = TAIL_EVENTS / SB_THREADS;   // consecutive events per thread
+
+__global__ void __launch_bounds__(SB_THREADS)
+    k_round_tail(int32_t M, Events ev, PState ps, int32_t omega, int32_t delta, int32_t phi,
+                 const int64_t* __restrict__ gp, int64_t* scal)
+{
+    __shared__ uint64_t w[TAIL_EVENTS];
+    __shared__ int32_t dv[TAIL_EVENTS / 2];   // two events per move at least
+    __shared__ Seg3 wseg[32];
+    __shared__ int64_t wg[32];
+    __shared__ int32_t wv[32];
+    __shared__ unsigned long long sbest;
+    __shared__ int simin;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int T = 2 * M + (int)scal[RS_NEV];   // <= TAIL_EVENTS (the events' capacity)
+    constexpr int IB = 12;
+    int N = 64;
+    while (N < T) N <<= 1;
+    for (int e = tid; e < N; e += SB_THREADS)
+        w[e] = e < T ? (ev.key[e] << IB) | (uint64_t)e : ~0ull;
+    for (int i = tid; i < M; i += SB_THREADS) dv[i] = 0;
+    if (tid == 0) {
+        sbest = 0;
+        simin = INT_MAX;
+    }
+    __syncthreads();
+    block_sort_words(w, N);
+    const uint64_t imask = (1ull << ev.ibits) - 1;
+    const int e0 = tid * TAIL_PER;
+    Seg3 v[TAIL_PER];
+    Seg3 run{0, 0, 0, 0};
+#pragma unroll
+    for (int r = 0; r < TAIL_PER; r++) {
+        int e = e0 + r;
+        Seg3 x{0, 0, 0, 0};
+        if (e < T) {
+            uint32_t o = (uint32_t)(w[e] & ((1u << IB) - 1));
+            uint64_t p = w[e] >> IB >> ev.ibits;
+            x = Seg3{ev.dsize[o], ev.dinp[o], ev.dpc[o], e == 0 || (w[e - 1] >> IB >> ev.ibits) != p};
+        }
+        run = r == 0 ? x : seg3_join(run, x);
+        v[r] = run;
+    }
+    Seg3 inc = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        Seg3 t = seg3_shfl_up(inc, o);
+        if (lane >= o) inc = seg3_join(t, inc);
+    }
+    if (lane == 31) wseg[warp] = inc;
+    __syncthreads();
+    if (warp == 0) {
+        Seg3 t = wseg[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            Seg3 u = seg3_shfl_up(t, o);
+            if (lane >= o) t = seg3_join(u, t);
+        }
+        wseg[lane] = t;
+    }
+    __syncthreads();
+    Seg3 before = seg3_shfl_up(inc, 1);
+    if (lane == 0) before = Seg3{0, 0, 0, 0};
+    if (warp > 0) before = lane == 0 ? wseg[warp - 1] : seg3_join(wseg[warp - 1], before);
+#pragma unroll
+    for (int r = 0; r < TAIL_PER; r++) {
+        int e = e0 + r;
+        if (e >= T) continue;
+        uint64_t key = w[e] >> IB, nxt = e + 1 < T ? w[e + 1] >> IB : ~0ull;
+        if (nxt == key) continue;   // the move has more events in this partition
+        Seg3 a = seg3_join(before, v[r]);
+        int32_t p = (int32_t)(key >> ev.ibits);
+        if (!violates(ps.size[p] + a.s, ps.inpins[p] + a.i, ps.pincnt[p] + a.c, omega, delta, phi))
+            continue;
+        // violated after this move until the partition's next one
+        atomicAdd(&dv[key & imask], 1);
+        if (e + 1 < T && (nxt >> ev.ibits) == (uint64_t)p) atomicAdd(&dv[nxt & imask], -1);
+    }
+    __syncthreads();
+    // prefix sums along the moves, two consecutive ones per thread
+    int64_t g[2];
+    int32_t d[2];
+#pragma unroll
+    for (int r = 0; r < 2; r++) {
+        int i = 2 * tid + r;
+        g[r] = i < M ? gp[i] : 0;
+        d[r] = i < M ? dv[i] : 0;
+    }
+    int64_t gi = warp_inclusive(g[0] + g[1]);
+    int32_t di = warp_inclusive(d[0] + d[1]);
+    if (lane == 31) {
+        wg[warp] = gi;
+        wv[warp] = di;
+    }
+    __syncthreads();
+    int64_t gb = gi - g[0] - g[1];
+    int32_t db = di - d[0] - d[1];
+    for (int x = 0; x < warp; x++) {
+        gb += wg[x];
+        db += wv[x];
+    }
+    int64_t G[2] = {gb + g[0], gb + g[0] + g[1]};
+    bool ok[2] = {2 * tid < M && db + d[0] == 0, 2 * tid + 1 < M && db + d[0] + d[1] == 0};
+    int64_t best = 0;
+    if (ok[0] && G[0] > best) best = G[0];
+    if (ok[1] && G[1] > best) best = G[1];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        int64_t b2 = __shfl_xor_sync(FULL, best, o);
+        best = b2 > best ? b2 : best;
+    }
+    if (lane == 0 && best > 0) atomicMax(&sbest, (unsigned long long)best);
+    __syncthreads();
+    best = (int64_t)sbest;
+    if (best <= 0) return;
+    if (ok[1] && G[1] == best) atomicMin(&simin, 2 * tid + 1);
+    if (ok[0] && G[0] == best) atomicMin(&simin, 2 * tid);
+    __syncthreads();
+    if (tid == 0) {
+        scal[RS_BEST] = best;
+        scal[RS_ISTAR] = simin;
     }
 }
 
-__global__ void k_round_init(int64_t* scal) { scal[RS_ISTAR] = INT64_MAX; }
+// the round's scalars: all zero but the prefix end (none) and Conn at its
+// start
+__global__ void k_round_begin(int64_t* scal, const int64_t* __restrict__ costv)
+{
+    int i = threadIdx.x;
+    if (i < SC_COUNT) scal[i] = i == RS_ISTAR ? INT64_MAX : (i == RS_COST ? *costv : 0);
+}
 
 // ---------------------------------------------------------------------------
 
@@ -1716,71 +1839,150 @@ Status level_cost(snnmap_hgraph* h, int32_t level, int32_t K, const int32_t* rho
 // pins and internal axons move between partitions, the hyperedges are
 // counted again, and their new contributions added back.
 
+// One warp per listed hyperedge: its enacted moves; if it holds any, its row
+// updates (levels with rows), its mark, and its old contributions out of the
+// partition state, Conn and the saves (the count pass adds the new ones).
 __global__ void __launch_bounds__(256)
-    k_pc_mark(Level L, const int32_t* __restrict__ moveidx, const int64_t* __restrict__ scal,
-              int32_t* hdirty, HedgeList hl)
+    k_prefix_hedges(Level L, PinCounts pc, const int32_t* __restrict__ moveidx, Moves mv,
+                    const int64_t* __restrict__ scal, RowsRef R, uint32_t* buf, int32_t* hdirty,
+                    const int32_t* __restrict__ rho, PState ps, int64_t* savev, int64_t* costv,
+                    HedgeList hl)
 {
     int64_t istar = scal[RS_BEST] > 0 ? scal[RS_ISTAR] : -1;
+    if (istar < 0) return;   // nothing is marked (the marks are cleared every round)
     int lane = threadIdx.x & 31;
+    unsigned lt = lanemask_lt();
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     int32_t nh = *hl.n;
     for (int64_t x = gw; x < nh; x += nw) {
         int32_t a = hl.a[x];
-        bool hit = false;
-        if (istar >= 0)
-            for (int64_t j = L.hoff[a] + lane; j < L.hoff[a + 1] && !hit; j += 32) {
-                int32_t mi = moveidx[L.hpins[j]];
-                if (mi >= 0 && mi <= istar) hit = true;
-            }
-        hit = __any_sync(FULL, hit);
-        if (lane == 0) hdirty[a] = hit ? 1 : 0;
-    }
-}
-
-// sign -1: remove the contributions of the marked hyperedges under the
-// current counts and rho; sign +1: add them
-__global__ void __launch_bounds__(256)
-    k_pc_contrib(Level L, PinCounts pc, const int32_t* __restrict__ hdirty,
-                 const int32_t* __restrict__ rho, PState ps, int64_t* savev, int64_t* costv,
-                 int sign, HedgeList hl)
-{
-    int lane = threadIdx.x & 31;
-    int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    int32_t nh = *hl.n;
-    for (int64_t x = gw; x < nh; x += nw) {
-        int32_t a = hl.a[x];
-        if (!hdirty[a]) continue;
         int64_t b = L.hoff[a], e = L.hoff[a + 1];
+        int sd = L.hsd[a];
+        int m = 0;
+        for (int64_t cb = b; cb < e; cb += 32) {
+            int64_t j = cb + lane;
+            int32_t mi = -1;
+            if (j < e) mi = moveidx[L.hpins[j]];
+            bool ap = mi >= 0 && mi <= istar;
+            unsigned mk = __ballot_sync(FULL, ap);
+            if (ap) buf[b + m + __popc(mk & lt)] = ((uint32_t)mi << 1) | ((j != b || sd) ? 1u : 0u);
+            m += __popc(mk);
+        }
+        if (m == 0) continue;
+        __syncwarp();
         int32_t lam = pc.lam[a];
         int64_t w = L.hw[a];
-        int64_t k = L.hk[a];
-        if (sign < 0) {
-            // the count pass adds inbound k and Conn itself for sign +1
-            for (int32_t r = lane; r < lam; r += 32)
-                if (pc.dcnt[b + r] > 0) atomicAdd((unsigned long long*)&ps.pincnt[pc.p[b + r]],
-                                                  (unsigned long long)(-k));
-            if (lane == 0 && lam > 1)
-                atomicAdd((unsigned long long*)costv, (unsigned long long)(-(w * (lam - 1))));
-        }
+        int32_t k = L.hk[a];
+        if (R.rowid) rows_cross(L, pc, mv, R, a, b, e, sd, lam, w, k, buf, m);
+        if (lane == 0) hdirty[a] = 1;
+        for (int32_t r = lane; r < lam; r += 32)
+            if (pc.dcnt[b + r] > 0)
+                atomicAdd((unsigned long long*)&ps.pincnt[pc.p[b + r]], (unsigned long long)(-(int64_t)k));
+        if (lane == 0 && lam > 1)
+            atomicAdd((unsigned long long*)costv, (unsigned long long)(-(w * (lam - 1))));
         for (int64_t j = b + lane; j < e; j += 32) {
-            int32_t x = L.hpins[j];
+            int32_t q = L.hpins[j];
             int32_t c, d;
-            lookup_count(pc, b, lam, rho[x], c, d);
-            if (c == 1) atomicAdd((unsigned long long*)&savev[x], (unsigned long long)(sign * w));
+            lookup_count(pc, b, lam, rho[q], c, d);
+            if (c == 1) atomicAdd((unsigned long long*)&savev[q], (unsigned long long)(-w));
         }
     }
 }
 
-// the enacted moves' own size, inbound pins and internal axons change
-// partition
-__global__ void k_ps_moves(int32_t M, Moves mv, Level L, const int64_t* __restrict__ scal, PState ps)
+// new contributions of hyperedge a to the saves (one warp)
+__device__ __forceinline__ void add_saves(const Level& L, const PinCounts& pc,
+                                          const int32_t* __restrict__ rho, int64_t* savev, int32_t a)
+{
+    const int lane = threadIdx.x & 31;
+    int64_t b = L.hoff[a], e = L.hoff[a + 1];
+    int32_t lam = pc.lam[a];
+    int64_t w = L.hw[a];
+    for (int64_t j = b + lane; j < e; j += 32) {
+        int32_t q = L.hpins[j];
+        int32_t c, d;
+        lookup_count(pc, b, lam, rho[q], c, d);
+        if (c == 1) atomicAdd((unsigned long long*)&savev[q], (unsigned long long)w);
+    }
+}
+
+// after the count pass over the size buckets: the saves of the marked
+// hyperedges, and the listed ones' marks back to zero for the next round
+__global__ void __launch_bounds__(256)
+    k_prefix_saves(Level L, PinCounts pc, const int32_t* __restrict__ rho, int64_t* savev,
+                   int32_t* hmark, int32_t* hdirty, HedgeList hl)
+{
+    int lane = threadIdx.x & 31;
+    int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    int32_t nh = *hl.n;
+    for (int64_t x = gw; x < nh; x += nw) {
+        int32_t a = hl.a[x];
+        if (hdirty[a]) add_saves(L, pc, rho, savev, a);
+        __syncwarp();
+        if (lane == 0) {
+            hmark[a] = 0;
+            hdirty[a] = 0;
+        }
+    }
+}
+
+// The count pass and the saves in one launch, a warp per listed hyperedge,
+// for short lists on levels without hyperedges of more than SEG_B1_CAP pins:
+// filtering the level's size buckets, counting them, and the two passes
+// after it were six launches over mostly a few hundred hyperedges.
+constexpr int64_t RECOUNT_MAX = 1 << 15;
+
+__global__ void __launch_bounds__(256)
+    k_prefix_recount(Level L, PinCountJob job, const int32_t* __restrict__ rho, int64_t* savev,
+                     int32_t* hmark, int32_t* hdirty, HedgeList hl)
+{
+    __shared__ __align__(16) uint32_t buf[8 * SEG_B1_CAP];
+    const int lane = threadIdx.x & 31;
+    uint32_t* s = buf + (threadIdx.x >> 5) * SEG_B1_CAP;
+    int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    int32_t nh = *hl.n;
+    for (int64_t x = gw; x < nh; x += nw) {
+        int32_t a = hl.a[x];
+        if (hdirty[a]) {
+            int n = job.len(a);
+            if (n <= 32) {
+                uint32_t v = lane < n ? job.load(a, lane) : KEY_PAD;
+                s[lane] = warp_bitonic32(v);
+                __syncwarp();
+            } else if (n <= 64) {
+                warp_sort_list<2>(job, a, n, s);
+            } else if (n <= 128) {
+                warp_sort_list<4>(job, a, n, s);
+            } else {
+                warp_sort_list<8>(job, a, n, s);
+            }
+            job.finish(a, s, n);
+            __syncwarp();
+            add_saves(L, job.pc, rho, savev, a);
+        }
+        __syncwarp();
+        if (lane == 0) {
+            hmark[a] = 0;
+            hdirty[a] = 0;
+        }
+    }
+}
+
+// the enacted moves: rho, and their own size, inbound pins and internal axons
+// change partition
+__global__ void k_apply(int32_t M, Moves mv, Level L, const int64_t* __restrict__ scal, PState ps,
+                        int32_t* rho, int32_t* moveidx)
 {
     int64_t istar = scal[RS_BEST] > 0 ? scal[RS_ISTAR] : -1;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= istar && i < M;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < M;
          i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t n = mv.n[i], f = mv.from[i], t = mv.to[i];
+        int32_t n = mv.n[i];
+        moveidx[n] = -1;
+        if (i > istar) continue;
+        int32_t f = mv.from[i], t = mv.to[i];
+        rho[n] = t;
         int64_t sz = L.vsize[n], ip = L.vinpins[n], ii = L.vinint[n];
         atomicAdd((unsigned long long*)&ps.size[f], (unsigned long long)(-sz));
         atomicAdd((unsigned long long*)&ps.size[t], (unsigned long long)sz);
@@ -1814,8 +2016,6 @@ __global__ void k_seg_meta_copy(const int32_t* __restrict__ meta, int32_t* meta2
 {
     for (int b = threadIdx.x; b < SEG_NB; b += blockDim.x) meta2[b] = meta[b];
 }
-
-__global__ void k_copy_i64(const int64_t* __restrict__ src, int64_t* dst) { *dst = *src; }
 
 // Per-level buffers that outlive a round: proposals (kept by vertices the
 // previous round did not touch), the vertices to evaluate, partition flags
@@ -1861,10 +2061,6 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     *rows = 0;
     *applied = 0;
     *gain = 0;
-    SNN_TRY(zero_scalars(h));
-    SNN_L k_round_init<<<1, 1, 0, s>>>(h->d_scal);
-    SNN_CUDA(cudaGetLastError());
-
     PinCounts pc = inc.pc;
     PState ps = inc.ps;
     {
@@ -1873,8 +2069,11 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
             SNN_CUDA(cudaMemsetAsync(inc.costv, 0, sizeof(int64_t), s));
             SNN_TRY(pin_counts_into(h, L, X, K, rho, pc, ps, inc.costv));
         }
-        SNN_L k_copy_i64<<<1, 1, 0, s>>>(inc.costv, h->d_scal + RS_COST);
-        SNN_L k_check_pstate<<<grid_for(K, 256), 256, 0, s>>>(K, ps, prm.omega, prm.delta, prm.phi, h->d_scal);
+        SNN_L k_round_begin<<<1, 32, 0, s>>>(h->d_scal, inc.costv);
+        // an enacted prefix is valid: the state can only be broken at the start
+        if (!inc.ready)
+            SNN_L k_check_pstate<<<grid_for(K, 256), 256, 0, s>>>(K, ps, prm.omega, prm.delta, prm.phi,
+                                                                 h->d_scal);
         SNN_CUDA(cudaGetLastError());
     }
     DenseRows& D = h->dense;
@@ -1887,11 +2086,8 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     }
     int32_t* pto = inc.pto;
     int64_t* pgain = inc.pgain;
-    int32_t *flag, *pos;
     int64_t* savev = inc.savev;
     int64_t* Wv = inc.Wv;
-    SNN_TRY(ar.alloc(&flag, V));
-    SNN_TRY(ar.alloc(&pos, V));
     if (!inc.ready) {
         prof.reset(new ProfScope(h, PS_SAVE));
         SNN_CUDA(cudaMemsetAsync(savev, 0, (size_t)(V > 0 ? V : 1) * 8, s));
@@ -1930,63 +2126,44 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
         SNN_TRY(gains<uint32_t>(h, L, pc, rho, ps, K, pto, pgain, savev, inc.dirty));
     }
     int gv = grid_for(V, 256);
-    SNN_L k_prop_stats<<<gv, 256, 0, s>>>(L, pto, pgain, savev, dense ? nullptr : inc.dirty,
-                                          prm.refine_nonpositive, flag, h->d_scal);
-    SNN_CUDA(cudaGetLastError());
-    SNN_TRY(scan_exclusive_i32(flag, pos, V, (int32_t*)(h->d_scal + RS_M), ar, s));
+    uint64_t *keys, *keys2;
+    uint32_t *vals, *vals2;
+    SNN_TRY(ar.alloc(&keys, V));
+    SNN_TRY(ar.alloc(&vals, V));
+    PropSums* sums;
+    SNN_TRY(ar.alloc(&sums, 1));
+    const int64_t bias = h->wsum;   // gains lie in [-wsum, wsum]
+    SNN_TRY(scan_run<PropSums>(PropIn{pto, savev, dense ? nullptr : inc.dirty, L.voff,
+                                      prm.refine_nonpositive},
+                               PropOut{pgain, bias, keys, vals}, V, sums, ar, s));
     prof.reset();
+    SNN_CUDA(cudaMemcpyAsync(h->h_tier + 2 * TIER_SLOTS, sums, sizeof(PropSums), cudaMemcpyDeviceToHost, s));
     SNN_TRY(read_scalars(h));
+    const int64_t* hs = h->h_tier + 2 * TIER_SLOTS;
     *cost = h->h_scal[RS_COST];
-    *n_active = (int32_t)h->h_scal[RS_ACT];
+    *n_active = (int32_t)hs[2];
     *rows = dense ? 1 : 0;
     if (h->h_scal[SC_STATUS] & ST_BADSTATE)
         return Status{SNNMAP_ERR_INVALID, "refinement input breaks a per-core limit"};
-    int32_t M = (int32_t)(h->h_scal[RS_M] & 0xffffffff);
-    int64_t maxg = h->h_scal[RS_MAXG];
-    int64_t ming = h->h_scal[RS_MING];   // <= 0: keys maxg - gain span maxg - ming
-    int64_t deg = h->h_scal[RS_DEG];
+    int32_t M = (int32_t)hs[0];
+    int64_t deg = hs[1];
     *n_props = M;
     if (M == 0) return Status{};
 
     // S8
     prof.reset(new ProfScope(h, PS_SORTMOVES));
-    uint64_t *keys, *keys2;
-    uint32_t *vals, *vals2;
-    SNN_TRY(ar.alloc(&keys, M));
     SNN_TRY(ar.alloc(&keys2, M));
-    SNN_TRY(ar.alloc(&vals, M));
     SNN_TRY(ar.alloc(&vals2, M));
-    SNN_L k_prop_keys<<<gv, 256, 0, s>>>(V, pto, pgain, pos, maxg, keys, vals);
-    SNN_CUDA(cudaGetLastError());
-    SNN_TRY(radix_sort_pairs(keys, vals, keys2, vals2, M, bits_for((uint64_t)(maxg - ming)), ar, s));
+    SNN_TRY(radix_sort_pairs(keys, vals, keys2, vals2, M, bits_for(2 * (uint64_t)bias), ar, s));
     Moves mv;
     SNN_TRY(ar.alloc(&mv.n, M));
     SNN_TRY(ar.alloc(&mv.from, M));
     SNN_TRY(ar.alloc(&mv.to, M));
     int gm = grid_for(M, 256);
-    SNN_L k_moves<<<gm, 256, 0, s>>>(M, vals, rho, pto, mv, moveidx);
-    SNN_CUDA(cudaGetLastError());
-    // the hyperedges holding a proposed move
-    int64_t nhl = std::max<int64_t>(1, std::min<int64_t>(L.E, deg));
-    int32_t *hla, *hln;
-    SNN_TRY(ar.alloc(&hla, nhl));
-    SNN_TRY(ar.alloc(&hln, 1));
-    SNN_CUDA(cudaMemsetAsync(hln, 0, sizeof(int32_t), s));
-    SNN_L k_prop_hedges<<<grid_for((int64_t)M * 32, 256), 256, 0, s>>>(M, mv, L, inc.hmark, hla, hln);
-    SNN_CUDA(cudaGetLastError());
-    HedgeList hl{hla, hln};
-    const int ghl = grid_for(nhl * 32, 256);
-
-    // S9
-    prof.reset(new ProfScope(h, PS_REPLAY));
     int64_t *gp, *G;
     int32_t *dv, *nviol;
     SNN_TRY(ar.alloc(&gp, M));
-    SNN_TRY(ar.alloc(&G, M));
     SNN_TRY(ar.alloc(&dv, M));
-    SNN_TRY(ar.alloc(&nviol, M));
-    SNN_CUDA(cudaMemsetAsync(gp, 0, (size_t)M * 8, s));
-    SNN_CUDA(cudaMemsetAsync(dv, 0, (size_t)M * 4, s));
     Events ev;
     ev.cap = 2 * (int64_t)M + 2 * deg;
     ev.ibits = bits_for((uint64_t)M);
@@ -1995,74 +2172,83 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     SNN_TRY(ar.alloc(&ev.dsize, ev.cap));
     SNN_TRY(ar.alloc(&ev.dinp, ev.cap));
     SNN_TRY(ar.alloc(&ev.dpc, ev.cap));
-    SNN_L k_size_events<<<gm, 256, 0, s>>>(M, mv, L, ev);
+    SNN_L k_moves<<<std::max(gm, gv), 256, 0, s>>>(M, vals, rho, pto, mv, moveidx, L, ev, gp, dv,
+                                                   inc.dirty, savev, inc.pst.save0);
     SNN_CUDA(cudaGetLastError());
+    // the hyperedges holding a proposed move
+    int64_t nhl = std::max<int64_t>(1, std::min<int64_t>(L.E, deg));
+    int32_t* hla;
+    int32_t* hln = (int32_t*)(h->d_scal + RS_NHL);
+    SNN_TRY(ar.alloc(&hla, nhl));
+    SNN_L k_prop_hedges<<<grid_for((int64_t)M * 32, 256), 256, 0, s>>>(M, mv, L, inc.hmark, hla, hln);
+    SNN_CUDA(cudaGetLastError());
+    HedgeList hl{hla, hln};
+    const int ghl = grid_for(nhl * 32, 256);
+
+    // S9
+    prof.reset(new ProfScope(h, PS_REPLAY));
     uint32_t* mvbuf;
     int32_t *hv, *hvc;
     SNN_TRY(ar.alloc(&mvbuf, L.P));
     SNN_TRY(ar.alloc(&hv, L.E));
     SNN_TRY(ar.alloc(&hvc, L.E));
+    const bool heavy = X.seg.n[SEG_BB1] + X.seg.n[SEG_BB2] + X.seg.n[SEG_BB3] > 0;
     if (L.E > 0) {
         SNN_L k_replay_warp<<<ghl, 256, 0, s>>>(L, pc, moveidx, mv, mvbuf, gp, ev, 2 * (int64_t)M, hv,
                                                 hvc, h->d_scal, hl);
-        SNN_CUDA(cudaGetLastError());
-        SNN_L k_replay_block<<<152 * 2, 256, 0, s>>>(L, pc, mv, mvbuf, gp, ev, 2 * (int64_t)M, hv, hvc,
-                                               h->d_scal);
+        // only a hyperedge of more than REPLAY_WARP_MAX pins holds more moves
+        if (heavy)
+            SNN_L k_replay_block<<<152 * 2, 256, 0, s>>>(L, pc, mv, mvbuf, gp, ev, 2 * (int64_t)M, hv, hvc,
+                                                   h->d_scal);
         SNN_CUDA(cudaGetLastError());
     }
-    prof.reset();
-    SNN_TRY(read_scalars(h));
-    if (h->h_scal[SC_STATUS] & ST_CAPACITY) return Status{SNNMAP_ERR_CUDA, "event buffer overflow"};
-    int64_t T = 2 * (int64_t)M + h->h_scal[RS_NEV];
-
-    // S10
-    prof.reset(new ProfScope(h, PS_VALIDITY));
-    uint64_t* ekey2;
-    uint32_t* eidx2;
-    SNN_TRY(ar.alloc(&ekey2, T));
-    SNN_TRY(ar.alloc(&eidx2, T));
-    int kbits = bits_for((uint64_t)K);
-    SNN_TRY(radix_sort_pairs(ev.key, ev.idx, ekey2, eidx2, T, ev.ibits + kbits, ar, s));
-    int32_t *pbeg, *pend;
-    SNN_TRY(ar.alloc(&pbeg, K));
-    SNN_TRY(ar.alloc(&pend, K));
-    SNN_CUDA(cudaMemsetAsync(pbeg, 0, (size_t)K * 4, s));
-    SNN_CUDA(cudaMemsetAsync(pend, 0, (size_t)K * 4, s));
-    SNN_L k_part_bounds<<<grid_for(T, 256), 256, 0, s>>>(T, ev.key, ev.ibits, pbeg, pend);
-    SNN_CUDA(cudaGetLastError());
-    SNN_L k_part_validity<<<grid_for((int64_t)K * 32, 256), 256, 0, s>>>(K, pbeg, pend, ev, ps, prm.omega,
-                                                                  prm.delta, prm.phi, dv);
-    SNN_CUDA(cudaGetLastError());
-
-    // S11
-    prof.reset(new ProfScope(h, PS_APPLY));
-    SNN_TRY(scan_inclusive_i64(gp, G, M, ar, s));
-    SNN_TRY(scan_inclusive_i32(dv, nviol, M, ar, s));
-    SNN_L k_best1<<<gm, 256, 0, s>>>(M, G, nviol, h->d_scal);
-    SNN_L k_best2<<<gm, 256, 0, s>>>(M, G, nviol, h->d_scal);
-    if (dense && L.E > 0) {
-        prof.reset(new ProfScope(h, PS_CROSS));
-        SNN_L k_dense_cross<<<ghl, 256, 0, s>>>(L, pc, moveidx, mv, h->d_scal, D.rowid, D.C, D.O,
-                                                D.M, D.cw, D.Kp, mvbuf, hl);
-        prof.reset(new ProfScope(h, PS_APPLY));
-    }
-    if (dense) {
-        // P* of the enacted prefix; k_ps_rows below decides the next round's
-        // proposals from the rows
-        SNN_CUDA(cudaMemsetAsync(inc.dirty, 0, (size_t)(V > 0 ? V : 1) * 4, s));
-        SNN_L k_ps_slots<<<gm, 256, 0, s>>>(M, mv, h->d_scal, inc.pst, inc.dirty);
+    if (ev.cap <= TAIL_EVENTS) {
+        // S10, S11
+        prof.reset(new ProfScope(h, PS_VALIDITY));
+        SNN_L k_round_tail<<<1, SB_THREADS, 0, s>>>(M, ev, ps, prm.omega, prm.delta, prm.phi, gp, h->d_scal);
         SNN_CUDA(cudaGetLastError());
-        if (inc.pst.save0 && V > 0)
-            SNN_CUDA(cudaMemcpyAsync(inc.pst.save0, savev, (size_t)V * 8, cudaMemcpyDeviceToDevice, s));
     } else {
-        // vertices the enacted prefix can affect, for the next round
-        SNN_CUDA(cudaMemsetAsync(inc.dirty, 0, (size_t)(V > 0 ? V : 1) * 4, s));
+        prof.reset();
+        SNN_TRY(read_scalars(h));
+        if (h->h_scal[SC_STATUS] & ST_CAPACITY) return Status{SNNMAP_ERR_CUDA, "event buffer overflow"};
+        int64_t T = 2 * (int64_t)M + h->h_scal[RS_NEV];
+
+        // S10
+        prof.reset(new ProfScope(h, PS_VALIDITY));
+        uint64_t* ekey2;
+        uint32_t* eidx2;
+        SNN_TRY(ar.alloc(&ekey2, T));
+        SNN_TRY(ar.alloc(&eidx2, T));
+        int kbits = bits_for((uint64_t)K);
+        SNN_TRY(radix_sort_pairs(ev.key, ev.idx, ekey2, eidx2, T, ev.ibits + kbits, ar, s));
+        int32_t *pbeg, *pend;
+        SNN_TRY(ar.alloc(&pbeg, 2 * (int64_t)K));
+        pend = pbeg + K;
+        SNN_CUDA(cudaMemsetAsync(pbeg, 0, (size_t)K * 8, s));
+        SNN_L k_part_bounds<<<grid_for(T, 256), 256, 0, s>>>(T, ev.key, ev.ibits, pbeg, pend);
+        SNN_CUDA(cudaGetLastError());
+        SNN_L k_part_validity<<<grid_for((int64_t)K * 32, 256), 256, 0, s>>>(K, pbeg, pend, ev, ps, prm.omega,
+                                                                      prm.delta, prm.phi, dv);
+        SNN_CUDA(cudaGetLastError());
+
+        // S11
+        prof.reset(new ProfScope(h, PS_APPLY));
+        SNN_TRY(ar.alloc(&G, M));
+        SNN_TRY(ar.alloc(&nviol, M));
+        SNN_TRY(scan_inclusive_i64(gp, G, M, ar, s));
+        SNN_TRY(scan_inclusive_i32(dv, nviol, M, ar, s));
+        SNN_L k_best1<<<gm, 256, 0, s>>>(M, G, nviol, h->d_scal);
+        SNN_L k_best2<<<gm, 256, 0, s>>>(M, G, nviol, h->d_scal);
+    }
+    prof.reset(new ProfScope(h, PS_APPLY));
+    // P* of the enacted prefix; when it is short, the rows (k_ps_rows) or the
+    // column update after the pin counts below decide the next round's
+    // proposals, otherwise the flags of the three rules here do
+    SNN_L k_ps_slots<<<gm, 256, 0, s>>>(M, mv, h->d_scal, inc.pst, inc.dirty);
+    SNN_CUDA(cudaGetLastError());
+    if (!dense && (!inc.pst.colc || 2 * (int64_t)M > PSTAR_MAX)) {
         SNN_CUDA(cudaMemsetAsync(inc.pchg, 0, (size_t)(K > 0 ? K : 1), s));
         SNN_CUDA(cudaMemsetAsync(inc.prel, 0, (size_t)(K > 0 ? K : 1), s));
-        // P* of the enacted prefix; when it is short the column update after
-        // the pin counts below decides the next round's proposals, otherwise
-        // the flags of the three rules below do
-        SNN_L k_ps_slots<<<gm, 256, 0, s>>>(M, mv, h->d_scal, inc.pst, inc.dirty);
         SNN_L k_inc_parts<<<gm, 256, 0, s>>>(M, mv, h->d_scal, ps, inc.vmax, prm.omega, prm.delta,
                                              prm.phi, inc.pchg, inc.prel, inc.pst.cnt);
         if (L.E > 0)
@@ -2070,37 +2256,41 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
                 L, pc, moveidx, mv, h->d_scal, inc.prel, mvbuf, inc.dirty, inc.pst.cnt);
         SNN_L k_inc_targets<<<gv, 256, 0, s>>>(V, pto, inc.pchg, inc.dirty, inc.pst.cnt);
         SNN_CUDA(cudaGetLastError());
-        if (inc.pst.save0 && V > 0)
-            SNN_CUDA(cudaMemcpyAsync(inc.pst.save0, savev, (size_t)V * 8, cudaMemcpyDeviceToDevice, s));
     }
     // carried pin counts: take out the hyperedges the prefix touches (old
     // counts, old rho), move, count them again, add them back
     prof.reset(new ProfScope(h, PS_PINCOUNT));
     if (L.E > 0) {
-        SNN_L k_pc_mark<<<ghl, 256, 0, s>>>(L, moveidx, h->d_scal, inc.hdirty, hl);
-        SNN_L k_pc_contrib<<<ghl, 256, 0, s>>>(L, pc, inc.hdirty, rho, ps, savev, inc.costv, -1, hl);
+        RowsRef R{dense ? D.rowid : nullptr, D.C, D.O, D.M, D.cw, D.Kp};
+        SNN_L k_prefix_hedges<<<ghl, 256, 0, s>>>(L, pc, moveidx, mv, h->d_scal, R, mvbuf, inc.hdirty, rho,
+                                                  ps, savev, inc.costv, hl);
         SNN_CUDA(cudaGetLastError());
     }
-    SNN_L k_ps_moves<<<gm, 256, 0, s>>>(M, mv, L, h->d_scal, ps);
-    SNN_L k_apply<<<gm, 256, 0, s>>>(M, mv, rho, moveidx, h->d_scal);
+    SNN_L k_apply<<<gm, 256, 0, s>>>(M, mv, L, h->d_scal, ps, rho, moveidx);
     SNN_CUDA(cudaGetLastError());
     if (L.E > 0) {
-        SNN_CUDA(cudaMemsetAsync(inc.hmeta, 0, 2 * SEG_NB * sizeof(int32_t), s));
-        SNN_L k_seg_meta_copy<<<1, 32, 0, s>>>(X.seg.meta, inc.hmeta);
-        SNN_L k_seg_filter<<<grid_for(L.E, 256), 256, 0, s>>>(X.seg.list, X.seg.meta, L.E, inc.hdirty,
-                                                             inc.hlist, inc.hmeta);
-        SNN_CUDA(cudaGetLastError());
-        SegBuckets db = X.seg;
-        db.list = inc.hlist;
-        db.meta = inc.hmeta;
-        int64_t* slots;
-        SNN_TRY(ar.alloc(&slots, COST_SLOTS));
-        SNN_CUDA(cudaMemsetAsync(slots, 0, COST_SLOTS * sizeof(int64_t), s));
-        PinCountJob job{L.hoff, L.hpins, L.hsd, L.hk, L.hw, rho, pc, ps.pincnt, slots};
-        SNN_TRY(seg_run(job, db, L.E, ar, s));
-        SNN_L k_cost_slots<<<1, 256, 0, s>>>(slots, inc.costv);
-        SNN_L k_pc_contrib<<<ghl, 256, 0, s>>>(L, pc, inc.hdirty, rho, ps, savev, inc.costv, 1, hl);
-        SNN_L k_hedges_clear<<<grid_for(nhl, 256), 256, 0, s>>>(hl, inc.hmark, inc.hdirty);
+        PinCountJob job{L.hoff, L.hpins, L.hsd, L.hk, L.hw, rho, pc, ps.pincnt, inc.costv};
+        job.cost_mask = 0;
+        if (nhl <= RECOUNT_MAX && X.seg.n[SEG_BB2] + X.seg.n[SEG_BB3] == 0) {
+            SNN_L k_prefix_recount<<<ghl, 256, 0, s>>>(L, job, rho, savev, inc.hmark, inc.hdirty, hl);
+        } else {
+            SNN_CUDA(cudaMemsetAsync(inc.hmeta, 0, 2 * SEG_NB * sizeof(int32_t), s));
+            SNN_L k_seg_meta_copy<<<1, 32, 0, s>>>(X.seg.meta, inc.hmeta);
+            SNN_L k_seg_filter<<<grid_for(L.E, 256), 256, 0, s>>>(X.seg.list, X.seg.meta, L.E, inc.hdirty,
+                                                                 inc.hlist, inc.hmeta);
+            SNN_CUDA(cudaGetLastError());
+            SegBuckets db = X.seg;
+            db.list = inc.hlist;
+            db.meta = inc.hmeta;
+            int64_t* slots;
+            SNN_TRY(ar.alloc(&slots, COST_SLOTS));
+            SNN_CUDA(cudaMemsetAsync(slots, 0, COST_SLOTS * sizeof(int64_t), s));
+            job.cost = slots;
+            job.cost_mask = COST_SLOTS - 1;
+            SNN_TRY(seg_run(job, db, L.E, ar, s));
+            SNN_L k_cost_slots<<<1, 256, 0, s>>>(slots, inc.costv);
+            SNN_L k_prefix_saves<<<ghl, 256, 0, s>>>(L, pc, rho, savev, inc.hmark, inc.hdirty, hl);
+        }
         SNN_CUDA(cudaGetLastError());
     }
     if (!dense) {
@@ -2125,6 +2315,7 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     }
     prof.reset();
     SNN_TRY(read_scalars(h));
+    if (h->h_scal[SC_STATUS] & ST_CAPACITY) return Status{SNNMAP_ERR_CUDA, "event buffer overflow"};
     int64_t best = h->h_scal[RS_BEST];
     int64_t istar = h->h_scal[RS_ISTAR];
     if (best > 0 && istar < M) {
@@ -2206,112 +2397,121 @@ void carry_close(snnmap_hgraph* h)
     C = Carry{};
 }
 
+// no move listed, every vertex to evaluate (unless inherited), no slot taken
+__global__ void k_refine_init(int32_t V, int32_t K, int32_t* moveidx, int32_t* dirty, PStar ps,
+                              int32_t base)
+{
+    int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t n = t0; n < V; n += step) {
+        moveidx[n] = -1;
+        if (dirty) dirty[n] = 1;
+    }
+    for (int64_t p = t0; p < K; p += step) ps.pslot[p] = -1;
+    if (t0 < 4) ps.cnt[t0] = (t0 & 1) ? 0 : base;
+}
+
 Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, int64_t* cost,
                     int64_t* cost_start)
 {
     Level& L = h->levels[level];
     cudaStream_t s = h->stream;
-    size_t nv = (size_t)(L.V > 0 ? L.V : 1), nk = (size_t)(K > 0 ? K : 1);
     int32_t* moveidx;
     IncState inc;
+    PStar& pst = inc.pst;
     Carry& CA = h->carry;
     const bool dense_level = h->dense.C && h->dense.level == level;
     const bool use_carry = CA.pto[0] && L.V <= CA.cap;
+    const int64_t V = L.V, E = L.E;
     bool inherited = false;
-    SNN_CUDA(dev_malloc(&moveidx, nv * sizeof(int32_t), s));
-    if (use_carry) {
-        int nb = 1 - CA.cur;
-        inc.pto = CA.pto[nb];
-        inc.pgain = CA.pgain[nb];
-        inc.dirty = CA.dirty[nb];
-        if (!dense_level && CA.level == level + 1 && L.V > 0) {
-            const Level& Lc = h->levels[level + 1];
-            int32_t* mcount;
-            SNN_TRY(h->scratch.alloc(&mcount, Lc.V));
-            SNN_CUDA(cudaMemsetAsync(mcount, 0, (size_t)(Lc.V > 0 ? Lc.V : 1) * 4, s));
-            SNN_L k_carry_count<<<grid_for(L.V, 256), 256, 0, s>>>(L.V, L.cid, mcount);
-            SNN_L k_carry<<<grid_for(L.V, 256), 256, 0, s>>>(L.V, L.cid, mcount, CA.pto[CA.cur],
-                                                            CA.pgain[CA.cur], CA.dirty[CA.cur],
-                                                            inc.pto, inc.pgain, inc.dirty);
-            SNN_CUDA(cudaGetLastError());
-            inherited = true;
-        }
-        CA.cur = nb;
-        CA.level = -1;
+    // the level's buffers, one allocation: the cleared ones first
+    Carver cv;
+    cv.add(&inc.hdirty, E);
+    cv.add(&inc.hmark, E);
+    cv.add(&inc.vmax, 3);
+    const size_t cleared = cv.total;
+    cv.add(&moveidx, V);
+    if (!use_carry) {
+        cv.add(&inc.pto, V);
+        cv.add(&inc.pgain, V);
+        cv.add(&inc.dirty, V);
+    }
+    cv.add(&inc.pchg, K);
+    cv.add(&inc.prel, K);
+    cv.add(&inc.pc.p, L.P);
+    cv.add(&inc.pc.cnt, L.P);
+    cv.add(&inc.pc.dcnt, L.P);
+    cv.add(&inc.pc.lam, E);
+    cv.add(&inc.ps.size, K);
+    cv.add(&inc.ps.inpins, K);
+    cv.add(&inc.ps.pincnt, K);
+    cv.add(&inc.costv, 1);
+    cv.add(&inc.savev, V);
+    cv.add(&inc.Wv, V);
+    cv.add(&inc.hlist, E);
+    cv.add(&inc.hmeta, 2 * SEG_NB);
+    cv.add(&pst.pslot, K);
+    cv.add(&pst.slots, PSTAR_MAX);
+    cv.add(&pst.cnt, 4);
+    void* block = nullptr;
+    SNN_CUDA(dev_malloc(&block, cv.total, s));
+    cv.assign(block);
+    // optional buffers. Rows levels need only the round-start saves besides
+    // the slot map; the others the columns too: without them every round
+    // takes the flag rules
+    Carver co;
+    size_t ccleared = 0;
+    if (!dense_level) {
+        co.add(&pst.hmask, E);
+        co.add(&pst.vt, V);
+        co.add(&pst.colc, (int64_t)PSTAR_MAX * V);
+        co.add(&pst.colo, (int64_t)PSTAR_MAX * V);
+        ccleared = co.total;
+        co.add(&pst.hl, E);
+    }
+    co.add(&pst.save0, V);
+    void* cols = nullptr;
+    if (dev_malloc(&cols, co.total, s) == cudaSuccess) {
+        co.assign(cols);
     } else {
-        SNN_CUDA(dev_malloc(&inc.pto, nv * 4, s));
-        SNN_CUDA(dev_malloc(&inc.pgain, nv * 8, s));
-        SNN_CUDA(dev_malloc(&inc.dirty, nv * 4, s));
+        cudaGetLastError();
+        cols = nullptr;
     }
-    SNN_CUDA(dev_malloc(&inc.pchg, nk, s));
-    SNN_CUDA(dev_malloc(&inc.prel, nk, s));
-    SNN_CUDA(dev_malloc(&inc.vmax, 3 * 4, s));
-    size_t np = (size_t)(L.P > 0 ? L.P : 1), ne = (size_t)(L.E > 0 ? L.E : 1);
-    SNN_CUDA(dev_malloc(&inc.pc.p, np * 4, s));
-    SNN_CUDA(dev_malloc(&inc.pc.cnt, np * 4, s));
-    SNN_CUDA(dev_malloc(&inc.pc.dcnt, np * 4, s));
-    SNN_CUDA(dev_malloc(&inc.pc.lam, ne * 4, s));
-    SNN_CUDA(dev_malloc(&inc.ps.size, nk * 8, s));
-    SNN_CUDA(dev_malloc(&inc.ps.inpins, nk * 8, s));
-    SNN_CUDA(dev_malloc(&inc.ps.pincnt, nk * 8, s));
-    SNN_CUDA(dev_malloc(&inc.costv, 8, s));
-    SNN_CUDA(dev_malloc(&inc.savev, nv * 8, s));
-    SNN_CUDA(dev_malloc(&inc.Wv, nv * 8, s));
-    SNN_CUDA(dev_malloc(&inc.hdirty, ne * 4, s));
-    SNN_CUDA(dev_malloc(&inc.hmark, ne * 4, s));
-    SNN_CUDA(cudaMemsetAsync(inc.hdirty, 0, ne * 4, s));
-    SNN_CUDA(cudaMemsetAsync(inc.hmark, 0, ne * 4, s));
-    SNN_CUDA(dev_malloc(&inc.hlist, ne * 4, s));
-    SNN_CUDA(dev_malloc(&inc.hmeta, 2 * SEG_NB * 4, s));
-    PStar& pst = inc.pst;
-    SNN_CUDA(dev_malloc(&pst.pslot, nk * 4, s));
-    SNN_CUDA(dev_malloc(&pst.slots, PSTAR_MAX * 4, s));
-    SNN_CUDA(dev_malloc(&pst.cnt, 4 * 4, s));
-    if (dense_level) {
-        // rows levels need only the round-start saves besides the slot map
-        if (dev_malloc(&pst.save0, nv * 8, s) != cudaSuccess) {
-            cudaGetLastError();
-            pst.save0 = nullptr;
+    auto give_back = [&]() {
+        cudaFreeAsync(block, s);
+        if (cols) cudaFreeAsync(cols, s);
+    };
+    auto setup = [&]() -> Status {
+        SNN_CUDA(cudaMemsetAsync(block, 0, cleared, s));
+        if (cols && ccleared) SNN_CUDA(cudaMemsetAsync(cols, 0, ccleared, s));
+        if (use_carry) {
+            int nb = 1 - CA.cur;
+            inc.pto = CA.pto[nb];
+            inc.pgain = CA.pgain[nb];
+            inc.dirty = CA.dirty[nb];
+            if (!dense_level && CA.level == level + 1 && L.V > 0) {
+                const Level& Lc = h->levels[level + 1];
+                int32_t* mcount;
+                SNN_TRY(h->scratch.alloc(&mcount, Lc.V));
+                SNN_CUDA(cudaMemsetAsync(mcount, 0, (size_t)(Lc.V > 0 ? Lc.V : 1) * 4, s));
+                SNN_L k_carry_count<<<grid_for(L.V, 256), 256, 0, s>>>(L.V, L.cid, mcount);
+                SNN_L k_carry<<<grid_for(L.V, 256), 256, 0, s>>>(L.V, L.cid, mcount, CA.pto[CA.cur],
+                                                                CA.pgain[CA.cur], CA.dirty[CA.cur],
+                                                                inc.pto, inc.pgain, inc.dirty);
+                SNN_CUDA(cudaGetLastError());
+                inherited = true;
+            }
+            CA.cur = nb;
+            CA.level = -1;
         }
-    } else {
-        // the column buffers are optional: without them every round takes
-        // the flag rules
-        size_t cols = (size_t)PSTAR_MAX * nv;
-        bool ok = dev_malloc(&pst.hmask, ne * 4, s) == cudaSuccess &&
-                  dev_malloc(&pst.hl, ne * 4, s) == cudaSuccess &&
-                  dev_malloc(&pst.colc, cols * 8, s) == cudaSuccess &&
-                  dev_malloc(&pst.colo, cols * 4, s) == cudaSuccess &&
-                  dev_malloc(&pst.vt, nv * 4, s) == cudaSuccess &&
-                  dev_malloc(&pst.save0, nv * 8, s) == cudaSuccess;
-        if (!ok) {
-            cudaGetLastError();
-            for (void* p : {(void*)pst.hmask, (void*)pst.hl, (void*)pst.colc, (void*)pst.colo,
-                            (void*)pst.vt, (void*)pst.save0})
-                if (p) cudaFreeAsync(p, s);
-            pst.hmask = nullptr;
-            pst.hl = nullptr;
-            pst.colc = nullptr;
-            pst.colo = nullptr;
-            pst.vt = nullptr;
-            pst.save0 = nullptr;
-        } else {
-            SNN_CUDA(cudaMemsetAsync(pst.hmask, 0, ne * 4, s));
-            SNN_CUDA(cudaMemsetAsync(pst.colc, 0, cols * 8, s));
-            SNN_CUDA(cudaMemsetAsync(pst.colo, 0, cols * 4, s));
-            SNN_CUDA(cudaMemsetAsync(pst.vt, 0, nv * 4, s));
-        }
-    }
-    {
-        int32_t base = (pst.colc || (dense_level && pst.save0)) ? 0 : (1 << 30);
-        int32_t hc[4] = {base, 0, base, 0};
-        SNN_CUDA(cudaMemcpyAsync(pst.cnt, hc, sizeof(hc), cudaMemcpyHostToDevice, s));
-        SNN_TRY(fill_i32(pst.pslot, -1, nk, s));
-    }
-    SNN_CUDA(cudaMemsetAsync(inc.vmax, 0, 3 * 4, s));
-    if (L.V > 0) SNN_L k_level_max<<<grid_for(L.V, 256), 256, 0, s>>>(L, inc.vmax);
-    SNN_CUDA(cudaGetLastError());
-    Status st = fill_i32(moveidx, -1, L.V, s);
-    if (st.ok() && !inherited) st = fill_i32(inc.dirty, 1, L.V, s);
+        // without the saves (and columns) the column update stays off
+        SNN_L k_refine_init<<<grid_for(std::max<int64_t>(V, K), 256), 256, 0, s>>>(
+            L.V, K, moveidx, inherited ? nullptr : inc.dirty, pst, cols ? 0 : (1 << 30));
+        if (!dense_level && L.V > 0) SNN_L k_level_max<<<grid_for(L.V, 256, 152 * 4), 256, 0, s>>>(L, inc.vmax);
+        SNN_CUDA(cudaGetLastError());
+        return Status{};
+    };
+    Status st = setup();
     int64_t c = 0;
     bool have_cost = false;
     for (int32_t r = 0; st.ok() && r < h->prm.max_refine_rounds; r++) {
@@ -2327,21 +2527,9 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
         have_cost = true;
         if (applied == 0) break;
     }
-    cudaFreeAsync(moveidx, s);
-    if (!use_carry)
-        for (void* p : {(void*)inc.pto, (void*)inc.pgain, (void*)inc.dirty}) cudaFreeAsync(p, s);
-    else if (st.ok() && !dense_level)
+    give_back();
+    if (use_carry && st.ok() && !dense_level)
         CA.level = level;   // the next finer level may inherit these proposals
-    for (void* p : {(void*)inc.pchg,
-                    (void*)inc.prel, (void*)inc.vmax, (void*)inc.pc.p, (void*)inc.pc.cnt,
-                    (void*)inc.pc.dcnt, (void*)inc.pc.lam, (void*)inc.ps.size,
-                    (void*)inc.ps.inpins, (void*)inc.ps.pincnt, (void*)inc.costv,
-                    (void*)inc.savev, (void*)inc.Wv, (void*)inc.hdirty, (void*)inc.hmark,
-                    (void*)inc.hlist,
-                    (void*)inc.hmeta, (void*)pst.pslot, (void*)pst.slots, (void*)pst.cnt,
-                    (void*)pst.hmask, (void*)pst.hl, (void*)pst.colc, (void*)pst.colo,
-                    (void*)pst.vt, (void*)pst.save0})
-        if (p) cudaFreeAsync(p, s);
     if (!st.ok()) return st;
     if (!have_cost) {
         SNN_TRY(level_cost(h, level, K, rho, &c));

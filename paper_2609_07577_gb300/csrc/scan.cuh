@@ -213,6 +213,34 @@ __global__ void __launch_bounds__(SCT_THREADS)
     if (total && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total = boff[blockIdx.x] + all;
 }
 
+// Sort of w[0..N) (shared memory, N a power of two in [64, SB_MAX]) by one
+// block of SB_THREADS, by a bitonic network; starts after and ends with a
+// barrier.
+constexpr int SB_MAX = 4096;
+constexpr int SB_THREADS = 1024;
+
+__device__ __forceinline__ void block_sort_words(uint64_t* w, int N)
+{
+    // a warp's 32 pairs of a step with stride <= 32 lie in one aligned run of
+    // 64 words, so only longer strides need the whole block
+    for (int k = 2; k <= N; k <<= 1) {
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int t = threadIdx.x; t < N / 2; t += SB_THREADS) {
+                int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
+                uint64_t a = w[i], b = w[i + j];
+                if ((a > b) == ((i & k) == 0)) {
+                    w[i] = b;
+                    w[i + j] = a;
+                }
+            }
+            // the next step's stride is j / 2, or k after the last of these
+            if (j > 32 || (j == 1 && k > 32)) __syncthreads();
+            else __syncwarp();
+        }
+    }
+    __syncthreads();
+}
+
 template <typename Tin, typename T>
 struct ScanLoad {
     const Tin* p;
