@@ -7,13 +7,13 @@
 // shared by every start. Sections of one depth are disjoint, so the label
 // propagation of every sibling pair of a depth, in every start, runs as one
 // set of jobs; each job stops on its own. At the start of a depth:
-//   k_ip_gain     one thread per position: the single-move cut drop G of
-//                 the node there (counts of its hyperedges on each side)
-//   k_ip_corr     one thread per L position: its row of the job's nL x nR
-//                 correction matrix (the thread is the row's only writer)
+//   k_ip_gain_corr  a warp (or block) per position: the single-move cut drop
+//                 G of the node there (counts of its hyperedges on each
+//                 side) and, in L, its row of the job's nL x nR correction
+//                 matrix
 // Then one round of all active jobs:
-//   k_ip_best_*   one thread per (x, y) pair: the steepest swap, ties to
-//                 the lowest x then y, in three passes of integer atomics
+//   k_ip_best     one thread per (x, y) pair: the steepest swap, ties to
+//                 the lowest x then y, in two passes of integer atomics
 //   k_ip_update   one block per job: stop, or swap and bring G and the
 //                 matrix up to date through the hyperedges of x and y only
 //                 (G deltas, weight changes of pairs of non-moving pins,
@@ -37,10 +37,10 @@ namespace ip = snn::initial;
 
 constexpr int kMaxStarts = 65535;   // gridDim.y
 
-// a pin repeated within its hyperedge; degrees of the nodes
+// a pin repeated within its hyperedge
 __global__ void k_ip_distinct(int64_t P, const int64_t* __restrict__ off,
                               const int32_t* __restrict__ pins, const int32_t* __restrict__ hid,
-                              int32_t* deg, int32_t* err)
+                              int32_t* err)
 {
     int bad = 0;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P;
@@ -49,21 +49,8 @@ __global__ void k_ip_distinct(int64_t P, const int64_t* __restrict__ off,
         int64_t e = off[hid[j] + 1];
         for (int64_t t = j + 1; t < e; t++)
             if (pins[t] == q) bad = 1;
-        atomicAdd(&deg[q], 1);
     }
     if (bad) atomicOr(err, 2);
-}
-
-// incidence lists: vinc[voff[q] ..] the hyperedges of node q (any order)
-__global__ void k_ip_fill(int64_t P, const int32_t* __restrict__ pins,
-                          const int32_t* __restrict__ hid, const int64_t* __restrict__ voff,
-                          int32_t* cursor, int32_t* vinc)
-{
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        int32_t q = pins[j];
-        vinc[voff[q] + atomicAdd(&cursor[q], 1)] = hid[j];
-    }
 }
 
 // seq and pos of every start from the initial orders; an order that is not
@@ -97,57 +84,70 @@ struct Jobs {
     const int64_t* pairoff;
 };
 
+// steepest swap of every job back to none; the count of jobs going on cleared
 __global__ void k_ip_reset(int32_t S, int32_t J, const int32_t* __restrict__ done, int64_t* bd,
-                           int32_t* bx, int32_t* by)
+                           unsigned long long* bxy, int32_t* active)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *active = 0;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < (int64_t)S * J;
          t += (int64_t)gridDim.x * blockDim.x) {
         if (done[t]) continue;
         bd[t] = 0;
-        bx[t] = INT32_MAX;
-        by[t] = INT32_MAX;
+        bxy[t] = ~0ull;
     }
 }
 
-__global__ void k_ip_gain(int32_t np, Jobs jb, const int32_t* __restrict__ done,
-                          const int64_t* __restrict__ voff, const int32_t* __restrict__ vinc,
-                          const int64_t* __restrict__ off, const int32_t* __restrict__ pins,
-                          const int64_t* __restrict__ eta, const int32_t* __restrict__ seq,
-                          const int32_t* __restrict__ pos, int64_t* G)
+// G of the node at each position of a depth's jobs and, for positions of L,
+// its row of the correction matrix (cleared before; ip::single_gain and
+// ip::corr_row, with the side counts of a hyperedge taken once for both). T
+// threads per position over the node's incidences: nodes of G_P are in
+// hundreds to thousands of hyperedges, so a thread per node walked a serial
+// chain (3.9 + 6.0 ms a depth for 64 starts of a 256-node G_P of 57,344
+// hyperedges).
+template <int T>
+__global__ void __launch_bounds__(256)
+    k_ip_gain_corr(int32_t np, int64_t pairs, Jobs jb, const int32_t* __restrict__ done,
+                   const int64_t* __restrict__ voff, const int32_t* __restrict__ vinc,
+                   const int64_t* __restrict__ off, const int32_t* __restrict__ pins,
+                   const int64_t* __restrict__ eta, const int32_t* __restrict__ seq,
+                   const int32_t* __restrict__ pos, int64_t* G, int64_t* M)
 {
+    __shared__ unsigned long long sh;
     int64_t s = blockIdx.y;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np;
-         i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t* ps = pos + s * np;
+    const int lane = threadIdx.x & (T - 1);
+    for (int64_t i = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T; i < np;
+         i += (int64_t)gridDim.x * (256 / T)) {
         int32_t k = jb.jobof[i];
-        if (k < 0 || done[s * jb.J + k]) continue;
-        int32_t x = seq[s * np + i];
-        int sd = ip::side_of((int32_t)i, jb.lo[k], jb.mid[k], jb.hi[k]);
-        G[s * np + x] = ip::single_gain(vinc, voff[x], voff[x + 1], off, pins, eta, pos + s * np, sd,
-                                        jb.lo[k], jb.mid[k], jb.hi[k]);
-    }
-}
-
-struct RowAdd {
-    int64_t* row;
-    __device__ void operator()(int32_t j, int64_t w) const { row[j] += w; }
-};
-
-__global__ void k_ip_corr(int32_t np, int64_t pairs, Jobs jb, const int32_t* __restrict__ done,
-                          const int64_t* __restrict__ voff, const int32_t* __restrict__ vinc,
-                          const int64_t* __restrict__ off, const int32_t* __restrict__ pins,
-                          const int64_t* __restrict__ eta, const int32_t* __restrict__ seq,
-                          const int32_t* __restrict__ pos, int64_t* M)
-{
-    int64_t s = blockIdx.y;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t k = jb.jobof[i];
-        if (k < 0 || done[s * jb.J + k] || i >= jb.mid[k]) continue;
-        int32_t x = seq[s * np + i];
-        int32_t nr = jb.hi[k] - jb.mid[k];
-        RowAdd add{M + s * pairs + jb.pairoff[k] + (i - jb.lo[k]) * (int64_t)nr};
-        ip::corr_row(vinc, voff[x], voff[x + 1], off, pins, eta, pos + s * np, jb.lo[k], jb.mid[k],
-                     jb.hi[k], add);
+        if (k < 0 || done[s * jb.J + k]) continue;   // the same for all T threads
+        const int32_t lo = jb.lo[k], mid = jb.mid[k], hi = jb.hi[k];
+        const int32_t x = seq[s * np + i];
+        const int sd = ip::side_of((int32_t)i, lo, mid, hi);
+        unsigned long long* row = (unsigned long long*)M + s * pairs + jb.pairoff[k] +
+                                  (i - lo) * (int64_t)(hi - mid);
+        int64_t g = 0;
+        for (int64_t t = voff[x] + lane; t < voff[x + 1]; t += T) {
+            int32_t a = vinc[t], cL, cR;
+            int64_t b = off[a], e = off[a + 1], w = eta[a];
+            ip::side_counts(pins, b, e, ps, lo, mid, hi, &cL, &cR);
+            g += w * ip::move_delta(sd, cL, cR);
+            if (sd != 1 || cR == 0 || (cL != 1 && cR != 1)) continue;
+            if (cL == 1 && cR == 1) w *= 2;
+            for (int64_t j = b; j < e; j++) {
+                int32_t q = ps[pins[j]];
+                if (ip::side_of(q, lo, mid, hi) == 2) atomicAdd(&row[q - mid], (unsigned long long)w);
+            }
+        }
+        g = warp_sum(g);
+        if (T > 32) {
+            if (threadIdx.x == 0) sh = 0;
+            __syncthreads();
+            if ((threadIdx.x & 31) == 0) atomicAdd(&sh, (unsigned long long)g);
+            __syncthreads();
+            g = (int64_t)sh;
+            __syncthreads();
+        }
+        if (lane == 0) G[s * np + x] = g;
     }
 }
 
@@ -166,7 +166,7 @@ __device__ __forceinline__ int32_t job_of_pair(const Jobs& jb, int64_t p)
 template <int PASS>
 __global__ void k_ip_best(int32_t np, int64_t pairs, Jobs jb, const int32_t* __restrict__ done,
                           const int32_t* __restrict__ seq, const int64_t* __restrict__ G,
-                          const int64_t* __restrict__ M, int64_t* bd, int32_t* bx, int32_t* by)
+                          const int64_t* __restrict__ M, int64_t* bd, unsigned long long* bxy)
 {
     int64_t s = blockIdx.y;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < pairs;
@@ -180,11 +180,10 @@ __global__ void k_ip_best(int32_t np, int64_t pairs, Jobs jb, const int32_t* __r
         int32_t y = seq[s * np + jb.mid[k] + (int32_t)(q % nr)];
         int64_t d = G[s * np + x] + G[s * np + y] - M[s * pairs + p];
         if (d <= 0) continue;
-        if (PASS == 0) atomicMax((long long*)&bd[t], (long long)d);
-        else if (PASS == 1) {
-            if (d == bd[t]) atomicMin(&bx[t], x);
-        } else {
-            if (d == bd[t] && x == bx[t]) atomicMin(&by[t], y);
+        if (PASS == 0) {
+            if (d > bd[t]) atomicMax((long long*)&bd[t], (long long)d);   // it only grows
+        } else if (d == bd[t]) {
+            atomicMin(&bxy[t], ((unsigned long long)(uint32_t)x << 32) | (uint32_t)y);
         }
     }
 }
@@ -226,8 +225,8 @@ struct ColAddAtomic {
 // One block per (job, start): stop when no swap lowers the cut, else swap
 // x and y and update G and the job's matrix incrementally.
 __global__ void k_ip_update(int32_t np, int64_t pairs, Jobs jb, int32_t* done, int32_t* it,
-                            const int64_t* __restrict__ bd, const int32_t* __restrict__ bx,
-                            const int32_t* __restrict__ by, const int64_t* __restrict__ voff,
+                            const int64_t* __restrict__ bd,
+                            const unsigned long long* __restrict__ bxy, const int64_t* __restrict__ voff,
                             const int32_t* __restrict__ vinc, const int64_t* __restrict__ off,
                             const int32_t* __restrict__ pins, const int64_t* __restrict__ eta,
                             int32_t* seq, int32_t* pos, int64_t* G, int64_t* M, int32_t* active)
@@ -248,7 +247,7 @@ __global__ void k_ip_update(int32_t np, int64_t pairs, Jobs jb, int32_t* done, i
     const int mode = s_mode;
     if (mode == 0) return;
     const int32_t lo = jb.lo[k], mid = jb.mid[k], hi = jb.hi[k], nr = hi - mid;
-    const int32_t x = bx[t], y = by[t];
+    const int32_t x = (int32_t)(bxy[t] >> 32), y = (int32_t)(uint32_t)bxy[t];
     int32_t* ps = pos + s * np;
     int64_t* Gs = G + s * np;
     int64_t* Mk = M + s * pairs + jb.pairoff[k];
@@ -460,12 +459,8 @@ Status initial_impl(int32_t np, int32_t ne, const int64_t* off, const int32_t* p
     SNN_TRY(gp_input(np, ne, off, pins, eta, ar, s, err, &P, &hid));
     if (np == 0) return Status{};
 
-    int32_t *deg, *cursor, *vinc, *seq, *pos, *seq2;
+    int32_t *vinc, *seq, *pos, *seq2;
     int64_t* voff;
-    SNN_TRY(ar.alloc(&deg, np));
-    SNN_TRY(ar.alloc(&cursor, np));
-    SNN_TRY(ar.alloc(&vinc, P));
-    SNN_TRY(ar.alloc(&voff, (int64_t)np + 1));
     SNN_TRY(ar.alloc(&seq, (int64_t)S * np));
     SNN_TRY(ar.alloc(&seq2, (int64_t)S * np));
     SNN_TRY(ar.alloc(&pos, (int64_t)S * np));
@@ -477,20 +472,14 @@ Status initial_impl(int32_t np, int32_t ne, const int64_t* off, const int32_t* p
     SNN_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     SNN_CUDA(cudaStreamSynchronize(s));
     if (herr) return invalid("an initial order that is not a permutation of the nodes");
-    SNN_CUDA(cudaMemsetAsync(deg, 0, sizeof(int32_t) * np, s));
-    SNN_CUDA(cudaMemsetAsync(cursor, 0, sizeof(int32_t) * np, s));
     if (P > 0) {
-        SNN_L k_ip_distinct<<<grid_for(P, 256), 256, 0, s>>>(P, off, pins, hid, deg, err);
+        SNN_L k_ip_distinct<<<grid_for(P, 256), 256, 0, s>>>(P, off, pins, hid, err);
         SNN_CUDA(cudaGetLastError());
     }
     SNN_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     SNN_CUDA(cudaStreamSynchronize(s));
     if (herr) return invalid("a pin repeated within a hyperedge");
-    SNN_TRY(scan_exclusive_i32_to_i64(deg, voff, np, voff + np, ar, s));
-    if (P > 0) {
-        SNN_L k_ip_fill<<<grid_for(P, 256), 256, 0, s>>>(P, pins, hid, voff, cursor, vinc);
-        SNN_CUDA(cudaGetLastError());
-    }
+    SNN_TRY(gp_incidence(np, P, pins, hid, ar, s, &voff, &vinc));
 
     // the bisection tree, shared by all starts
     HostTree ht(np);
@@ -522,17 +511,24 @@ Status initial_impl(int32_t np, int32_t ne, const int64_t* off, const int32_t* p
         if ((int32_t)js.size() > max_jobs) max_jobs = (int32_t)js.size();
     }
     int64_t *G, *M, *bd;
-    int32_t *jobof, *done, *it, *bx, *by, *active;
+    int32_t *jobof, *done, *it, *active;
+    unsigned long long* bxy;
     SNN_TRY(ar.alloc(&G, (int64_t)S * np));
     SNN_TRY(ar.alloc(&M, (int64_t)S * max_pairs));
     SNN_TRY(ar.alloc(&jobof, np));
     SNN_TRY(ar.alloc(&done, (int64_t)S * max_jobs));
     SNN_TRY(ar.alloc(&it, (int64_t)S * max_jobs));
     SNN_TRY(ar.alloc(&bd, (int64_t)S * max_jobs));
-    SNN_TRY(ar.alloc(&bx, (int64_t)S * max_jobs));
-    SNN_TRY(ar.alloc(&by, (int64_t)S * max_jobs));
+    SNN_TRY(ar.alloc(&bxy, (int64_t)S * max_jobs));
     SNN_TRY(ar.alloc(&active, 1));
     const dim3 gpos = grid2(np, S);
+    // a warp per node while the nodes of all starts fill the GPU with warps,
+    // a block per node below that
+    const bool warps = (int64_t)np * S >= 152 * 32;
+    const int capn = 152 * 32 / S > 0 ? 152 * 32 / S : 1;
+    const dim3 gnode((unsigned)grid_for(np, warps ? 8 : 1, capn), (unsigned)S);
+    // a swap's block takes one hyperedge of the two nodes per thread
+    const int updt = 2 * P / np >= 512 ? 512 : 128;
     for (int32_t d = 0; d <= ht.maxd; d++) {
         const std::vector<int32_t>& js = jobs_at[d];
         if (js.empty()) continue;
@@ -571,20 +567,17 @@ Status initial_impl(int32_t np, int32_t ne, const int64_t* off, const int32_t* p
         SNN_CUDA(cudaGetLastError());
         const dim3 gpair = grid2(pairs, S);
         const int gjob = grid_for((int64_t)S * J, 256);
-        SNN_L k_ip_gain<<<gpos, 256, 0, s>>>(np, jb, done, voff, vinc, off, pins, eta, seq, pos, G);
         SNN_CUDA(cudaMemsetAsync(M, 0, sizeof(int64_t) * S * pairs, s));
-        SNN_L k_ip_corr<<<gpos, 256, 0, s>>>(np, pairs, jb, done, voff, vinc, off, pins, eta, seq,
-                                             pos, M);
+        auto gc = warps ? k_ip_gain_corr<32> : k_ip_gain_corr<256>;
+        SNN_L gc<<<gnode, 256, 0, s>>>(np, pairs, jb, done, voff, vinc, off, pins, eta, seq, pos, G, M);
         SNN_CUDA(cudaGetLastError());
         const dim3 gupd((unsigned)J, (unsigned)S);
         for (;;) {
-            SNN_L k_ip_reset<<<gjob, 256, 0, s>>>(S, J, done, bd, bx, by);
-            SNN_L k_ip_best<0><<<gpair, 256, 0, s>>>(np, pairs, jb, done, seq, G, M, bd, bx, by);
-            SNN_L k_ip_best<1><<<gpair, 256, 0, s>>>(np, pairs, jb, done, seq, G, M, bd, bx, by);
-            SNN_L k_ip_best<2><<<gpair, 256, 0, s>>>(np, pairs, jb, done, seq, G, M, bd, bx, by);
-            SNN_CUDA(cudaMemsetAsync(active, 0, sizeof(int32_t), s));
-            SNN_L k_ip_update<<<gupd, 128, 0, s>>>(np, pairs, jb, done, it, bd, bx, by, voff, vinc, off,
-                                                   pins, eta, seq, pos, G, M, active);
+            SNN_L k_ip_reset<<<gjob, 256, 0, s>>>(S, J, done, bd, bxy, active);
+            SNN_L k_ip_best<0><<<gpair, 256, 0, s>>>(np, pairs, jb, done, seq, G, M, bd, bxy);
+            SNN_L k_ip_best<1><<<gpair, 256, 0, s>>>(np, pairs, jb, done, seq, G, M, bd, bxy);
+            SNN_L k_ip_update<<<gupd, updt, 0, s>>>(np, pairs, jb, done, it, bd, bxy, voff, vinc, off,
+                                                    pins, eta, seq, pos, G, M, active);
             SNN_CUDA(cudaGetLastError());
             int32_t hact = 0;
             SNN_CUDA(cudaMemcpyAsync(&hact, active, sizeof(int32_t), cudaMemcpyDeviceToHost, s));

@@ -221,6 +221,10 @@ bool device_pointer(const void* p);
 Status gp_input(int32_t np, int32_t ne, const int64_t* off, const int32_t* pins,
                 const int64_t* eta, Arena& ar, cudaStream_t s, int32_t* err, int64_t* P_out,
                 int32_t** hid_out);
+// incidence lists of G_P's nodes (arena): hyperedges vinc[voff[q] ..] of node
+// q, one entry per pin entry, in any order
+Status gp_incidence(int32_t np, int64_t P, const int32_t* pins, const int32_t* hid, Arena& ar,
+                    cudaStream_t s, int64_t** voff, int32_t** vinc);
 // S3: next level from h->match
 Status contract_level(snnmap_hgraph* h);
 // after a contraction of `src`: candidates of src carried to src + 1

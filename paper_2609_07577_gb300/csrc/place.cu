@@ -9,9 +9,8 @@
 // one matching call covers all of them.
 //
 // One round:
-//   k_pl_force    one thread per pin entry: its hyperedge's share of Eq.
-//                 force of the pin's node towards the four adjacent cores,
-//                 added into F with int64 atomics (exact, order-free)
+//   k_pl_force    a warp (or block) per node: Eq. force towards the four
+//                 adjacent cores, from counts of pins on each side
 //   k_pl_propose  one thread per core: Eq. tension and the core's proposal
 //   match_forest  Eq. matching with tension as the score
 //   k_pl_flag     one swap per matched pair, counted per start
@@ -19,8 +18,8 @@
 //   radix sorts   stable by key, then stable by start: per start,
 //                 decreasing tension, ties by the lower core
 //   k_pl_rank     each swapping core's rank within its start, and its mate
-//   k_pl_reeval   one thread per pin entry of a swapping node: its
-//                 hyperedge's share of the re-evaluated tension
+//   k_pl_reeval   a warp (or block) per swapping node: its share of the
+//                 re-evaluated tension
 //   scan, k_pl_best, k_pl_first   the best positive prefix per start
 //   k_pl_apply    the prefix's swaps applied to gamma and pi
 #include "internal.cuh"
@@ -106,6 +105,45 @@ Status gp_input(int32_t np, int32_t ne, const int64_t* off, const int32_t* pins,
     return Status{};
 }
 
+// incidence lists of G_P's nodes, one entry per pin entry
+__global__ void k_gp_degree(int64_t P, const int32_t* __restrict__ pins, int32_t* deg)
+{
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P;
+         j += (int64_t)gridDim.x * blockDim.x)
+        atomicAdd(&deg[pins[j]], 1);
+}
+
+__global__ void k_gp_fill(int64_t P, const int32_t* __restrict__ pins,
+                          const int32_t* __restrict__ hid, const int64_t* __restrict__ voff,
+                          int32_t* cursor, int32_t* vinc)
+{
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P;
+         j += (int64_t)gridDim.x * blockDim.x) {
+        int32_t q = pins[j];
+        vinc[voff[q] + atomicAdd(&cursor[q], 1)] = hid[j];
+    }
+}
+
+Status gp_incidence(int32_t np, int64_t P, const int32_t* pins, const int32_t* hid, Arena& ar,
+                    cudaStream_t s, int64_t** voff, int32_t** vinc)
+{
+    int32_t* deg;   // and the cursors behind the degrees
+    SNN_TRY(ar.alloc(&deg, 2 * (int64_t)np));
+    SNN_TRY(ar.alloc(voff, (int64_t)np + 1));
+    SNN_TRY(ar.alloc(vinc, P));
+    if (np > 0) SNN_CUDA(cudaMemsetAsync(deg, 0, 2 * sizeof(int32_t) * (size_t)np, s));
+    if (P > 0) {
+        SNN_L k_gp_degree<<<grid_for(P, 256), 256, 0, s>>>(P, pins, deg);
+        SNN_CUDA(cudaGetLastError());
+    }
+    SNN_TRY(scan_exclusive_i32_to_i64(deg, *voff, np, *voff + np, ar, s));
+    if (P > 0) {
+        SNN_L k_gp_fill<<<grid_for(P, 256), 256, 0, s>>>(P, pins, hid, *voff, deg + np, *vinc);
+        SNN_CUDA(cudaGetLastError());
+    }
+    return Status{};
+}
+
 }  // namespace snn
 
 namespace {
@@ -140,27 +178,82 @@ __global__ void k_pl_init_stats(int32_t S, int64_t* st)
         st[i] = i >= (int64_t)PS_FIRST * S ? INT64_MAX : 0;
 }
 
-__global__ void k_pl_force(int64_t P, int32_t np, int32_t width, int32_t height,
-                           const int32_t* __restrict__ hid, const int64_t* __restrict__ off,
-                           const int32_t* __restrict__ pins, const int64_t* __restrict__ eta,
-                           const int32_t* __restrict__ g, const int32_t* __restrict__ act,
-                           int64_t* F)
+// lattice coordinates of every start's nodes
+__global__ void k_pl_xy(int64_t n, int32_t width, const int32_t* __restrict__ g, int2* xy)
 {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        xy[i] = make_int2(g[i] % width, g[i] / width);
+}
+
+__device__ __forceinline__ int32_t xy_dist(int2 u, int2 v) { return abs(u.x - v.x) + abs(u.y - v.y); }
+
+// sum of v over the T threads (32 or the whole block of 256) of a node; the
+// result is valid in the first of them
+template <int T>
+__device__ __forceinline__ int64_t node_sum(int64_t v, unsigned long long* sh)
+{
+    v = warp_sum(v);
+    if (T == 32) return v;
+    __syncthreads();
+    if (threadIdx.x == 0) *sh = 0;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) atomicAdd(sh, (unsigned long long)v);
+    __syncthreads();
+    return (int64_t)*sh;
+}
+
+// Eq. force of every node towards its four neighbours, T threads per node
+// over its incidences, summed in registers. On a lattice the force towards a
+// neighbour only counts pins: moving one row up brings every pin above one
+// hop nearer and every other one hop farther away, and a pin on the
+// neighbour itself counts one less (the max(., 1) of Eq. force). So a pin
+// costs four comparisons and no distance; with a thread per pin entry, five
+// distances a pin (their coordinates by division) and four 64-bit atomics a
+// pin entry, a round took 1.05 ms for 64 starts of a 256-node G_P with
+// 57,344 hyperedges.
+template <int T>
+__global__ void __launch_bounds__(256)
+    k_pl_force(int32_t np, int32_t width, int32_t height, const int64_t* __restrict__ voff,
+               const int32_t* __restrict__ vinc, const int64_t* __restrict__ off,
+               const int32_t* __restrict__ pins, const int64_t* __restrict__ eta,
+               const int2* __restrict__ xy, const int32_t* __restrict__ act, int64_t* F)
+{
+    __shared__ unsigned long long sh;
     int64_t s = blockIdx.y;
     if (!act[s]) return;
-    const int32_t* gs = g + s * np;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        int32_t a = hid[j], p = pins[j];
-        int32_t h = gs[p];
-        int32_t nb[4];
-        place::neighbours(width, height, h, nb);
+    const int2* xs = xy + s * np;
+    const int lane = threadIdx.x & (T - 1);
+    for (int64_t p = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T; p < np;
+         p += (int64_t)gridDim.x * (256 / T)) {
+        int2 c = xs[p];
         int64_t f[4] = {0, 0, 0, 0};
-        place::force_terms(pins, off[a], off[a + 1], gs, p, h, nb, width, f);
-        int64_t w = eta[a];
-        unsigned long long* Fp = (unsigned long long*)(F + (s * np + p) * 4);
-        for (int d = 0; d < 4; d++)
-            if (f[d] != 0 && w != 0) atomicAdd(&Fp[d], (unsigned long long)(w * f[d]));
+        for (int64_t t = voff[p] + lane; t < voff[p + 1]; t += T) {
+            int32_t a = vinc[t];
+            int64_t e = off[a + 1];
+            int n = 0, l[4] = {0, 0, 0, 0};   // twice the pins beyond, less those on the neighbour
+            for (int64_t j = off[a]; j < e; j++) {
+                int32_t q = pins[j];
+                if (q == (int32_t)p) continue;
+                int2 d = xs[q];
+                int dx = d.x - c.x, dy = d.y - c.y;
+                n++;
+                l[0] += dy < 0 ? 2 : 0;
+                l[1] += dx < 0 ? 2 : 0;
+                l[2] += dx > 0 ? 2 : 0;
+                l[3] += dy > 0 ? 2 : 0;
+                if (abs(dx) + abs(dy) == 1) l[dy < 0 ? 0 : (dx < 0 ? 1 : (dx > 0 ? 2 : 3))]--;
+            }
+            int64_t w = eta[a];
+#pragma unroll
+            for (int d = 0; d < 4; d++) f[d] += w * (l[d] - n);
+        }
+        bool in[4] = {c.y > 0, c.x > 0, c.x + 1 < width, c.y + 1 < height};
+#pragma unroll
+        for (int d = 0; d < 4; d++) {
+            int64_t v = node_sum<T>(f[d], &sh);
+            if (lane == 0) F[(s * np + p) * 4 + d] = in[d] ? v : 0;
+        }
     }
 }
 
@@ -252,27 +345,46 @@ __global__ void k_pl_rank(int64_t ns, int32_t nh, const uint32_t* __restrict__ v
     }
 }
 
-__global__ void k_pl_reeval(int64_t P, int32_t np, int32_t nh, int32_t width,
-                            const int32_t* __restrict__ hid, const int64_t* __restrict__ off,
-                            const int32_t* __restrict__ pins, const int64_t* __restrict__ eta,
-                            const int32_t* __restrict__ g, const int32_t* __restrict__ rank,
-                            const int32_t* __restrict__ mate, const int32_t* __restrict__ segbeg,
-                            int64_t* Tn)
+// Re-evaluated tension: each swapping node's force towards its swap's other
+// core with every earlier swap of its start applied (place::core_before), T
+// threads per node over its incidences; nodes outside swaps cost nothing.
+template <int T>
+__global__ void __launch_bounds__(256)
+    k_pl_reeval(int32_t np, int32_t nh, int32_t width, const int64_t* __restrict__ voff,
+                const int32_t* __restrict__ vinc, const int64_t* __restrict__ off,
+                const int32_t* __restrict__ pins, const int64_t* __restrict__ eta,
+                const int32_t* __restrict__ g, const int2* __restrict__ cxy,
+                const int32_t* __restrict__ rank, const int32_t* __restrict__ mate,
+                const int32_t* __restrict__ segbeg, int64_t* Tn)
 {
+    __shared__ unsigned long long sh;
     int64_t s = blockIdx.y;
     const int32_t* gs = g + s * np;
     const int32_t* rs = rank + s * nh;
     const int32_t* ms = mate + s * nh;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        int32_t p = pins[j];
+    const int lane = threadIdx.x & (T - 1);
+    for (int64_t p = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T; p < np;
+         p += (int64_t)gridDim.x * (256 / T)) {
         int32_t h = gs[p];
         int32_t r = rs[h];
-        if (r == NO_RANK) continue;
-        int32_t a = hid[j];
-        int64_t v = place::reeval_terms(pins, off[a], off[a + 1], gs, rs, ms, p, h, ms[h], r, width);
-        if (v != 0 && eta[a] != 0)
-            atomicAdd((unsigned long long*)&Tn[segbeg[s] + r], (unsigned long long)(eta[a] * v));
+        if (r == NO_RANK) continue;   // the same for all T threads
+        int2 ch = cxy[h], ck = cxy[ms[h]];
+        int64_t v = 0;
+        for (int64_t t = voff[p] + lane; t < voff[p + 1]; t += T) {
+            int32_t a = vinc[t];
+            int64_t e = off[a + 1];
+            int64_t x = 0;
+            for (int64_t j = off[a]; j < e; j++) {
+                int32_t q = pins[j];
+                if (q == (int32_t)p) continue;
+                int2 c = cxy[place::core_before(rs, ms, gs[q], r)];
+                x += xy_dist(ch, c) - max(xy_dist(ck, c), 1);
+            }
+            v += eta[a] * x;
+        }
+        v = node_sum<T>(v, &sh);
+        if (lane == 0 && v != 0)
+            atomicAdd((unsigned long long*)&Tn[segbeg[s] + r], (unsigned long long)v);
     }
 }
 
@@ -326,18 +438,21 @@ __global__ void k_pl_apply(int64_t ns, int32_t nh, int32_t np, const uint32_t* _
     }
 }
 
-__global__ void k_pl_trd(int64_t P, int32_t np, int32_t width, const int32_t* __restrict__ hid,
+__global__ void k_pl_trd(int64_t P, int32_t np, const int32_t* __restrict__ hid,
                          const int64_t* __restrict__ off, const int32_t* __restrict__ pins,
-                         const int64_t* __restrict__ eta, const int32_t* __restrict__ g,
+                         const int64_t* __restrict__ eta, const int2* __restrict__ xy,
                          int64_t* acc)
 {
     int64_t s = blockIdx.y;
-    const int32_t* gs = g + s * np;
+    const int2* xs = xy + s * np;
     int64_t sum = 0;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P;
          j += (int64_t)gridDim.x * blockDim.x) {
         int32_t a = hid[j];
-        sum += eta[a] * place::trd_terms(pins, j, off[a + 1], gs, width);
+        int64_t e = off[a + 1], x = 0;
+        int2 c = xs[pins[j]];
+        for (int64_t i = j + 1; i < e; i++) x += xy_dist(c, xs[pins[i]]);
+        sum += eta[a] * x;
     }
     sum = warp_sum(sum);
     if ((threadIdx.x & 31) == 0 && sum != 0) atomicAdd((unsigned long long*)&acc[s], (unsigned long long)sum);
@@ -348,6 +463,16 @@ dim3 grid2(int64_t n, int32_t S)
 {
     int cap = 152 * 32 / S;
     return dim3((unsigned)grid_for(n, 256, cap > 0 ? cap : 1), (unsigned)S);
+}
+
+// a warp per node while the nodes of all starts fill the GPU with warps, a
+// block per node below that
+inline bool warp_per_node(int64_t np, int32_t S) { return np * S >= 152 * 32; }
+
+dim3 node_grid(int64_t np, int32_t S)
+{
+    int cap = 152 * 32 / S;
+    return dim3((unsigned)grid_for(np, warp_per_node(np, S) ? 8 : 1, cap > 0 ? cap : 1), (unsigned)S);
 }
 
 struct Input {
@@ -422,6 +547,23 @@ Status refine_impl(Input& in, int32_t* g, int32_t max_rounds, cudaStream_t s, in
     std::vector<int64_t> h_st((size_t)PS_N * S);
     std::vector<std::vector<snnmap_place_log>> logs(S);
     SNN_CUDA(cudaMemcpyAsync(act, h_act.data(), sizeof(int32_t) * S, cudaMemcpyHostToDevice, s));
+    int64_t* voff;
+    int32_t* vinc;
+    int2 *nxy, *cxy;
+    SNN_TRY(gp_incidence(np, in.P, in.pins, hid, ar, s, &voff, &vinc));
+    SNN_TRY(ar.alloc(&nxy, (int64_t)S * np));
+    SNN_TRY(ar.alloc(&cxy, in.nh));
+    {
+        int32_t* id;
+        Arena::Mark mk = ar.mark();
+        SNN_TRY(ar.alloc(&id, in.nh));
+        SNN_TRY(iota_i32(id, in.nh, s));
+        SNN_L k_pl_xy<<<grid_for(in.nh, 256), 256, 0, s>>>(in.nh, in.width, id, cxy);
+        SNN_CUDA(cudaGetLastError());
+        ar.rewind(mk);
+    }
+    const bool warps = warp_per_node(np, S);
+    const dim3 gnode = node_grid(np, S);
     int32_t active = S;
     const dim3 gn = grid2(in.P, S), gc = grid2(nh, S);
     for (int32_t round = 0; round < max_rounds && active > 0; round++) {
@@ -429,8 +571,10 @@ Status refine_impl(Input& in, int32_t* g, int32_t max_rounds, cudaStream_t s, in
         SNN_CUDA(cudaMemsetAsync(F, 0, sizeof(int64_t) * S * (int64_t)np * 4, s));
         SNN_L k_pl_init_stats<<<1, 256, 0, s>>>(S, st);
         if (in.P > 0) {
-            SNN_L k_pl_force<<<gn, 256, 0, s>>>(in.P, np, in.width, in.height, hid, in.off,
-                                                in.pins, in.eta, g, act, F);
+            SNN_L k_pl_xy<<<grid_for((int64_t)S * np, 256), 256, 0, s>>>((int64_t)S * np, in.width, g, nxy);
+            auto force = warps ? k_pl_force<32> : k_pl_force<256>;
+            SNN_L force<<<gnode, 256, 0, s>>>(np, in.width, in.height, voff, vinc, in.off, in.pins,
+                                              in.eta, nxy, act, F);
         }
         SNN_L k_pl_propose<<<gc, 256, 0, s>>>(nh, np, in.width, in.height, act, pi, F, cand,
                                               cscore, st + (int64_t)PS_PROPS * S);
@@ -474,8 +618,9 @@ Status refine_impl(Input& in, int32_t* g, int32_t max_rounds, cudaStream_t s, in
             SNN_L k_pl_rank<<<grid_for(ns, 256), 256, 0, s>>>(ns, nh, vals, match, segbeg, rank, mate);
             SNN_CUDA(cudaMemsetAsync(Tn, 0, sizeof(int64_t) * ns, s));
             if (in.P > 0) {
-                SNN_L k_pl_reeval<<<gn, 256, 0, s>>>(in.P, np, nh, in.width, hid, in.off, in.pins,
-                                                     in.eta, g, rank, mate, segbeg, Tn);
+                auto reeval = warps ? k_pl_reeval<32> : k_pl_reeval<256>;
+                SNN_L reeval<<<gnode, 256, 0, s>>>(np, nh, in.width, voff, vinc, in.off, in.pins, in.eta,
+                                                   g, cxy, rank, mate, segbeg, Tn);
             }
             SNN_CUDA(cudaGetLastError());
             SNN_TRY(scan_inclusive_i64(Tn, C, ns, ar, s));
@@ -540,8 +685,12 @@ Status trd_impl(Input& in, const int32_t* g, cudaStream_t s, int64_t* trd_out)
     SNN_TRY(ar.alloc(&acc, in.S));
     SNN_CUDA(cudaMemsetAsync(acc, 0, sizeof(int64_t) * in.S, s));
     if (in.P > 0) {
-        SNN_L k_pl_trd<<<grid2(in.P, in.S), 256, 0, s>>>(in.P, in.np, in.width, hid, in.off,
-                                                         in.pins, in.eta, g, acc);
+        int2* nxy;
+        const int64_t n = (int64_t)in.S * in.np;
+        SNN_TRY(ar.alloc(&nxy, n));
+        SNN_L k_pl_xy<<<grid_for(n, 256), 256, 0, s>>>(n, in.width, g, nxy);
+        SNN_L k_pl_trd<<<grid2(in.P, in.S), 256, 0, s>>>(in.P, in.np, hid, in.off, in.pins, in.eta, nxy,
+                                                         acc);
         SNN_CUDA(cudaGetLastError());
     }
     SNN_CUDA(cudaMemcpyAsync(trd_out, acc, sizeof(int64_t) * in.S, cudaMemcpyDeviceToHost, s));
