@@ -361,13 +361,23 @@ static int snnmap_partition_impl(snnmap_hgraph* h, void* stream, int32_t* d_rho_
     // once the level above needed at least four evaluations per vertex
     // (rounds times the share of vertices evaluated), as on power-law
     // graphs whose levels run many rounds with every vertex active.
+    // The rows are allocated for the levels that keep them by the first rule,
+    // known here from the level sizes (a finer level's rows may be the whole
+    // budget: 38 GB for the 1,048,576-neuron conv network's level 0, which
+    // never uses them, and mapping and unmapping those took 100 of its 700
+    // ms); a busier level opens them again at the full size, every row fresh.
     int32_t lb = nl;
+    auto fresh_rows = [&](int32_t l) {
+        return 2 * ((int64_t)h->levels[l].V - h->levels[l + 1].V);
+    };
     {
         int64_t rb = snn::dense_row_budget(h);
         int64_t per = ((((int64_t)K + 3) & ~(int64_t)3) * 8 + 20);
         if (rb > 0 && !h->wide && !h->wzero && h->wsum <= INT32_MAX)
             for (int32_t l = nl - 1; l >= 0 && (int64_t)h->levels[l].V * per <= rb; l--) lb = l;
-        if (lb < nl && !snn::dense_open(h, K, h->levels[lb].V).ok()) {
+        int32_t lk = nl - 1;
+        while (lk > lb && 4 * fresh_rows(lk - 1) <= h->levels[lk - 1].V) lk--;
+        if (lb < nl && !snn::dense_open(h, K, h->levels[lk].V).ok()) {
             snn::dense_close(h);
             cudaGetLastError();
             lb = nl;
@@ -390,15 +400,23 @@ static int snnmap_partition_impl(snnmap_hgraph* h, void* stream, int32_t* d_rho_
             std::swap(cur, oth);
             if (l >= lb) {
                 int64_t V = h->levels[l].V;
-                int64_t fresh = 2 * (V - h->levels[l + 1].V);
                 bool busy = evals_above >= 4.0;
                 snn::ProfScope prof(h, snn::PS_ROWS);
-                if (h->dense.level == l + 1 && (4 * fresh <= V || busy)) {
+                bool keep = h->dense.C && h->dense.level == l + 1 && (4 * fresh_rows(l) <= V || busy);
+                if (keep && V <= h->dense.cap) {
                     s2 = snn::dense_descend(h, l);
                     rows_here = true;
-                } else if (h->dense.level != l + 1 && busy) {
-                    s2 = snn::dense_begin(h, l);
-                    rows_here = true;
+                } else if (keep || (busy && (!h->dense.C || h->dense.level != l + 1))) {
+                    bool room = h->dense.C && V <= h->dense.cap;
+                    if (!room) room = snn::dense_open(h, K, h->levels[lb].V).ok();
+                    if (room) {
+                        s2 = snn::dense_begin(h, l);
+                        rows_here = true;
+                    } else {
+                        cudaGetLastError();
+                        snn::dense_close(h);
+                        lb = nl;   // no room: histograms from here down
+                    }
                 }
             } else if (h->dense.C) {
                 snn::dense_close(h);
