@@ -43,6 +43,7 @@ template <typename S_>
 struct AffPol {
     using S = S_;
     static constexpr bool kOptimistic = false;
+    static constexpr bool kMasks = false;
     struct Acc {
         __device__ Acc() {}
         __device__ void add(const Acc&) {}
@@ -50,6 +51,7 @@ struct AffPol {
     };
     static __device__ Acc warp_reduce(const Acc& a) { return a; }
 
+    const HRec* rec = nullptr;   // the level's records, or null: its arrays
     Level L;
     int32_t V;
     int64_t keys;
@@ -74,12 +76,14 @@ struct AffPol {
     __device__ int64_t seg_len(int64_t i) const
     {
         int32_t a = (int32_t)((uint32_t)L.vinc[i] & ~SRC_BIT);
+        if (rec) return rec[a].n();
         return L.hoff[a + 1] - L.hoff[a];
     }
     __device__ Seg<S> seg(int64_t i, Acc&) const
     {
         uint32_t inc = (uint32_t)L.vinc[i];
         int32_t a = (int32_t)(inc & ~SRC_BIT);
+        if (rec) return rec_seg<S>(rec[a], inc);
         Seg<S> g;
         g.sd = L.hsd[a];
         g.nd = !(inc & SRC_BIT) || g.sd;
@@ -96,7 +100,9 @@ struct AffPol {
         uint32_t o;
     };
     static __device__ Item none() { return Item{-1, 0, 0u}; }
-    __device__ Item load(int32_t n, const Seg<S>& g, int32_t off) const
+    using Own = int4;
+    __device__ Own own(int32_t n) const { return prefilter ? vst[n] : make_int4(0, 0, 0, 0); }
+    __device__ Item load(int32_t n, const Own& a, const Seg<S>& g, int32_t off) const
     {
         Item it;
         it.m = L.hpins[g.b + off];
@@ -108,7 +114,7 @@ struct AffPol {
         if (it.m == n) {
             it.m = -1;
         } else if (prefilter) {
-            int4 a = vst[n], b = vst[it.m];
+            int4 b = vst[it.m];
             if ((int64_t)a.x + b.x > omega || (int64_t)a.y + b.y > phi) it.m = -1;
         }
         return it;
@@ -138,6 +144,16 @@ struct AffPol {
         cov[n] = bk < 0 ? 0 : (int32_t)bo;
     }
 };
+
+__global__ void k_pack_hedges(Level L, HRec* rec)
+{
+    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < L.E;
+         a += (int64_t)gridDim.x * blockDim.x) {
+        int64_t b = L.hoff[a];
+        rec[a] = HRec{b, L.hw[a], (uint32_t)L.hk[a],
+                      (uint32_t)(L.hoff[a + 1] - b) | (uint32_t)L.hsd[a] << 31, 0, 0};
+    }
+}
 
 // (size, inbound pins, inbound axons) of every vertex in one 16-byte entry, so
 // a neighbour's state is one gather in the histograms' hot loops
@@ -324,7 +340,12 @@ static Status affinity(snnmap_hgraph* h, Level& L)
     SNN_TRY(h->scratch.alloc(&vst, L.V));
     SNN_L k_pack_state<<<grid_for(L.V, 256), 256, 0, h->stream>>>(L, vst);
     SNN_CUDA(cudaGetLastError());
+    HRec* rec;
+    SNN_TRY(h->scratch.alloc(&rec, L.E));
+    if (L.E > 0) SNN_L k_pack_hedges<<<grid_for(L.E, 256), 256, 0, h->stream>>>(L, rec);
+    SNN_CUDA(cudaGetLastError());
     AffPol<S> pol;
+    pol.rec = rec;
     pol.vst = vst;
     pol.vmin = vmin;
     pol.prefilter = 2 * (int64_t)vm[2] > h->prm.omega || 2 * (int64_t)vm[3] > h->prm.phi;
@@ -562,6 +583,7 @@ template <typename S_>
 struct AffNewPol {
     using S = S_;
     static constexpr bool kOptimistic = false;
+    static constexpr bool kMasks = false;
     struct Acc {
         __device__ Acc() {}
         __device__ void add(const Acc&) {}
@@ -573,7 +595,7 @@ struct AffNewPol {
     int32_t V;
     int64_t keys;
     int32_t omega, delta, phi;
-    const int64_t* loff;
+    const HRec* rec;         // of the lists
     const uint32_t* lpins;
     AffCarry ac;
     bool prefilter;
@@ -587,21 +609,12 @@ struct AffNewPol {
     __device__ int64_t ve(int32_t n) const { return L.voff[n + 1]; }
     __device__ int64_t seg_len(int64_t i) const
     {
-        int32_t a = (int32_t)((uint32_t)L.vinc[i] & ~SRC_BIT);
-        return loff[a + 1] - loff[a];
+        return rec[(int32_t)((uint32_t)L.vinc[i] & ~SRC_BIT)].n();
     }
     __device__ Seg<S> seg(int64_t i, Acc&) const
     {
         uint32_t inc = (uint32_t)L.vinc[i];
-        int32_t a = (int32_t)(inc & ~SRC_BIT);
-        Seg<S> g;
-        g.sd = L.hsd[a];
-        g.nd = !(inc & SRC_BIT) || g.sd;
-        g.b = loff[a];
-        g.len = (int32_t)(loff[a + 1] - g.b);
-        g.w = (S)L.hw[a];
-        g.k = (uint32_t)L.hk[a];
-        return g;
+        return rec_seg<S>(rec[(int32_t)(inc & ~SRC_BIT)], inc);
     }
     struct Item {
         int32_t m;
@@ -609,7 +622,9 @@ struct AffNewPol {
         uint32_t o;
     };
     static __device__ Item none() { return Item{-1, 0, 0u}; }
-    __device__ Item load(int32_t n, const Seg<S>& g, int32_t off) const
+    using Own = int4;
+    __device__ Own own(int32_t n) const { return prefilter ? vst[n] : make_int4(0, 0, 0, 0); }
+    __device__ Item load(int32_t, const Own& a, const Seg<S>& g, int32_t off) const
     {
         uint32_t e = lpins[g.b + off];
         Item it;
@@ -617,7 +632,7 @@ struct AffNewPol {
         it.w = g.w;
         it.o = (g.nd && !(e & NOT_DEST)) ? g.k : 0u;
         if (prefilter) {
-            int4 a = vst[n], b = vst[it.m];
+            int4 b = vst[it.m];
             if ((int64_t)a.x + b.x > omega || (int64_t)a.y + b.y > phi) it.m = -1;
         }
         return it;
@@ -700,14 +715,18 @@ Status aff_carry(snnmap_hgraph* h, int32_t src)
     return Status{};
 }
 
-// exclusive list positions, closed by the end of the last list
+// exclusive list positions, closed by the end of the last list, and the
+// lists' records
 struct ListPlaces {
     int64_t* off;
     int64_t n;
+    Level L;
+    HRec* rec;
     __device__ void operator()(int64_t i, int64_t ex, int64_t v) const
     {
         off[i] = ex;
         if (i == n - 1) off[n] = ex + v;
+        rec[i] = HRec{ex, L.hw[i], (uint32_t)L.hk[i], (uint32_t)v | (uint32_t)L.hsd[i] << 31, 0, 0};
     }
 };
 
@@ -731,7 +750,10 @@ static Status affinity_carried(snnmap_hgraph* h, Level& L, bool* done)
     SNN_L k_level_min<<<grid_for(L.V, 256, 152 * 4), 256, 0, s>>>(L, vmin);
     if (E > 0) SNN_HEDGE_LAUNCH(hedge_lanes(L.P, E), k_ac_count, E, s, L, C.kind, lcnt, work);
     SNN_CUDA(cudaGetLastError());
-    SNN_TRY(scan_run<int64_t>(ScanLoad<int32_t, int64_t>{lcnt}, ListPlaces{loff, E}, E, work + 2, ar, s));
+    HRec* lrec;
+    SNN_TRY(ar.alloc(&lrec, E));
+    SNN_TRY(scan_run<int64_t>(ScanLoad<int32_t, int64_t>{lcnt}, ListPlaces{loff, E, L, lrec}, E, work + 2, ar,
+                              s));
     int64_t* hv = h->h_tier + 2 * TIER_SLOTS;   // pinned
     SNN_CUDA(cudaMemcpyAsync(hv, work, 5 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     SNN_CUDA(cudaStreamSynchronize(s));
@@ -762,7 +784,7 @@ static Status affinity_carried(snnmap_hgraph* h, Level& L, bool* done)
         pol.omega = h->prm.omega;
         pol.delta = h->prm.delta;
         pol.phi = h->prm.phi;
-        pol.loff = loff;
+        pol.rec = lrec;
         pol.lpins = lpins;
         pol.ac = C;
         pol.prefilter = prefilter;

@@ -19,14 +19,15 @@
 //               vertex then reduces the table.
 // Key spaces of up to 24,576 keys take arrays instead of the tables of the
 // block tier (up to 4,096 keys) and of the big and split tiers (k_ht_dense).
-// The hash tiers visit a chunk of 32 incidences at a time with their segments
-// flattened into one range, so all 32 lanes load consecutive elements even
-// when segments are short.
+// In the warp tier a warp flattens 32 incidences at a time (warp_visit); in
+// the others a group of 4 to 32 lanes (the vertex's mean segment) takes an
+// incidence (group_visit).
 //
 // A Policy supplies:
 //   typedef S (score type), struct Acc (per-thread sums, with add(Acc) and
 //   __device__ Acc reduce over a warp)
 //   int32_t V (vertices), key space bound `keys`
+//   static constexpr bool kMasks                    segments carry HRec's run masks
 //   static constexpr bool kOptimistic               try the warp tier even when the
 //                                                   bound exceeds its table (few keys expected)
 //   __device__ bool skip(n)                         n needs no histogram (result
@@ -34,7 +35,8 @@
 //   __device__ int64_t seg_len(int64_t i)           segment length of incidence i
 //   __device__ int64_t vb(n), ve(n)                 incidence range of vertex n
 //   __device__ Seg<S> seg(int64_t i, Acc&)          segment of incidence i
-//   struct Item, Item load(n, const Seg<S>&, off)   one element's reads; none() an empty Item
+//   struct Own, Own own(n)                          what load reads of the visiting vertex
+//   struct Item, Item load(n, Own, const Seg<S>&, off)  one element's reads; none() an empty Item
 //   __device__ bool put(n, const Item&, table, Acc&)  its table update
 //   (apart, so that several elements' loads are in flight per thread)
 //   __device__ void consider(n, key, int64 sc, uint32 ov, const Acc& total,
@@ -44,7 +46,10 @@
 #include "common.cuh"
 #include "histo_tiers.cuh"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
+#include <climits>
 #include <type_traits>
 
 namespace snn {
@@ -55,6 +60,14 @@ __device__ __forceinline__ bool better(int64_t s1, int32_t m1, int64_t s2, int32
     if (m1 < 0) return false;
     if (m2 < 0) return true;
     return s1 > s2 || (s1 == s2 && m1 < m2);
+}
+
+// first slot probed for key m: the high bits of a multiplicative hash (the
+// golden ratio's), scaled to the table; runs of consecutive ids, which a
+// hyperedge's sorted pins often are, land spread over it
+__device__ __forceinline__ uint32_t table_slot(int32_t m, uint32_t mask)
+{
+    return __umulhi((uint32_t)m * 0x9e3779b1u, mask + 1);
 }
 
 // Open-addressing slots: key (-1 empty), summed weight, summed overlap.
@@ -76,7 +89,7 @@ struct Table {
     // returns false if m has no slot within the first max_probes probed
     __device__ __forceinline__ bool try_add(int32_t m, S w, uint32_t o, uint32_t max_probes) const
     {
-        uint32_t slot = hash32((uint32_t)m) & mask;
+        uint32_t slot = table_slot(m, mask);
         for (uint32_t probe = 0; probe < max_probes; probe++) {
             int32_t k = *(volatile int32_t*)&key[slot];
             if (k == -1) {
@@ -112,6 +125,22 @@ __device__ __forceinline__ Table<S> carve_table(unsigned char* base, int64_t cap
     return t;
 }
 
+// What the histograms read of a hyperedge, in one 32-byte sector: a vertex's
+// incidences name hyperedges all over the level, so offsets, weight,
+// multiplicity and flags in arrays of their own cost a sector each (the
+// gains of the 262,144-neuron conv network's first round read 20 million
+// segments of about nine partitions).
+struct alignas(32) HRec {
+    int64_t b;       // first element
+    int64_t w;
+    uint32_t k;
+    uint32_t len;    // elements; bit 31: selfdst
+    uint32_t dm;     // pin counts: bit r set when run r (r < 32) has destinations
+    uint32_t sm;     // pin counts: bit r set when run r (r < 32) is a single pin
+    __device__ int32_t n() const { return (int32_t)(len & 0x7fffffffu); }
+    __device__ int sd() const { return (int)(len >> 31); }
+};
+
 // One incidence's segment: elements [b, b+len) of a per-hyperedge array,
 // with the hyperedge's weight w, multiplicity k, whether the visiting vertex
 // is one of its destinations (nd) and its selfdst flag (sd).
@@ -122,19 +151,67 @@ struct Seg {
     S w;
     uint32_t k;
     int nd, sd;
+    uint32_t dm, sm;   // as HRec (refinement)
 };
 
-// One warp visits incidences [i0, ve) of vertex n, 32 at a time every
-// `stride`, flattening their segments. Returns false if an insert failed.
+// the segment of an incidence word (hyperedge id and source bit)
+template <typename S>
+__device__ __forceinline__ Seg<S> rec_seg(const HRec& r, uint32_t inc)
+{
+    Seg<S> g;
+    g.sd = r.sd();
+    g.nd = !(inc & SRC_BIT) || g.sd;
+    g.b = r.b;
+    g.len = r.n();
+    g.w = (S)r.w;
+    g.k = r.k;
+    g.dm = r.dm;
+    g.sm = r.sm;
+    return g;
+}
+
+// Slots whose weight and overlap share one word, value = weight << sb |
+// overlap, for vertices whose sums over all incidences bound both within 32
+// bits: one shared-memory atomic an element instead of two.
+struct PackedTable {
+    int32_t* key;
+    uint32_t* val;
+    uint32_t mask;
+    uint32_t probes;
+    int sb;
+    __device__ __forceinline__ bool add(int32_t m, uint32_t w, uint32_t o) const
+    {
+        uint32_t slot = table_slot(m, mask);
+        for (uint32_t probe = 0; probe < probes; probe++) {
+            int32_t k = *(volatile int32_t*)&key[slot];
+            if (k == -1) {
+                int32_t prev = atomicCAS(&key[slot], -1, m);
+                k = prev == -1 ? m : prev;
+            }
+            if (k == m) {
+                atomicAdd(&val[slot], (w << sb) + o);
+                return true;
+            }
+            slot = (slot + 1) & mask;
+        }
+        return false;
+    }
+};
+
+// One warp visits incidences [vb, ve) of vertex n, 32 at a time with their
+// segments flattened into one range, so that all 32 lanes load consecutive
+// elements even when segments are short or uneven; two steps' loads are in
+// flight. Returns false if an insert failed.
 template <typename S, class Pol, class Tb>
-__device__ bool warp_visit(const Pol& pol, int32_t n, int64_t i0, int64_t ve, int64_t stride,
-                           const Tb& t, typename Pol::Acc& acc)
+__device__ bool warp_visit(const Pol& pol, int32_t n, int64_t vb, int64_t ve, const Tb& t,
+                           typename Pol::Acc& acc)
 {
     int lane = threadIdx.x & 31;
     bool ok = true;
-    for (int64_t ib = i0; ib < ve; ib += stride) {
+    const typename Pol::Own own = pol.own(n);
+    for (int64_t ib = vb; ib < ve; ib += 32) {
         int64_t i = ib + lane;
-        Seg<S> sg{0, 0, 0, 0, 0, 0};
+        Seg<S> sg{};
         if (i < ve) sg = pol.seg(i, acc);
         int32_t pre = sg.len;
 #pragma unroll
@@ -144,27 +221,149 @@ __device__ bool warp_visit(const Pol& pol, int32_t n, int64_t i0, int64_t ve, in
         }
         int32_t total = __shfl_sync(FULL, pre, 31);
         pre -= sg.len;
-        for (int32_t vbase = 0; vbase < total; vbase += 32) {
-            int32_t v = vbase + lane;
-            int32_t lo = 0;
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1) {
-                int32_t c = lo + step;
-                int32_t pc = __shfl_sync(FULL, pre, c & 31);
-                if (c < 32 && pc <= v) lo = c;
+        const int flags = sg.nd << 1 | sg.sd;
+        // nonempty segments in order (src: lane of the r-th), so that within a
+        // window of 32 elements the segment of one is the number of segments
+        // starting at or before it, less one
+        const unsigned some = __ballot_sync(FULL, sg.len > 0);
+        int src = lane;
+        if (some != FULL) {
+            src = 0;
+            unsigned rest = some;
+            for (int r = 0; rest; r++) {
+                if (lane == r) src = __ffs(rest) - 1;
+                rest &= rest - 1;
             }
-            Seg<S> g;
-            g.b = __shfl_sync(FULL, sg.b, lo);
-            g.len = __shfl_sync(FULL, sg.len, lo);
-            g.w = __shfl_sync(FULL, sg.w, lo);
-            g.k = __shfl_sync(FULL, sg.k, lo);
-            g.nd = __shfl_sync(FULL, sg.nd, lo);
-            g.sd = __shfl_sync(FULL, sg.sd, lo);
-            int32_t pt = __shfl_sync(FULL, pre, lo);
-            if (v < total && !pol.put(n, pol.load(n, g, v - pt), t, acc)) ok = false;
+        }
+        int before = 0;   // nonempty segments that start before the window
+        constexpr int U = 2;
+        for (int32_t vbase = 0; vbase < total; vbase += 32 * U) {
+            typename Pol::Item it[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int32_t w0 = vbase + 32 * u, v = w0 + lane;
+                const int32_t d = pre - w0;
+                const unsigned starts =
+                    __reduce_or_sync(FULL, sg.len > 0 && d >= 0 && d < 32 ? 1u << d : 0u);
+                int r = before + __popc(starts & (lanemask_lt() | (1u << lane))) - 1;
+                before += __popc(starts);
+                const int lo = __shfl_sync(FULL, src, r & 31);
+                Seg<S> g;
+                g.b = __shfl_sync(FULL, sg.b, lo);
+                g.len = 0;
+                g.w = __shfl_sync(FULL, sg.w, lo);
+                g.k = __shfl_sync(FULL, sg.k, lo);
+                int f = __shfl_sync(FULL, flags, lo);
+                g.nd = f >> 1;
+                g.sd = f & 1;
+                if (Pol::kMasks) {
+                    g.dm = __shfl_sync(FULL, sg.dm, lo);
+                    g.sm = __shfl_sync(FULL, sg.sm, lo);
+                }
+                int32_t pt = __shfl_sync(FULL, pre, lo);
+                it[u] = v < total ? pol.load(n, own, g, v - pt) : Pol::none();
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) ok = pol.put(n, it[u], t, acc) && ok;
         }
     }
     return __all_sync(FULL, ok);
+}
+
+// lanes (log2) that take one incidence of a vertex with this many incidences
+// and elements: its mean segment, a power of two in [4, 32]
+__device__ __forceinline__ int group_log(int64_t deg, int64_t work)
+{
+    int64_t mean = deg > 0 ? (work + deg - 1) / deg : 32;
+    return mean <= 4 ? 2 : (mean <= 8 ? 3 : (mean <= 16 ? 4 : 5));
+}
+
+// T threads (whole warps; tid 0..T-1) visit incidences [vb, ve) of vertex n,
+// a group of 2^glog lanes per incidence and U incidences in flight per group.
+// The group's lanes hold the same segment in registers, so an element costs
+// its load and its table update; the flattened form before (tiles of
+// incidences, a shared-memory prefix and a search per element) spent most of
+// its instructions on finding the segment. Segments longer than eight rounds
+// of their group are finished by its whole warp; those longer than T go to
+// slong (if any) for the whole block, which would otherwise wait for one of
+// its warps (a vertex of the 1,048,576-neuron power-law network meets 47
+// pins a hyperedge on average, but up to 16,384). Returns false in lanes
+// whose insert failed.
+constexpr int HT_NLONG = 256;
+
+template <typename S, int T, int U, class Pol, class Tb>
+__device__ __forceinline__ bool group_visit(const Pol& pol, int32_t n, int64_t vb, int64_t ve,
+                                            int glog, int tid, const Tb& t,
+                                            typename Pol::Acc& acc, int64_t* slong = nullptr,
+                                            int32_t* nlong = nullptr)
+{
+    const int lane = tid & 31, G = 1 << glog, gl = lane & (G - 1);
+    const int grp = tid >> glog, ngrp = T >> glog;
+    bool ok = true;
+    const typename Pol::Own own = pol.own(n);
+    typename Pol::Acc other;   // a segment's own terms count once, in its first lane
+    for (int64_t base = vb; base < ve; base += (int64_t)U * ngrp) {
+        Seg<S> g[U];
+        typename Pol::Item it[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            int64_t i = base + (int64_t)u * ngrp + grp;
+            g[u] = Seg<S>{};
+            if (i < ve) g[u] = pol.seg(i, gl == 0 ? acc : other);
+        }
+        if (slong) {
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                bool lg = g[u].len > T;
+                int32_t at = HT_NLONG;
+                if (lg && gl == 0) at = atomicAdd(nlong, 1);
+                if (!__any_sync(FULL, lg)) continue;
+                at = __shfl_sync(FULL, at, lane & ~(G - 1));
+                if (lg && at < HT_NLONG) {
+                    if (gl == 0) slong[at] = base + (int64_t)u * ngrp + grp;
+                    g[u].len = 0;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            it[u] = gl < g[u].len ? pol.load(n, own, g[u], gl) : Pol::none();
+#pragma unroll
+        for (int u = 0; u < U; u++) ok = pol.put(n, it[u], t, acc) && ok;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const bool lg = G < 32 && g[u].len > 8 * G;
+            if (!lg) {
+                for (int32_t off = gl + G; off < g[u].len; off += 2 * G) {
+                    typename Pol::Item a = pol.load(n, own, g[u], off);
+                    typename Pol::Item b =
+                        off + G < g[u].len ? pol.load(n, own, g[u], off + G) : Pol::none();
+                    ok = pol.put(n, a, t, acc) && ok;
+                    ok = pol.put(n, b, t, acc) && ok;
+                }
+            }
+            unsigned m = G < 32 ? __ballot_sync(FULL, lg && gl == 0) : 0u;
+            while (m) {
+                int src = __ffs(m) - 1;
+                m &= m - 1;
+                Seg<S> w;
+                w.b = __shfl_sync(FULL, g[u].b, src);
+                w.len = __shfl_sync(FULL, g[u].len, src);
+                w.w = __shfl_sync(FULL, g[u].w, src);
+                w.k = __shfl_sync(FULL, g[u].k, src);
+                w.nd = __shfl_sync(FULL, g[u].nd, src);
+                w.sd = __shfl_sync(FULL, g[u].sd, src);
+                if (Pol::kMasks) {
+                    w.dm = __shfl_sync(FULL, g[u].dm, src);
+                    w.sm = __shfl_sync(FULL, g[u].sm, src);
+                }
+                for (int32_t off = G + lane; off < w.len; off += 32)
+                    ok = pol.put(n, pol.load(n, own, w, off), t, acc) && ok;
+            }
+        }
+        if (!__all_sync(FULL, ok)) break;
+    }
+    return ok;
 }
 
 template <typename S>
@@ -283,10 +482,13 @@ __global__ void __launch_bounds__(256)
     __shared__ unsigned long long part;
     int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t nt = *ntodo;
-    for (int64_t base = (int64_t)blockIdx.x * 8; base < nt; base += (int64_t)gridDim.x * 8) {
+    // consecutive vertices go to different blocks: few vertices (a tail level's
+    // merged ones) then have a block each
+    for (int64_t base = blockIdx.x; base < nt; base += (int64_t)gridDim.x * 8) {
+        const int64_t mine = base + (int64_t)warp * gridDim.x;
         bool longer = false;
-        if (base + warp < nt) {
-            int32_t n = todo[base + warp];
+        if (mine < nt) {
+            int32_t n = todo[mine];
             int64_t vb = pol.vb(n), ve = pol.ve(n);
             longer = ve - vb > HT_WORK_LONG;
             if (!longer) {
@@ -298,8 +500,8 @@ __global__ void __launch_bounds__(256)
             }
         }
         if (!__syncthreads_or(longer)) continue;
-        for (int x = 0; x < 8 && base + x < nt; x++) {
-            int32_t n = todo[base + x];
+        for (int x = 0; x < 8 && base + (int64_t)x * gridDim.x < nt; x++) {
+            int32_t n = todo[base + (int64_t)x * gridDim.x];
             int64_t vb = pol.vb(n), ve = pol.ve(n);
             if (ve - vb <= HT_WORK_LONG) continue;
             if (threadIdx.x == 0) part = 0;
@@ -416,7 +618,7 @@ __global__ void __launch_bounds__(HT_WARPS * 32)
         // (policies that expect few keys) try it and move on if it fills
         bool sure = bound <= HT_WLOAD;
         t.probes = sure ? (uint32_t)cap : 32u;
-        bool ok = warp_visit<S>(pol, n, vb, ve, 32, t, acc);
+        bool ok = warp_visit<S>(pol, n, vb, ve, t, acc);
         __syncwarp();
         if (!ok) {
             clear_slots(t, lane, cap, 32);
@@ -450,90 +652,45 @@ __device__ __forceinline__ int32_t seg_find(const int32_t* spre, int32_t n, int3
     return lo;
 }
 
-// Block-wide visit of incidences [vb, ve): tiles of blockDim incidences, one
-// per thread, segment lengths scanned across the block, then every thread
-// takes elements v = tid, tid + blockDim, ... of the tile's flattened range
-// and finds its segment in shared memory (the elements of a thread are
-// increasing, so its search resumes where the previous one ended).
-template <typename S, class Pol, int T>
-__device__ bool block_visit(const Pol& pol, int32_t n, int64_t vb, int64_t ve, const Table<S>& t,
-                            typename Pol::Acc& acc, Seg<S>* sseg, int32_t* spre, int32_t* swarp,
-                            int* sfail)
-{
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nw = T / 32;
-    bool ok = true;
-    for (int64_t tile = vb; tile < ve; tile += T) {
-        int64_t i = tile + threadIdx.x;
-        Seg<S> sg{0, 0, 0, 0, 0, 0};
-        if (i < ve) sg = pol.seg(i, acc);
-        int32_t inc = sg.len;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int32_t t2 = __shfl_up_sync(FULL, inc, o);
-            if (lane >= o) inc += t2;
-        }
-        if (lane == 31) swarp[warp] = inc;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int32_t run = 0;
-            for (int w = 0; w < nw; w++) {
-                int32_t c = swarp[w];
-                swarp[w] = run;
-                run += c;
-            }
-            swarp[nw] = run;
-        }
-        __syncthreads();
-        spre[threadIdx.x] = swarp[warp] + inc - sg.len;
-        sseg[threadIdx.x] = sg;
-        int32_t total = swarp[nw];
-        __syncthreads();
-        int32_t lo = 0;
-        constexpr int U = 4;   // elements in flight per thread
-        for (int32_t v0 = threadIdx.x; v0 < total && ok; v0 += U * T) {
-            typename Pol::Item it[U];
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                int32_t v = v0 + u * T;
-                if (v < total) {
-                    lo = seg_find(spre, T, lo, v);
-                    it[u] = pol.load(n, sseg[lo], v - spre[lo]);
-                } else {
-                    it[u] = Pol::none();
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < U; u++) ok = pol.put(n, it[u], t, acc) && ok;
-        }
-        if (!ok) *sfail = 1;
-        __syncthreads();
-        if (*sfail) break;
-    }
-    return *sfail == 0;
-}
-
 // Block (T threads) per vertex with a CAP-slot shared table; vertices whose
-// keys do not fit are pushed to tier `next`.
+// keys do not fit are pushed to tier `next`. What bounds it is the stream of
+// shared-memory operations and the instructions around them, so a vertex
+// whose summed weights and multiplicities fit one 32-bit word together uses
+// packed sums.
+//
+// Vertices of more than T / 4 incidences are visited by groups of lanes
+// (group_visit): with enough incidences per warp their uneven lengths even
+// out, and an element needs no search (level 0 of the 1,048,576-neuron conv
+// network: 40.1 -> 29.7 ms, packed sums included). Vertices of fewer keep
+// the flattened form (their segments' prefix in shared memory, a search per
+// element): on level 0 of the 1,048,576-neuron power-law network, 16
+// incidences of 8 to 16,384 pins each, the groups left most of the block
+// waiting for the longest (12.7 ms flattened, 15.3 by groups).
 template <class Pol, int T, int CAP, int TIER, int NEXT>
 __global__ void __launch_bounds__(T)
-    k_ht_block(Pol pol, int32_t* lists, int64_t* cnt, int64_t* scap, const int64_t* __restrict__ workv)
+    k_ht_block(Pol pol, int32_t* lists, int64_t* cnt, int64_t* scap, const int64_t* __restrict__ workv,
+               int64_t leave)
 {
     using S = typename Pol::S;
     using Acc = typename Pol::Acc;
     extern __shared__ __align__(16) unsigned char ht_dyn[];
-    __shared__ __align__(16) unsigned char sseg_raw[sizeof(Seg<S>) * T];
-    __shared__ int32_t spre[T];
-    __shared__ int32_t swarp[T / 32 + 1];
     __shared__ int sfail;
+    __shared__ int64_t slong[HT_NLONG];
+    __shared__ int32_t nlong;
+    constexpr int FLAT = T / 4;   // most incidences of the flattened form
+    __shared__ __align__(16) unsigned char sseg_raw[sizeof(Seg<S>) * FLAT];
+    __shared__ int32_t spre[FLAT];
+    __shared__ int32_t swarp[FLAT / 32];
+    Seg<S>* sseg = (Seg<S>*)sseg_raw;
+    __shared__ unsigned long long ssum[2];
     __shared__ __align__(16) unsigned char wacc_raw[sizeof(Acc) * (T / 32)];
     __shared__ int64_t rs[T / 32];
     __shared__ int32_t rk[T / 32];
     __shared__ uint32_t ro[T / 32];
-    Seg<S>* sseg = (Seg<S>*)sseg_raw;
     Acc* wacc = (Acc*)wacc_raw;
     const int nwarps = T / 32;
     int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (cnt[TIER] <= leave) return;   // so few that the big tier's blocks take them
     Table<S> t = carve_table<S>(ht_dyn, CAP);
     t.probes = 64;   // a vertex that clusters the table this much moves on
     clear_slots(t, threadIdx.x, CAP, T);
@@ -544,18 +701,119 @@ __global__ void __launch_bounds__(T)
         if (threadIdx.x == 0) {
             snext = (int64_t)atomicAdd((unsigned long long*)&cnt[HT_CNT_NEXT + TIER], 1ull);
             sfail = 0;
+            nlong = 0;
+            ssum[0] = ssum[1] = 0;
         }
         __syncthreads();
         int64_t idx = snext;
         if (idx >= nl) break;
         int32_t n = list[idx];
         int64_t vb = pol.vb(n), ve = pol.ve(n);
+        const int deg = ve - vb < (int64_t)INT_MAX ? (int)(ve - vb) : INT_MAX;
+        const bool flat = deg <= FLAT;
+        const int glog = group_log(ve - vb, workv[n]);
         Acc acc;
-        bool ok = block_visit<S, Pol, T>(pol, n, vb, ve, t, acc, sseg, spre, swarp, &sfail);
+        bool ok;
+        int sb = -1;
+        int32_t total = 0;
+        unsigned long long wsum = 0, ksum = 0;
+        if (flat) {
+            if (threadIdx.x < FLAT) {   // whole warps
+                Seg<S> g{};
+                if ((int)threadIdx.x < deg) g = pol.seg(vb + threadIdx.x, acc);
+                sseg[threadIdx.x] = g;
+                wsum = g.w;
+                ksum = g.k;
+                int32_t inc = g.len;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    int32_t t2 = __shfl_up_sync(FULL, inc, o);
+                    if (lane >= o) inc += t2;
+                }
+                spre[threadIdx.x] = inc - g.len;
+                if (lane == 31) swarp[warp] = inc;
+            }
+        } else if (sizeof(S) == 4) {
+            Acc other;
+            for (int64_t i = vb + threadIdx.x; i < ve; i += T) {
+                Seg<S> g = pol.seg(i, other);
+                wsum += g.w;
+                ksum += g.k;
+            }
+        }
+        // bounds of a key's weight and overlap: the sums over all incidences
+        if (sizeof(S) == 4 && vb + (threadIdx.x & ~31) < ve) {
+            wsum = warp_sum(wsum);
+            ksum = warp_sum(ksum);
+            if (lane == 0) {
+                atomicAdd(&ssum[0], wsum);
+                atomicAdd(&ssum[1], ksum);
+            }
+        }
+        __syncthreads();
+        if (flat) {
+            int32_t before = 0;
+#pragma unroll
+            for (int w = 0; w < FLAT / 32; w++) {
+                if (w < warp) before += swarp[w];
+                total += swarp[w];
+            }
+            if (threadIdx.x < FLAT && before) spre[threadIdx.x] += before;
+            __syncthreads();
+        }
+        if constexpr (sizeof(S) == 4) {
+            int wb = 64 - __clzll((long long)ssum[0]), kb = 64 - __clzll((long long)ssum[1]);
+            if (wb + kb <= 32) sb = kb;
+        }
+        auto visit = [&](const auto& tb) {
+            const typename Pol::Own own = pol.own(n);
+            bool k = true;
+            if (flat) {
+                constexpr int U = 4;   // elements in flight per thread
+                int32_t lo = 0;
+                for (int32_t v0 = threadIdx.x; v0 < total && k; v0 += U * T) {
+                    typename Pol::Item it[U];
+#pragma unroll
+                    for (int u = 0; u < U; u++) {
+                        int32_t v = v0 + u * T;
+                        if (v < total) {
+                            lo = seg_find(spre, deg, lo, v);
+                            it[u] = pol.load(n, own, sseg[lo], v - spre[lo]);
+                        } else {
+                            it[u] = Pol::none();
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; u++) k = pol.put(n, it[u], tb, acc) && k;
+                }
+                return k;
+            }
+            k = group_visit<S, T, 2>(pol, n, vb, ve, glog, threadIdx.x, tb, acc, slong, &nlong);
+            __syncthreads();
+            const int nlg = nlong < HT_NLONG ? nlong : HT_NLONG;
+            Acc other;   // the segments' own terms are in already
+            for (int x = 0; x < nlg && k; x++) {
+                Seg<S> g = pol.seg(slong[x], other);
+                for (int32_t off = threadIdx.x; off < g.len && k; off += 2 * T) {
+                    typename Pol::Item a = pol.load(n, own, g, off);
+                    typename Pol::Item b = off + T < g.len ? pol.load(n, own, g, off + T) : Pol::none();
+                    k = pol.put(n, a, tb, acc) && k;
+                    k = pol.put(n, b, tb, acc) && k;
+                }
+            }
+            return k;
+        };
+        if constexpr (sizeof(S) == 4) {
+            if (sb >= 0) ok = visit(PackedTable{t.key, (uint32_t*)t.sc, t.mask, t.probes, sb});
+            else ok = visit(t);
+        } else {
+            ok = visit(t);
+        }
+        if (!ok) sfail = 1;
         Acc wa = Pol::warp_reduce(acc);
         if (lane == 0) wacc[warp] = wa;
         __syncthreads();
-        if (!ok) {
+        if (sfail) {
             clear_slots(t, threadIdx.x, CAP, T);
             if (threadIdx.x == 0) ht_push(pol, NEXT, n, workv[n], lists, cnt, scap);
             __syncthreads();
@@ -566,7 +824,19 @@ __global__ void __launch_bounds__(T)
         int64_t bs = 0;
         int32_t bk = -1;
         uint32_t bo = 0;
-        scan_slots<S>(pol, n, t, threadIdx.x, CAP, T, tot, bs, bk, bo);
+        if (sb >= 0) {
+            const uint32_t omask = (1u << sb) - 1;   // sb < 32: a weight of 0 needs no bit
+            for (int i = threadIdx.x; i < CAP; i += T) {
+                int32_t k = t.key[i];
+                if (k < 0) continue;
+                uint32_t v = (uint32_t)t.sc[i];
+                t.key[i] = -1;
+                t.sc[i] = 0;
+                pol.consider(n, k, (int64_t)(v >> sb), v & omask, tot, bs, bk, bo);
+            }
+        } else {
+            scan_slots<S>(pol, n, t, threadIdx.x, CAP, T, tot, bs, bk, bo);
+        }
         warp_argmax(bs, bk, bo);
         if (lane == 0) {
             rs[warp] = bs;
@@ -593,11 +863,9 @@ __global__ void __launch_bounds__(T)
 // handed on, no split tier and no wait for its sizes. Presence of a key is a
 // nonzero sum, so every weight has to be positive (the callers know).
 //
-// A group of G lanes takes an incidence (G: the mean segment, a power of
-// two) and loops over its segment, U incidences in flight per group, since a
-// block walking one heavy super-node's incidences is a chain of gathers
-// (incidence -> hyperedge -> pins); segments longer than HT_DENSE_LONG are
-// left to the whole block.
+// Four incidences are in flight per group, since a block walking one heavy
+// super-node's incidences is a chain of gathers (incidence -> hyperedge ->
+// pins).
 //
 // Clearing, scanning and occupancy bound it from above: a vertex costs the
 // whole key range once, so vertices of little work stay on the hash tiers
@@ -605,8 +873,6 @@ __global__ void __launch_bounds__(T)
 constexpr int64_t HT_DENSE_KEYS = 24 * 1024;   // 192 KB of 32-bit sum pairs
 constexpr int64_t HT_DENSE_SMALL = 4 * 1024;   // 32 KB: several 256-thread blocks per SM
 constexpr int64_t HT_DENSE_BWORK = 8192;       // most elements a 256-thread block takes there
-constexpr int HT_DENSE_LONG = 1024;
-constexpr int HT_DENSE_NLONG = 256;
 
 template <typename S>
 struct DenseTable {
@@ -620,27 +886,93 @@ struct DenseTable {
     }
 };
 
+
+// one vertex by one block: its elements into the arrays, the sums of the
+// policy's per-vertex terms into wacc[0..T/32)
+template <class Pol, int T>
+__device__ __forceinline__ void dense_count(const Pol& pol, int32_t n, int64_t vb, int64_t ve, int glog,
+                                            const DenseTable<typename Pol::S>& t,
+                                            typename Pol::Acc* wacc, int64_t* slong, int32_t* nlong)
+{
+    using S = typename Pol::S;
+    using Acc = typename Pol::Acc;
+    const typename Pol::Own own = pol.own(n);
+    Acc acc, other;
+    group_visit<S, T, 4>(pol, n, vb, ve, glog, threadIdx.x, t, acc, slong, nlong);
+    __syncthreads();
+    const int nlg = *nlong < HT_NLONG ? *nlong : HT_NLONG;
+    for (int x = 0; x < nlg; x++) {
+        Seg<S> g = pol.seg(slong[x], other);   // its own terms are in already
+        for (int32_t off = threadIdx.x; off < g.len; off += T)
+            pol.put(n, pol.load(n, own, g, off), t, acc);
+    }
+    Acc wa = Pol::warp_reduce(acc);
+    if ((threadIdx.x & 31) == 0) wacc[threadIdx.x >> 5] = wa;
+    __syncthreads();
+}
+
+struct HtBest {
+    int64_t s;
+    int32_t k;
+    uint32_t o;
+};
+
+// best of the block's threads, valid in thread 0
+template <int T>
+__device__ __forceinline__ HtBest block_best(int64_t bs, int32_t bk, uint32_t bo, HtBest* wbest)
+{
+    warp_argmax(bs, bk, bo);
+    if ((threadIdx.x & 31) == 0) wbest[threadIdx.x >> 5] = HtBest{bs, bk, bo};
+    __syncthreads();
+    HtBest b = wbest[0];
+    if (threadIdx.x == 0)
+        for (int w = 1; w < T / 32; w++)
+            if (better(wbest[w].s, wbest[w].k, b.s, b.k)) b = wbest[w];
+    return b;
+}
+
+// one vertex by one block, to its result
+template <class Pol, int T>
+__device__ __forceinline__ void dense_vertex(const Pol& pol, int32_t n, int64_t work, int32_t keys,
+                                             const DenseTable<typename Pol::S>& t,
+                                             typename Pol::Acc* wacc, HtBest* wbest, int64_t* slong,
+                                             int32_t* nlong)
+{
+    using S = typename Pol::S;
+    const int64_t vb = pol.vb(n), ve = pol.ve(n);
+    dense_count<Pol, T>(pol, n, vb, ve, group_log(ve - vb, work), t, wacc, slong, nlong);
+    typename Pol::Acc tot = wacc[0];
+    for (int w = 1; w < T / 32; w++) tot.add(wacc[w]);
+    int64_t bs = 0;
+    int32_t bk = -1;
+    uint32_t bo = 0;
+    for (int32_t k = threadIdx.x; k < keys; k += T) {
+        S v = t.sc[k];
+        if (v == 0) continue;
+        uint32_t o = t.ov[k];
+        t.sc[k] = 0;
+        t.ov[k] = 0;
+        pol.consider(n, k, (int64_t)v, o, tot, bs, bk, bo);
+    }
+    HtBest b = block_best<T>(bs, bk, bo, wbest);
+    if (threadIdx.x == 0) pol.write(n, b.s, b.k, b.o, tot);
+    __syncthreads();
+}
+
 template <class Pol, int T, int TIER>
 __global__ void __launch_bounds__(T)
-    k_ht_dense(Pol pol, const int32_t* __restrict__ lists, int64_t* cnt, int32_t keys, int glog)
+    k_ht_dense(Pol pol, const int32_t* __restrict__ lists, int64_t* cnt, int32_t keys,
+               const int64_t* __restrict__ workv)
 {
     using S = typename Pol::S;
     using Acc = typename Pol::Acc;
     extern __shared__ __align__(16) unsigned char ht_dyn[];
-    __shared__ int64_t slong[HT_DENSE_NLONG];
+    __shared__ int64_t slong[HT_NLONG];
     __shared__ int32_t nlong;
     __shared__ __align__(16) unsigned char wacc_raw[sizeof(Acc) * (T / 32)];
-    __shared__ int64_t rs[T / 32];
-    __shared__ int32_t rk[T / 32];
-    __shared__ uint32_t ro[T / 32];
+    __shared__ HtBest wbest[T / 32];
     __shared__ int64_t snext;
-    Acc* wacc = (Acc*)wacc_raw;
     DenseTable<S> t{(S*)ht_dyn, (uint32_t*)(ht_dyn + (size_t)keys * sizeof(S))};
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int G = 1 << glog, gl = threadIdx.x & (G - 1), grp = threadIdx.x >> glog;
-    const int ngrp = T >> glog;
-    const unsigned gmask = G == 32 ? FULL : ((1u << G) - 1) << (lane & ~(G - 1));
-    constexpr int U = 4;
     const int32_t* list = lists + (int64_t)TIER * pol.V;
     const int64_t nl = cnt[TIER];
     if (nl == 0) return;
@@ -657,77 +989,123 @@ __global__ void __launch_bounds__(T)
         const int64_t idx = snext;
         if (idx >= nl) break;
         const int32_t n = list[idx];
-        const int64_t vb = pol.vb(n), ve = pol.ve(n);
-        Acc acc, other;   // a segment's own terms count once, in its first lane
-        for (int64_t i0 = vb + grp; i0 < ve; i0 += (int64_t)U * ngrp) {
-            Seg<S> g[U];
-            typename Pol::Item it[U];
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                int64_t i = i0 + (int64_t)u * ngrp;
-                g[u] = Seg<S>{0, 0, 0, 0, 0, 0};
-                if (i < ve) g[u] = pol.seg(i, gl == 0 ? acc : other);
-                if (g[u].len > HT_DENSE_LONG) {
-                    int32_t at = HT_DENSE_NLONG;
-                    if (gl == 0) at = atomicAdd(&nlong, 1);
-                    at = __shfl_sync(gmask, at, lane & ~(G - 1));
-                    if (at < HT_DENSE_NLONG) {
-                        if (gl == 0) slong[at] = i;
-                        g[u].len = 0;
-                    }
-                }
+        dense_vertex<Pol, T>(pol, n, workv[n], keys, t, (Acc*)wacc_raw, wbest, slong, &nlong);
+    }
+}
+
+// The big tier. While it holds few vertices (a tail level has a handful for
+// the whole GPU), a cluster of eight blocks takes one, each block counting an
+// eighth of its incidences into its own arrays; the sums are joined through
+// distributed shared memory, an eighth of the keys per block. One block alone
+// is bound by its SM's shared-memory atomics (67 to 177 us for the one merged
+// super-node of a level of the 12,007-neuron power-law network, 23 with the
+// cluster). With more than HT_SOLO vertices every block takes its own (the
+// 60,052-neuron layered network: 65 us a level, 113 with clusters). A block
+// tier of at most `leave` vertices is taken here as well: their latency on
+// 256 threads each would be the level's (79 us).
+constexpr int HT_DENSE_CTAS = 8;
+constexpr int64_t HT_SOLO = 38;       // two waves of clusters
+constexpr int64_t HT_LEAVE = 304;     // two waves of blocks
+
+template <class Pol, int T>
+__global__ void __cluster_dims__(HT_DENSE_CTAS, 1, 1) __launch_bounds__(T)
+    k_ht_dense_big(Pol pol, const int32_t* __restrict__ lists, int64_t* cnt, int32_t keys,
+                   const int64_t* __restrict__ workv, int64_t leave)
+{
+    namespace cg = cooperative_groups;
+    using S = typename Pol::S;
+    using Acc = typename Pol::Acc;
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ __align__(16) unsigned char ht_dyn[];
+    __shared__ int64_t slong[HT_NLONG];
+    __shared__ int32_t nlong;
+    __shared__ __align__(16) unsigned char wacc_raw[sizeof(Acc) * (T / 32)];
+    __shared__ HtBest wbest[T / 32];
+    __shared__ HtBest sbest;
+    __shared__ int64_t snext;
+    Acc* wacc = (Acc*)wacc_raw;
+    DenseTable<S> t{(S*)ht_dyn, (uint32_t*)(ht_dyn + (size_t)keys * sizeof(S))};
+    const int rank = (int)cl.block_rank();
+    const int64_t nb = cnt[HT_TIER_BLOCK] <= leave ? cnt[HT_TIER_BLOCK] : 0;
+    const int64_t nl = nb + cnt[HT_TIER_BIG];
+    if (nl == 0) return;   // every block
+    auto vertex = [&](int64_t idx) {
+        return idx < nb ? lists[(int64_t)HT_TIER_BLOCK * pol.V + idx]
+                        : lists[(int64_t)HT_TIER_BIG * pol.V + (idx - nb)];
+    };
+    unsigned long long* next = (unsigned long long*)&cnt[HT_CNT_NEXT + HT_TIER_BIG];
+    for (int32_t k = threadIdx.x; k < keys; k += T) {
+        t.sc[k] = 0;
+        t.ov[k] = 0;
+    }
+    if (nl > HT_SOLO) {
+        for (;;) {
+            if (threadIdx.x == 0) {
+                snext = (int64_t)atomicAdd(next, 1ull);
+                nlong = 0;
             }
-#pragma unroll
-            for (int u = 0; u < U; u++)
-                it[u] = gl < g[u].len ? pol.load(n, g[u], gl) : Pol::none();
-#pragma unroll
-            for (int u = 0; u < U; u++) pol.put(n, it[u], t, acc);
-#pragma unroll
-            for (int u = 0; u < U; u++)
-                for (int32_t off = gl + G; off < g[u].len; off += G)
-                    pol.put(n, pol.load(n, g[u], off), t, acc);
+            __syncthreads();
+            const int64_t idx = snext;
+            if (idx >= nl) return;
+            const int32_t n = vertex(idx);
+            dense_vertex<Pol, T>(pol, n, workv[n], keys, t, wacc, wbest, slong, &nlong);
         }
-        __syncthreads();
-        const int nlg = nlong < HT_DENSE_NLONG ? nlong : HT_DENSE_NLONG;
-        for (int x = 0; x < nlg; x++) {
-            Seg<S> g = pol.seg(slong[x], other);   // its own terms are in already
-            for (int32_t off = threadIdx.x; off < g.len; off += T)
-                pol.put(n, pol.load(n, g, off), t, acc);
+    }
+    for (;;) {
+        if (threadIdx.x == 0) {
+            if (rank == 0) snext = (int64_t)atomicAdd(next, 1ull);
+            nlong = 0;
         }
-        Acc wa = Pol::warp_reduce(acc);
-        if (lane == 0) wacc[warp] = wa;
-        __syncthreads();
-        Acc tot = wacc[0];
-        for (int w = 1; w < T / 32; w++) tot.add(wacc[w]);
+        cl.sync();
+        const int64_t idx = *cl.map_shared_rank(&snext, 0);
+        if (idx >= nl) break;
+        const int32_t n = vertex(idx);
+        const int64_t v0 = pol.vb(n), deg = pol.ve(n) - v0;
+        dense_count<Pol, T>(pol, n, v0 + deg * rank / HT_DENSE_CTAS, v0 + deg * (rank + 1) / HT_DENSE_CTAS,
+                            group_log(deg, workv[n]), t, wacc, slong, &nlong);
+        if (threadIdx.x == 0)
+            for (int w = 1; w < T / 32; w++) wacc[0].add(wacc[w]);
+        cl.sync();   // counts and sums of all blocks are in
+        Acc tot = *cl.map_shared_rank(&wacc[0], 0);
+        for (int r = 1; r < HT_DENSE_CTAS; r++) tot.add(*cl.map_shared_rank(&wacc[0], r));
         int64_t bs = 0;
         int32_t bk = -1;
         uint32_t bo = 0;
-        for (int32_t k = threadIdx.x; k < keys; k += T) {
-            S v = t.sc[k];
+        const S* sc[HT_DENSE_CTAS];
+        const uint32_t* ov[HT_DENSE_CTAS];
+#pragma unroll
+        for (int r = 0; r < HT_DENSE_CTAS; r++) {
+            sc[r] = cl.map_shared_rank(t.sc, r);
+            ov[r] = cl.map_shared_rank(t.ov, r);
+        }
+        for (int32_t k = rank * T + threadIdx.x; k < keys; k += HT_DENSE_CTAS * T) {
+            S v = 0;
+#pragma unroll
+            for (int r = 0; r < HT_DENSE_CTAS; r++) v += sc[r][k];
             if (v == 0) continue;
-            uint32_t o = t.ov[k];
-            t.sc[k] = 0;
-            t.ov[k] = 0;
+            uint32_t o = 0;
+#pragma unroll
+            for (int r = 0; r < HT_DENSE_CTAS; r++) o += ov[r][k];
             pol.consider(n, k, (int64_t)v, o, tot, bs, bk, bo);
         }
-        warp_argmax(bs, bk, bo);
-        if (lane == 0) {
-            rs[warp] = bs;
-            rk[warp] = bk;
-            ro[warp] = bo;
+        HtBest b = block_best<T>(bs, bk, bo, wbest);
+        if (threadIdx.x == 0) sbest = b;
+        cl.sync();   // every block has read the arrays
+        if (rank == 0 && threadIdx.x == 0) {
+            for (int r = 1; r < HT_DENSE_CTAS; r++) {
+                HtBest c = *cl.map_shared_rank(&sbest, r);
+                if (better(c.s, c.k, b.s, b.k)) b = c;
+            }
+            pol.write(n, b.s, b.k, b.o, tot);
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int w = 1; w < T / 32; w++)
-                if (better(rs[w], rk[w], bs, bk)) {
-                    bs = rs[w];
-                    bk = rk[w];
-                    bo = ro[w];
-                }
-            pol.write(n, bs, bk, bo, tot);
+        for (int32_t k = threadIdx.x; k < keys; k += T) {
+            if (t.sc[k]) {
+                t.sc[k] = 0;
+                t.ov[k] = 0;
+            }
         }
-        __syncthreads();
     }
+    cl.sync();   // no block leaves while another reads its shared memory
 }
 
 // Split tier. The incidences of the split vertices are laid out flat
@@ -835,7 +1213,8 @@ __global__ void __launch_bounds__(HT_WARPS * 32)
                      const int64_t* __restrict__ od, int64_t D,
                      const int64_t* __restrict__ item_f0, int64_t nitems,
                      const int64_t* __restrict__ toff, const int64_t* __restrict__ scap,
-                     unsigned char* pool, typename Pol::Acc* gacc, int32_t* ovf, uint32_t probes)
+                     unsigned char* pool, typename Pol::Acc* gacc, int32_t* ovf, uint32_t probes,
+                     const int64_t* __restrict__ workv)
 {
     using S = typename Pol::S;
     using Acc = typename Pol::Acc;
@@ -858,14 +1237,16 @@ __global__ void __launch_bounds__(HT_WARPS * 32)
         if (probes) g.probes = probes;
         Acc acc;
         bool ok;
+        const int glog = group_log(od[j + 1] - od[j], workv[n]);
         if (scap[j] <= HT_WCAP) {
             Table<S> p = priv;
             p.mask = (uint32_t)(scap[j] - 1);
             p.probes = (uint32_t)scap[j];
-            ok = warp_visit<S>(pol, n, vb, ve, 32, p, acc);
+            ok = __all_sync(FULL, (group_visit<S, 32, 2>(pol, n, vb, ve, glog, lane, p, acc)));
+            __syncwarp();
             ok = flush_private(p, scap[j], g) && ok;
         } else {
-            ok = warp_visit<S>(pol, n, vb, ve, 32, g, acc);
+            ok = __all_sync(FULL, (group_visit<S, 32, 2>(pol, n, vb, ve, glog, lane, g, acc)));
         }
         if (!ok && lane == 0) ovf[j] = 1;
         Acc wa = Pol::warp_reduce(acc);
@@ -1005,7 +1386,7 @@ Status run_split(const Pol& pol, Arena& ar, cudaStream_t s, const int32_t* sl, i
     SNN_L k_ht_split_visit<Pol><<<(int)std::min<int64_t>(ceil_div(items, HT_WARPS), 152 * 8),
                                   HT_WARPS * 32, wsm, s>>>(pol, sl, ns, od, D, item_f0, items, toff,
                                                            scap, pool, gacc, ovf,
-                                                           limit > 0 ? 256u : 0u);
+                                                           limit > 0 ? 256u : 0u, workv);
     SNN_CUDA(cudaGetLastError());
     SNN_L k_ht_split_scan<Pol><<<(int)std::min<int64_t>(ns, 152 * 4), 1024, 0, s>>>(pol, sl, ns, toff,
                                                                                     scap, pool, gacc, ovf);
@@ -1094,7 +1475,7 @@ Status run_histogram(const Pol& pol, Arena& ar, cudaStream_t s, int64_t* d_cnt, 
     int64_t* ntodo = d_cnt + HT_CNT_TODO;
     SNN_TRY(ar.alloc(&todo, V));
     SNN_L k_ht_skip<Pol><<<grid_for(V, 256), 256, 0, s>>>(pol, workv, todo, ntodo);
-    SNN_L k_ht_work<Pol><<<grid_for(V, 8), 256, 0, s>>>(pol, workv, todo, ntodo);
+    SNN_L k_ht_work<Pol><<<grid_for(V, 8, 152 * 16), 256, 0, s>>>(pol, workv, todo, ntodo);
     SNN_CUDA(cudaGetLastError());
     SNN_L k_ht_classify<Pol><<<grid_for(V, 256), 256, 0, s>>>(pol, workv, lists, d_cnt, scap, tiers, dense_big);
     SNN_CUDA(cudaGetLastError());
@@ -1110,25 +1491,30 @@ Status run_histogram(const Pol& pol, Arena& ar, cudaStream_t s, int64_t* d_cnt, 
                            s>>>(pol, lists, d_cnt, workv, scap);
     SNN_CUDA(cudaGetLastError());
     const size_t dsm = (size_t)key_space * (sizeof(S) + sizeof(uint32_t));
-    int glog = 2;   // lanes per incidence: the level's mean hyperedge size
-    while (glog < 5 && (1 << glog) < hedge_lanes(pol.L.P, pol.L.E)) glog++;
-    if (dense_block) {
-        auto kd = k_ht_dense<Pol, HT_BTHREADS, HT_TIER_BLOCK>;
-        SNN_L kd<<<(int)std::min<int64_t>(V, 152 * 6), HT_BTHREADS, dsm, s>>>(pol, lists, d_cnt,
-                                                                              key_space, glog);
-    } else {
+    if constexpr (sizeof(S) == 4) {
+        if (dense_block) {
+            auto kd = k_ht_dense<Pol, HT_BTHREADS, HT_TIER_BLOCK>;
+            SNN_L kd<<<(int)std::min<int64_t>(V, 152 * 6), HT_BTHREADS, dsm, s>>>(pol, lists, d_cnt,
+                                                                                  key_space, workv);
+        }
+        if (dense_big) {
+            auto kd = k_ht_dense_big<Pol, 1024>;
+            const int64_t leave = dense_block ? 0 : HT_LEAVE;
+            if (!dense_block) {
+                SNN_TRY(set_smem(kb, bsm));
+                SNN_L kb<<<(int)std::min<int64_t>(V, 152 * 8), HT_BTHREADS, bsm, s>>>(pol, lists, d_cnt,
+                                                                                      scap, workv, leave);
+            }
+            SNN_TRY(set_smem(kd, (size_t)HT_DENSE_KEYS * 8));
+            SNN_L kd<<<19 * HT_DENSE_CTAS, 1024, dsm, s>>>(pol, lists, d_cnt, key_space, workv, leave);
+        }
+    }
+    if (!dense_big) {
         SNN_TRY(set_smem(kb, bsm));
         SNN_L kb<<<(int)std::min<int64_t>(V, 152 * 8), HT_BTHREADS, bsm, s>>>(pol, lists, d_cnt, scap,
-                                                                              workv);
-    }
-    SNN_CUDA(cudaGetLastError());
-    if (dense_big) {
-        auto kd = k_ht_dense<Pol, 1024, HT_TIER_BIG>;
-        SNN_TRY(set_smem(kd, (size_t)HT_DENSE_KEYS * (sizeof(S) + sizeof(uint32_t))));
-        SNN_L kd<<<(int)std::min<int64_t>(V, 152), 1024, dsm, s>>>(pol, lists, d_cnt, key_space, glog);
-    } else {
+                                                                              workv, 0);
         SNN_TRY(set_smem(kg, gsm));
-        SNN_L kg<<<152, HT_GTHREADS, gsm, s>>>(pol, lists, d_cnt, scap, workv);
+        SNN_L kg<<<152, HT_GTHREADS, gsm, s>>>(pol, lists, d_cnt, scap, workv, 0);
     }
     SNN_CUDA(cudaGetLastError());
     if (!split) return Status{};

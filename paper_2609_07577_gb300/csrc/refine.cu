@@ -55,6 +55,7 @@ struct PinCounts {
     int32_t* cnt;
     int32_t* dcnt;
     int32_t* lam;
+    HRec* rec;     // per hyperedge: first entry, omega, k, lam and masks of its first 32 entries
 };
 
 struct PState {
@@ -166,6 +167,7 @@ struct PinCountJob {
             R += __popc(mr);
         }
         // pass 2: starts -> counts
+        uint32_t dm = 0, sm = 0;
         for (int c = 0; c < R; c += 32) {
             int r = c + lane;
             int st = 0, nx = 0, dsx = -1;
@@ -175,22 +177,28 @@ struct PinCountJob {
                 dsx = pc.dcnt[base + r];
             }
             __syncwarp();
+            int dc = r < R && dsx >= 0 ? nx - dsx : 0;
             if (r < R) {
-                int dc = dsx >= 0 ? nx - dsx : 0;
                 pc.cnt[base + r] = nx - st;
                 pc.dcnt[base + r] = dc;
                 if (dc > 0) add_inbound(pc.p[base + r], hk[a]);
             }
-            __syncwarp();
+            unsigned md = __ballot_sync(FULL, dc > 0), ms = __ballot_sync(FULL, r < R && nx - st == 1);
+            if (c == 0) {
+                dm = md;
+                sm = ms;
+            }
         }
         if (lane == 0) {
             pc.lam[a] = R;
+            pc.rec[a] = HRec{base, hw[a], (uint32_t)hk[a], (uint32_t)R | (uint32_t)hsd[a] << 31, dm, sm};
             if (R > 1) atomicAdd((unsigned long long*)&cost[a & cost_mask], (unsigned long long)(hw[a] * (R - 1)));
         }
     }
     __device__ void finish_thread(int32_t a, const uint32_t* s, int n, int st) const
     {
         int64_t base = hoff[a];
+        uint32_t dm = 0, sm = 0;   // at most SEG_T_CAP runs
         int R = 0, c = 0, d = 0;
         for (int i = 0; i < n; i++) {
             uint32_t p = s[(i) * st] >> 1;
@@ -199,6 +207,8 @@ struct PinCountJob {
                 pc.cnt[base + R] = c;
                 pc.dcnt[base + R] = d;
                 if (d > 0) add_inbound((int32_t)(s[(i - 1) * st] >> 1), hk[a]);
+                dm |= (uint32_t)(d > 0) << R;
+                sm |= (uint32_t)(c == 1) << R;
                 R++;
                 c = 0;
                 d = 0;
@@ -211,9 +221,12 @@ struct PinCountJob {
             pc.cnt[base + R] = c;
             pc.dcnt[base + R] = d;
             if (d > 0) add_inbound((int32_t)(s[(n - 1) * st] >> 1), hk[a]);
+            dm |= (uint32_t)(d > 0) << R;
+            sm |= (uint32_t)(c == 1) << R;
             R++;
         }
         pc.lam[a] = R;
+        pc.rec[a] = HRec{base, hw[a], (uint32_t)hk[a], (uint32_t)R | (uint32_t)hsd[a] << 31, dm, sm};
         if (R > 1) atomicAdd((unsigned long long*)&cost[a & cost_mask], (unsigned long long)(hw[a] * (R - 1)));
     }
 };
@@ -334,6 +347,7 @@ struct GainPol {
     using S = S_;
     // a vertex meets few partitions even when its bound is large
     static constexpr bool kOptimistic = true;
+    static constexpr bool kMasks = true;
     struct Acc {
         int64_t W, save;   // summed omega of incident hyperedges; of those n is the last pin of
         __device__ Acc() : W(0), save(0) {}
@@ -379,16 +393,9 @@ struct GainPol {
     __device__ Seg<S> seg(int64_t i, Acc& acc) const
     {
         uint32_t inc = (uint32_t)L.vinc[i];
-        int32_t a = (int32_t)(inc & ~SRC_BIT);
-        Seg<S> g;
-        g.sd = L.hsd[a];
-        g.nd = !(inc & SRC_BIT) || g.sd;
-        g.b = L.hoff[a];
-        g.len = pc.lam[a];
-        g.w = (S)L.hw[a];
-        g.k = (uint32_t)L.hk[a];
-        acc.W += L.hw[a];
-        return g;
+        HRec r = pc.rec[(int32_t)(inc & ~SRC_BIT)];
+        acc.W += r.w;
+        return rec_seg<S>(r, inc);
     }
     // one element: partition p (-1: nothing to add, -2: weight w to save)
     struct Item {
@@ -397,15 +404,23 @@ struct GainPol {
         uint32_t o;
     };
     static __device__ Item none() { return Item{-1, 0, 0u}; }
-    __device__ Item load(int32_t n, const Seg<S>& g, int32_t off) const
+    struct Own {
+        int32_t part, size, inpins;
+    };
+    __device__ Own own(int32_t n) const { return Own{rho[n], L.vsize[n], L.vinpins[n]}; }
+    __device__ Item load(int32_t, const Own& o, const Seg<S>& g, int32_t off) const
     {
         int64_t e = g.b + off;
         int32_t p = pc.p[e];
-        if (p == rho[n]) return Item{pc.cnt[e] == 1 ? -2 : -1, g.w, 0u};
+        if (p == o.part) {
+            bool one = off < 32 ? (g.sm >> off) & 1 : pc.cnt[e] == 1;
+            return Item{one ? -2 : -1, g.w, 0u};
+        }
         // a partition that cannot take n by size or inbound pins is never
         // the chosen move: leave it out of the table
-        if (ps.size[p] + L.vsize[n] > omega || ps.inpins[p] + L.vinpins[n] > phi) return none();
-        return Item{p, g.w, (g.nd && pc.dcnt[e] > 0) ? g.k : 0u};
+        if (ps.size[p] + o.size > omega || ps.inpins[p] + o.inpins > phi) return none();
+        bool in = off < 32 ? (g.dm >> off) & 1 : pc.dcnt[e] > 0;
+        return Item{p, g.w, (g.nd && in) ? g.k : 0u};
     }
     template <class Tb>
     __device__ bool put(int32_t, const Item& it, const Tb& t, Acc& acc) const
@@ -471,6 +486,7 @@ struct RowPol {
     using S = S_;
     // a row holds every adjacent partition: warp tables would overflow
     static constexpr bool kOptimistic = false;
+    static constexpr bool kMasks = true;
     struct Acc {
         __device__ Acc() {}
         __device__ void add(const Acc&) {}
@@ -500,15 +516,7 @@ struct RowPol {
     __device__ Seg<S> seg(int64_t i, Acc&) const
     {
         uint32_t inc = (uint32_t)L.vinc[i];
-        int32_t a = (int32_t)(inc & ~SRC_BIT);
-        Seg<S> g;
-        g.sd = L.hsd[a];
-        g.nd = !(inc & SRC_BIT) || g.sd;
-        g.b = L.hoff[a];
-        g.len = pc.lam[a];
-        g.w = (S)L.hw[a];
-        g.k = (uint32_t)L.hk[a];
-        return g;
+        return rec_seg<S>(pc.rec[(int32_t)(inc & ~SRC_BIT)], inc);
     }
     struct Item {
         int32_t p;
@@ -516,10 +524,13 @@ struct RowPol {
         uint32_t o;
     };
     static __device__ Item none() { return Item{-1, 0, 0u}; }
-    __device__ Item load(int32_t, const Seg<S>& g, int32_t off) const
+    struct Own {};
+    __device__ Own own(int32_t) const { return Own{}; }
+    __device__ Item load(int32_t, const Own&, const Seg<S>& g, int32_t off) const
     {
         int64_t e = g.b + off;
-        return Item{pc.p[e], g.w, (g.nd && pc.dcnt[e] > 0) ? g.k : 0u};
+        bool in = off < 32 ? (g.dm >> off) & 1 : pc.dcnt[e] > 0;
+        return Item{pc.p[e], g.w, (g.nd && in) ? g.k : 0u};
     }
     template <class Tb>
     __device__ bool put(int32_t, const Item& it, const Tb& t, Acc&) const
@@ -577,17 +588,36 @@ __global__ void __launch_bounds__(256)
         int32_t bk = -1;
         const int64_t nq = ((int64_t)K + 3) >> 2;
         unsigned long long msk = M[rw];   // the same word in every lane
-        while (msk) {
-            int c = __ffsll((long long)msk) - 1;
-            msk &= msk - 1;
-            int64_t q0 = (int64_t)c * (cw >> 2);
-            int64_t q1 = q0 + (cw >> 2) < nq ? q0 + (cw >> 2) : nq;
-            for (int64_t q = q0 + lane; q < q1; q += 32) {
-                int4 c4 = row[q];
-                int cv[4] = {c4.x, c4.y, c4.z, c4.w};
+        // marked entries four loads at a time, in increasing order: row entry
+        // it of the marked ones, 32 int4 per step (cw >> 2 of them a chunk)
+        const int per = (cw >> 2) > 32 ? (cw >> 2) / 32 : 1;   // steps per chunk
+        int step = 0, c = -1;
+        while (msk || step > 0) {
+            constexpr int U = 4;
+            int4 c4[U];
+            int64_t qq[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                if (step == 0 && msk) {
+                    c = __ffsll((long long)msk) - 1;
+                    msk &= msk - 1;
+                    step = per;
+                }
+                qq[u] = nq;
+                if (step > 0) {
+                    int64_t q0 = (int64_t)c * (cw >> 2);
+                    int64_t q = q0 + (int64_t)(per - step) * 32 + lane;
+                    if (q < q0 + (cw >> 2)) qq[u] = q;
+                    step--;
+                }
+                c4[u] = qq[u] < nq ? row[qq[u]] : make_int4(0, 0, 0, 0);
+            }
+#pragma unroll
+            for (int v = 0; v < U; v++) {
+                int cv[4] = {c4[v].x, c4[v].y, c4[v].z, c4[v].w};
 #pragma unroll
                 for (int u = 0; u < 4; u++) {
-                    int32_t p = (int32_t)(4 * q + u);
+                    int32_t p = (int32_t)(4 * qq[v] + u);
                     int64_t g = (int64_t)cv[u] - T;
                     // default: positive gains only (bs starts at 0); variant:
                     // any adjacent partition (conn > 0), the first one found
@@ -966,6 +996,38 @@ __global__ void __launch_bounds__(256)
                 uint32_t old = atomicOr(&ps.hmask[a], bit);
                 if (old == 0) ps.hl[atomicAdd(&ps.cnt[1], 1)] = a;
             }
+        }
+    }
+}
+
+// The same from the pin counts: every hyperedge looks its partitions up in the
+// slot map. A heavy super-node of a P* partition is in most hyperedges, and
+// one warp walking its incidence list took 60 to 170 us a round on tail
+// levels; this reads one word per (hyperedge, partition) of the level, so it
+// takes the levels of up to PS_MARK_PINS pins.
+constexpr int64_t PS_MARK_PINS = 16 << 20;
+
+template <int G>
+__global__ void __launch_bounds__(256)
+    k_ps_mark_counts(Level L, PinCounts pc, const int64_t* __restrict__ scal, PStar ps)
+{
+    if (!pstar_on(scal, ps.cnt)) return;
+    const int lane = threadIdx.x & (G - 1);
+    const unsigned gmask = (G == 32 ? FULL : ((1u << (G & 31)) - 1)) << ((threadIdx.x & 31) & ~(G - 1));
+    int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
+    int64_t nw = ((int64_t)gridDim.x * blockDim.x) / G;
+    for (int64_t a = gw; a < L.E; a += nw) {
+        int64_t b = L.hoff[a];
+        int32_t lam = pc.lam[a];
+        uint32_t m = 0;
+        for (int32_t r = lane; r < lam; r += G) {
+            int32_t sl = ps.pslot[pc.p[b + r]];
+            if (sl >= 0) m |= 1u << sl;
+        }
+        m = __reduce_or_sync(gmask, m);
+        if (lane == 0 && m) {
+            ps.hmask[a] = m;
+            ps.hl[atomicAdd(&ps.cnt[1], 1)] = (int32_t)a;
         }
     }
 }
@@ -1811,6 +1873,7 @@ static Status pin_counts(snnmap_hgraph* h, Level& L, LevelExtra& X, int32_t K, c
     SNN_TRY(ar.alloc(&pc.cnt, L.P));
     SNN_TRY(ar.alloc(&pc.dcnt, L.P));
     SNN_TRY(ar.alloc(&pc.lam, L.E));
+    SNN_TRY(ar.alloc(&pc.rec, L.E));
     SNN_TRY(ar.alloc(&ps.size, K));
     SNN_TRY(ar.alloc(&ps.inpins, K));
     SNN_TRY(ar.alloc(&ps.pincnt, K));
@@ -2296,7 +2359,12 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     if (!dense) {
         prof.reset(new ProfScope(h, PS_GAINS));
         if (inc.pst.colc && V > 0) {
-            SNN_L k_ps_mark<<<grid_for(V, 256), 256, 0, s>>>(L, rho, h->d_scal, inc.pst);
+            if (L.P <= PS_MARK_PINS) {
+                SNN_HEDGE_LAUNCH(hedge_lanes(L.P, 2 * (int64_t)L.E), k_ps_mark_counts, L.E, s, L, pc,
+                                 h->d_scal, inc.pst);
+            } else {
+                SNN_L k_ps_mark<<<grid_for(V, 256), 256, 0, s>>>(L, rho, h->d_scal, inc.pst);
+            }
             SNN_L k_ps_cols<<<152 * 8, 256, 0, s>>>(L, pc, rho, h->d_scal, inc.pst);
             SNN_L k_ps_combine<<<gv, 256, 0, s>>>(L, rho, h->d_scal, inc.pst, ps, savev, Wv, prm.omega,
                                                   prm.delta, prm.phi, prm.refine_nonpositive, pto,
@@ -2442,6 +2510,7 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
     cv.add(&inc.pc.cnt, L.P);
     cv.add(&inc.pc.dcnt, L.P);
     cv.add(&inc.pc.lam, E);
+    cv.add(&inc.pc.rec, E);
     cv.add(&inc.ps.size, K);
     cv.add(&inc.ps.inpins, K);
     cv.add(&inc.ps.pincnt, K);

@@ -15,7 +15,7 @@
 // hyperedge can only vanish if all its pins fall into one super-node). So
 // the next level's matrix is a gather of the previous one at the
 // representatives, plus fresh rows (a histogram, ScorePol) for the merged
-// super-nodes, mirrored into their columns.
+// super-nodes, stored into their columns as well.
 #include "histo.cuh"
 #include "internal.cuh"
 
@@ -25,6 +25,7 @@ template <typename S_>
 struct ScorePol {
     using S = S_;
     static constexpr bool kOptimistic = false;
+    static constexpr bool kMasks = false;
     struct Acc {
         __device__ Acc() {}
         __device__ void add(const Acc&) {}
@@ -67,7 +68,9 @@ struct ScorePol {
         uint32_t o;
     };
     static __device__ Item none() { return Item{-1, 0, 0u}; }
-    __device__ Item load(int32_t n, const Seg<S>& g, int32_t off) const
+    struct Own {};
+    __device__ Own own(int32_t) const { return Own{}; }
+    __device__ Item load(int32_t n, const Own&, const Seg<S>& g, int32_t off) const
     {
         int32_t m = L.hpins[g.b + off];
         int md = off != 0 || g.sd;   // pin 0 is the source
@@ -78,14 +81,14 @@ struct ScorePol {
     {
         return it.m < 0 || t.add(it.m, it.w, it.o);
     }
-    // every neighbour lands in the row (stores: a vertex redone by a later
-    // tier overwrites its partial entries)
+    // every neighbour lands in the row and, mirrored, in the column (stores: a
+    // vertex redone by a later tier overwrites its partial entries)
     __device__ void consider(int32_t n, int32_t m, int64_t s, uint32_t o, const Acc&, int64_t&,
                              int32_t&, uint32_t&) const
     {
-        int64_t r = (int64_t)n * Vs + m;
-        Sm[r] = (int32_t)s;
-        OVm[r] = (int32_t)o;
+        int64_t r = (int64_t)n * Vs + m, c = (int64_t)m * Vs + n;
+        Sm[r] = Sm[c] = (int32_t)s;
+        OVm[r] = OVm[c] = (int32_t)o;
     }
     __device__ void write(int32_t, int64_t, int32_t, uint32_t, const Acc&) const {}
 };
@@ -155,8 +158,8 @@ __global__ void k_mat_reps(int32_t V, const int32_t* __restrict__ cid,
     }
 }
 
-// S2[i][j] = S[rep(i)][rep(j)] (one block per row); rows of merged vertices
-// are cleared for their fresh sums
+// S2[i][j] = S[rep(i)][rep(j)] (one block per row); rows and columns of
+// merged vertices are cleared for their fresh sums
 __global__ void __launch_bounds__(256)
     k_mat_gather(int32_t V2, const int32_t* __restrict__ repof, const int32_t* __restrict__ fresh,
                  const int32_t* __restrict__ Sm,
@@ -174,24 +177,9 @@ __global__ void __launch_bounds__(256)
         }
         for (int64_t j = threadIdx.x; j < V2; j += blockDim.x) {
             int64_t c = repof[j];
-            S2[dst + j] = Sm[src + c];
-            OV2[dst + j] = OVm[src + c];
-        }
-    }
-}
-
-// column u of every fresh vertex u mirrors its row (one warp per vertex)
-__global__ void k_mat_mirror(int32_t V, const int32_t* __restrict__ fresh, int32_t* Sm, int32_t* OVm,
-                             int64_t Vs)
-{
-    int lane = threadIdx.x & 31;
-    int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t u = gw; u < V; u += nw) {
-        if (!fresh[u]) continue;
-        for (int64_t x = lane; x < V; x += 32) {
-            Sm[x * Vs + u] = Sm[u * Vs + x];
-            OVm[x * Vs + u] = OVm[u * Vs + x];
+            bool f = fresh[j];
+            S2[dst + j] = f ? 0 : Sm[src + c];
+            OV2[dst + j] = f ? 0 : OVm[src + c];
         }
     }
 }
@@ -307,8 +295,6 @@ Status mat_descend(snnmap_hgraph* h, int32_t src)
     M.Vs = Vs2;
     if (L.V > 0) {
         SNN_TRY(mat_rows(h, L, fresh));
-        SNN_L k_mat_mirror<<<grid_for((int64_t)L.V * 32, 256), 256, 0, s>>>(L.V, fresh, M.S, M.OV, M.Vs);
-        SNN_CUDA(cudaGetLastError());
     }
     M.level = src + 1;
     return Status{};
