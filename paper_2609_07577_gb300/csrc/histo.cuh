@@ -172,10 +172,15 @@ __device__ __forceinline__ Seg<S> rec_seg(const HRec& r, uint32_t inc)
 
 // Slots whose weight and overlap share one word, value = weight << sb |
 // overlap, for vertices whose sums over all incidences bound both within 32
-// bits: one shared-memory atomic an element instead of two.
+// bits: one shared-memory atomic an element instead of two. LIST: the slots
+// in use are listed, so the result of a large table costs a read per key
+// instead of one per slot.
+template <bool LIST>
 struct PackedTable {
     int32_t* key;
     uint32_t* val;
+    uint16_t* used;    // LIST: slots in use, *nused of them
+    int32_t* nused;
     uint32_t mask;
     uint32_t probes;
     int sb;
@@ -187,6 +192,14 @@ struct PackedTable {
             if (k == -1) {
                 int32_t prev = atomicCAS(&key[slot], -1, m);
                 k = prev == -1 ? m : prev;
+                if (LIST && prev == -1) {
+                    const unsigned am = __activemask();
+                    const int leader = __ffs(am) - 1;
+                    int32_t at = 0;
+                    if ((int)(threadIdx.x & 31) == leader) at = atomicAdd(nused, __popc(am));
+                    at = __shfl_sync(am, at, leader);
+                    used[at + __popc(am & lanemask_lt())] = (uint16_t)slot;
+                }
             }
             if (k == m) {
                 atomicAdd(&val[slot], (w << sb) + o);
@@ -531,62 +544,128 @@ __device__ __forceinline__ void ht_push(const Pol& pol, int tier, int32_t n, int
     }
 }
 
+// vertex n (of this thread; n >= V: none) into its tier's list, or its result
+// when there is nothing to count; whole warps
+template <class Pol>
+__device__ __forceinline__ void ht_place(const Pol& pol, int64_t n, int64_t work, int32_t* lists,
+                                         int64_t* cnt, int64_t* scap, const HtTiers& tiers, bool dense)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = lanemask_lt();
+    int tier = -1;
+    if (n < pol.V) {
+        if (work <= 0) {
+            // skipped, or nothing to count: the empty table's result (no key,
+            // zero sums) without a histogram
+            pol.write((int32_t)n, 0, -1, 0, typename Pol::Acc());
+        } else {
+            int64_t bound = work < pol.keys ? work : pol.keys;
+            // few keys but much work: many warps into one small table, or
+            // (dense) a block's arrays
+            if (bound <= HT_WLOAD && (work <= tiers.wwork || !dense))
+                tier = work <= tiers.wwork ? HT_TIER_WARP : HT_TIER_SPLIT;
+            else if (Pol::kOptimistic && work <= tiers.wwork) tier = HT_TIER_WARP;
+            else if (work <= tiers.bwork) tier = HT_TIER_BLOCK;
+            else if (work <= tiers.gwork) tier = HT_TIER_BIG;
+            else tier = HT_TIER_SPLIT;
+        }
+    }
+    for (int t = 0; t < HT_NTIER; t++) {
+        unsigned m = __ballot_sync(FULL, tier == t);
+        if (!m) continue;
+        int leader = __ffs(m) - 1;
+        int64_t pos = 0;
+        if (lane == leader) pos = (int64_t)atomicAdd((unsigned long long*)&cnt[t], (unsigned long long)__popc(m));
+        pos = __shfl_sync(FULL, pos, leader);
+        if (tier == t) {
+            int64_t p = pos + __popc(m & lt);
+            lists[(int64_t)t * pol.V + p] = (int32_t)n;
+            if (t == HT_TIER_SPLIT) {
+                int64_t bound = work < pol.keys ? work : pol.keys;
+                scap[p] = pow2_ceil(2 * (bound > 16 ? bound : 16));
+            }
+        }
+    }
+    int64_t ws = warp_sum(tier >= 0 ? work : 0);
+    int64_t vs = __popc(__ballot_sync(FULL, tier >= 0));
+    if (lane == 0 && vs) {
+        atomicAdd((unsigned long long*)&cnt[HT_CNT_WORK], (unsigned long long)ws);
+        atomicAdd((unsigned long long*)&cnt[HT_CNT_VERTS], (unsigned long long)vs);
+    }
+}
+
 template <class Pol>
 __global__ void __launch_bounds__(256)
     k_ht_classify(Pol pol, const int64_t* __restrict__ workv, int32_t* lists, int64_t* cnt,
                   int64_t* scap, HtTiers tiers, bool dense)
 {
-    int lane = threadIdx.x & 31;
-    unsigned lt = lanemask_lt();
-    int64_t wsum = 0, vsum = 0;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < pol.V;
          base += (int64_t)gridDim.x * blockDim.x) {
         int64_t n = base + threadIdx.x;
-        int tier = -1;
-        int64_t work = 0;
-        if (n < pol.V) {
-            work = workv[n];
-            if (work <= 0) {
-                // skipped, or nothing to count: the empty table's result
-                // (no key, zero sums) without a histogram
-                pol.write((int32_t)n, 0, -1, 0, typename Pol::Acc());
-            } else {
-                wsum += work;
-                vsum++;
-                int64_t bound = work < pol.keys ? work : pol.keys;
-                // few keys but much work: many warps into one small table, or
-                // (dense) a block's arrays
-                if (bound <= HT_WLOAD && (work <= tiers.wwork || !dense))
-                    tier = work <= tiers.wwork ? HT_TIER_WARP : HT_TIER_SPLIT;
-                else if (Pol::kOptimistic && work <= tiers.wwork) tier = HT_TIER_WARP;
-                else if (work <= tiers.bwork) tier = HT_TIER_BLOCK;
-                else if (work <= tiers.gwork) tier = HT_TIER_BIG;
-                else tier = HT_TIER_SPLIT;
-            }
-        }
-        for (int t = 0; t < HT_NTIER; t++) {
-            unsigned m = __ballot_sync(FULL, tier == t);
-            if (!m) continue;
-            int leader = __ffs(m) - 1;
-            int64_t pos = 0;
-            if (lane == leader) pos = (int64_t)atomicAdd((unsigned long long*)&cnt[t], (unsigned long long)__popc(m));
-            pos = __shfl_sync(FULL, pos, leader);
-            if (tier == t) {
-                int64_t p = pos + __popc(m & lt);
-                lists[(int64_t)t * pol.V + p] = (int32_t)n;
-                if (t == HT_TIER_SPLIT) {
-                    int64_t bound = work < pol.keys ? work : pol.keys;
-                    scap[p] = pow2_ceil(2 * (bound > 16 ? bound : 16));
-                }
-            }
+        ht_place(pol, n, n < pol.V ? workv[n] : -1, lists, cnt, scap, tiers, dense);
+    }
+}
+
+// The three passes above in one launch, for levels of up to HT_PLAN_V
+// vertices, where launches cost more than the work: a block takes 32 vertices
+// a grid apart, a warp per listed one sums its segments (the block those of a
+// long list), then the first warp classifies them. (Not 32 consecutive ones:
+// super-nodes of like size have consecutive ids, and a block that got the
+// largest of a 60,000-neuron layered network took 83 us.)
+constexpr int32_t HT_PLAN_V = 1 << 16;
+
+template <class Pol>
+__global__ void __launch_bounds__(256)
+    k_ht_plan(Pol pol, int64_t* workv, int32_t* lists, int64_t* cnt, int64_t* scap, HtTiers tiers,
+              bool dense)
+{
+    __shared__ int64_t work[32];
+    __shared__ unsigned smask;
+    __shared__ unsigned long long part;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t mine = blockIdx.x + (int64_t)lane * gridDim.x;
+    if (warp == 0) {
+        work[lane] = -1;
+        unsigned m = __ballot_sync(FULL, mine < pol.V && !pol.skip((int32_t)mine));
+        if (lane == 0) smask = m;
+    }
+    __syncthreads();
+    unsigned m = smask, lng = 0;
+    // the r-th listed vertex to warp r % 8
+    for (int r = 0; m; r++) {
+        int t = __ffs(m) - 1;
+        m &= m - 1;
+        int32_t n = (int32_t)(blockIdx.x + (int64_t)t * gridDim.x);
+        int64_t vb = pol.vb(n), ve = pol.ve(n);
+        if (ve - vb > HT_WORK_LONG) {
+            lng |= 1u << t;
+        } else if ((r & 7) == warp) {
+            int64_t w = 0;
+#pragma unroll 4
+            for (int64_t i = vb + lane; i < ve; i += 32) w += pol.seg_len(i);
+            w = warp_sum(w);
+            if (lane == 0) work[t] = w;
         }
     }
-    wsum = warp_sum(wsum);
-    vsum = warp_sum(vsum);
-    if (lane == 0 && vsum) {
-        atomicAdd((unsigned long long*)&cnt[HT_CNT_WORK], (unsigned long long)wsum);
-        atomicAdd((unsigned long long*)&cnt[HT_CNT_VERTS], (unsigned long long)vsum);
+    while (lng) {   // the same in every thread
+        int t = __ffs(lng) - 1;
+        lng &= lng - 1;
+        int32_t n = (int32_t)(blockIdx.x + (int64_t)t * gridDim.x);
+        int64_t vb = pol.vb(n), ve = pol.ve(n);
+        if (threadIdx.x == 0) part = 0;
+        __syncthreads();
+        int64_t w = 0;
+#pragma unroll 4
+        for (int64_t i = vb + threadIdx.x; i < ve; i += 256) w += pol.seg_len(i);
+        w = warp_sum(w);
+        if (lane == 0) atomicAdd(&part, (unsigned long long)w);
+        __syncthreads();
+        if (threadIdx.x == 0) work[t] = (int64_t)part;
     }
+    __syncthreads();
+    if (warp != 0) return;
+    if (mine < pol.V) workv[mine] = work[lane];
+    ht_place(pol, mine, work[lane], lists, cnt, scap, tiers, dense);
 }
 
 template <class Pol>
@@ -666,8 +745,14 @@ __device__ __forceinline__ int32_t seg_find(const int32_t* spre, int32_t n, int3
 // element): on level 0 of the 1,048,576-neuron power-law network, 16
 // incidences of 8 to 16,384 pins each, the groups left most of the block
 // waiting for the longest (12.7 ms flattened, 15.3 by groups).
+//
+// Held to 32 registers so that eight blocks share an SM: at 6 blocks (40
+// registers) the two networks above take 36.8 and 20.1 ms, at 5 39.5 and
+// 21.5, at 8 31.9 and 19.2, a few spilled words included.
+constexpr int HT_BLOCKS = 8;
+
 template <class Pol, int T, int CAP, int TIER, int NEXT>
-__global__ void __launch_bounds__(T)
+__global__ void __launch_bounds__(T, CAP <= 2048 ? HT_BLOCKS : 1)
     k_ht_block(Pol pol, int32_t* lists, int64_t* cnt, int64_t* scap, const int64_t* __restrict__ workv,
                int64_t leave)
 {
@@ -691,8 +776,20 @@ __global__ void __launch_bounds__(T)
     const int nwarps = T / 32;
     int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (cnt[TIER] <= leave) return;   // so few that the big tier's blocks take them
+    // pt shares t's slots: its sums take the place of the weights, its list
+    // that of the overlaps, which are cleared when an unpacked vertex follows
     Table<S> t = carve_table<S>(ht_dyn, CAP);
     t.probes = 64;   // a vertex that clusters the table this much moves on
+    constexpr bool LIST = CAP > 4096;
+    __shared__ int32_t nused;
+    PackedTable<LIST> pt;
+    pt.key = t.key;
+    pt.val = (uint32_t*)t.sc;
+    pt.used = (uint16_t*)t.ov;
+    pt.nused = &nused;
+    pt.mask = t.mask;
+    pt.probes = t.probes;
+    bool listed = false;   // the list has overwritten overlaps
     clear_slots(t, threadIdx.x, CAP, T);
     const int32_t* list = lists + (int64_t)TIER * pol.V;
     int64_t nl = cnt[TIER];
@@ -702,6 +799,7 @@ __global__ void __launch_bounds__(T)
             snext = (int64_t)atomicAdd((unsigned long long*)&cnt[HT_CNT_NEXT + TIER], 1ull);
             sfail = 0;
             nlong = 0;
+            nused = 0;
             ssum[0] = ssum[1] = 0;
         }
         __syncthreads();
@@ -764,6 +862,13 @@ __global__ void __launch_bounds__(T)
         if constexpr (sizeof(S) == 4) {
             int wb = 64 - __clzll((long long)ssum[0]), kb = 64 - __clzll((long long)ssum[1]);
             if (wb + kb <= 32) sb = kb;
+            if (LIST && sb < 0 && listed) {   // the same for the whole block
+                clear_slots(t, threadIdx.x, CAP, T);
+                listed = false;
+                __syncthreads();
+            }
+            if (LIST && sb >= 0) listed = true;
+            pt.sb = sb;
         }
         auto visit = [&](const auto& tb) {
             const typename Pol::Own own = pol.own(n);
@@ -804,7 +909,7 @@ __global__ void __launch_bounds__(T)
             return k;
         };
         if constexpr (sizeof(S) == 4) {
-            if (sb >= 0) ok = visit(PackedTable{t.key, (uint32_t*)t.sc, t.mask, t.probes, sb});
+            if (sb >= 0) ok = visit(pt);
             else ok = visit(t);
         } else {
             ok = visit(t);
@@ -825,13 +930,15 @@ __global__ void __launch_bounds__(T)
         int32_t bk = -1;
         uint32_t bo = 0;
         if (sb >= 0) {
-            const uint32_t omask = (1u << sb) - 1;   // sb < 32: a weight of 0 needs no bit
-            for (int i = threadIdx.x; i < CAP; i += T) {
-                int32_t k = t.key[i];
-                if (k < 0) continue;
-                uint32_t v = (uint32_t)t.sc[i];
-                t.key[i] = -1;
-                t.sc[i] = 0;
+            const uint32_t omask = (1u << sb) - 1;   // sb < 32: multiplicities sum below 2^31
+            const int nk = LIST ? nused : CAP;
+            for (int x = threadIdx.x; x < nk; x += T) {
+                int i = LIST ? pt.used[x] : x;
+                int32_t k = pt.key[i];
+                if (!LIST && k < 0) continue;
+                uint32_t v = pt.val[i];
+                pt.key[i] = -1;
+                pt.val[i] = 0;
                 pol.consider(n, k, (int64_t)(v >> sb), v & omask, tot, bs, bk, bo);
             }
         } else {
@@ -1471,13 +1578,19 @@ Status run_histogram(const Pol& pol, Arena& ar, cudaStream_t s, int64_t* d_cnt, 
     SNN_TRY(ar.alloc(&scap, V));
     SNN_TRY(ar.alloc(&workv, V));
     SNN_CUDA(cudaMemsetAsync(d_cnt, 0, HT_NCNT * sizeof(int64_t), s));
-    int32_t* todo;
-    int64_t* ntodo = d_cnt + HT_CNT_TODO;
-    SNN_TRY(ar.alloc(&todo, V));
-    SNN_L k_ht_skip<Pol><<<grid_for(V, 256), 256, 0, s>>>(pol, workv, todo, ntodo);
-    SNN_L k_ht_work<Pol><<<grid_for(V, 8, 152 * 16), 256, 0, s>>>(pol, workv, todo, ntodo);
-    SNN_CUDA(cudaGetLastError());
-    SNN_L k_ht_classify<Pol><<<grid_for(V, 256), 256, 0, s>>>(pol, workv, lists, d_cnt, scap, tiers, dense_big);
+    if (V <= HT_PLAN_V) {
+        SNN_L k_ht_plan<Pol><<<(int)ceil_div(V, 32), 256, 0, s>>>(pol, workv, lists, d_cnt, scap, tiers,
+                                                                  dense_big);
+    } else {
+        int32_t* todo;
+        int64_t* ntodo = d_cnt + HT_CNT_TODO;
+        SNN_TRY(ar.alloc(&todo, V));
+        SNN_L k_ht_skip<Pol><<<grid_for(V, 256), 256, 0, s>>>(pol, workv, todo, ntodo);
+        SNN_L k_ht_work<Pol><<<grid_for(V, 8, 152 * 16), 256, 0, s>>>(pol, workv, todo, ntodo);
+        SNN_CUDA(cudaGetLastError());
+        SNN_L k_ht_classify<Pol><<<grid_for(V, 256), 256, 0, s>>>(pol, workv, lists, d_cnt, scap, tiers,
+                                                                  dense_big);
+    }
     SNN_CUDA(cudaGetLastError());
     size_t wsm = (size_t)HT_WARPS * HT_WCAP * slot_bytes<S>();
     size_t bsm = (size_t)HT_BCAP * slot_bytes<S>();
