@@ -47,6 +47,9 @@ enum : int {
     RS_NHL = 11,       // listed hyperedges (int32)
 };
 
+// pinned host words the kernels of a round write (snnmap_hgraph::h_tier)
+enum : int { HW_COST = 0, HW_BAD, HW_PROPS, HW_STATUS = HW_PROPS + 3, HW_BEST, HW_ISTAR };
+
 constexpr int REPLAY_WARP_MAX = 32;
 constexpr int PSTAR_MAX = 16;   // partitions of P* the column update takes
 
@@ -246,16 +249,6 @@ __device__ __forceinline__ bool violates(int64_t sz, int64_t ip, int64_t pc, int
                                          int32_t delta, int32_t phi)
 {
     return sz > omega || ip > phi || pc > delta;
-}
-
-__global__ void k_check_pstate(int32_t K, PState ps, int32_t omega, int32_t delta, int32_t phi,
-                               int64_t* scal)
-{
-    int bad = 0;
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < K;
-         p += (int64_t)gridDim.x * blockDim.x)
-        if (violates(ps.size[p], ps.inpins[p], ps.pincnt[p], omega, delta, phi)) bad = 1;
-    if (__any_sync(FULL, bad) && (threadIdx.x & 31) == 0) atomicOr((int*)&scal[SC_STATUS], ST_BADSTATE);
 }
 
 // counts of partition p in hyperedge a at round start (entries sorted by p)
@@ -1179,8 +1172,9 @@ __global__ void k_ps_rows(Level L, const int32_t* __restrict__ rho,
     }
 }
 
-// slot map and counters back to empty
-__global__ void k_ps_reset(int32_t M, Moves mv, const int64_t* __restrict__ scal, PStar ps)
+// slot map and counters back to empty; the round's result to the host's words
+__global__ void k_ps_reset(int32_t M, Moves mv, const int64_t* __restrict__ scal, PStar ps,
+                           int64_t* host)
 {
     int64_t istar = scal[RS_BEST] > 0 ? scal[RS_ISTAR] : -1;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= istar && i < M;
@@ -1191,6 +1185,9 @@ __global__ void k_ps_reset(int32_t M, Moves mv, const int64_t* __restrict__ scal
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ps.cnt[0] = ps.cnt[2];
         ps.cnt[1] = 0;
+        host[HW_STATUS] = scal[SC_STATUS];
+        host[HW_BEST] = scal[RS_BEST];
+        host[HW_ISTAR] = scal[RS_ISTAR];
     }
 }
 
@@ -1693,15 +1690,40 @@ __global__ void __launch_bounds__(SB_THREADS)
     }
 }
 
-// the round's scalars: all zero but the prefix end (none) and Conn at its
-// start
-__global__ void k_round_begin(int64_t* scal, const int64_t* __restrict__ costv)
+// The round's scalars: all zero but the prefix end (none). First round: Conn
+// from its partial sums, and whether the partitions are within their limits
+// (an enacted prefix is valid, so the state can only be broken at the start).
+// Conn and that finding go straight to the host's words (pinned, HW_BAD
+// cleared by the host, read after the proposals' wait), which saves a copy a
+// round.
+__global__ void __launch_bounds__(1024)
+    k_round_begin(int64_t* scal, int64_t* costv, const int64_t* __restrict__ slots, int32_t K, PState ps,
+                  int32_t omega, int32_t delta, int32_t phi, int64_t* host)
 {
-    int i = threadIdx.x;
-    if (i < SC_COUNT) scal[i] = i == RS_ISTAR ? INT64_MAX : (i == RS_COST ? *costv : 0);
+    __shared__ unsigned long long sum;
+    const int i = threadIdx.x;
+    if (slots) {
+        for (int64_t p = blockIdx.x * (int64_t)blockDim.x + i; p < K; p += (int64_t)gridDim.x * blockDim.x)
+            if (violates(ps.size[p], ps.inpins[p], ps.pincnt[p], omega, delta, phi)) host[HW_BAD] = 1;
+    }
+    if (blockIdx.x != 0) return;
+    if (i < SC_COUNT) scal[i] = i == RS_ISTAR ? INT64_MAX : 0;
+    if (!slots) {
+        if (i == 0) host[HW_COST] = *costv;
+        return;
+    }
+    if (i == 0) sum = 0;
+    __syncthreads();
+    if (i < COST_SLOTS) {
+        int64_t v = warp_sum(slots[i]);
+        if ((i & 31) == 0) atomicAdd(&sum, (unsigned long long)v);
+    }
+    __syncthreads();
+    if (i == 0) {
+        *costv = (int64_t)sum;
+        host[HW_COST] = (int64_t)sum;
+    }
 }
-
-// ---------------------------------------------------------------------------
 
 template <typename S>
 static Status gains(snnmap_hgraph* h, Level& L, const PinCounts& pc, const int32_t* rho,
@@ -1840,44 +1862,20 @@ Status dense_descend(snnmap_hgraph* h, int32_t level)
     return Status{};
 }
 
-// pin counts + partition state + Conn for rho, into buffers the caller owns
-// (Conn is added to *cost)
+// pin counts + partition state + the COST_SLOTS partial sums of Conn for rho,
+// into buffers the caller owns (state and sums cleared)
 static Status pin_counts_into(snnmap_hgraph* h, Level& L, LevelExtra& X, int32_t K,
-                              const int32_t* rho, PinCounts& pc, PState& ps, int64_t* cost)
+                              const int32_t* rho, PinCounts& pc, PState& ps, int64_t* slots)
 {
     cudaStream_t s = h->stream;
     Arena& ar = h->scratch;
-    SNN_CUDA(cudaMemsetAsync(ps.size, 0, (size_t)K * 8, s));
-    SNN_CUDA(cudaMemsetAsync(ps.inpins, 0, (size_t)K * 8, s));
-    SNN_CUDA(cudaMemsetAsync(ps.pincnt, 0, (size_t)K * 8, s));
     if (L.V > 0) {
         SNN_L k_pstate_vertices<<<grid_for(L.V, 256), 256, 0, s>>>(L, rho, ps);
         SNN_CUDA(cudaGetLastError());
     }
-    int64_t* slots;
-    SNN_TRY(ar.alloc(&slots, COST_SLOTS));
-    SNN_CUDA(cudaMemsetAsync(slots, 0, COST_SLOTS * sizeof(int64_t), s));
     PinCountJob job{L.hoff, L.hpins, L.hsd, L.hk, L.hw, rho, pc, ps.pincnt, slots};
     if (K <= PC_SMEM_K && L.E >= 16 * (int64_t)K) job.K = K;
-    SNN_TRY(seg_run(job, X.seg, L.E, ar, s));
-    SNN_L k_cost_slots<<<1, 256, 0, s>>>(slots, cost);
-    SNN_CUDA(cudaGetLastError());
-    return Status{};
-}
-
-static Status pin_counts(snnmap_hgraph* h, Level& L, LevelExtra& X, int32_t K, const int32_t* rho,
-                         PinCounts& pc, PState& ps)
-{
-    Arena& ar = h->scratch;
-    SNN_TRY(ar.alloc(&pc.p, L.P));
-    SNN_TRY(ar.alloc(&pc.cnt, L.P));
-    SNN_TRY(ar.alloc(&pc.dcnt, L.P));
-    SNN_TRY(ar.alloc(&pc.lam, L.E));
-    SNN_TRY(ar.alloc(&pc.rec, L.E));
-    SNN_TRY(ar.alloc(&ps.size, K));
-    SNN_TRY(ar.alloc(&ps.inpins, K));
-    SNN_TRY(ar.alloc(&ps.pincnt, K));
-    return pin_counts_into(h, L, X, K, rho, pc, ps, h->d_scal + RS_COST);
+    return seg_run(job, X.seg, L.E, ar, s);
 }
 
 Status level_cost(snnmap_hgraph* h, int32_t level, int32_t K, const int32_t* rho, int64_t* cost)
@@ -1887,7 +1885,25 @@ Status level_cost(snnmap_hgraph* h, int32_t level, int32_t K, const int32_t* rho
     SNN_TRY(zero_scalars(h));
     PinCounts pc;
     PState ps;
-    SNN_TRY(pin_counts(h, L, X, K, rho, pc, ps));
+    Arena& ar = h->scratch;
+    SNN_TRY(ar.alloc(&pc.p, L.P));
+    SNN_TRY(ar.alloc(&pc.cnt, L.P));
+    SNN_TRY(ar.alloc(&pc.dcnt, L.P));
+    SNN_TRY(ar.alloc(&pc.lam, L.E));
+    SNN_TRY(ar.alloc(&pc.rec, L.E));
+    int64_t* slots;
+    Carver cv;
+    cv.add(&ps.size, K);
+    cv.add(&ps.inpins, K);
+    cv.add(&ps.pincnt, K);
+    cv.add(&slots, COST_SLOTS);
+    char* base;
+    SNN_TRY(ar.alloc(&base, (int64_t)cv.total));
+    cv.assign(base);
+    SNN_CUDA(cudaMemsetAsync(base, 0, cv.total, h->stream));
+    SNN_TRY(pin_counts_into(h, L, X, K, rho, pc, ps, slots));
+    SNN_L k_cost_slots<<<1, 256, 0, h->stream>>>(slots, h->d_scal + RS_COST);
+    SNN_CUDA(cudaGetLastError());
     SNN_TRY(read_scalars(h));
     h->scratch.reset();
     *cost = h->h_scal[RS_COST];
@@ -2096,6 +2112,7 @@ struct IncState {
     PinCounts pc;
     PState ps;
     int64_t* costv = nullptr;
+    int64_t* slots = nullptr;    // partial sums of Conn of the first round
     int64_t* savev = nullptr;
     int64_t* Wv = nullptr;
     int32_t* hdirty = nullptr;   // per hyperedge
@@ -2126,17 +2143,14 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     *gain = 0;
     PinCounts pc = inc.pc;
     PState ps = inc.ps;
+    int64_t* host = h->h_tier + 2 * TIER_SLOTS;   // pinned, written by the kernels
     {
         ProfScope prof(h, PS_PINCOUNT);
-        if (!inc.ready) {
-            SNN_CUDA(cudaMemsetAsync(inc.costv, 0, sizeof(int64_t), s));
-            SNN_TRY(pin_counts_into(h, L, X, K, rho, pc, ps, inc.costv));
-        }
-        SNN_L k_round_begin<<<1, 32, 0, s>>>(h->d_scal, inc.costv);
-        // an enacted prefix is valid: the state can only be broken at the start
-        if (!inc.ready)
-            SNN_L k_check_pstate<<<grid_for(K, 256), 256, 0, s>>>(K, ps, prm.omega, prm.delta, prm.phi,
-                                                                 h->d_scal);
+        if (!inc.ready) SNN_TRY(pin_counts_into(h, L, X, K, rho, pc, ps, inc.slots));
+        host[HW_BAD] = 0;
+        SNN_L k_round_begin<<<inc.ready ? 1 : grid_for(K, 1024, 152), inc.ready ? 32 : 1024, 0, s>>>(h->d_scal, inc.costv,
+                                                                inc.ready ? nullptr : inc.slots, K, ps,
+                                                                prm.omega, prm.delta, prm.phi, host);
         SNN_CUDA(cudaGetLastError());
     }
     DenseRows& D = h->dense;
@@ -2153,8 +2167,6 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     int64_t* Wv = inc.Wv;
     if (!inc.ready) {
         prof.reset(new ProfScope(h, PS_SAVE));
-        SNN_CUDA(cudaMemsetAsync(savev, 0, (size_t)(V > 0 ? V : 1) * 8, s));
-        SNN_CUDA(cudaMemsetAsync(Wv, 0, (size_t)(V > 0 ? V : 1) * 8, s));
         if (L.E > 0 && !h->wide && V <= SAVE_SMEM_V) {
             auto launch = [&](auto kern) -> Status {
                 SNN_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2193,20 +2205,19 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     uint32_t *vals, *vals2;
     SNN_TRY(ar.alloc(&keys, V));
     SNN_TRY(ar.alloc(&vals, V));
-    PropSums* sums;
-    SNN_TRY(ar.alloc(&sums, 1));
     const int64_t bias = h->wsum;   // gains lie in [-wsum, wsum]
-    SNN_TRY(scan_run<PropSums>(PropIn{pto, savev, dense ? nullptr : inc.dirty, L.voff,
+    for (int i = 0; i < 3; i++) host[HW_PROPS + i] = 0;
+    if (V > 0)
+        SNN_TRY(scan_run<PropSums>(PropIn{pto, savev, dense ? nullptr : inc.dirty, L.voff,
                                       prm.refine_nonpositive},
-                               PropOut{pgain, bias, keys, vals}, V, sums, ar, s));
+                               PropOut{pgain, bias, keys, vals}, V, (PropSums*)(host + HW_PROPS), ar, s));
     prof.reset();
-    SNN_CUDA(cudaMemcpyAsync(h->h_tier + 2 * TIER_SLOTS, sums, sizeof(PropSums), cudaMemcpyDeviceToHost, s));
-    SNN_TRY(read_scalars(h));
-    const int64_t* hs = h->h_tier + 2 * TIER_SLOTS;
-    *cost = h->h_scal[RS_COST];
+    SNN_CUDA(cudaStreamSynchronize(s));
+    const int64_t* hs = host + HW_PROPS;
+    *cost = host[HW_COST];
     *n_active = (int32_t)hs[2];
     *rows = dense ? 1 : 0;
-    if (h->h_scal[SC_STATUS] & ST_BADSTATE)
+    if (host[HW_BAD])
         return Status{SNNMAP_ERR_INVALID, "refinement input breaks a per-core limit"};
     int32_t M = (int32_t)hs[0];
     int64_t deg = hs[1];
@@ -2370,7 +2381,7 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
                                                   prm.delta, prm.phi, prm.refine_nonpositive, pto,
                                                   pgain, inc.dirty);
         }
-        SNN_L k_ps_reset<<<gm, 256, 0, s>>>(M, mv, h->d_scal, inc.pst);
+        SNN_L k_ps_reset<<<gm, 256, 0, s>>>(M, mv, h->d_scal, inc.pst, host);
         SNN_CUDA(cudaGetLastError());
     } else {
         prof.reset(new ProfScope(h, PS_GAINS));
@@ -2378,14 +2389,14 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
             SNN_L k_ps_rows<<<gv, 256, 0, s>>>(L, rho, h->d_scal, inc.pst, ps, savev, Wv, D.rowid, D.C,
                                                D.O, D.Kp, prm.omega, prm.delta, prm.phi,
                                                prm.refine_nonpositive, pto, pgain, inc.dirty);
-        SNN_L k_ps_reset<<<gm, 256, 0, s>>>(M, mv, h->d_scal, inc.pst);
+        SNN_L k_ps_reset<<<gm, 256, 0, s>>>(M, mv, h->d_scal, inc.pst, host);
         SNN_CUDA(cudaGetLastError());
     }
     prof.reset();
-    SNN_TRY(read_scalars(h));
-    if (h->h_scal[SC_STATUS] & ST_CAPACITY) return Status{SNNMAP_ERR_CUDA, "event buffer overflow"};
-    int64_t best = h->h_scal[RS_BEST];
-    int64_t istar = h->h_scal[RS_ISTAR];
+    SNN_CUDA(cudaStreamSynchronize(s));
+    if (host[HW_STATUS] & ST_CAPACITY) return Status{SNNMAP_ERR_CUDA, "event buffer overflow"};
+    int64_t best = host[HW_BEST];
+    int64_t istar = host[HW_ISTAR];
     if (best > 0 && istar < M) {
         *applied = (int32_t)(istar + 1);
         *gain = best;
@@ -2497,6 +2508,12 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
     cv.add(&inc.hdirty, E);
     cv.add(&inc.hmark, E);
     cv.add(&inc.vmax, 3);
+    cv.add(&inc.ps.size, K);
+    cv.add(&inc.ps.inpins, K);
+    cv.add(&inc.ps.pincnt, K);
+    cv.add(&inc.slots, COST_SLOTS);
+    cv.add(&inc.savev, V);
+    cv.add(&inc.Wv, V);
     const size_t cleared = cv.total;
     cv.add(&moveidx, V);
     if (!use_carry) {
@@ -2511,12 +2528,7 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
     cv.add(&inc.pc.dcnt, L.P);
     cv.add(&inc.pc.lam, E);
     cv.add(&inc.pc.rec, E);
-    cv.add(&inc.ps.size, K);
-    cv.add(&inc.ps.inpins, K);
-    cv.add(&inc.ps.pincnt, K);
     cv.add(&inc.costv, 1);
-    cv.add(&inc.savev, V);
-    cv.add(&inc.Wv, V);
     cv.add(&inc.hlist, E);
     cv.add(&inc.hmeta, 2 * SEG_NB);
     cv.add(&pst.pslot, K);
