@@ -361,23 +361,16 @@ static int snnmap_partition_impl(snnmap_hgraph* h, void* stream, int32_t* d_rho_
     // once the level above needed at least four evaluations per vertex
     // (rounds times the share of vertices evaluated), as on power-law
     // graphs whose levels run many rounds with every vertex active.
-    // The rows are allocated for the levels that keep them by the first rule,
-    // known here from the level sizes (a finer level's rows may be the whole
-    // budget: 38 GB for the 1,048,576-neuron conv network's level 0, which
-    // never uses them, and mapping and unmapping those took 100 of its 700
-    // ms); a busier level opens them again at the full size, every row fresh.
+    // The rows' memory grows with the levels that take them (dense_grow): the
+    // finest level's would be the whole budget, 38 GB for the 1,048,576-neuron
+    // conv network, whose rows end at 426,000 vertices.
     int32_t lb = nl;
-    auto fresh_rows = [&](int32_t l) {
-        return 2 * ((int64_t)h->levels[l].V - h->levels[l + 1].V);
-    };
     {
         int64_t rb = snn::dense_row_budget(h);
         int64_t per = ((((int64_t)K + 3) & ~(int64_t)3) * 8 + 20);
         if (rb > 0 && !h->wide && !h->wzero && h->wsum <= INT32_MAX)
             for (int32_t l = nl - 1; l >= 0 && (int64_t)h->levels[l].V * per <= rb; l--) lb = l;
-        int32_t lk = nl - 1;
-        while (lk > lb && 4 * fresh_rows(lk - 1) <= h->levels[lk - 1].V) lk--;
-        if (lb < nl && !snn::dense_open(h, K, h->levels[lk].V).ok()) {
+        if (lb < nl && (!snn::dense_open(h, K, h->levels[lb].V).ok() || !snn::dense_grow(h, K).ok())) {
             snn::dense_close(h);
             cudaGetLastError();
             lb = nl;
@@ -402,23 +395,19 @@ static int snnmap_partition_impl(snnmap_hgraph* h, void* stream, int32_t* d_rho_
                 int64_t V = h->levels[l].V;
                 bool busy = evals_above >= 4.0;
                 snn::ProfScope prof(h, snn::PS_ROWS);
-                bool keep = h->dense.C && h->dense.level == l + 1 && (4 * fresh_rows(l) <= V || busy);
-                if (keep && V <= h->dense.cap) {
-                    s2 = snn::dense_descend(h, l);
-                    rows_here = true;
-                } else if (keep || (busy && (!h->dense.C || h->dense.level != l + 1))) {
-                    bool room = h->dense.C && V <= h->dense.cap;
-                    if (!room) room = snn::dense_open(h, K, h->levels[lb].V).ok();
-                    if (room) {
-                        s2 = snn::dense_begin(h, l);
+                int64_t fresh = 2 * (V - h->levels[l + 1].V);
+                bool keep = h->dense.level == l + 1;
+                if (keep ? 4 * fresh <= V || busy : busy) {
+                    if (snn::dense_grow(h, V).ok()) {
+                        s2 = keep ? snn::dense_descend(h, l) : snn::dense_begin(h, l);
                         rows_here = true;
                     } else {
-                        cudaGetLastError();
+                        cudaGetLastError();   // no room: histograms from here down
                         snn::dense_close(h);
-                        lb = nl;   // no room: histograms from here down
+                        lb = nl;
                     }
                 }
-            } else if (h->dense.C) {
+            } else {
                 snn::dense_close(h);
             }
             if (!s2.ok()) break;
@@ -427,7 +416,7 @@ static int snnmap_partition_impl(snnmap_hgraph* h, void* stream, int32_t* d_rho_
             rows_here = true;
             if (!s2.ok()) break;
         }
-        if (!rows_here && h->dense.C) h->dense.level = -1;
+        if (!rows_here) h->dense.level = -1;
         int64_t c0 = 0;
         size_t r0 = h->rlog.size();
         s2 = snn::refine_level(h, l, K, cur, &cost, l == nl - 1 ? &c0 : nullptr);

@@ -116,7 +116,8 @@ Status level_alloc(snnmap_hgraph* h, Level& L, LevelExtra& X, int32_t V, int32_t
     c.assign(p);
     L.block = p;
     L.bytes = c.total;
-    if (!L.cid) SNN_CUDA(dev_malloc((void**)&L.cid, (size_t)(V > 0 ? V : 1) * 4, h->stream));
+    if (!L.cid) SNN_CUDA(dev_malloc((void**)&L.cid, (size_t)(V > 0 ? V : 1) * 5, h->stream));
+    L.pr = (uint8_t*)(L.cid + V);
     L.resident = true;
     return Status{};
 }
@@ -124,9 +125,9 @@ Status level_alloc(snnmap_hgraph* h, Level& L, LevelExtra& X, int32_t V, int32_t
 int64_t held_bytes(const snnmap_hgraph* h)
 {
     int64_t t = (int64_t)h->scratch.held() + (int64_t)h->cap_v * 20;
-    if (h->dense.C) t += h->dense.cap * (h->dense.Kp * 8 + 20);
+    if (h->dense.rowid) t += h->dense.rows * h->dense.Kp * 8 + h->dense.cap * 20;
     if (h->mat.S) t += h->mat.cap * 16;
-    for (auto& L : h->levels) t += (int64_t)L.bytes + 4 * (int64_t)L.V;
+    for (auto& L : h->levels) t += (int64_t)L.bytes + 5 * (int64_t)L.V;
     return t;
 }
 
@@ -147,13 +148,13 @@ void level_release(snnmap_hgraph* h, Level& L)
 {
     if (!L.resident) return;
     if (L.block) cudaFreeAsync(L.block, h->stream);
-    int32_t* cid = L.cid;
     Level k;
     k.V = L.V;
     k.E = L.E;
     k.P = L.P;
     k.maxlen = L.maxlen;
-    k.cid = cid;
+    k.cid = L.cid;
+    k.pr = L.pr;
     L = k;
 }
 

@@ -128,6 +128,7 @@ struct Level {
     int32_t* vincnt = nullptr;
     int32_t* vinint = nullptr;
     int32_t* cid = nullptr;      // map to the next level (own allocation, always kept)
+    uint8_t* pr = nullptr;       // behind cid: 1 lower, 2 upper member of a matched pair, 0 unmatched
     int32_t maxlen = 0;          // longest hyperedge
     void* block = nullptr;       // single allocation holding every array but cid
     size_t bytes = 0;

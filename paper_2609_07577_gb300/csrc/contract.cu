@@ -49,12 +49,13 @@ struct NextState {
 };
 
 __global__ void k_cid_map(int32_t V, const int32_t* __restrict__ match,
-                          const int32_t* __restrict__ repidx, int32_t* cid)
+                          const int32_t* __restrict__ repidx, int32_t* cid, uint8_t* pr)
 {
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
         int32_t m = match[n];
         cid[n] = repidx[(m < 0 || (int32_t)n < m) ? (int32_t)n : m];
+        pr[n] = m < 0 ? 0 : ((int32_t)n < m ? 1 : 2);
     }
 }
 
@@ -578,7 +579,7 @@ Status contract_level(snnmap_hgraph* h)
         ProfScope prof(h, PS_CONTRACT);
         SNN_TRY(scan_run<int32_t>(RepFlag{h->match}, ScanStore<int32_t, false>{repidx}, V,
                                   (int32_t*)(h->d_scal + SC_A), ar, s));
-        SNN_L k_cid_map<<<grid_for(V, 256), 256, 0, s>>>(V, h->match, repidx, L.cid);
+        SNN_L k_cid_map<<<grid_for(V, 256), 256, 0, s>>>(V, h->match, repidx, L.cid, L.pr);
         SNN_CUDA(cudaGetLastError());
     }
     h->levels.emplace_back();

@@ -38,15 +38,27 @@ extern const char* const kStageNames[PS_N];
 }  // namespace snn
 
 namespace snn {
+// Where row r's Kp entries of C and O lie: rows are kept in chunks of 2^shift.
+struct RowTab {
+    int32_t* const* tab = nullptr;   // device: C and O of every chunk
+    int32_t shift = 0;
+    int64_t Kp = 0;
+    __device__ int64_t at(int32_t r) const { return (int64_t)(r & ((1 << shift) - 1)) * Kp; }
+    __device__ int32_t* C(int32_t r) const { return tab[2 * (r >> shift)] + at(r); }
+    __device__ int32_t* O(int32_t r) const { return tab[2 * (r >> shift) + 1] + at(r); }
+};
+
 // Connection rows of the refinement levels that fit the row budget: C and O
-// hold cap rows of Kp (K rounded up to 4) int32 entries; rowid maps the
+// hold rows of Kp (K rounded up to 4) int32 entries, in chunks allocated as
+// finer levels need them (`rows` of at most `cap` so far); rowid maps the
 // current level's vertices to rows.
 struct DenseRows {
     int32_t K = 0;
     int64_t Kp = 0;
     int64_t cap = 0;
-    int32_t* C = nullptr;
-    int32_t* O = nullptr;
+    int64_t rows = 0;
+    RowTab tab;
+    std::vector<int32_t*> chunks;   // one allocation each, C then O
     int32_t* rowid = nullptr;
     int32_t* rowid2 = nullptr;
     int32_t* fresh = nullptr;
@@ -73,15 +85,17 @@ struct ScoreMat {
 };
 
 // Proposals, gains and re-evaluation flags of the last histogram-refined
-// level, double-buffered so the next finer level can inherit them through
-// its cid map (cap vertices each).
+// level, and saves and W of the last level, double-buffered so the next finer
+// level can inherit them through its cid map (cap vertices each).
 struct Carry {
     int32_t* pto[2] = {nullptr, nullptr};
     int64_t* pgain[2] = {nullptr, nullptr};
     int32_t* dirty[2] = {nullptr, nullptr};
+    int64_t* save[2] = {nullptr, nullptr};   // saves, then W of the level's V vertices
     int cur = 0;
     int64_t cap = 0;
-    int32_t level = -1;   // level whose final state buffers[cur] hold (-1: none)
+    int32_t level = -1;   // level whose final proposals buffers[cur] hold (-1: none)
+    int32_t slevel = -1;  // level whose final saves save[cur] holds (-1: none)
 };
 
 // Candidates carried through a contraction (coarsen.cu, aff_carry): for each
@@ -255,10 +269,12 @@ Status mat_affinity(snnmap_hgraph* h, int32_t level, bool* done);
 Status mat_descend(snnmap_hgraph* h, int32_t src);
 void mat_close(snnmap_hgraph* h);
 
-// connection rows: allocation for `rows` vertices and K partitions; rows of
-// every vertex of `level` (the coarsest refined level) marked fresh; descent
-// from level+1 to `level` after projection; release
-Status dense_open(snnmap_hgraph* h, int32_t K, int64_t rows);
+// connection rows for K partitions and up to `cap` vertices; memory for at
+// least `rows` of them; rows of every vertex of `level` (the coarsest refined
+// level) marked fresh; descent from level+1 to `level` after projection;
+// release
+Status dense_open(snnmap_hgraph* h, int32_t K, int64_t cap);
+Status dense_grow(snnmap_hgraph* h, int64_t rows);
 Status dense_begin(snnmap_hgraph* h, int32_t level);
 Status dense_descend(snnmap_hgraph* h, int32_t level);
 void dense_close(snnmap_hgraph* h);

@@ -493,9 +493,7 @@ struct RowPol {
     int64_t keys;
     const int32_t* fresh;
     const int32_t* rowid;
-    int32_t* C;
-    int32_t* O;
-    int64_t Kp;
+    RowTab tab;
     unsigned long long* M;
     int32_t cw;
 
@@ -536,9 +534,8 @@ struct RowPol {
                              int32_t&, uint32_t&) const
     {
         int32_t row = rowid[n];
-        int64_t r = (int64_t)row * Kp + p;
-        C[r] = (int32_t)conn;
-        O[r] = (int32_t)o;
+        tab.C(row)[p] = (int32_t)conn;
+        tab.O(row)[p] = (int32_t)o;
         unsigned long long bit = 1ull << (p / cw);
         if (!(M[row] & bit)) atomicOr(&M[row], bit);   // a set bit is never cleared here
     }
@@ -553,9 +550,9 @@ struct RowPol {
 __global__ void __launch_bounds__(256)
     k_dense_best(Level L, const int32_t* __restrict__ rho, PState ps,
                  const int64_t* __restrict__ savev, const int64_t* __restrict__ Wv,
-                 const int32_t* __restrict__ rowid, const int32_t* __restrict__ C,
-                 const int32_t* __restrict__ O, const unsigned long long* __restrict__ M,
-                 int32_t cw, int64_t Kp, int32_t K, int32_t omega, int32_t delta, int32_t phi,
+                 const int32_t* __restrict__ rowid, RowTab tab,
+                 const unsigned long long* __restrict__ M, int32_t cw, int32_t K, int32_t omega,
+                 int32_t delta, int32_t phi,
                  int nonpos, int32_t* pto, int64_t* pgain, const int32_t* __restrict__ dirty)
 {
     int lane = threadIdx.x & 31;
@@ -575,8 +572,8 @@ __global__ void __launch_bounds__(256)
         int32_t own = rho[n];
         int64_t sz = L.vsize[n], ip = L.vinpins[n], ic = L.vincnt[n];
         int32_t rw = rowid[n];
-        int64_t r0 = (int64_t)rw * Kp;
-        const int4* row = reinterpret_cast<const int4*>(C + r0);
+        const int4* row = reinterpret_cast<const int4*>(tab.C(rw));
+        const int32_t* ov = tab.O(rw);
         int64_t bs = 0;
         int32_t bk = -1;
         const int64_t nq = ((int64_t)K + 3) >> 2;
@@ -617,7 +614,7 @@ __global__ void __launch_bounds__(256)
                     // seeds bs
                     if (p < K && (g > bs || (nonpos && bk < 0 && cv[u] > 0)) && cv[u] > 0 &&
                         p != own && ps.size[p] + sz <= omega && ps.inpins[p] + ip <= phi &&
-                        ps.pincnt[p] + ic - (int64_t)O[r0 + p] <= delta) {
+                        ps.pincnt[p] + ic - (int64_t)ov[p] <= delta) {
                         bs = g;
                         bk = p;
                     }
@@ -642,10 +639,9 @@ __global__ void __launch_bounds__(256)
 
 struct RowsRef {
     const int32_t* rowid;   // null: the level has no rows
-    int32_t *C, *O;
+    RowTab tab;
     unsigned long long* M;
     int32_t cw;
-    int64_t Kp;
 };
 
 // Row updates of hyperedge a for the enacted prefix (one warp): the moves of
@@ -660,10 +656,8 @@ __device__ __forceinline__ void rows_cross(const Level& L, const PinCounts& pc, 
 {
     const int lane = threadIdx.x & 31;
     const int32_t* rowid = R.rowid;
-    int32_t *C = R.C, *O = R.O;
     unsigned long long* M = R.M;
     const int32_t cw = R.cw;
-    const int64_t Kp = R.Kp;
     {
         for (int ib = 0; ib < m; ib += 32) {
             int ii = ib + lane;
@@ -708,11 +702,10 @@ __device__ __forceinline__ void rows_cross(const Level& L, const PinCounts& pc, 
                     int ds = __shfl_sync(FULL, rd[u], src);
                     for (int64_t j = b + lane; j < e; j += 32) {
                         int32_t rw = rowid[L.hpins[j]];
-                        int64_t r = (int64_t)rw * Kp + p;
-                        if (cs) atomicAdd(&C[r], (int32_t)(cs * w));
+                        if (cs) atomicAdd(R.tab.C(rw) + p, (int32_t)(cs * w));
                         unsigned long long bit = 1ull << (p / cw);
                         if (cs > 0 && !(M[rw] & bit)) atomicOr(&M[rw], bit);
-                        if (ds && (j != b || sd)) atomicAdd(&O[r], ds * k);
+                        if (ds && (j != b || sd)) atomicAdd(R.tab.O(rw) + p, ds * k);
                     }
                 }
             }
@@ -720,45 +713,29 @@ __device__ __forceinline__ void rows_cross(const Level& L, const PinCounts& pc, 
     }
 }
 
-// descent to the next finer level: member counts and smallest member per
-// coarse vertex
-__global__ void k_dense_members(int32_t V, const int32_t* __restrict__ cid, int32_t* mcount,
-                                int32_t* first)
-{
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
-         n += (int64_t)gridDim.x * blockDim.x) {
-        atomicAdd(&mcount[cid[n]], 1);
-        atomicMin(&first[cid[n]], (int32_t)n);
+// descent to the next finer level: the lower member of a pair keeps its
+// super-node's row, the upper one takes row Vc + (its rank among the upper
+// ones); both are to be computed afresh
+struct UpperMember {
+    const uint8_t* pr;
+    __device__ int32_t operator()(int64_t n) const { return pr[n] == 2; }
+};
+struct RowIds {
+    const uint8_t* pr;
+    const int32_t *cid, *rowc;
+    int32_t Vc;
+    int32_t *rowf, *fresh;
+    __device__ void operator()(int64_t n, int32_t before, int32_t upper) const
+    {
+        rowf[n] = upper ? Vc + before : rowc[cid[n]];
+        fresh[n] = pr[n] != 0;
     }
-}
-
-__global__ void k_dense_flags(int32_t V, const int32_t* __restrict__ cid,
-                              const int32_t* __restrict__ mcount, const int32_t* __restrict__ first,
-                              int32_t* nonrep, int32_t* fresh)
-{
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
-         n += (int64_t)gridDim.x * blockDim.x) {
-        int32_t c = cid[n];
-        nonrep[n] = first[c] != (int32_t)n;
-        fresh[n] = mcount[c] > 1;
-    }
-}
-
-// the smaller member keeps its super-node's row, the other takes row
-// Vc + (its rank among non-representatives)
-__global__ void k_dense_rowid(int32_t V, int32_t Vc, const int32_t* __restrict__ cid,
-                              const int32_t* __restrict__ nonrep, const int32_t* __restrict__ idx,
-                              const int32_t* __restrict__ rowc, int32_t* rowf)
-{
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
-         n += (int64_t)gridDim.x * blockDim.x)
-        rowf[n] = nonrep[n] ? Vc + idx[n] : rowc[cid[n]];
-}
+};
 
 // clears the rows of vertices flagged fresh (one warp per vertex)
 __global__ void k_dense_zero(int32_t V, const int32_t* __restrict__ fresh,
-                             const int32_t* __restrict__ rowid, int32_t* C, int32_t* O,
-                             unsigned long long* M, int64_t Kp)
+                             const int32_t* __restrict__ rowid, RowTab tab,
+                             unsigned long long* M)
 {
     int lane = threadIdx.x & 31;
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -766,9 +743,9 @@ __global__ void k_dense_zero(int32_t V, const int32_t* __restrict__ fresh,
     for (int64_t n = gw; n < V; n += nw) {
         if (!fresh[n]) continue;
         if (lane == 0) M[rowid[n]] = 0;
-        int4* c = reinterpret_cast<int4*>(C + (int64_t)rowid[n] * Kp);
-        int4* o = reinterpret_cast<int4*>(O + (int64_t)rowid[n] * Kp);
-        for (int64_t q = lane; q < Kp / 4; q += 32) {
+        int4* c = reinterpret_cast<int4*>(tab.C(rowid[n]));
+        int4* o = reinterpret_cast<int4*>(tab.O(rowid[n]));
+        for (int64_t q = lane; q < tab.Kp / 4; q += 32) {
             c[q] = make_int4(0, 0, 0, 0);
             o[q] = make_int4(0, 0, 0, 0);
         }
@@ -1129,8 +1106,7 @@ __global__ void k_ps_combine(Level L, const int32_t* __restrict__ rho,
 __global__ void k_ps_rows(Level L, const int32_t* __restrict__ rho,
                           const int64_t* __restrict__ scal, PStar ps, PState st,
                           const int64_t* __restrict__ savev, const int64_t* __restrict__ Wv,
-                          const int32_t* __restrict__ rowid, const int32_t* __restrict__ C,
-                          const int32_t* __restrict__ O, int64_t Kp, int32_t omega,
+                          const int32_t* __restrict__ rowid, RowTab tab, int32_t omega,
                           int32_t delta, int32_t phi, int nonpos, int32_t* pto, int64_t* pgain,
                           int32_t* dirty)
 {
@@ -1152,15 +1128,15 @@ __global__ void k_ps_rows(Level L, const int32_t* __restrict__ rho,
         }
         int64_t bs = q >= 0 ? pgain[n] + ds : 0;
         int32_t bk = q;
-        int64_t r0 = (int64_t)rowid[n] * Kp;
+        const int32_t *C = tab.C(rowid[n]), *O = tab.O(rowid[n]);
         int64_t sw = savev[n] - Wv[n];
         int32_t own = rho[n];
         for (int sl = 0; sl < ns; sl++) {
             int32_t p = ps.slots[sl];
-            int64_t c = C[r0 + p];
+            int64_t c = C[p];
             if (p == own || c <= 0) continue;
             bool feas = st.size[p] + L.vsize[n] <= omega && st.inpins[p] + L.vinpins[n] <= phi &&
-                        st.pincnt[p] + L.vincnt[n] - (int64_t)O[r0 + p] <= delta;
+                        st.pincnt[p] + L.vincnt[n] - (int64_t)O[p] <= delta;
             if (feas && better(sw + c, p, bs, bk)) {
                 bs = sw + c;
                 bk = p;
@@ -1762,9 +1738,7 @@ static Status dense_fresh(snnmap_hgraph* h, Level& L, const PinCounts& pc)
     pol.keys = D.K;
     pol.fresh = D.fresh;
     pol.rowid = D.rowid;
-    pol.C = D.C;
-    pol.O = D.O;
-    pol.Kp = D.Kp;
+    pol.tab = D.tab;
     pol.M = D.M;
     pol.cw = D.cw;
     int64_t* cnt;
@@ -1781,16 +1755,22 @@ int64_t dense_row_budget(const snnmap_hgraph* h)
     return (int64_t)(tot / 4);
 }
 
-Status dense_open(snnmap_hgraph* h, int32_t K, int64_t rows)
+// rows per chunk: about 1 GB of C and O
+constexpr int64_t ROW_CHUNK_BYTES = (int64_t)1 << 30;
+
+Status dense_open(snnmap_hgraph* h, int32_t K, int64_t cap)
 {
     dense_close(h);
     DenseRows& D = h->dense;
     cudaStream_t s = h->stream;
     D.K = K;
     D.Kp = ((int64_t)K + 3) & ~(int64_t)3;
-    D.cap = rows > 0 ? rows : 1;
-    SNN_CUDA(dev_malloc(&D.C, (size_t)(D.cap * D.Kp) * 4, s));
-    SNN_CUDA(dev_malloc(&D.O, (size_t)(D.cap * D.Kp) * 4, s));
+    D.cap = cap > 0 ? cap : 1;
+    D.tab.Kp = D.Kp;
+    while (((int64_t)1 << D.tab.shift) < D.cap && ((int64_t)2 << D.tab.shift) * D.Kp * 8 <= ROW_CHUNK_BYTES)
+        D.tab.shift++;
+    const int64_t nchunks = ceil_div(D.cap, (int64_t)1 << D.tab.shift);
+    SNN_CUDA(dev_malloc((void**)&D.tab.tab, (size_t)nchunks * 2 * sizeof(int32_t*), s));
     SNN_CUDA(dev_malloc(&D.rowid, (size_t)D.cap * 4, s));
     SNN_CUDA(dev_malloc(&D.rowid2, (size_t)D.cap * 4, s));
     SNN_CUDA(dev_malloc(&D.fresh, (size_t)D.cap * 4, s));
@@ -1802,12 +1782,38 @@ Status dense_open(snnmap_hgraph* h, int32_t K, int64_t rows)
     return Status{};
 }
 
+Status dense_grow(snnmap_hgraph* h, int64_t rows)
+{
+    DenseRows& D = h->dense;
+    if (!D.rowid || rows > D.cap) return Status{SNNMAP_ERR_STATE, "connection rows: capacity"};
+    const int64_t per = (int64_t)1 << D.tab.shift;
+    const size_t had = D.chunks.size(), need = (size_t)ceil_div(std::max<int64_t>(rows - D.rows, 0), per);
+    std::vector<int32_t*> ptrs;
+    ptrs.reserve(2 * need);
+    D.chunks.reserve(had + need);   // so that no chunk is lost to a failed host allocation
+    while (D.rows < rows) {
+        const int64_t n = std::min<int64_t>(per, D.cap - D.rows);
+        int32_t* c = nullptr;
+        SNN_CUDA(dev_malloc(&c, (size_t)(n * D.Kp) * 8, h->stream));
+        D.chunks.push_back(c);
+        ptrs.push_back(c);
+        ptrs.push_back(c + n * D.Kp);
+        D.rows += n;
+    }
+    if (!ptrs.empty())
+        SNN_CUDA(cudaMemcpyAsync((void*)(D.tab.tab + 2 * had), ptrs.data(), ptrs.size() * sizeof(int32_t*),
+                                 cudaMemcpyHostToDevice, h->stream));
+    return Status{};
+}
+
 void dense_close(snnmap_hgraph* h)
 {
     DenseRows& D = h->dense;
-    for (int32_t* p : {D.C, D.O, D.rowid, D.rowid2, D.fresh})
+    for (int32_t* p : D.chunks) cudaFreeAsync(p, h->stream);
+    for (int32_t* p : {D.rowid, D.rowid2, D.fresh})
         if (p) cudaFreeAsync(p, h->stream);
     if (D.M) cudaFreeAsync(D.M, h->stream);
+    if (D.tab.tab) cudaFreeAsync((void*)D.tab.tab, h->stream);
     D = DenseRows{};
 }
 
@@ -1815,12 +1821,12 @@ Status dense_begin(snnmap_hgraph* h, int32_t level)
 {
     DenseRows& D = h->dense;
     const Level& L = h->levels[level];
-    if (!D.C || L.V > D.cap) return Status{SNNMAP_ERR_STATE, "connection rows: capacity"};
+    if (L.V > D.rows) return Status{SNNMAP_ERR_STATE, "connection rows: capacity"};
     SNN_TRY(iota_i32(D.rowid, L.V, h->stream));
     SNN_TRY(fill_i32(D.fresh, 1, L.V, h->stream));
     if (L.V > 0) {
         SNN_L k_dense_zero<<<grid_for((int64_t)L.V * 32, 256), 256, 0, h->stream>>>(L.V, D.fresh, D.rowid,
-                                                                            D.C, D.O, D.M, D.Kp);
+                                                                            D.tab, D.M);
         SNN_CUDA(cudaGetLastError());
     }
     D.level = level;
@@ -1833,28 +1839,16 @@ Status dense_descend(snnmap_hgraph* h, int32_t level)
     DenseRows& D = h->dense;
     const Level& L = h->levels[level];
     int32_t Vc = h->levels[level + 1].V;
-    if (!D.C || D.level != level + 1 || L.V > D.cap)
+    if (D.level != level + 1 || L.V > D.rows)
         return Status{SNNMAP_ERR_STATE, "connection rows: descent out of order"};
     cudaStream_t s = h->stream;
     Arena& ar = h->scratch;
-    int32_t *mcount, *first, *nonrep, *idx;
-    SNN_TRY(ar.alloc(&mcount, Vc));
-    SNN_TRY(ar.alloc(&first, Vc));
-    SNN_TRY(ar.alloc(&nonrep, L.V));
-    SNN_TRY(ar.alloc(&idx, L.V));
-    SNN_CUDA(cudaMemsetAsync(mcount, 0, (size_t)(Vc > 0 ? Vc : 1) * 4, s));
-    SNN_TRY(fill_i32(first, INT_MAX, Vc, s));
     if (L.V > 0) {
-        int g = grid_for(L.V, 256);
-        SNN_L k_dense_members<<<g, 256, 0, s>>>(L.V, L.cid, mcount, first);
-        SNN_L k_dense_flags<<<g, 256, 0, s>>>(L.V, L.cid, mcount, first, nonrep, D.fresh);
-        SNN_CUDA(cudaGetLastError());
-        SNN_TRY(scan_exclusive_i32(nonrep, idx, L.V, nullptr, ar, s));
-        SNN_L k_dense_rowid<<<g, 256, 0, s>>>(L.V, Vc, L.cid, nonrep, idx, D.rowid, D.rowid2);
-        SNN_CUDA(cudaGetLastError());
+        SNN_TRY(scan_run<int32_t>(UpperMember{L.pr}, RowIds{L.pr, L.cid, D.rowid, Vc, D.rowid2, D.fresh}, L.V,
+                                  (int32_t*)nullptr, ar, s));
         std::swap(D.rowid, D.rowid2);
-        SNN_L k_dense_zero<<<grid_for((int64_t)L.V * 32, 256), 256, 0, s>>>(L.V, D.fresh, D.rowid, D.C,
-                                                                     D.O, D.M, D.Kp);
+        SNN_L k_dense_zero<<<grid_for((int64_t)L.V * 32, 256), 256, 0, s>>>(L.V, D.fresh, D.rowid, D.tab,
+                                                                     D.M);
         SNN_CUDA(cudaGetLastError());
     }
     D.level = level;
@@ -2121,7 +2115,52 @@ struct IncState {
     int32_t* hmeta = nullptr;    // their bucket starts and counts (2 * SEG_NB)
     bool ready = false;          // set once the first round computed them
     PStar pst;                   // column update of proposals after short prefixes
+    int64_t members = 0;         // members of pairs whose saves are to be computed (0: all vertices')
+    int32_t* mlist = nullptr;
+    int32_t* mcnt = nullptr;
 };
+
+// saves and W of the listed vertices (cleared before) from their hyperedges;
+// the four blocks of a column share a vertex's incidences
+__global__ void __launch_bounds__(256)
+    k_save_members(Level L, PinCounts pc, const int32_t* __restrict__ rho,
+                   const int32_t* __restrict__ list, const int32_t* __restrict__ nlist, int64_t* savev,
+                   int64_t* Wv)
+{
+    __shared__ unsigned long long sum[2];
+    const int32_t nl = *nlist;
+    for (int32_t x = blockIdx.x; x < nl; x += gridDim.x) {
+        const int32_t n = list[x];
+        const int64_t vb = L.voff[n], ve = L.voff[n + 1];
+        if (vb + (int64_t)blockIdx.y * 1024 >= ve) continue;   // the whole block
+        if (threadIdx.x < 2) sum[threadIdx.x] = 0;
+        __syncthreads();
+        const int32_t p = rho[n];
+        int64_t W = 0, save = 0;
+        for (int64_t t = vb + (int64_t)blockIdx.y * 1024; t < ve; t += 4 * 1024) {
+            const int64_t te = t + 1024 < ve ? t + 1024 : ve;
+            for (int64_t i = t + threadIdx.x; i < te; i += 256) {
+                HRec r = pc.rec[(int32_t)((uint32_t)L.vinc[i] & ~SRC_BIT)];
+                W += r.w;
+                int32_t c, d;
+                lookup_count(pc, r.b, r.n(), p, c, d);
+                if (c == 1) save += r.w;
+            }
+        }
+        W = warp_sum(W);
+        save = warp_sum(save);
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(&sum[0], (unsigned long long)W);
+            atomicAdd(&sum[1], (unsigned long long)save);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            if (sum[0]) atomicAdd((unsigned long long*)&Wv[n], sum[0]);
+            if (sum[1]) atomicAdd((unsigned long long*)&savev[n], sum[1]);
+        }
+        __syncthreads();
+    }
+}
 
 // One round; *applied = moves enacted, *gain = Conn removed, *cost = Conn at
 // round start.
@@ -2154,7 +2193,7 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
         SNN_CUDA(cudaGetLastError());
     }
     DenseRows& D = h->dense;
-    const bool dense = D.C && D.level == level;
+    const bool dense = D.level == level;
     std::unique_ptr<ProfScope> prof;
     if (dense && D.pending) {
         prof.reset(new ProfScope(h, PS_ROWS));
@@ -2167,7 +2206,12 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     int64_t* Wv = inc.Wv;
     if (!inc.ready) {
         prof.reset(new ProfScope(h, PS_SAVE));
-        if (L.E > 0 && !h->wide && V <= SAVE_SMEM_V) {
+        if (inc.mlist) {
+            if (inc.members > 0)
+                SNN_L k_save_members<<<dim3((unsigned)std::min<int64_t>(inc.members, 152 * 16), 4), 256, 0,
+                                       s>>>(L, pc, rho, inc.mlist, inc.mcnt, savev, Wv);
+            SNN_CUDA(cudaGetLastError());
+        } else if (L.E > 0 && !h->wide && V <= SAVE_SMEM_V) {
             auto launch = [&](auto kern) -> Status {
                 SNN_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               SAVE_SMEM_V * 8));
@@ -2191,7 +2235,7 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     if (dense) {
         if (V > 0) {
             SNN_L k_dense_best<<<grid_for((int64_t)V * 32, 256), 256, 0, s>>>(
-                L, rho, ps, savev, Wv, D.rowid, D.C, D.O, D.M, D.cw, D.Kp, K, prm.omega, prm.delta,
+                L, rho, ps, savev, Wv, D.rowid, D.tab, D.M, D.cw, K, prm.omega, prm.delta,
                 prm.phi, prm.refine_nonpositive, pto, pgain, inc.dirty);
             SNN_CUDA(cudaGetLastError());
         }
@@ -2335,7 +2379,7 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     // counts, old rho), move, count them again, add them back
     prof.reset(new ProfScope(h, PS_PINCOUNT));
     if (L.E > 0) {
-        RowsRef R{dense ? D.rowid : nullptr, D.C, D.O, D.M, D.cw, D.Kp};
+        RowsRef R{dense ? D.rowid : nullptr, D.tab, D.M, D.cw};
         SNN_L k_prefix_hedges<<<ghl, 256, 0, s>>>(L, pc, moveidx, mv, h->d_scal, R, mvbuf, inc.hdirty, rho,
                                                   ps, savev, inc.costv, hl);
         SNN_CUDA(cudaGetLastError());
@@ -2386,8 +2430,8 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     } else {
         prof.reset(new ProfScope(h, PS_GAINS));
         if (V > 0)
-            SNN_L k_ps_rows<<<gv, 256, 0, s>>>(L, rho, h->d_scal, inc.pst, ps, savev, Wv, D.rowid, D.C,
-                                               D.O, D.Kp, prm.omega, prm.delta, prm.phi,
+            SNN_L k_ps_rows<<<gv, 256, 0, s>>>(L, rho, h->d_scal, inc.pst, ps, savev, Wv, D.rowid, D.tab,
+                                               prm.omega, prm.delta, prm.phi,
                                                prm.refine_nonpositive, pto, pgain, inc.dirty);
         SNN_L k_ps_reset<<<gm, 256, 0, s>>>(M, mv, h->d_scal, inc.pst, host);
         SNN_CUDA(cudaGetLastError());
@@ -2430,14 +2474,7 @@ Status check_rho(snnmap_hgraph* h, int32_t level, int32_t K, const int32_t* rho)
 // super-node's proposal, gain and flag (its conn, overlap, save, W and the
 // partition state are unchanged by projection); both members of a pair are
 // evaluated.
-__global__ void k_carry_count(int32_t V, const int32_t* __restrict__ cid, int32_t* mcount)
-{
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
-         n += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&mcount[cid[n]], 1);
-}
-
-__global__ void k_carry(int32_t V, const int32_t* __restrict__ cid, const int32_t* __restrict__ mcount,
+__global__ void k_carry(int32_t V, const int32_t* __restrict__ cid, const uint8_t* __restrict__ pr,
                         const int32_t* __restrict__ pto_c, const int64_t* __restrict__ pgain_c,
                         const int32_t* __restrict__ dirty_c, int32_t* pto, int64_t* pgain,
                         int32_t* dirty)
@@ -2447,7 +2484,7 @@ __global__ void k_carry(int32_t V, const int32_t* __restrict__ cid, const int32_
         int32_t c = cid[n];
         pto[n] = pto_c[c];
         pgain[n] = pgain_c[c];
-        dirty[n] = (mcount[c] > 1 || dirty_c[c]) ? 1 : 0;
+        dirty[n] = (pr[n] || dirty_c[c]) ? 1 : 0;
     }
 }
 
@@ -2460,9 +2497,11 @@ Status carry_open(snnmap_hgraph* h, int64_t cap)
         SNN_CUDA(dev_malloc(&C.pto[b], n * 4, h->stream));
         SNN_CUDA(dev_malloc(&C.pgain[b], n * 8, h->stream));
         SNN_CUDA(dev_malloc(&C.dirty[b], n * 4, h->stream));
+        SNN_CUDA(dev_malloc(&C.save[b], n * 16, h->stream));
     }
     C.cap = cap;
     C.level = -1;
+    C.slevel = -1;
     C.cur = 0;
     return Status{};
 }
@@ -2471,20 +2510,41 @@ void carry_close(snnmap_hgraph* h)
 {
     Carry& C = h->carry;
     for (int b = 0; b < 2; b++)
-        for (void* p : {(void*)C.pto[b], (void*)C.pgain[b], (void*)C.dirty[b]})
+        for (void* p : {(void*)C.pto[b], (void*)C.pgain[b], (void*)C.dirty[b], (void*)C.save[b]})
             if (p) cudaFreeAsync(p, h->stream);
     C = Carry{};
 }
 
-// no move listed, every vertex to evaluate (unless inherited), no slot taken
+// Saves and W inherited from the next coarser level (cid null: none). An
+// unmatched vertex keeps its super-node's: its hyperedges map one to one onto
+// that super-node's with the same summed omega, and it is its partition's last
+// pin in the same ones. The members of pairs are listed and computed from
+// their hyperedges (k_save_members), which took every vertex before.
+struct SaveIn {
+    const int32_t* cid;
+    const uint8_t* pr;
+    const int64_t *sc, *wc;
+    int64_t *save, *W;
+    int32_t *mlist, *mcnt;
+};
+
+// no move listed, every vertex to evaluate (unless inherited), no slot taken,
+// saves inherited
 __global__ void k_refine_init(int32_t V, int32_t K, int32_t* moveidx, int32_t* dirty, PStar ps,
-                              int32_t base)
+                              int32_t base, SaveIn si)
 {
     int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     int64_t step = (int64_t)gridDim.x * blockDim.x;
     for (int64_t n = t0; n < V; n += step) {
         moveidx[n] = -1;
         if (dirty) dirty[n] = 1;
+        if (si.cid) {
+            bool pair = si.pr[n] != 0;
+            int32_t c = si.cid[n];
+            si.save[n] = pair ? 0 : si.sc[c];
+            si.W[n] = pair ? 0 : si.wc[c];
+            if (pair) si.mlist[atomicAdd(si.mcnt, 1)] = (int32_t)n;
+        }
     }
     for (int64_t p = t0; p < K; p += step) ps.pslot[p] = -1;
     if (t0 < 4) ps.cnt[t0] = (t0 & 1) ? 0 : base;
@@ -2499,7 +2559,7 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
     IncState inc;
     PStar& pst = inc.pst;
     Carry& CA = h->carry;
-    const bool dense_level = h->dense.C && h->dense.level == level;
+    const bool dense_level = h->dense.level == level;
     const bool use_carry = CA.pto[0] && L.V <= CA.cap;
     const int64_t V = L.V, E = L.E;
     bool inherited = false;
@@ -2512,10 +2572,16 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
     cv.add(&inc.ps.inpins, K);
     cv.add(&inc.ps.pincnt, K);
     cv.add(&inc.slots, COST_SLOTS);
-    cv.add(&inc.savev, V);
-    cv.add(&inc.Wv, V);
+    const bool inherit_save =
+        use_carry && CA.slevel == level + 1 && 8 * (V - h->levels[level + 1].V) <= V;
+    if (inherit_save) cv.add(&inc.mcnt, 1);
+    if (!use_carry) {
+        cv.add(&inc.savev, V);
+        cv.add(&inc.Wv, V);
+    }
     const size_t cleared = cv.total;
     cv.add(&moveidx, V);
+    if (inherit_save) cv.add(&inc.mlist, 2 * (V - h->levels[level + 1].V));
     if (!use_carry) {
         cv.add(&inc.pto, V);
         cv.add(&inc.pgain, V);
@@ -2562,6 +2628,7 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
         cudaFreeAsync(block, s);
         if (cols) cudaFreeAsync(cols, s);
     };
+    SaveIn si{};
     auto setup = [&]() -> Status {
         SNN_CUDA(cudaMemsetAsync(block, 0, cleared, s));
         if (cols && ccleared) SNN_CUDA(cudaMemsetAsync(cols, 0, ccleared, s));
@@ -2570,13 +2637,19 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
             inc.pto = CA.pto[nb];
             inc.pgain = CA.pgain[nb];
             inc.dirty = CA.dirty[nb];
+            inc.savev = CA.save[nb];
+            inc.Wv = CA.save[nb] + V;
+            if (inherit_save) {
+                inc.members = 2 * (V - h->levels[level + 1].V);
+                const int64_t* from = CA.save[CA.cur];
+                si = SaveIn{L.cid, L.pr, from, from + h->levels[level + 1].V, inc.savev, inc.Wv,
+                            inc.mlist, inc.mcnt};
+            } else {
+                SNN_CUDA(cudaMemsetAsync(inc.savev, 0, (size_t)V * 16, s));
+            }
+            CA.slevel = -1;
             if (!dense_level && CA.level == level + 1 && L.V > 0) {
-                const Level& Lc = h->levels[level + 1];
-                int32_t* mcount;
-                SNN_TRY(h->scratch.alloc(&mcount, Lc.V));
-                SNN_CUDA(cudaMemsetAsync(mcount, 0, (size_t)(Lc.V > 0 ? Lc.V : 1) * 4, s));
-                SNN_L k_carry_count<<<grid_for(L.V, 256), 256, 0, s>>>(L.V, L.cid, mcount);
-                SNN_L k_carry<<<grid_for(L.V, 256), 256, 0, s>>>(L.V, L.cid, mcount, CA.pto[CA.cur],
+                SNN_L k_carry<<<grid_for(L.V, 256), 256, 0, s>>>(L.V, L.cid, L.pr, CA.pto[CA.cur],
                                                                 CA.pgain[CA.cur], CA.dirty[CA.cur],
                                                                 inc.pto, inc.pgain, inc.dirty);
                 SNN_CUDA(cudaGetLastError());
@@ -2587,7 +2660,7 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
         }
         // without the saves (and columns) the column update stays off
         SNN_L k_refine_init<<<grid_for(std::max<int64_t>(V, K), 256), 256, 0, s>>>(
-            L.V, K, moveidx, inherited ? nullptr : inc.dirty, pst, cols ? 0 : (1 << 30));
+            L.V, K, moveidx, inherited ? nullptr : inc.dirty, pst, cols ? 0 : (1 << 30), si);
         if (!dense_level && L.V > 0) SNN_L k_level_max<<<grid_for(L.V, 256, 152 * 4), 256, 0, s>>>(L, inc.vmax);
         SNN_CUDA(cudaGetLastError());
         return Status{};
@@ -2609,6 +2682,7 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
         if (applied == 0) break;
     }
     give_back();
+    if (use_carry && st.ok() && inc.ready) CA.slevel = level;   // saves, for the next finer level
     if (use_carry && st.ok() && !dense_level)
         CA.level = level;   // the next finer level may inherit these proposals
     if (!st.ok()) return st;
