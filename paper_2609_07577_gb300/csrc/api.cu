@@ -86,6 +86,7 @@ void drop_levels_above(snnmap_hgraph* h, size_t keep)
 
 __global__ void k_mark_used(int32_t V, const int32_t* __restrict__ rho, uint8_t* used)
 {
+    snn::after_previous();
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x)
         used[rho[n]] = 1;
@@ -93,6 +94,7 @@ __global__ void k_mark_used(int32_t V, const int32_t* __restrict__ rho, uint8_t*
 
 __global__ void k_count_used(int32_t K, const uint8_t* __restrict__ used, int64_t* out)
 {
+    snn::after_previous();
     int c = 0;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < K;
          p += (int64_t)gridDim.x * blockDim.x)
@@ -107,8 +109,9 @@ snn::Status count_nonempty(snnmap_hgraph* h, int32_t V, int32_t K, const int32_t
     SNN_TRY(h->scratch.alloc(&used, K));
     SNN_CUDA(cudaMemsetAsync(used, 0, (size_t)K, h->stream));
     SNN_TRY(snn::zero_scalars(h));
-    if (V > 0) SNN_L k_mark_used<<<snn::grid_for(V, 256), 256, 0, h->stream>>>(V, rho, used);
-    if (K > 0) SNN_L k_count_used<<<snn::grid_for(K, 256), 256, 0, h->stream>>>(K, used, h->d_scal + snn::SC_A);
+    if (V > 0) snn::enqueue(k_mark_used, snn::grid_for(V, 256), 256, 0, h->stream, V, rho, used);
+    if (K > 0) snn::enqueue(k_count_used, snn::grid_for(K, 256), 256, 0, h->stream, K, used,
+                            h->d_scal + snn::SC_A);
     SNN_CUDA(cudaGetLastError());
     SNN_TRY(snn::read_scalars(h));
     *out = (int32_t)h->h_scal[snn::SC_A];

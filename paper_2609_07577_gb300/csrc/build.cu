@@ -172,6 +172,7 @@ __global__ void __launch_bounds__(1024)
     k_seg_lists(const int64_t* __restrict__ hoff, int32_t E, SegStart st, int32_t* cursor,
                 int32_t* meta, int32_t* list)
 {
+    after_previous();
     __shared__ int32_t wc[SEG_NB][32];
     __shared__ int32_t base[SEG_NB];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -223,7 +224,7 @@ Status seg_lists(const int64_t* hoff, int32_t E, int32_t maxlen, SegBuckets& b, 
         st.n[i] = b.n[i];
         run += b.n[i];
     }
-    SNN_L k_seg_lists<<<grid_for(E, 1024, 152 * 2), 1024, 0, s>>>(hoff, E, st, cursor, b.meta, b.list);
+    enqueue(k_seg_lists, grid_for(E, 1024, 152 * 2), 1024, 0, s, hoff, E, st, cursor, b.meta, b.list);
     SNN_CUDA(cudaGetLastError());
     return Status{};
 }
@@ -236,6 +237,7 @@ Status seg_lists(const int64_t* hoff, int32_t E, int32_t maxlen, SegBuckets& b, 
 // runs over whole warps so the match covers all 32 lanes.
 __global__ void k_count_deg(const int32_t* __restrict__ pins, int64_t P, int32_t* deg)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < P;
@@ -253,6 +255,7 @@ __global__ void k_csc_fill(const int64_t* __restrict__ hoff, const int32_t* __re
                            int32_t E, const int64_t* __restrict__ voff, int32_t* cursor,
                            int32_t* vinc)
 {
+    after_previous();
     int lane = threadIdx.x & (G - 1);
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -278,6 +281,7 @@ constexpr int CSC_THREADS = 1024;
 __global__ void __launch_bounds__(CSC_THREADS)
     k_deg_smem(const int32_t* __restrict__ pins, int64_t P, int32_t V, int32_t* deg)
 {
+    after_previous();
     extern __shared__ int32_t sdeg[];
     for (int32_t v = threadIdx.x; v < V; v += CSC_THREADS) sdeg[v] = 0;
     __syncthreads();
@@ -306,6 +310,7 @@ __global__ void __launch_bounds__(CSC_THREADS)
     k_csc_smem(const int64_t* __restrict__ hoff, const int32_t* __restrict__ pins, int32_t E,
                int64_t P, int32_t V, const int64_t* __restrict__ voff, int32_t* cursor, int32_t* vinc)
 {
+    after_previous();
     extern __shared__ int32_t sdeg[];
     __shared__ int32_t se[2];
     if (threadIdx.x < 2) se[threadIdx.x] = hedge_at(hoff, E, P * (blockIdx.x + threadIdx.x) / gridDim.x);
@@ -347,9 +352,9 @@ Status build_incidence(snnmap_hgraph* h, Level& L)
         if (small) {
             SNN_CUDA(cudaFuncSetAttribute(k_deg_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           CSC_SMEM_V * 4));
-            SNN_L k_deg_smem<<<nb, CSC_THREADS, sm, s>>>(L.hpins, L.P, L.V, deg);
+            enqueue(k_deg_smem, nb, CSC_THREADS, sm, s, L.hpins, L.P, L.V, deg);
         } else {
-            SNN_L k_count_deg<<<grid_for(L.P, 256), 256, 0, s>>>(L.hpins, L.P, deg);
+            enqueue(k_count_deg, grid_for(L.P, 256), 256, 0, s, L.hpins, L.P, deg);
         }
         SNN_CUDA(cudaGetLastError());
     }
@@ -359,8 +364,8 @@ Status build_incidence(snnmap_hgraph* h, Level& L)
             auto launch = [&](auto kern) -> Status {
                 SNN_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               CSC_SMEM_V * 4));
-                SNN_L kern<<<nb, CSC_THREADS, sm, s>>>(L.hoff, L.hpins, L.E, L.P, L.V, L.voff, cursor,
-                                                       L.vinc);
+                enqueue(kern, nb, CSC_THREADS, sm, s, L.hoff, L.hpins, L.E, L.P, L.V, L.voff, cursor,
+                        L.vinc);
                 return Status{};
             };
             switch (hedge_lanes(L.P, L.E)) {
@@ -384,6 +389,7 @@ Status build_incidence(snnmap_hgraph* h, Level& L)
 __global__ void k_in_hedges(const int64_t* __restrict__ off, const int32_t* __restrict__ w,
                             int32_t E, int32_t* kept, int64_t* klen, int64_t* scal)
 {
+    after_previous();
     SegTally tally;
     int32_t bad = 0;
     int64_t mx = 0, wsum = 0;
@@ -419,6 +425,7 @@ __global__ void k_in_hedges(const int64_t* __restrict__ off, const int32_t* __re
 
 __global__ void k_in_pins(const int32_t* __restrict__ pins, int64_t P, int32_t V, int64_t* scal)
 {
+    after_previous();
     int bad = 0;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P;
          j += (int64_t)gridDim.x * blockDim.x) {
@@ -433,6 +440,7 @@ __global__ void k_copy_hedges(const int64_t* __restrict__ off, const int32_t* __
                               const int32_t* __restrict__ kept, const int32_t* __restrict__ newid,
                               const int64_t* __restrict__ newoff, Level L)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -452,6 +460,7 @@ __global__ void k_copy_hedges(const int64_t* __restrict__ off, const int32_t* __
 
 __global__ void k_set_last_off(int64_t* hoff, int32_t E, const int64_t* P)
 {
+    after_previous();
     hoff[E] = *P;
 }
 
@@ -495,6 +504,7 @@ struct BuildCheckJob {
 __global__ void k_count_inpins(const int64_t* __restrict__ hoff, const int32_t* __restrict__ pins,
                                int32_t E, int32_t* inpins)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -505,6 +515,7 @@ __global__ void k_count_inpins(const int64_t* __restrict__ hoff, const int32_t* 
 
 __global__ void k_vertex_init(Level L, int32_t delta, int32_t phi, int64_t* scal)
 {
+    after_previous();
     int bad = 0;
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < L.V;
          n += (int64_t)gridDim.x * blockDim.x) {
@@ -537,11 +548,11 @@ Status build_level0(snnmap_hgraph* h, int32_t V, int32_t E, const int64_t* d_off
     SNN_TRY(ar.alloc(&klen, E));
     SNN_TRY(ar.alloc(&newoff, E));
     if (E > 0) {
-        SNN_L k_in_hedges<<<grid_for(E, 256, 152 * 8), 256, 0, s>>>(d_off, d_w, E, kept, klen, h->d_scal);
+        enqueue(k_in_hedges, grid_for(E, 256, 152 * 8), 256, 0, s, d_off, d_w, E, kept, klen, h->d_scal);
         SNN_CUDA(cudaGetLastError());
     }
     if (Pin > 0) {
-        SNN_L k_in_pins<<<grid_for(Pin, 256), 256, 0, s>>>(d_pins, Pin, V, h->d_scal);
+        enqueue(k_in_pins, grid_for(Pin, 256), 256, 0, s, d_pins, Pin, V, h->d_scal);
         SNN_CUDA(cudaGetLastError());
     }
     SNN_TRY(scan_exclusive_i32(kept, newid, E, (int32_t*)(h->d_scal + SC_A), ar, s));
@@ -564,11 +575,11 @@ Status build_level0(snnmap_hgraph* h, int32_t V, int32_t E, const int64_t* d_off
     SNN_TRY(level_alloc(h, L, X, V, E0, P0));
     L.maxlen = maxlen;
     if (E > 0) {
-        SNN_L k_copy_hedges<<<grid_for((int64_t)E * 32, 256), 256, 0, s>>>(d_off, d_pins, d_w, E, kept,
-                                                                      newid, newoff, L);
+        enqueue(k_copy_hedges, grid_for((int64_t)E * 32, 256), 256, 0, s, d_off, d_pins, d_w, E, kept,
+                newid, newoff, L);
         SNN_CUDA(cudaGetLastError());
     }
-    SNN_L k_set_last_off<<<1, 1, 0, s>>>(L.hoff, E0, h->d_scal + SC_B);
+    enqueue(k_set_last_off, 1, 1, 0, s, L.hoff, E0, h->d_scal + SC_B);
     SNN_CUDA(cudaGetLastError());
     X.pair_terms = terms;
     for (int i = 0; i < SEG_NB; i++) X.seg.n[i] = (int32_t)h->h_scal[SC_SEG + i];
@@ -583,11 +594,12 @@ Status build_level0(snnmap_hgraph* h, int32_t V, int32_t E, const int64_t* d_off
     }
     if (V > 0) SNN_CUDA(cudaMemsetAsync(L.vinpins, 0, (size_t)V * sizeof(int32_t), s));
     if (E0 > 0) {
-        SNN_L k_count_inpins<<<grid_for((int64_t)E0 * 32, 256), 256, 0, s>>>(L.hoff, L.hpins, E0, L.vinpins);
+        enqueue(k_count_inpins, grid_for((int64_t)E0 * 32, 256), 256, 0, s, L.hoff, L.hpins, E0,
+                L.vinpins);
         SNN_CUDA(cudaGetLastError());
     }
     if (V > 0) {
-        SNN_L k_vertex_init<<<grid_for(V, 256), 256, 0, s>>>(L, h->prm.delta, h->prm.phi, h->d_scal);
+        enqueue(k_vertex_init, grid_for(V, 256), 256, 0, s, L, h->prm.delta, h->prm.phi, h->d_scal);
         SNN_CUDA(cudaGetLastError());
     }
     SNN_TRY(build_incidence(h, L));

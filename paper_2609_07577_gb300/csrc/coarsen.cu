@@ -147,6 +147,7 @@ struct AffPol {
 
 __global__ void k_pack_hedges(Level L, HRec* rec)
 {
+    after_previous();
     for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < L.E;
          a += (int64_t)gridDim.x * blockDim.x) {
         int64_t b = L.hoff[a];
@@ -159,6 +160,7 @@ __global__ void k_pack_hedges(Level L, HRec* rec)
 // a neighbour's state is one gather in the histograms' hot loops
 __global__ void k_pack_state(Level L, int4* vst)
 {
+    after_previous();
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < L.V;
          n += (int64_t)gridDim.x * blockDim.x)
         vst[n] = make_int4(L.vsize[n], L.vinpins[n], L.vincnt[n], 0);
@@ -174,6 +176,7 @@ __global__ void __launch_bounds__(256)
     k_child_best_score(int32_t V, const int32_t* __restrict__ cand,
                        const int64_t* __restrict__ cscore, unsigned long long* bestsc, int64_t* scal)
 {
+    after_previous();
     int k = 0;
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
@@ -188,6 +191,7 @@ __global__ void k_child_best_id(int32_t V, const int32_t* __restrict__ cand,
                                 const int64_t* __restrict__ cscore,
                                 const unsigned long long* __restrict__ bestsc, uint32_t* bc)
 {
+    after_previous();
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
         int32_t c = cand[n];
@@ -224,6 +228,7 @@ __global__ void __launch_bounds__(256)
     k_match(int32_t V, const int32_t* __restrict__ cand, const uint32_t* __restrict__ bc,
             int32_t* match, int64_t* scal)
 {
+    after_previous();
     int longer = 0, pairs = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < V;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -250,6 +255,7 @@ __global__ void __launch_bounds__(256)
 __global__ void k_jump_init(int32_t V, const int32_t* __restrict__ cand,
                             const uint32_t* __restrict__ bc, int32_t* nxt, uint8_t* pj)
 {
+    after_previous();
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
         int32_t l = chain_link(cand, bc, (int32_t)n);
@@ -261,6 +267,7 @@ __global__ void k_jump_init(int32_t V, const int32_t* __restrict__ cand,
 __global__ void k_jump(int32_t V, const int32_t* __restrict__ nxt, const uint8_t* __restrict__ pj,
                        int32_t* nxt2, uint8_t* pj2, int64_t* scal)
 {
+    after_previous();
     int c = 0;
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
@@ -283,6 +290,7 @@ __global__ void __launch_bounds__(256)
     k_match_jumped(int32_t V, const int32_t* __restrict__ cand, const uint32_t* __restrict__ bc,
                    const uint8_t* __restrict__ pj, int32_t* match, int64_t* scal)
 {
+    after_previous();
     int pairs = 0;
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
@@ -299,6 +307,7 @@ __global__ void __launch_bounds__(256)
 // vm[3]: the largest (all start cleared)
 __global__ void __launch_bounds__(256) k_level_min(Level L, uint32_t* vm)
 {
+    after_previous();
     __shared__ uint32_t sv[4];
     if (threadIdx.x < 4) sv[threadIdx.x] = 0;
     __syncthreads();
@@ -331,18 +340,18 @@ static Status affinity(snnmap_hgraph* h, Level& L)
     uint32_t* vmin;
     SNN_TRY(h->scratch.alloc(&vmin, 4));
     SNN_CUDA(cudaMemsetAsync(vmin, 0, 4 * sizeof(int32_t), h->stream));
-    SNN_L k_level_min<<<grid_for(L.V, 256, 152 * 4), 256, 0, h->stream>>>(L, vmin);
+    enqueue(k_level_min, grid_for(L.V, 256, 152 * 4), 256, 0, h->stream, L, vmin);
     SNN_CUDA(cudaGetLastError());
     int32_t vm[4];
     SNN_CUDA(cudaMemcpyAsync(vm, vmin, sizeof(vm), cudaMemcpyDeviceToHost, h->stream));
     SNN_CUDA(cudaStreamSynchronize(h->stream));
     int4* vst;
     SNN_TRY(h->scratch.alloc(&vst, L.V));
-    SNN_L k_pack_state<<<grid_for(L.V, 256), 256, 0, h->stream>>>(L, vst);
+    enqueue(k_pack_state, grid_for(L.V, 256), 256, 0, h->stream, L, vst);
     SNN_CUDA(cudaGetLastError());
     HRec* rec;
     SNN_TRY(h->scratch.alloc(&rec, L.E));
-    if (L.E > 0) SNN_L k_pack_hedges<<<grid_for(L.E, 256), 256, 0, h->stream>>>(L, rec);
+    if (L.E > 0) enqueue(k_pack_hedges, grid_for(L.E, 256), 256, 0, h->stream, L, rec);
     SNN_CUDA(cudaGetLastError());
     AffPol<S> pol;
     pol.rec = rec;
@@ -431,6 +440,7 @@ __global__ void k_ac_prep(int32_t V, const int32_t* __restrict__ cid,
                           const int64_t* __restrict__ cscore, const int32_t* __restrict__ cov,
                           AffCarry ac)
 {
+    after_previous();
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
         int32_t x = cid[n];
@@ -468,6 +478,7 @@ template <int G>
 __global__ void __launch_bounds__(256)
     k_ac_count(Level L, const uint8_t* __restrict__ kind, int32_t* lcnt, int64_t* work)
 {
+    after_previous();
     constexpr int PER = 32 / G;
     int lane = threadIdx.x & (G - 1);
     int grp = (threadIdx.x & 31) / G;
@@ -505,6 +516,7 @@ __global__ void __launch_bounds__(256)
     k_ac_fill(Level L, const uint8_t* __restrict__ kind, const int64_t* __restrict__ loff,
               uint32_t* lpins)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     unsigned lt = lanemask_lt();
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -533,6 +545,7 @@ __global__ void __launch_bounds__(256)
 __global__ void __launch_bounds__(256)
     k_ac_check(Level L, AffCarry ac, int32_t omega, int32_t delta, int32_t phi)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -707,8 +720,8 @@ Status aff_carry(snnmap_hgraph* h, int32_t src)
         C.cap = (int64_t)n;
     }
     if (F.V > 0) {
-        SNN_L k_ac_prep<<<grid_for(F.V, 256), 256, 0, h->stream>>>(F.V, F.cid, h->match, h->cand,
-                                                                  h->cscore, h->cov, C);
+        enqueue(k_ac_prep, grid_for(F.V, 256), 256, 0, h->stream, F.V, F.cid, h->match, h->cand,
+                h->cscore, h->cov, C);
         SNN_CUDA(cudaGetLastError());
     }
     C.level = src + 1;
@@ -747,7 +760,7 @@ static Status affinity_carried(snnmap_hgraph* h, Level& L, bool* done)
     SNN_TRY(ar.alloc(&loff, E + 1));
     SNN_CUDA(cudaMemsetAsync(work, 0, 5 * sizeof(int64_t), s));
     uint32_t* vmin = (uint32_t*)(work + 3);
-    SNN_L k_level_min<<<grid_for(L.V, 256, 152 * 4), 256, 0, s>>>(L, vmin);
+    enqueue(k_level_min, grid_for(L.V, 256, 152 * 4), 256, 0, s, L, vmin);
     if (E > 0) SNN_HEDGE_LAUNCH(hedge_lanes(L.P, E), k_ac_count, E, s, L, C.kind, lcnt, work);
     SNN_CUDA(cudaGetLastError());
     HRec* lrec;
@@ -766,12 +779,12 @@ static Status affinity_carried(snnmap_hgraph* h, Level& L, bool* done)
     uint32_t* lpins;
     SNN_TRY(ar.alloc(&lpins, hv[2]));
     if (E > 0 && hv[2] > 0)
-        SNN_L k_ac_fill<<<grid_for(E * 32, 256), 256, 0, s>>>(L, C.kind, loff, lpins);
+        enqueue(k_ac_fill, grid_for(E * 32, 256), 256, 0, s, L, C.kind, loff, lpins);
     SNN_CUDA(cudaGetLastError());
     bool prefilter = 2 * (int64_t)vm[2] > h->prm.omega || 2 * (int64_t)vm[3] > h->prm.phi;
     int4* vst;
     SNN_TRY(ar.alloc(&vst, L.V));
-    SNN_L k_pack_state<<<grid_for(L.V, 256), 256, 0, s>>>(L, vst);
+    enqueue(k_pack_state, grid_for(L.V, 256), 256, 0, s, L, vst);
     SNN_CUDA(cudaGetLastError());
     int64_t* cnt;
     SNN_TRY(ar.alloc(&cnt, HT_NCNT));
@@ -795,8 +808,7 @@ static Status affinity_carried(snnmap_hgraph* h, Level& L, bool* done)
         SNN_TRY(run_histogram(pol, ar, s, cnt, h->h_scal + 12, h->d_scal, h->tiers, L.V, !h->wzero));
         SNN_CUDA(cudaMemcpyAsync(h->h_tier, cnt, HT_NCNT * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     }
-    SNN_L k_ac_check<<<grid_for(L.V, 256), 256, 0, s>>>(L, C, h->prm.omega, h->prm.delta,
-                                                        h->prm.phi);
+    enqueue(k_ac_check, grid_for(L.V, 256), 256, 0, s, L, C, h->prm.omega, h->prm.delta, h->prm.phi);
     SNN_CUDA(cudaGetLastError());
     {
         AffPol<S> pol;
@@ -841,9 +853,9 @@ static Status match_into(int32_t V, const int32_t* cand, const int64_t* cscore, 
     SNN_TRY(ar.alloc(&base, (int64_t)c.total));
     c.assign(base);
     SNN_CUDA(cudaMemsetAsync(base, 0, c.total, s));
-    SNN_L k_child_best_score<<<g, 256, 0, s>>>(V, cand, cscore, bestsc, d_scal);
-    SNN_L k_child_best_id<<<g, 256, 0, s>>>(V, cand, cscore, bestsc, bc);
-    SNN_L k_match<<<g, 256, 0, s>>>(V, cand, bc, match, d_scal);
+    enqueue(k_child_best_score, g, 256, 0, s, V, cand, cscore, bestsc, d_scal);
+    enqueue(k_child_best_id, g, 256, 0, s, V, cand, cscore, bestsc, bc);
+    enqueue(k_match, g, 256, 0, s, V, cand, bc, match, d_scal);
     SNN_CUDA(cudaGetLastError());
     auto read = [&]() -> Status {
         SNN_CUDA(cudaMemcpyAsync(h_scal, d_scal, SC_COUNT * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
@@ -859,18 +871,18 @@ static Status match_into(int32_t V, const int32_t* cand, const int64_t* cscore, 
         SNN_TRY(ar.alloc(&nxt2, V));
         SNN_TRY(ar.alloc(&pj, V));
         SNN_TRY(ar.alloc(&pj2, V));
-        SNN_L k_jump_init<<<g, 256, 0, s>>>(V, cand, bc, nxt, pj);
+        enqueue(k_jump_init, g, 256, 0, s, V, cand, bc, nxt, pj);
         SNN_CUDA(cudaGetLastError());
         for (int it = 0; it < 40; it++) {
             SNN_CUDA(cudaMemsetAsync(d_scal + SC_B, 0, 2 * sizeof(int64_t), s));
-            SNN_L k_jump<<<g, 256, 0, s>>>(V, nxt, pj, nxt2, pj2, d_scal);
+            enqueue(k_jump, g, 256, 0, s, V, nxt, pj, nxt2, pj2, d_scal);
             SNN_CUDA(cudaGetLastError());
             std::swap(nxt, nxt2);
             std::swap(pj, pj2);
             SNN_TRY(read());
             if (h_scal[SC_B] == 0) break;
         }
-        SNN_L k_match_jumped<<<g, 256, 0, s>>>(V, cand, bc, pj, match, d_scal);
+        enqueue(k_match_jumped, g, 256, 0, s, V, cand, bc, pj, match, d_scal);
         SNN_CUDA(cudaGetLastError());
         SNN_TRY(read());
     }

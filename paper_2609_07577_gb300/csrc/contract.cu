@@ -51,6 +51,7 @@ struct NextState {
 __global__ void k_cid_map(int32_t V, const int32_t* __restrict__ match,
                           const int32_t* __restrict__ repidx, int32_t* cid, uint8_t* pr)
 {
+    after_previous();
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
         int32_t m = match[n];
@@ -71,6 +72,7 @@ __global__ void k_next_state(Level S, const int32_t* __restrict__ map,
                              const int32_t* __restrict__ cov, const int32_t* __restrict__ dropped,
                              Level N)
 {
+    after_previous();
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < S.V;
          n += (int64_t)gridDim.x * blockDim.x) {
         int32_t m = match[n];
@@ -93,6 +95,7 @@ __global__ void k_next_state(Level S, const int32_t* __restrict__ map,
 // member sums per coarse vertex
 __global__ void k_sum_state(Level S, const int32_t* __restrict__ map, NextState ns)
 {
+    after_previous();
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < S.V;
          n += (int64_t)gridDim.x * blockDim.x) {
         int32_t u = map[n];
@@ -106,6 +109,7 @@ __global__ void k_sum_state(Level S, const int32_t* __restrict__ map, NextState 
 // hold the internal counts on entry)
 __global__ void k_in_count(Level N)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -119,6 +123,7 @@ __global__ void k_in_count(Level N)
 
 __global__ void k_compose(int64_t n, int32_t* c, const int32_t* __restrict__ next)
 {
+    after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
         c[i] = next[c[i]];
@@ -218,6 +223,7 @@ __global__ void k_dedup_keys(int32_t E, const int32_t* __restrict__ tlen,
                              const uint64_t* __restrict__ thash, uint64_t dropped_hi,
                              uint64_t* keys, uint32_t* vals)
 {
+    after_previous();
     for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < E;
          a += (int64_t)gridDim.x * blockDim.x) {
         uint64_t hi = tlen[a] > 0 ? (uint64_t)(uint32_t)tpins[hoff[a]] : dropped_hi;
@@ -229,6 +235,7 @@ __global__ void k_dedup_keys(int32_t E, const int32_t* __restrict__ tlen,
 
 __global__ void k_run_heads(int32_t E, const uint64_t* __restrict__ keys, int32_t* headpos)
 {
+    after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < E;
          i += (int64_t)gridDim.x * blockDim.x)
         headpos[i] = (i == 0 || keys[i] != keys[i - 1]) ? (int32_t)i : 0;
@@ -274,6 +281,7 @@ __global__ void k_dedup_insert(int32_t E, const int32_t* __restrict__ tlen,
                                const int32_t* __restrict__ hk, int64_t* tw, int32_t* tk,
                                DedupTable t, int round)
 {
+    after_previous();
     for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < E;
          a += (int64_t)gridDim.x * blockDim.x) {
         if (round > 0 && t.rep[a] != REP_PENDING) continue;
@@ -305,6 +313,7 @@ __global__ void __launch_bounds__(256)
                     const int64_t* __restrict__ hw, const int32_t* __restrict__ hk, int64_t* tw,
                     int32_t* tk, DedupTable t, int round, int64_t* scal)
 {
+    after_previous();
     SegTally tally;
     int pending = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < E;
@@ -360,6 +369,7 @@ __global__ void k_dedup_rep(int32_t E, const uint64_t* __restrict__ keys,
                             const int32_t* __restrict__ tlen, const uint8_t* __restrict__ tsd,
                             int32_t* rep, int32_t* head)
 {
+    after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < E;
          i += (int64_t)gridDim.x * blockDim.x) {
         int32_t a = (int32_t)vals[i];
@@ -381,6 +391,7 @@ __global__ void k_dedup_accum(int32_t E, const uint32_t* __restrict__ vals,
                               const int32_t* __restrict__ hk, int64_t* tw, int32_t* tk,
                               int64_t* newlen, int32_t* gid)
 {
+    after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < E;
          i += (int64_t)gridDim.x * blockDim.x) {
         int32_t r = rep[i];
@@ -406,6 +417,7 @@ __global__ void k_dedup_emit(int32_t E, const uint32_t* __restrict__ vals,
                              const int64_t* __restrict__ tw, const int32_t* __restrict__ tk,
                              const int64_t* __restrict__ newoff, Level N)
 {
+    after_previous();
     int lane = threadIdx.x & (G - 1);
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -434,6 +446,7 @@ __global__ void k_level_emit(int32_t E, const int32_t* __restrict__ rep,
                              const int32_t* __restrict__ tk, const int64_t* __restrict__ newoff,
                              Level N)
 {
+    after_previous();
     int lane = threadIdx.x & (G - 1);
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -453,7 +466,11 @@ __global__ void k_level_emit(int32_t E, const int32_t* __restrict__ rep,
     }
 }
 
-__global__ void k_set_off_end(int64_t* hoff, int32_t E, int64_t P) { hoff[E] = P; }
+__global__ void k_set_off_end(int64_t* hoff, int32_t E, int64_t P)
+{
+    after_previous();
+    hoff[E] = P;
+}
 
 // Materializes levels[dst] from the resident levels[src] through `map`
 // (int32[V(src)] into the new level's ids). The new level's vertex count is
@@ -507,10 +524,10 @@ Status build_coarse(snnmap_hgraph* h, int32_t src, const int32_t* map, int32_t V
     int ge = grid_for(E, 256);
     for (int round = 0;; round++) {
         if (E > 0) {
-            SNN_L k_dedup_insert<<<ge, 256, 0, s>>>(E, tlen, L.hoff, tpins, thash, L.hw, L.hk, tw, tk,
-                                                    dt, round);
-            SNN_L k_dedup_resolve<<<grid_for(E, 256, 152 * 8), 256, 0, s>>>(E, tlen, L.hoff, tpins, tsd, L.hw, L.hk, tw, tk, dt,
-                                                     round, h->d_scal);
+            enqueue(k_dedup_insert, ge, 256, 0, s, E, tlen, L.hoff, tpins, thash, L.hw, L.hk, tw, tk,
+                    dt, round);
+            enqueue(k_dedup_resolve, grid_for(E, 256, 152 * 8), 256, 0, s, E, tlen, L.hoff, tpins, tsd,
+                    L.hw, L.hk, tw, tk, dt, round, h->d_scal);
             SNN_CUDA(cudaGetLastError());
         }
         SNN_TRY(scan_run<Sum2>(RepSizes{dt.rep, tlen}, RepPlaces{gid, newoff}, E,
@@ -539,13 +556,14 @@ Status build_coarse(snnmap_hgraph* h, int32_t src, const int32_t* map, int32_t V
     for (int i = 0; i < SEG_NB; i++) NX.seg.n[i] = (int32_t)h->h_scal[SC_SEG + i];
     prof.reset(new ProfScope(h, PS_CONTRACT));
     if (match && V > 0) {
-        SNN_L k_next_state<<<grid_for(V, 256), 256, 0, s>>>(L, map, match, cand, cov, dropped, N);
+        enqueue(k_next_state, grid_for(V, 256), 256, 0, s, L, map, match, cand, cov, dropped, N);
         SNN_CUDA(cudaGetLastError());
     } else if (V2 > 0) {
         SNN_CUDA(cudaMemsetAsync(N.vsize, 0, (size_t)V2 * 4, s));
         SNN_CUDA(cudaMemsetAsync(N.vinpins, 0, (size_t)V2 * 4, s));
         SNN_CUDA(cudaMemcpyAsync(N.vinint, dropped, (size_t)V2 * 4, cudaMemcpyDeviceToDevice, s));
-        SNN_L k_sum_state<<<grid_for(V, 256), 256, 0, s>>>(L, map, NextState{N.vsize, N.vinpins, N.vinint});
+        enqueue(k_sum_state, grid_for(V, 256), 256, 0, s, L, map, NextState{N.vsize, N.vinpins,
+                N.vinint});
         SNN_CUDA(cudaGetLastError());
         SNN_CUDA(cudaMemcpyAsync(N.vincnt, N.vinint, (size_t)V2 * 4, cudaMemcpyDeviceToDevice, s));
     }
@@ -554,7 +572,7 @@ Status build_coarse(snnmap_hgraph* h, int32_t src, const int32_t* map, int32_t V
                      tw, tk, newoff, N);
     SNN_CUDA(cudaGetLastError());
     if (E2 > 0 && !match) {
-        SNN_L k_in_count<<<grid_for((int64_t)E2 * 32, 256), 256, 0, s>>>(N);
+        enqueue(k_in_count, grid_for((int64_t)E2 * 32, 256), 256, 0, s, N);
         SNN_CUDA(cudaGetLastError());
     }
     SNN_TRY(seg_lists(N.hoff, E2, N.maxlen, NX.seg, cursor, s));
@@ -579,7 +597,7 @@ Status contract_level(snnmap_hgraph* h)
         ProfScope prof(h, PS_CONTRACT);
         SNN_TRY(scan_run<int32_t>(RepFlag{h->match}, ScanStore<int32_t, false>{repidx}, V,
                                   (int32_t*)(h->d_scal + SC_A), ar, s));
-        SNN_L k_cid_map<<<grid_for(V, 256), 256, 0, s>>>(V, h->match, repidx, L.cid, L.pr);
+        enqueue(k_cid_map, grid_for(V, 256), 256, 0, s, V, h->match, repidx, L.cid, L.pr);
         SNN_CUDA(cudaGetLastError());
     }
     h->levels.emplace_back();
@@ -603,6 +621,7 @@ Status contract_level(snnmap_hgraph* h)
 __global__ void k_gp_internal(int32_t E, const int32_t* __restrict__ tlen,
                               const int64_t* __restrict__ hw, int64_t* out)
 {
+    after_previous();
     int64_t w = 0;
     for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < E;
          a += (int64_t)gridDim.x * blockDim.x)
@@ -659,16 +678,17 @@ Status emit_gp(snnmap_hgraph* h, int32_t K, const int32_t* rho)
     SNN_TRY(ar.alloc(&newoff, E));
     int ge = grid_for(E, 256);
     if (E > 0) {
-        SNN_L k_gp_internal<<<ge, 256, 0, s>>>(E, tlen, L.hw, h->d_scal + SC_D);
-        SNN_L k_dedup_keys<<<ge, 256, 0, s>>>(E, tlen, L.hoff, tpins, thash, (uint64_t)K, keys, vals);
+        enqueue(k_gp_internal, ge, 256, 0, s, E, tlen, L.hw, h->d_scal + SC_D);
+        enqueue(k_dedup_keys, ge, 256, 0, s, E, tlen, L.hoff, tpins, thash, (uint64_t)K, keys, vals);
         SNN_CUDA(cudaGetLastError());
         SNN_TRY(radix_sort_pairs(keys, vals, keys2, vals2, E, 32 + bits_for((uint64_t)K), ar, s));
-        SNN_L k_run_heads<<<ge, 256, 0, s>>>(E, keys, headpos);
+        enqueue(k_run_heads, ge, 256, 0, s, E, keys, headpos);
         SNN_CUDA(cudaGetLastError());
     }
     SNN_TRY(scan_inclusive_max_i32(headpos, runstart, E, ar, s));
     if (E > 0) {
-        SNN_L k_dedup_rep<<<ge, 256, 0, s>>>(E, keys, vals, runstart, L.hoff, tpins, tlen, tsd, rep, head);
+        enqueue(k_dedup_rep, ge, 256, 0, s, E, keys, vals, runstart, L.hoff, tpins, tlen, tsd, rep,
+                head);
         SNN_CUDA(cudaGetLastError());
     }
     SNN_TRY(scan_exclusive_i32(head, gidh, E, (int32_t*)(h->d_scal + SC_B), ar, s));
@@ -676,7 +696,7 @@ Status emit_gp(snnmap_hgraph* h, int32_t K, const int32_t* rho)
         SNN_CUDA(cudaMemsetAsync(tw, 0, (size_t)E * sizeof(int64_t), s));
         SNN_CUDA(cudaMemsetAsync(tk, 0, (size_t)E * sizeof(int32_t), s));
         SNN_CUDA(cudaMemsetAsync(newlen, 0, (size_t)E * sizeof(int64_t), s));
-        SNN_L k_dedup_accum<<<ge, 256, 0, s>>>(E, vals, rep, gidh, tlen, L.hw, L.hk, tw, tk, newlen, gid);
+        enqueue(k_dedup_accum, ge, 256, 0, s, E, vals, rep, gidh, tlen, L.hw, L.hk, tw, tk, newlen, gid);
         SNN_CUDA(cudaGetLastError());
     }
     SNN_TRY(scan_exclusive_i64(newlen, newoff, E, h->d_scal + SC_C, ar, s));
@@ -704,7 +724,7 @@ Status emit_gp(snnmap_hgraph* h, int32_t K, const int32_t* rho)
                          tlen, tsd, tw, tk, newoff, N);
         SNN_CUDA(cudaGetLastError());
     }
-    SNN_L k_set_off_end<<<1, 1, 0, s>>>(G.hoff, E2, P2);
+    enqueue(k_set_off_end, 1, 1, 0, s, G.hoff, E2, P2);
     SNN_CUDA(cudaGetLastError());
     SNN_CUDA(cudaStreamSynchronize(s));
     ar.reset();
@@ -746,7 +766,7 @@ Status ensure_resident(snnmap_hgraph* h, int32_t l)
     if (S.V > 0)
         SNN_CUDA(cudaMemcpyAsync(c, S.cid, (size_t)S.V * 4, cudaMemcpyDeviceToDevice, s));
     for (int32_t m = j + 1; m < l; m++) {
-        SNN_L k_compose<<<grid_for(S.V, 256), 256, 0, s>>>(S.V, c, h->levels[m].cid);
+        enqueue(k_compose, grid_for(S.V, 256), 256, 0, s, S.V, c, h->levels[m].cid);
         SNN_CUDA(cudaGetLastError());
     }
     SNN_TRY(zero_scalars(h));

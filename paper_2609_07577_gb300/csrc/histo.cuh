@@ -463,6 +463,7 @@ __host__ __device__ inline int64_t pow2_ceil(int64_t x)
 template <class Pol>
 __global__ void __launch_bounds__(256) k_ht_skip(Pol pol, int64_t* work, int32_t* todo, int64_t* ntodo)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     unsigned lt = lanemask_lt();
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < pol.V;
@@ -492,6 +493,7 @@ template <class Pol>
 __global__ void __launch_bounds__(256)
     k_ht_work(Pol pol, int64_t* work, const int32_t* __restrict__ todo, const int64_t* __restrict__ ntodo)
 {
+    after_previous();
     __shared__ unsigned long long part;
     int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t nt = *ntodo;
@@ -599,6 +601,7 @@ __global__ void __launch_bounds__(256)
     k_ht_classify(Pol pol, const int64_t* __restrict__ workv, int32_t* lists, int64_t* cnt,
                   int64_t* scap, HtTiers tiers, bool dense)
 {
+    after_previous();
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < pol.V;
          base += (int64_t)gridDim.x * blockDim.x) {
         int64_t n = base + threadIdx.x;
@@ -619,6 +622,7 @@ __global__ void __launch_bounds__(256)
     k_ht_plan(Pol pol, int64_t* workv, int32_t* lists, int64_t* cnt, int64_t* scap, HtTiers tiers,
               bool dense)
 {
+    after_previous();
     __shared__ int64_t work[32];
     __shared__ unsigned smask;
     __shared__ unsigned long long part;
@@ -673,6 +677,7 @@ __global__ void __launch_bounds__(HT_WARPS * 32)
     k_ht_warp(Pol pol, int32_t* lists, int64_t* cnt, const int64_t* __restrict__ workv,
               int64_t* scap)
 {
+    after_previous();
     using S = typename Pol::S;
     using Acc = typename Pol::Acc;
     extern __shared__ __align__(16) unsigned char ht_dyn[];
@@ -756,6 +761,7 @@ __global__ void __launch_bounds__(T, CAP <= 2048 ? HT_BLOCKS : 1)
     k_ht_block(Pol pol, int32_t* lists, int64_t* cnt, int64_t* scap, const int64_t* __restrict__ workv,
                int64_t leave)
 {
+    after_previous();
     using S = typename Pol::S;
     using Acc = typename Pol::Acc;
     extern __shared__ __align__(16) unsigned char ht_dyn[];
@@ -1071,6 +1077,7 @@ __global__ void __launch_bounds__(T)
     k_ht_dense(Pol pol, const int32_t* __restrict__ lists, int64_t* cnt, int32_t keys,
                const int64_t* __restrict__ workv)
 {
+    after_previous();
     using S = typename Pol::S;
     using Acc = typename Pol::Acc;
     extern __shared__ __align__(16) unsigned char ht_dyn[];
@@ -1119,6 +1126,7 @@ __global__ void __cluster_dims__(HT_DENSE_CTAS, 1, 1) __launch_bounds__(T)
     k_ht_dense_big(Pol pol, const int32_t* __restrict__ lists, int64_t* cnt, int32_t keys,
                    const int64_t* __restrict__ workv, int64_t leave)
 {
+    after_previous();
     namespace cg = cooperative_groups;
     using S = typename Pol::S;
     using Acc = typename Pol::Acc;
@@ -1239,6 +1247,7 @@ __global__ void k_ht_split_deg(Pol pol, const int32_t* __restrict__ slist, int64
                                const int64_t* __restrict__ workv, int64_t* total_work,
                                int64_t* scap, int64_t limit)
 {
+    after_previous();
     int64_t w = 0;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < ns;
          j += (int64_t)gridDim.x * blockDim.x) {
@@ -1258,6 +1267,7 @@ template <class Pol>
 __global__ void k_ht_split_len(Pol pol, const int32_t* __restrict__ slist, int64_t ns,
                                const int64_t* __restrict__ od, int64_t D, int64_t* len)
 {
+    after_previous();
     for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < D;
          f += (int64_t)gridDim.x * blockDim.x) {
         int64_t j = find_owner(od, ns, f);
@@ -1269,6 +1279,7 @@ static __global__ void k_ht_split_starts(int64_t ns, const int64_t* __restrict__
                                   const int64_t* __restrict__ x, const int64_t* __restrict__ len,
                                   int32_t* start, int64_t item)
 {
+    after_previous();
     for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < D;
          f += (int64_t)gridDim.x * blockDim.x) {
         int64_t j = find_owner(od, ns, f);
@@ -1286,6 +1297,7 @@ static __global__ void k_ht_split_starts(int64_t ns, const int64_t* __restrict__
 static __global__ void k_ht_split_items(int64_t D, const int32_t* __restrict__ start,
                                  const int32_t* __restrict__ pos, int64_t* item_f0)
 {
+    after_previous();
     for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < D;
          f += (int64_t)gridDim.x * blockDim.x)
         if (start[f]) item_f0[pos[f]] = f;
@@ -1323,6 +1335,7 @@ __global__ void __launch_bounds__(HT_WARPS * 32)
                      unsigned char* pool, typename Pol::Acc* gacc, int32_t* ovf, uint32_t probes,
                      const int64_t* __restrict__ workv)
 {
+    after_previous();
     using S = typename Pol::S;
     using Acc = typename Pol::Acc;
     extern __shared__ __align__(16) unsigned char ht_dyn[];
@@ -1368,6 +1381,7 @@ __global__ void __launch_bounds__(1024)
                     unsigned char* pool, const typename Pol::Acc* gacc,
                     const int32_t* __restrict__ ovf)
 {
+    after_previous();
     using S = typename Pol::S;
     __shared__ int64_t rs[32];
     __shared__ int32_t rk[32];
@@ -1406,6 +1420,7 @@ __global__ void __launch_bounds__(1024)
 static __global__ void k_ht_collect_ovf(const int32_t* __restrict__ slist, int64_t ns,
                                         const int32_t* __restrict__ ovf, int32_t* out, int64_t* cnt)
 {
+    after_previous();
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < ns;
          j += (int64_t)gridDim.x * blockDim.x)
         if (ovf[j]) out[atomicAdd((unsigned long long*)cnt, 1ull)] = slist[j];
@@ -1415,6 +1430,7 @@ template <typename S>
 __global__ void k_ht_pool_clear(unsigned char* pool, const int64_t* __restrict__ toff,
                                 const int64_t* __restrict__ scap, int64_t ns)
 {
+    after_previous();
     for (int64_t j = blockIdx.x; j < ns; j += gridDim.x) {
         Table<S> t = carve_table<S>(pool + toff[j] * slot_bytes<S>(), scap[j]);
         clear_slots(t, threadIdx.x, scap[j], blockDim.x);
@@ -1451,8 +1467,8 @@ Status run_split(const Pol& pol, Arena& ar, cudaStream_t s, const int32_t* sl, i
     SNN_TRY(ar.alloc(&ovf, ns));
     SNN_CUDA(cudaMemsetAsync(tot, 0, 4 * sizeof(int64_t), s));
     SNN_CUDA(cudaMemsetAsync(ovf, 0, (size_t)ns * sizeof(int32_t), s));
-    SNN_L k_ht_split_deg<Pol><<<grid_for(ns, 256), 256, 0, s>>>(pol, sl, ns, deg, workv, tot + 2, scap,
-                                                              limit);
+    enqueue(k_ht_split_deg<Pol>, grid_for(ns, 256), 256, 0, s, pol, sl, ns, deg, workv, tot + 2, scap,
+            limit);
     SNN_CUDA(cudaGetLastError());
     SNN_TRY(scan_exclusive_i64(scap, toff, ns, tot, ar, s));
     SNN_TRY(scan_exclusive_i64(deg, od, ns, od + ns, ar, s));
@@ -1470,13 +1486,13 @@ Status run_split(const Pol& pol, Arena& ar, cudaStream_t s, const int32_t* sl, i
     SNN_TRY(ar.alloc(&start, D));
     SNN_TRY(ar.alloc(&pos, D));
     SNN_TRY(ar.alloc(&item_f0, D));
-    SNN_L k_ht_split_len<Pol><<<grid_for(D, 256), 256, 0, s>>>(pol, sl, ns, od, D, len);
+    enqueue(k_ht_split_len<Pol>, grid_for(D, 256), 256, 0, s, pol, sl, ns, od, D, len);
     SNN_CUDA(cudaGetLastError());
     SNN_TRY(scan_exclusive_i64(len, x, D, nullptr, ar, s));
-    SNN_L k_ht_split_starts<<<grid_for(D, 256), 256, 0, s>>>(ns, od, D, x, len, start, item);
+    enqueue(k_ht_split_starts, grid_for(D, 256), 256, 0, s, ns, od, D, x, len, start, item);
     SNN_CUDA(cudaGetLastError());
     SNN_TRY(scan_exclusive_i32(start, pos, D, (int32_t*)(tot + 1), ar, s));
-    SNN_L k_ht_split_items<<<grid_for(D, 256), 256, 0, s>>>(D, start, pos, item_f0);
+    enqueue(k_ht_split_items, grid_for(D, 256), 256, 0, s, D, start, pos, item_f0);
     SNN_CUDA(cudaGetLastError());
     SNN_CUDA(cudaMemcpyAsync(h_cnt, tot + 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     SNN_CUDA(cudaStreamSynchronize(s));
@@ -1486,20 +1502,19 @@ Status run_split(const Pol& pol, Arena& ar, cudaStream_t s, const int32_t* sl, i
     SNN_TRY(ar.alloc(&pool, slots * (int64_t)slot_bytes<S>()));
     SNN_TRY(ar.alloc(&gacc, ns));
     SNN_CUDA(cudaMemsetAsync(gacc, 0, (size_t)ns * sizeof(typename Pol::Acc), s));
-    SNN_L k_ht_pool_clear<S><<<(int)std::min<int64_t>(ns, 152 * 8), 256, 0, s>>>(pool, toff, scap, ns);
+    enqueue(k_ht_pool_clear<S>, (int)std::min<int64_t>(ns, 152 * 8), 256, 0, s, pool, toff, scap, ns);
     SNN_CUDA(cudaGetLastError());
     size_t wsm = (size_t)HT_WARPS * HT_WCAP * slot_bytes<S>();
     SNN_TRY(set_smem(k_ht_split_visit<Pol>, wsm));
-    SNN_L k_ht_split_visit<Pol><<<(int)std::min<int64_t>(ceil_div(items, HT_WARPS), 152 * 8),
-                                  HT_WARPS * 32, wsm, s>>>(pol, sl, ns, od, D, item_f0, items, toff,
-                                                           scap, pool, gacc, ovf,
-                                                           limit > 0 ? 256u : 0u, workv);
+    enqueue(k_ht_split_visit<Pol>, (int)std::min<int64_t>(ceil_div(items, HT_WARPS), 152 * 8),
+            HT_WARPS * 32, wsm, s, pol, sl, ns, od, D, item_f0, items, toff, scap, pool, gacc, ovf,
+            limit > 0 ? 256u : 0u, workv);
     SNN_CUDA(cudaGetLastError());
-    SNN_L k_ht_split_scan<Pol><<<(int)std::min<int64_t>(ns, 152 * 4), 1024, 0, s>>>(pol, sl, ns, toff,
-                                                                                    scap, pool, gacc, ovf);
+    enqueue(k_ht_split_scan<Pol>, (int)std::min<int64_t>(ns, 152 * 4), 1024, 0, s, pol, sl, ns, toff,
+            scap, pool, gacc, ovf);
     SNN_CUDA(cudaGetLastError());
     if (limit > 0) {
-        SNN_L k_ht_collect_ovf<<<grid_for(ns, 256), 256, 0, s>>>(sl, ns, ovf, again, nagain);
+        enqueue(k_ht_collect_ovf, grid_for(ns, 256), 256, 0, s, sl, ns, ovf, again, nagain);
         SNN_CUDA(cudaGetLastError());
         SNN_CUDA(cudaMemcpyAsync(h_cnt, nagain, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
         SNN_CUDA(cudaStreamSynchronize(s));
@@ -1512,6 +1527,7 @@ template <class Pol>
 __global__ void k_ht_split_caps(Pol pol, const int32_t* __restrict__ slist, int64_t ns,
                                 const int64_t* __restrict__ workv, int64_t limit, int64_t* caps)
 {
+    after_previous();
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < ns;
          j += (int64_t)gridDim.x * blockDim.x) {
         int64_t work = workv[slist[j]];
@@ -1534,7 +1550,7 @@ Status split_cuts(const Pol& pol, Arena& ar, cudaStream_t s, const int32_t* sl, 
     int64_t *caps, *pre;
     SNN_TRY(ar.alloc(&caps, ns));
     SNN_TRY(ar.alloc(&pre, ns));
-    SNN_L k_ht_split_caps<Pol><<<grid_for(ns, 256), 256, 0, s>>>(pol, sl, ns, workv, limit, caps);
+    enqueue(k_ht_split_caps<Pol>, grid_for(ns, 256), 256, 0, s, pol, sl, ns, workv, limit, caps);
     SNN_CUDA(cudaGetLastError());
     SNN_TRY(scan_inclusive_i64(caps, pre, ns, ar, s));
     std::vector<int64_t> hp((size_t)ns);
@@ -1579,17 +1595,17 @@ Status run_histogram(const Pol& pol, Arena& ar, cudaStream_t s, int64_t* d_cnt, 
     SNN_TRY(ar.alloc(&workv, V));
     SNN_CUDA(cudaMemsetAsync(d_cnt, 0, HT_NCNT * sizeof(int64_t), s));
     if (V <= HT_PLAN_V) {
-        SNN_L k_ht_plan<Pol><<<(int)ceil_div(V, 32), 256, 0, s>>>(pol, workv, lists, d_cnt, scap, tiers,
-                                                                  dense_big);
+        enqueue(k_ht_plan<Pol>, (int)ceil_div(V, 32), 256, 0, s, pol, workv, lists, d_cnt, scap, tiers,
+                dense_big);
     } else {
         int32_t* todo;
         int64_t* ntodo = d_cnt + HT_CNT_TODO;
         SNN_TRY(ar.alloc(&todo, V));
-        SNN_L k_ht_skip<Pol><<<grid_for(V, 256), 256, 0, s>>>(pol, workv, todo, ntodo);
-        SNN_L k_ht_work<Pol><<<grid_for(V, 8, 152 * 16), 256, 0, s>>>(pol, workv, todo, ntodo);
+        enqueue(k_ht_skip<Pol>, grid_for(V, 256), 256, 0, s, pol, workv, todo, ntodo);
+        enqueue(k_ht_work<Pol>, grid_for(V, 8, 152 * 16), 256, 0, s, pol, workv, todo, ntodo);
         SNN_CUDA(cudaGetLastError());
-        SNN_L k_ht_classify<Pol><<<grid_for(V, 256), 256, 0, s>>>(pol, workv, lists, d_cnt, scap, tiers,
-                                                                  dense_big);
+        enqueue(k_ht_classify<Pol>, grid_for(V, 256), 256, 0, s, pol, workv, lists, d_cnt, scap, tiers,
+                dense_big);
     }
     SNN_CUDA(cudaGetLastError());
     size_t wsm = (size_t)HT_WARPS * HT_WCAP * slot_bytes<S>();
@@ -1600,34 +1616,34 @@ Status run_histogram(const Pol& pol, Arena& ar, cudaStream_t s, int64_t* d_cnt, 
     // set on every call: the attribute is per device, and handles on other
     // host threads may reach this point concurrently
     SNN_TRY(set_smem(k_ht_warp<Pol>, wsm));
-    SNN_L k_ht_warp<Pol><<<(int)std::min<int64_t>(ceil_div(V, HT_WARPS), 152 * 8), HT_WARPS * 32, wsm,
-                           s>>>(pol, lists, d_cnt, workv, scap);
+    enqueue(k_ht_warp<Pol>, (int)std::min<int64_t>(ceil_div(V, HT_WARPS), 152 * 8), HT_WARPS * 32, wsm,
+            s, pol, lists, d_cnt, workv, scap);
     SNN_CUDA(cudaGetLastError());
     const size_t dsm = (size_t)key_space * (sizeof(S) + sizeof(uint32_t));
     if constexpr (sizeof(S) == 4) {
         if (dense_block) {
             auto kd = k_ht_dense<Pol, HT_BTHREADS, HT_TIER_BLOCK>;
-            SNN_L kd<<<(int)std::min<int64_t>(V, 152 * 6), HT_BTHREADS, dsm, s>>>(pol, lists, d_cnt,
-                                                                                  key_space, workv);
+            enqueue(kd, (int)std::min<int64_t>(V, 152 * 6), HT_BTHREADS, dsm, s, pol, lists, d_cnt,
+                    key_space, workv);
         }
         if (dense_big) {
             auto kd = k_ht_dense_big<Pol, 1024>;
             const int64_t leave = dense_block ? 0 : HT_LEAVE;
             if (!dense_block) {
                 SNN_TRY(set_smem(kb, bsm));
-                SNN_L kb<<<(int)std::min<int64_t>(V, 152 * 8), HT_BTHREADS, bsm, s>>>(pol, lists, d_cnt,
-                                                                                      scap, workv, leave);
+                enqueue(kb, (int)std::min<int64_t>(V, 152 * 8), HT_BTHREADS, bsm, s, pol, lists, d_cnt,
+                        scap, workv, leave);
             }
             SNN_TRY(set_smem(kd, (size_t)HT_DENSE_KEYS * 8));
-            SNN_L kd<<<19 * HT_DENSE_CTAS, 1024, dsm, s>>>(pol, lists, d_cnt, key_space, workv, leave);
+            enqueue(kd, 19 * HT_DENSE_CTAS, 1024, dsm, s, pol, lists, d_cnt, key_space, workv, leave);
         }
     }
     if (!dense_big) {
         SNN_TRY(set_smem(kb, bsm));
-        SNN_L kb<<<(int)std::min<int64_t>(V, 152 * 8), HT_BTHREADS, bsm, s>>>(pol, lists, d_cnt, scap,
-                                                                              workv, 0);
+        enqueue(kb, (int)std::min<int64_t>(V, 152 * 8), HT_BTHREADS, bsm, s, pol, lists, d_cnt, scap,
+                workv, 0);
         SNN_TRY(set_smem(kg, gsm));
-        SNN_L kg<<<152, HT_GTHREADS, gsm, s>>>(pol, lists, d_cnt, scap, workv, 0);
+        enqueue(kg, 152, HT_GTHREADS, gsm, s, pol, lists, d_cnt, scap, workv, 0);
     }
     SNN_CUDA(cudaGetLastError());
     if (!split) return Status{};

@@ -42,6 +42,7 @@ __global__ void k_ip_distinct(int64_t P, const int64_t* __restrict__ off,
                               const int32_t* __restrict__ pins, const int32_t* __restrict__ hid,
                               int32_t* err)
 {
+    snn::after_previous();
     int bad = 0;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P;
          j += (int64_t)gridDim.x * blockDim.x) {
@@ -58,6 +59,7 @@ __global__ void k_ip_distinct(int64_t P, const int64_t* __restrict__ off,
 __global__ void k_ip_seq(int32_t np, const int32_t* __restrict__ seq0, int32_t* seq, int32_t* pos,
                          int32_t* err)
 {
+    snn::after_previous();
     int64_t s = blockIdx.y;
     int bad = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np;
@@ -74,6 +76,7 @@ __global__ void k_ip_seq(int32_t np, const int32_t* __restrict__ seq0, int32_t* 
 __global__ void k_ip_jobof(int32_t J, const int32_t* __restrict__ jlo, const int32_t* __restrict__ jhi,
                            int32_t* jobof)
 {
+    snn::after_previous();
     for (int32_t k = blockIdx.x; k < J; k += gridDim.x)
         for (int32_t i = jlo[k] + threadIdx.x; i < jhi[k]; i += blockDim.x) jobof[i] = k;
 }
@@ -88,6 +91,7 @@ struct Jobs {
 __global__ void k_ip_reset(int32_t S, int32_t J, const int32_t* __restrict__ done, int64_t* bd,
                            unsigned long long* bxy, int32_t* active)
 {
+    snn::after_previous();
     if (blockIdx.x == 0 && threadIdx.x == 0) *active = 0;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < (int64_t)S * J;
          t += (int64_t)gridDim.x * blockDim.x) {
@@ -112,6 +116,7 @@ __global__ void __launch_bounds__(256)
                    const int64_t* __restrict__ eta, const int32_t* __restrict__ seq,
                    const int32_t* __restrict__ pos, int64_t* G, int64_t* M)
 {
+    snn::after_previous();
     __shared__ unsigned long long sh;
     int64_t s = blockIdx.y;
     const int32_t* ps = pos + s * np;
@@ -168,6 +173,7 @@ __global__ void k_ip_best(int32_t np, int64_t pairs, Jobs jb, const int32_t* __r
                           const int32_t* __restrict__ seq, const int64_t* __restrict__ G,
                           const int64_t* __restrict__ M, int64_t* bd, unsigned long long* bxy)
 {
+    snn::after_previous();
     int64_t s = blockIdx.y;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < pairs;
          p += (int64_t)gridDim.x * blockDim.x) {
@@ -231,6 +237,7 @@ __global__ void k_ip_update(int32_t np, int64_t pairs, Jobs jb, int32_t* done, i
                             const int32_t* __restrict__ pins, const int64_t* __restrict__ eta,
                             int32_t* seq, int32_t* pos, int64_t* G, int64_t* M, int32_t* active)
 {
+    snn::after_previous();
     __shared__ int s_mode;   // 0 skip, 1 swap then stop, 2 swap and go on
     const int64_t s = blockIdx.y;
     const int32_t k = blockIdx.x;
@@ -307,6 +314,7 @@ __global__ void k_ip_conn(int64_t P, int32_t np, Tree T, const int32_t* __restri
                           const int64_t* __restrict__ eta, const int32_t* __restrict__ pos,
                           int64_t* conn)
 {
+    snn::after_previous();
     int64_t s = blockIdx.y;
     const int32_t* ps = pos + s * np;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P;
@@ -334,6 +342,7 @@ __global__ void k_ip_conn(int64_t P, int32_t np, Tree T, const int32_t* __restri
 // when its child more connected to the sibling does not face it
 __global__ void k_ip_flip(Tree T, const int64_t* __restrict__ conn, uint8_t* flip)
 {
+    snn::after_previous();
     int64_t s = blockIdx.y;
     for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < T.nn; v += gridDim.x * blockDim.x) {
         uint8_t f = 0;
@@ -350,6 +359,7 @@ __global__ void k_ip_flip(Tree T, const int64_t* __restrict__ conn, uint8_t* fli
 __global__ void k_ip_fold(int32_t np, Tree T, const uint8_t* __restrict__ flip,
                           const int32_t* __restrict__ seq, int32_t* seq_out)
 {
+    snn::after_previous();
     int64_t s = blockIdx.y;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < np; i += gridDim.x * blockDim.x)
         seq_out[s * np + ip::folded_position(T.lo, T.hi, T.kid, flip + s * T.nn, i)] =
@@ -358,6 +368,7 @@ __global__ void k_ip_fold(int32_t np, Tree T, const uint8_t* __restrict__ flip,
 
 __global__ void k_ip_hkeys(int32_t width, int32_t nh, uint32_t n2, uint64_t* keys, uint32_t* vals)
 {
+    snn::after_previous();
     for (int32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < nh; h += gridDim.x * blockDim.x) {
         keys[h] = ip::hilbert_index(n2, (uint32_t)(h % width), (uint32_t)(h / width));
         vals[h] = (uint32_t)h;
@@ -367,6 +378,7 @@ __global__ void k_ip_hkeys(int32_t width, int32_t nh, uint32_t n2, uint64_t* key
 __global__ void k_ip_gamma(int32_t np, const int32_t* __restrict__ seq_out,
                            const uint32_t* __restrict__ order, int32_t* gamma)
 {
+    snn::after_previous();
     int64_t s = blockIdx.y;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < np; i += gridDim.x * blockDim.x)
         gamma[s * np + seq_out[s * np + i]] = (int32_t)order[i];
@@ -391,7 +403,7 @@ Status hilbert_order(int32_t width, int32_t height, uint32_t* order, Arena& ar, 
     SNN_TRY(ar.alloc(&keys, nh));
     SNN_TRY(ar.alloc(&keys2, nh));
     SNN_TRY(ar.alloc(&vals2, nh));
-    SNN_L k_ip_hkeys<<<grid_for(nh, 256), 256, 0, s>>>(width, nh, n2, keys, order);
+    snn::enqueue(k_ip_hkeys, grid_for(nh, 256), 256, 0, s, width, nh, n2, keys, order);
     SNN_CUDA(cudaGetLastError());
     SNN_TRY(radix_sort_pairs(keys, order, keys2, vals2, nh, bits_for((uint64_t)n2 * n2 - 1), ar, s));
     return Status{};
@@ -466,14 +478,14 @@ Status initial_impl(int32_t np, int32_t ne, const int64_t* off, const int32_t* p
     SNN_TRY(ar.alloc(&pos, (int64_t)S * np));
     SNN_CUDA(cudaMemsetAsync(err, 0, sizeof(int32_t), s));
     SNN_TRY(fill_i32(pos, -1, (int64_t)S * np, s));
-    SNN_L k_ip_seq<<<grid2(np, S), 256, 0, s>>>(np, seq0, seq, pos, err);
+    snn::enqueue(k_ip_seq, grid2(np, S), 256, 0, s, np, seq0, seq, pos, err);
     SNN_CUDA(cudaGetLastError());
     int32_t herr = 0;
     SNN_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     SNN_CUDA(cudaStreamSynchronize(s));
     if (herr) return invalid("an initial order that is not a permutation of the nodes");
     if (P > 0) {
-        SNN_L k_ip_distinct<<<grid_for(P, 256), 256, 0, s>>>(P, off, pins, hid, err);
+        snn::enqueue(k_ip_distinct, grid_for(P, 256), 256, 0, s, P, off, pins, hid, err);
         SNN_CUDA(cudaGetLastError());
     }
     SNN_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
@@ -561,7 +573,7 @@ Status initial_impl(int32_t np, int32_t ne, const int64_t* off, const int32_t* p
         jb.pairoff = jpo;
         jb.jobof = jobof;
         SNN_TRY(fill_i32(jobof, -1, np, s));
-        SNN_L k_ip_jobof<<<grid_for(J, 1, 152 * 8), 128, 0, s>>>(J, jlo, jhi, jobof);
+        snn::enqueue(k_ip_jobof, grid_for(J, 1, 152 * 8), 128, 0, s, J, jlo, jhi, jobof);
         SNN_CUDA(cudaMemsetAsync(done, 0, sizeof(int32_t) * S * J, s));
         SNN_CUDA(cudaMemsetAsync(it, 0, sizeof(int32_t) * S * J, s));
         SNN_CUDA(cudaGetLastError());
@@ -569,15 +581,16 @@ Status initial_impl(int32_t np, int32_t ne, const int64_t* off, const int32_t* p
         const int gjob = grid_for((int64_t)S * J, 256);
         SNN_CUDA(cudaMemsetAsync(M, 0, sizeof(int64_t) * S * pairs, s));
         auto gc = warps ? k_ip_gain_corr<32> : k_ip_gain_corr<256>;
-        SNN_L gc<<<gnode, 256, 0, s>>>(np, pairs, jb, done, voff, vinc, off, pins, eta, seq, pos, G, M);
+        snn::enqueue(gc, gnode, 256, 0, s, np, pairs, jb, done, voff, vinc, off, pins, eta, seq, pos,
+                     G, M);
         SNN_CUDA(cudaGetLastError());
         const dim3 gupd((unsigned)J, (unsigned)S);
         for (;;) {
-            SNN_L k_ip_reset<<<gjob, 256, 0, s>>>(S, J, done, bd, bxy, active);
-            SNN_L k_ip_best<0><<<gpair, 256, 0, s>>>(np, pairs, jb, done, seq, G, M, bd, bxy);
-            SNN_L k_ip_best<1><<<gpair, 256, 0, s>>>(np, pairs, jb, done, seq, G, M, bd, bxy);
-            SNN_L k_ip_update<<<gupd, updt, 0, s>>>(np, pairs, jb, done, it, bd, bxy, voff, vinc, off,
-                                                    pins, eta, seq, pos, G, M, active);
+            snn::enqueue(k_ip_reset, gjob, 256, 0, s, S, J, done, bd, bxy, active);
+            snn::enqueue(k_ip_best<0>, gpair, 256, 0, s, np, pairs, jb, done, seq, G, M, bd, bxy);
+            snn::enqueue(k_ip_best<1>, gpair, 256, 0, s, np, pairs, jb, done, seq, G, M, bd, bxy);
+            snn::enqueue(k_ip_update, gupd, updt, 0, s, np, pairs, jb, done, it, bd, bxy, voff, vinc,
+                         off, pins, eta, seq, pos, G, M, active);
             SNN_CUDA(cudaGetLastError());
             int32_t hact = 0;
             SNN_CUDA(cudaMemcpyAsync(&hact, active, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
@@ -596,14 +609,14 @@ Status initial_impl(int32_t np, int32_t ne, const int64_t* off, const int32_t* p
     SNN_TRY(ar.alloc(&order, nh));
     SNN_CUDA(cudaMemsetAsync(conn, 0, sizeof(int64_t) * S * T.nn, s));
     if (P > 0) {
-        SNN_L k_ip_conn<<<grid2(P, S), 256, 0, s>>>(P, np, T, hid, off, pins, eta, pos, conn);
+        snn::enqueue(k_ip_conn, grid2(P, S), 256, 0, s, P, np, T, hid, off, pins, eta, pos, conn);
     }
-    SNN_L k_ip_flip<<<grid2(T.nn, S), 256, 0, s>>>(T, conn, flip);
+    snn::enqueue(k_ip_flip, grid2(T.nn, S), 256, 0, s, T, conn, flip);
     int32_t* seq_out = seq_out_user ? seq_out_user : seq2;
-    SNN_L k_ip_fold<<<gpos, 256, 0, s>>>(np, T, flip, seq, seq_out);
+    snn::enqueue(k_ip_fold, gpos, 256, 0, s, np, T, flip, seq, seq_out);
     SNN_CUDA(cudaGetLastError());
     SNN_TRY(hilbert_order(width, height, order, ar, s));
-    SNN_L k_ip_gamma<<<gpos, 256, 0, s>>>(np, seq_out, order, gamma);
+    snn::enqueue(k_ip_gamma, gpos, 256, 0, s, np, seq_out, order, gamma);
     SNN_CUDA(cudaGetLastError());
     SNN_CUDA(cudaStreamSynchronize(s));
     return Status{};

@@ -38,6 +38,7 @@ namespace {
 __global__ void k_gp_check(int32_t ne, int64_t P, int32_t np, const int64_t* __restrict__ off,
                            const int32_t* __restrict__ pins, int32_t* err)
 {
+    snn::after_previous();
     int bad = 0;
     int64_t n = (int64_t)ne > P ? (int64_t)ne : P;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -51,6 +52,7 @@ __global__ void k_gp_check(int32_t ne, int64_t P, int32_t np, const int64_t* __r
 // hyperedge of every pin entry (offsets already checked)
 __global__ void k_gp_hid(int32_t ne, const int64_t* __restrict__ off, int32_t* hid)
 {
+    snn::after_previous();
     for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < ne;
          a += (int64_t)gridDim.x * blockDim.x)
         for (int64_t j = off[a]; j < off[a + 1]; j++) hid[j] = (int32_t)a;
@@ -89,7 +91,7 @@ Status gp_input(int32_t np, int32_t ne, const int64_t* off, const int32_t* pins,
     SNN_TRY(ar.alloc(&hid, P));
     SNN_CUDA(cudaMemsetAsync(err, 0, sizeof(int32_t), s));
     if (ne > 0 || P > 0) {
-        SNN_L k_gp_check<<<grid_for(ne > P ? ne : P, 256), 256, 0, s>>>(ne, P, np, off, pins, err);
+        snn::enqueue(k_gp_check, grid_for(ne > P ? ne : P, 256), 256, 0, s, ne, P, np, off, pins, err);
         SNN_CUDA(cudaGetLastError());
     }
     int32_t herr = 0;
@@ -97,7 +99,7 @@ Status gp_input(int32_t np, int32_t ne, const int64_t* off, const int32_t* pins,
     SNN_CUDA(cudaStreamSynchronize(s));
     if (herr) return Status{SNNMAP_ERR_INVALID, "malformed offsets or a pin out of range"};
     if (ne > 0) {
-        SNN_L k_gp_hid<<<grid_for(ne, 256), 256, 0, s>>>(ne, off, hid);
+        snn::enqueue(k_gp_hid, grid_for(ne, 256), 256, 0, s, ne, off, hid);
         SNN_CUDA(cudaGetLastError());
     }
     *P_out = P;
@@ -108,6 +110,7 @@ Status gp_input(int32_t np, int32_t ne, const int64_t* off, const int32_t* pins,
 // incidence lists of G_P's nodes, one entry per pin entry
 __global__ void k_gp_degree(int64_t P, const int32_t* __restrict__ pins, int32_t* deg)
 {
+    snn::after_previous();
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P;
          j += (int64_t)gridDim.x * blockDim.x)
         atomicAdd(&deg[pins[j]], 1);
@@ -117,6 +120,7 @@ __global__ void k_gp_fill(int64_t P, const int32_t* __restrict__ pins,
                           const int32_t* __restrict__ hid, const int64_t* __restrict__ voff,
                           int32_t* cursor, int32_t* vinc)
 {
+    snn::after_previous();
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P;
          j += (int64_t)gridDim.x * blockDim.x) {
         int32_t q = pins[j];
@@ -133,12 +137,12 @@ Status gp_incidence(int32_t np, int64_t P, const int32_t* pins, const int32_t* h
     SNN_TRY(ar.alloc(vinc, P));
     if (np > 0) SNN_CUDA(cudaMemsetAsync(deg, 0, 2 * sizeof(int32_t) * (size_t)np, s));
     if (P > 0) {
-        SNN_L k_gp_degree<<<grid_for(P, 256), 256, 0, s>>>(P, pins, deg);
+        snn::enqueue(k_gp_degree, grid_for(P, 256), 256, 0, s, P, pins, deg);
         SNN_CUDA(cudaGetLastError());
     }
     SNN_TRY(scan_exclusive_i32_to_i64(deg, *voff, np, *voff + np, ar, s));
     if (P > 0) {
-        SNN_L k_gp_fill<<<grid_for(P, 256), 256, 0, s>>>(P, pins, hid, *voff, deg + np, *vinc);
+        snn::enqueue(k_gp_fill, grid_for(P, 256), 256, 0, s, P, pins, hid, *voff, deg + np, *vinc);
         SNN_CUDA(cudaGetLastError());
     }
     return Status{};
@@ -160,6 +164,7 @@ constexpr int kMaxStarts = 65535;   // gridDim.y
 __global__ void k_pl_occupy(int32_t np, int32_t nh, const int32_t* __restrict__ g, int32_t* pi,
                             int32_t* err)
 {
+    snn::after_previous();
     int64_t s = blockIdx.y;
     int bad = 0;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < np;
@@ -173,6 +178,7 @@ __global__ void k_pl_occupy(int32_t np, int32_t nh, const int32_t* __restrict__ 
 
 __global__ void k_pl_init_stats(int32_t S, int64_t* st)
 {
+    snn::after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (int64_t)PS_N * S;
          i += (int64_t)gridDim.x * blockDim.x)
         st[i] = i >= (int64_t)PS_FIRST * S ? INT64_MAX : 0;
@@ -181,6 +187,7 @@ __global__ void k_pl_init_stats(int32_t S, int64_t* st)
 // lattice coordinates of every start's nodes
 __global__ void k_pl_xy(int64_t n, int32_t width, const int32_t* __restrict__ g, int2* xy)
 {
+    snn::after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
         xy[i] = make_int2(g[i] % width, g[i] / width);
@@ -219,6 +226,7 @@ __global__ void __launch_bounds__(256)
                const int32_t* __restrict__ pins, const int64_t* __restrict__ eta,
                const int2* __restrict__ xy, const int32_t* __restrict__ act, int64_t* F)
 {
+    snn::after_previous();
     __shared__ unsigned long long sh;
     int64_t s = blockIdx.y;
     if (!act[s]) return;
@@ -262,6 +270,7 @@ __global__ void k_pl_propose(int32_t nh, int32_t np, int32_t width, int32_t heig
                              const int64_t* __restrict__ F, int32_t* cand, int64_t* cscore,
                              int64_t* st_props)
 {
+    snn::after_previous();
     int64_t s = blockIdx.y;
     bool on = act[s] != 0;
     int c = 0;
@@ -283,6 +292,7 @@ __global__ void k_pl_propose(int32_t nh, int32_t np, int32_t width, int32_t heig
 __global__ void k_pl_flag(int32_t nh, const int32_t* __restrict__ match, int32_t* flag,
                           int64_t* st_swaps)
 {
+    snn::after_previous();
     int64_t s = blockIdx.y;
     int c = 0;
     for (int64_t h = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; h < nh;
@@ -302,6 +312,7 @@ __global__ void k_pl_compact(int32_t nh, int32_t np, int32_t width, int32_t heig
                              const int32_t* __restrict__ pos, uint64_t* keys, uint32_t* vals,
                              int32_t* err)
 {
+    snn::after_previous();
     int64_t s = blockIdx.y;
     int bad = 0;
     for (int64_t h = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; h < nh;
@@ -323,6 +334,7 @@ __global__ void k_pl_compact(int32_t nh, int32_t np, int32_t width, int32_t heig
 __global__ void k_pl_startkey(int64_t ns, int32_t nh, const uint32_t* __restrict__ vals,
                               uint64_t* keys)
 {
+    snn::after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ns;
          i += (int64_t)gridDim.x * blockDim.x)
         keys[i] = vals[i] / (uint32_t)nh;
@@ -332,6 +344,7 @@ __global__ void k_pl_rank(int64_t ns, int32_t nh, const uint32_t* __restrict__ v
                           const int32_t* __restrict__ match, const int32_t* __restrict__ segbeg,
                           int32_t* rank, int32_t* mate)
 {
+    snn::after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ns;
          i += (int64_t)gridDim.x * blockDim.x) {
         int64_t x = vals[i];
@@ -357,6 +370,7 @@ __global__ void __launch_bounds__(256)
                 const int32_t* __restrict__ rank, const int32_t* __restrict__ mate,
                 const int32_t* __restrict__ segbeg, int64_t* Tn)
 {
+    snn::after_previous();
     __shared__ unsigned long long sh;
     int64_t s = blockIdx.y;
     const int32_t* gs = g + s * np;
@@ -398,6 +412,7 @@ __global__ void k_pl_best(int64_t ns, int32_t nh, const uint32_t* __restrict__ v
                           const int32_t* __restrict__ segbeg, const int64_t* __restrict__ C,
                           int64_t* st_best)
 {
+    snn::after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ns;
          i += (int64_t)gridDim.x * blockDim.x) {
         int64_t s = vals[i] / (uint32_t)nh;
@@ -410,6 +425,7 @@ __global__ void k_pl_first(int64_t ns, int32_t nh, const uint32_t* __restrict__ 
                            const int32_t* __restrict__ segbeg, const int64_t* __restrict__ C,
                            const int64_t* __restrict__ st_best, int64_t* st_first)
 {
+    snn::after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ns;
          i += (int64_t)gridDim.x * blockDim.x) {
         int64_t s = vals[i] / (uint32_t)nh;
@@ -423,6 +439,7 @@ __global__ void k_pl_apply(int64_t ns, int32_t nh, int32_t np, const uint32_t* _
                            const int32_t* __restrict__ match, const int32_t* __restrict__ segbeg,
                            const int64_t* __restrict__ st_first, int32_t* pi, int32_t* g)
 {
+    snn::after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ns;
          i += (int64_t)gridDim.x * blockDim.x) {
         int64_t x = vals[i];
@@ -443,6 +460,7 @@ __global__ void k_pl_trd(int64_t P, int32_t np, const int32_t* __restrict__ hid,
                          const int64_t* __restrict__ eta, const int2* __restrict__ xy,
                          int64_t* acc)
 {
+    snn::after_previous();
     int64_t s = blockIdx.y;
     const int2* xs = xy + s * np;
     int64_t sum = 0;
@@ -502,7 +520,7 @@ Status prepare(Input& in, const int32_t* g, Arena& ar, cudaStream_t s, int32_t**
     SNN_CUDA(cudaMemsetAsync(err, 0, sizeof(int32_t), s));
     SNN_TRY(fill_i32(pi, -1, in.nh * in.S, s));
     if (in.np > 0) {
-        SNN_L k_pl_occupy<<<grid2(in.np, in.S), 256, 0, s>>>(in.np, (int32_t)in.nh, g, pi, err);
+        snn::enqueue(k_pl_occupy, grid2(in.np, in.S), 256, 0, s, in.np, (int32_t)in.nh, g, pi, err);
         SNN_CUDA(cudaGetLastError());
     }
     int32_t herr = 0;
@@ -558,7 +576,7 @@ Status refine_impl(Input& in, int32_t* g, int32_t max_rounds, cudaStream_t s, in
         Arena::Mark mk = ar.mark();
         SNN_TRY(ar.alloc(&id, in.nh));
         SNN_TRY(iota_i32(id, in.nh, s));
-        SNN_L k_pl_xy<<<grid_for(in.nh, 256), 256, 0, s>>>(in.nh, in.width, id, cxy);
+        snn::enqueue(k_pl_xy, grid_for(in.nh, 256), 256, 0, s, in.nh, in.width, id, cxy);
         SNN_CUDA(cudaGetLastError());
         ar.rewind(mk);
     }
@@ -569,19 +587,20 @@ Status refine_impl(Input& in, int32_t* g, int32_t max_rounds, cudaStream_t s, in
     for (int32_t round = 0; round < max_rounds && active > 0; round++) {
         Arena::Mark mk = ar.mark();
         SNN_CUDA(cudaMemsetAsync(F, 0, sizeof(int64_t) * S * (int64_t)np * 4, s));
-        SNN_L k_pl_init_stats<<<1, 256, 0, s>>>(S, st);
+        snn::enqueue(k_pl_init_stats, 1, 256, 0, s, S, st);
         if (in.P > 0) {
-            SNN_L k_pl_xy<<<grid_for((int64_t)S * np, 256), 256, 0, s>>>((int64_t)S * np, in.width, g, nxy);
+            snn::enqueue(k_pl_xy, grid_for((int64_t)S * np, 256), 256, 0, s, (int64_t)S * np, in.width,
+                         g, nxy);
             auto force = warps ? k_pl_force<32> : k_pl_force<256>;
-            SNN_L force<<<gnode, 256, 0, s>>>(np, in.width, in.height, voff, vinc, in.off, in.pins,
-                                              in.eta, nxy, act, F);
+            snn::enqueue(force, gnode, 256, 0, s, np, in.width, in.height, voff, vinc, in.off, in.pins,
+                         in.eta, nxy, act, F);
         }
-        SNN_L k_pl_propose<<<gc, 256, 0, s>>>(nh, np, in.width, in.height, act, pi, F, cand,
-                                              cscore, st + (int64_t)PS_PROPS * S);
+        snn::enqueue(k_pl_propose, gc, 256, 0, s, nh, np, in.width, in.height, act, pi, F, cand,
+                     cscore, st + (int64_t)PS_PROPS * S);
         SNN_CUDA(cudaGetLastError());
         int64_t pairs = 0;
         SNN_TRY(match_forest((int32_t)V, cand, cscore, match, scal, ar, s, &pairs));
-        SNN_L k_pl_flag<<<gc, 256, 0, s>>>(nh, match, flag, st + (int64_t)PS_SWAPS * S);
+        snn::enqueue(k_pl_flag, gc, 256, 0, s, nh, match, flag, st + (int64_t)PS_SWAPS * S);
         SNN_CUDA(cudaGetLastError());
         SNN_CUDA(cudaMemcpyAsync(h_st.data(), st, sizeof(int64_t) * PS_N * S, cudaMemcpyDeviceToHost, s));
         SNN_CUDA(cudaStreamSynchronize(s));
@@ -604,33 +623,33 @@ Status refine_impl(Input& in, int32_t* g, int32_t max_rounds, cudaStream_t s, in
             SNN_TRY(ar.alloc(&Tn, ns));
             SNN_TRY(ar.alloc(&C, ns));
             SNN_CUDA(cudaMemsetAsync(err, 0, sizeof(int32_t), s));
-            SNN_L k_pl_compact<<<gc, 256, 0, s>>>(nh, np, in.width, in.height, match, pi, F, flag,
-                                                  pos, keys, vals, err);
+            snn::enqueue(k_pl_compact, gc, 256, 0, s, nh, np, in.width, in.height, match, pi, F, flag,
+                         pos, keys, vals, err);
             SNN_CUDA(cudaGetLastError());
             SNN_TRY(radix_sort_pairs(keys, vals, keys2, vals2, ns, 63, ar, s));
             if (S > 1) {
-                SNN_L k_pl_startkey<<<grid_for(ns, 256), 256, 0, s>>>(ns, nh, vals, keys);
+                snn::enqueue(k_pl_startkey, grid_for(ns, 256), 256, 0, s, ns, nh, vals, keys);
                 SNN_CUDA(cudaGetLastError());
                 SNN_TRY(radix_sort_pairs(keys, vals, keys2, vals2, ns, bits_for((uint64_t)(S - 1)),
                                          ar, s));
             }
             SNN_TRY(fill_i32(rank, NO_RANK, V, s));
-            SNN_L k_pl_rank<<<grid_for(ns, 256), 256, 0, s>>>(ns, nh, vals, match, segbeg, rank, mate);
+            snn::enqueue(k_pl_rank, grid_for(ns, 256), 256, 0, s, ns, nh, vals, match, segbeg, rank,
+                         mate);
             SNN_CUDA(cudaMemsetAsync(Tn, 0, sizeof(int64_t) * ns, s));
             if (in.P > 0) {
                 auto reeval = warps ? k_pl_reeval<32> : k_pl_reeval<256>;
-                SNN_L reeval<<<gnode, 256, 0, s>>>(np, nh, in.width, voff, vinc, in.off, in.pins, in.eta,
-                                                   g, cxy, rank, mate, segbeg, Tn);
+                snn::enqueue(reeval, gnode, 256, 0, s, np, nh, in.width, voff, vinc, in.off, in.pins,
+                             in.eta, g, cxy, rank, mate, segbeg, Tn);
             }
             SNN_CUDA(cudaGetLastError());
             SNN_TRY(scan_inclusive_i64(Tn, C, ns, ar, s));
-            SNN_L k_pl_best<<<grid_for(ns, 256), 256, 0, s>>>(ns, nh, vals, segbeg, C,
-                                                              st + (int64_t)PS_BEST * S);
-            SNN_L k_pl_first<<<grid_for(ns, 256), 256, 0, s>>>(ns, nh, vals, segbeg, C,
-                                                               st + (int64_t)PS_BEST * S,
-                                                               st + (int64_t)PS_FIRST * S);
-            SNN_L k_pl_apply<<<grid_for(ns, 256), 256, 0, s>>>(ns, nh, np, vals, match, segbeg,
-                                                               st + (int64_t)PS_FIRST * S, pi, g);
+            snn::enqueue(k_pl_best, grid_for(ns, 256), 256, 0, s, ns, nh, vals, segbeg, C,
+                         st + (int64_t)PS_BEST * S);
+            snn::enqueue(k_pl_first, grid_for(ns, 256), 256, 0, s, ns, nh, vals, segbeg, C,
+                         st + (int64_t)PS_BEST * S, st + (int64_t)PS_FIRST * S);
+            snn::enqueue(k_pl_apply, grid_for(ns, 256), 256, 0, s, ns, nh, np, vals, match, segbeg,
+                         st + (int64_t)PS_FIRST * S, pi, g);
             SNN_CUDA(cudaGetLastError());
             int32_t herr = 0;
             SNN_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
@@ -688,9 +707,9 @@ Status trd_impl(Input& in, const int32_t* g, cudaStream_t s, int64_t* trd_out)
         int2* nxy;
         const int64_t n = (int64_t)in.S * in.np;
         SNN_TRY(ar.alloc(&nxy, n));
-        SNN_L k_pl_xy<<<grid_for(n, 256), 256, 0, s>>>(n, in.width, g, nxy);
-        SNN_L k_pl_trd<<<grid2(in.P, in.S), 256, 0, s>>>(in.P, in.np, hid, in.off, in.pins, in.eta, nxy,
-                                                         acc);
+        snn::enqueue(k_pl_xy, grid_for(n, 256), 256, 0, s, n, in.width, g, nxy);
+        snn::enqueue(k_pl_trd, grid2(in.P, in.S), 256, 0, s, in.P, in.np, hid, in.off, in.pins, in.eta,
+                     nxy, acc);
         SNN_CUDA(cudaGetLastError());
     }
     SNN_CUDA(cudaMemcpyAsync(trd_out, acc, sizeof(int64_t) * in.S, cudaMemcpyDeviceToHost, s));

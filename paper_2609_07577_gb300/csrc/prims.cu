@@ -166,6 +166,7 @@ size_t Arena::held() const
 template <typename T>
 __global__ void k_fill(T* p, T v, int64_t n)
 {
+    after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
         p[i] = v;
@@ -173,6 +174,7 @@ __global__ void k_fill(T* p, T v, int64_t n)
 
 __global__ void k_iota(int32_t* p, int64_t n)
 {
+    after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
         p[i] = (int32_t)i;
@@ -181,7 +183,7 @@ __global__ void k_iota(int32_t* p, int64_t n)
 Status fill_i32(int32_t* p, int32_t v, int64_t n, cudaStream_t s)
 {
     if (n <= 0) return Status{};
-    SNN_L k_fill<int32_t><<<grid_for(n, 256), 256, 0, s>>>(p, v, n);
+    enqueue(k_fill<int32_t>, grid_for(n, 256), 256, 0, s, p, v, n);
     SNN_CUDA(cudaGetLastError());
     return Status{};
 }
@@ -189,7 +191,7 @@ Status fill_i32(int32_t* p, int32_t v, int64_t n, cudaStream_t s)
 Status fill_i64(int64_t* p, int64_t v, int64_t n, cudaStream_t s)
 {
     if (n <= 0) return Status{};
-    SNN_L k_fill<int64_t><<<grid_for(n, 256), 256, 0, s>>>(p, v, n);
+    enqueue(k_fill<int64_t>, grid_for(n, 256), 256, 0, s, p, v, n);
     SNN_CUDA(cudaGetLastError());
     return Status{};
 }
@@ -197,7 +199,7 @@ Status fill_i64(int64_t* p, int64_t v, int64_t n, cudaStream_t s)
 Status iota_i32(int32_t* p, int64_t n, cudaStream_t s)
 {
     if (n <= 0) return Status{};
-    SNN_L k_iota<<<grid_for(n, 256), 256, 0, s>>>(p, n);
+    enqueue(k_iota, grid_for(n, 256), 256, 0, s, p, n);
     SNN_CUDA(cudaGetLastError());
     return Status{};
 }
@@ -280,6 +282,7 @@ constexpr int RS_TILE = RS_THREADS * RS_ROUNDS;
 __global__ void __launch_bounds__(RS_THREADS)
     k_rs_upsweep(const uint64_t* keys, int64_t n, int shift, uint32_t* counts, int nblk)
 {
+    after_previous();
     __shared__ uint32_t hist[256];
     for (int i = threadIdx.x; i < 256; i += RS_THREADS) hist[i] = 0;
     __syncthreads();
@@ -296,6 +299,7 @@ __global__ void __launch_bounds__(RS_THREADS)
     k_rs_downsweep(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout,
                    int64_t n, int shift, const uint32_t* offs, int nblk)
 {
+    after_previous();
     __shared__ uint32_t wcnt[RS_WARPS][256];
     __shared__ uint32_t boff[256];
     __shared__ uint32_t tmp[RS_WARPS][32];
@@ -364,6 +368,7 @@ __global__ void __cluster_dims__(RSC_CTAS, 1, 1) __launch_bounds__(RSC_THREADS)
     k_rs_cluster(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t* vals_alt, int32_t n,
                  int passes)
 {
+    after_previous();
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     __shared__ uint32_t wcnt[RSC_WARPS][256];
@@ -478,6 +483,7 @@ __global__ void __cluster_dims__(RSC_CTAS, 1, 1) __launch_bounds__(RSC_THREADS)
 __global__ void __launch_bounds__(SB_THREADS)
     k_sort_block(uint64_t* keys, uint32_t* vals, int32_t n, int N, int ibits)
 {
+    after_previous();
     __shared__ uint64_t w[SB_MAX];
     uint32_t v[SB_MAX / SB_THREADS];
     const uint64_t imask = (1ull << ibits) - 1;
@@ -511,14 +517,14 @@ Status radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint
         int N = 64, ib = bits_for((uint64_t)(n - 1));
         while (N < n) N <<= 1;
         if (end_bit + ib < 64) {   // the padding stays above every word
-            SNN_L k_sort_block<<<1, SB_THREADS, 0, s>>>(keys, vals, (int32_t)n, N, ib);
+            enqueue(k_sort_block, 1, SB_THREADS, 0, s, keys, vals, (int32_t)n, N, ib);
             SNN_CUDA(cudaGetLastError());
             return Status{};
         }
     }
     if (n <= RSC_MAX) {
-        SNN_L k_rs_cluster<<<RSC_CTAS, RSC_THREADS, 0, s>>>(keys, vals, keys_alt, vals_alt, (int32_t)n,
-                                                            passes);
+        enqueue(k_rs_cluster, RSC_CTAS, RSC_THREADS, 0, s, keys, vals, keys_alt, vals_alt, (int32_t)n,
+                passes);
         SNN_CUDA(cudaGetLastError());
         return Status{};
     }
@@ -529,11 +535,11 @@ Status radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint
     uint32_t *vi = vals, *vo = vals_alt;
     for (int p = 0; p < passes; p++) {
         int shift = 8 * p;
-        SNN_L k_rs_upsweep<<<nblk, RS_THREADS, 0, s>>>(ki, n, shift, counts, nblk);
+        enqueue(k_rs_upsweep, nblk, RS_THREADS, 0, s, ki, n, shift, counts, nblk);
         SNN_CUDA(cudaGetLastError());
         SNN_TRY((scan_plain<uint32_t, uint32_t, false>(counts, counts, (int64_t)256 * nblk,
                                                        (uint32_t*)nullptr, ar, s)));
-        SNN_L k_rs_downsweep<<<nblk, RS_THREADS, 0, s>>>(ki, vi, ko, vo, n, shift, counts, nblk);
+        enqueue(k_rs_downsweep, nblk, RS_THREADS, 0, s, ki, vi, ko, vo, n, shift, counts, nblk);
         SNN_CUDA(cudaGetLastError());
         uint64_t* tk = ki; ki = ko; ko = tk;
         uint32_t* tv = vi; vi = vo; vo = tv;

@@ -73,6 +73,7 @@ struct PState {
 __global__ void k_project(int32_t V, const int32_t* __restrict__ cid,
                           const int32_t* __restrict__ rc, int32_t* rf)
 {
+    after_previous();
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x)
         rf[n] = rc[cid[n]];
@@ -82,7 +83,7 @@ Status project(snnmap_hgraph* h, int32_t level, const int32_t* rho_coarse, int32
 {
     Level& L = h->levels[level];
     if (L.V > 0) {
-        SNN_L k_project<<<grid_for(L.V, 256), 256, 0, h->stream>>>(L.V, L.cid, rho_coarse, rho_fine);
+        enqueue(k_project, grid_for(L.V, 256), 256, 0, h->stream, L.V, L.cid, rho_coarse, rho_fine);
         SNN_CUDA(cudaGetLastError());
     }
     return Status{};
@@ -97,6 +98,7 @@ constexpr int COST_SLOTS = 256;
 
 __global__ void k_cost_slots(const int64_t* __restrict__ slots, int64_t* out)
 {
+    after_previous();
     int64_t v = 0;
     for (int i = threadIdx.x; i < COST_SLOTS; i += blockDim.x) v += slots[i];
     v = warp_sum(v);
@@ -236,6 +238,7 @@ struct PinCountJob {
 
 __global__ void k_pstate_vertices(Level L, const int32_t* __restrict__ rho, PState ps)
 {
+    after_previous();
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < L.V;
          n += (int64_t)gridDim.x * blockDim.x) {
         int32_t p = rho[n];
@@ -279,6 +282,7 @@ template <int G>
 __global__ void __launch_bounds__(256)
     k_save(Level L, PinCounts pc, const int32_t* __restrict__ rho, int64_t* savev, int64_t* Wv)
 {
+    after_previous();
     int lane = threadIdx.x & (G - 1);
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -306,6 +310,7 @@ template <int G>
 __global__ void __launch_bounds__(SAVE_THREADS)
     k_save_smem(Level L, PinCounts pc, const int32_t* __restrict__ rho, int64_t* savev, int64_t* Wv)
 {
+    after_previous();
     extern __shared__ uint32_t ssum[];   // W, then save
     uint32_t *sW = ssum, *sS = ssum + L.V;
     for (int32_t v = threadIdx.x; v < 2 * L.V; v += SAVE_THREADS) ssum[v] = 0;
@@ -555,6 +560,7 @@ __global__ void __launch_bounds__(256)
                  int32_t delta, int32_t phi,
                  int nonpos, int32_t* pto, int64_t* pgain, const int32_t* __restrict__ dirty)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -737,6 +743,7 @@ __global__ void k_dense_zero(int32_t V, const int32_t* __restrict__ fresh,
                              const int32_t* __restrict__ rowid, RowTab tab,
                              unsigned long long* M)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -765,6 +772,7 @@ __global__ void k_dense_zero(int32_t V, const int32_t* __restrict__ fresh,
 
 __global__ void k_level_max(Level L, int32_t* vmax)
 {
+    after_previous();
     int32_t a = 0, b = 0, c = 0;
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < L.V;
          n += (int64_t)gridDim.x * blockDim.x) {
@@ -792,6 +800,7 @@ __global__ void k_inc_parts(int32_t M, Moves mv, const int64_t* __restrict__ sca
                             int32_t phi, uint8_t* pchg, uint8_t* prel,
                             const int32_t* __restrict__ pstar_n)
 {
+    after_previous();
     if (*pstar_n <= PSTAR_MAX) return;   // the column update below handles this round
     int64_t istar = scal[RS_BEST] > 0 ? scal[RS_ISTAR] : -1;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= istar && i < M;
@@ -816,6 +825,7 @@ __global__ void __launch_bounds__(256)
                  const int64_t* __restrict__ scal, const uint8_t* __restrict__ prel, uint32_t* buf,
                  int32_t* dirty, const int32_t* __restrict__ pstar_n)
 {
+    after_previous();
     if (*pstar_n <= PSTAR_MAX) return;
     int64_t istar = scal[RS_BEST] > 0 ? scal[RS_ISTAR] : -1;
     if (istar < 0) return;
@@ -880,6 +890,7 @@ __global__ void k_inc_targets(int32_t V, const int32_t* __restrict__ pto,
                               const uint8_t* __restrict__ pchg, int32_t* dirty,
                               const int32_t* __restrict__ pstar_n)
 {
+    after_previous();
     if (*pstar_n <= PSTAR_MAX) return;
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x)
@@ -925,6 +936,7 @@ __device__ __forceinline__ bool pstar_on(const int64_t* scal, const int32_t* cnt
 __global__ void k_ps_slots(int32_t M, Moves mv, const int64_t* __restrict__ scal, PStar ps,
                            int32_t* dirty)
 {
+    after_previous();
     int64_t istar = scal[RS_BEST] > 0 ? scal[RS_ISTAR] : -1;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= istar && i < M;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -948,6 +960,7 @@ __global__ void k_ps_slots(int32_t M, Moves mv, const int64_t* __restrict__ scal
 __global__ void __launch_bounds__(256)
     k_ps_mark(Level L, const int32_t* __restrict__ rho, const int64_t* __restrict__ scal, PStar ps)
 {
+    after_previous();
     if (!pstar_on(scal, ps.cnt)) return;
     int lane = threadIdx.x & 31;
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -981,6 +994,7 @@ template <int G>
 __global__ void __launch_bounds__(256)
     k_ps_mark_counts(Level L, PinCounts pc, const int64_t* __restrict__ scal, PStar ps)
 {
+    after_previous();
     if (!pstar_on(scal, ps.cnt)) return;
     const int lane = threadIdx.x & (G - 1);
     const unsigned gmask = (G == 32 ? FULL : ((1u << (G & 31)) - 1)) << ((threadIdx.x & 31) & ~(G - 1));
@@ -1009,6 +1023,7 @@ __global__ void __launch_bounds__(256)
     k_ps_cols(Level L, PinCounts pc, const int32_t* __restrict__ rho,
               const int64_t* __restrict__ scal, PStar ps)
 {
+    after_previous();
     if (!pstar_on(scal, ps.cnt)) return;
     int lane = threadIdx.x & 31;
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -1052,6 +1067,7 @@ __global__ void k_ps_combine(Level L, const int32_t* __restrict__ rho,
                              int32_t omega, int32_t delta, int32_t phi, int nonpos, int32_t* pto,
                              int64_t* pgain, int32_t* dirty)
 {
+    after_previous();
     if (!pstar_on(scal, ps.cnt)) return;
     int32_t ns = ps.cnt[0];
     int64_t V = L.V;
@@ -1110,6 +1126,7 @@ __global__ void k_ps_rows(Level L, const int32_t* __restrict__ rho,
                           int32_t delta, int32_t phi, int nonpos, int32_t* pto, int64_t* pgain,
                           int32_t* dirty)
 {
+    after_previous();
     if (scal[RS_BEST] <= 0) return;
     bool on = ps.cnt[0] <= PSTAR_MAX;
     int32_t ns = on ? ps.cnt[0] : 0;
@@ -1152,6 +1169,7 @@ __global__ void k_ps_rows(Level L, const int32_t* __restrict__ rho,
 __global__ void k_ps_reset(int32_t M, Moves mv, const int64_t* __restrict__ scal, PStar ps,
                            int64_t* host)
 {
+    after_previous();
     int64_t istar = scal[RS_BEST] > 0 ? scal[RS_ISTAR] : -1;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= istar && i < M;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -1226,6 +1244,7 @@ struct PropOut {
 __global__ void __launch_bounds__(256)
     k_prop_hedges(int32_t M, Moves mv, Level L, int32_t* hmark, int32_t* list, int32_t* n)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1259,6 +1278,7 @@ __global__ void k_moves(int32_t M, const uint32_t* __restrict__ vals, const int3
                         Events ev, int64_t* gp, int32_t* dv, int32_t* dirty,
                         const int64_t* __restrict__ savev, int64_t* save0)
 {
+    after_previous();
     const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t step = (int64_t)gridDim.x * blockDim.x;
     for (int64_t n = t0; n < L.V; n += step) {
@@ -1328,6 +1348,7 @@ __global__ void __launch_bounds__(256)
                   uint32_t* mvbuf, int64_t* gp, Events ev, int64_t evbase, int32_t* heavy,
                   int32_t* heavycnt, int64_t* scal, HedgeList hl)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     unsigned lt = lanemask_lt();
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -1391,6 +1412,7 @@ __global__ void __launch_bounds__(256)
                    Events ev, int64_t evbase, const int32_t* __restrict__ heavy,
                    const int32_t* __restrict__ heavycnt, int64_t* scal)
 {
+    after_previous();
     int32_t nh = (int32_t)scal[RS_NHV];
     for (int32_t h = blockIdx.x; h < nh; h += gridDim.x) {
         int32_t a = heavy[h];
@@ -1426,6 +1448,7 @@ __global__ void __launch_bounds__(256)
 __global__ void k_part_bounds(int64_t T, const uint64_t* __restrict__ key, int ibits, int32_t* pbeg,
                               int32_t* pend)
 {
+    after_previous();
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < T;
          e += (int64_t)gridDim.x * blockDim.x) {
         uint64_t p = key[e] >> ibits;
@@ -1438,6 +1461,7 @@ __global__ void __launch_bounds__(256)
     k_part_validity(int32_t K, const int32_t* __restrict__ pbeg, const int32_t* __restrict__ pend,
                     Events ev, PState ps, int32_t omega, int32_t delta, int32_t phi, int32_t* dv)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     unsigned lt = lanemask_lt();
     uint64_t imask = (ev.ibits >= 64) ? ~0ull : ((1ull << ev.ibits) - 1);
@@ -1496,6 +1520,7 @@ __global__ void __launch_bounds__(256)
 __global__ void k_best1(int32_t M, const int64_t* __restrict__ G, const int32_t* __restrict__ nviol,
                         int64_t* scal)
 {
+    after_previous();
     int64_t best = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < M;
          i += (int64_t)gridDim.x * blockDim.x)
@@ -1512,6 +1537,7 @@ __global__ void k_best1(int32_t M, const int64_t* __restrict__ G, const int32_t*
 __global__ void k_best2(int32_t M, const int64_t* __restrict__ G, const int32_t* __restrict__ nviol,
                         int64_t* scal)
 {
+    after_previous();
     int64_t best = scal[RS_BEST];
     if (best <= 0) return;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < M;
@@ -1548,6 +1574,7 @@ __global__ void __launch_bounds__(SB_THREADS)
     k_round_tail(int32_t M, Events ev, PState ps, int32_t omega, int32_t delta, int32_t phi,
                  const int64_t* __restrict__ gp, int64_t* scal)
 {
+    after_previous();
     __shared__ uint64_t w[TAIL_EVENTS];
     __shared__ int32_t dv[TAIL_EVENTS / 2];   // two events per move at least
     __shared__ Seg3 wseg[32];
@@ -1676,6 +1703,7 @@ __global__ void __launch_bounds__(1024)
     k_round_begin(int64_t* scal, int64_t* costv, const int64_t* __restrict__ slots, int32_t K, PState ps,
                   int32_t omega, int32_t delta, int32_t phi, int64_t* host)
 {
+    after_previous();
     __shared__ unsigned long long sum;
     const int i = threadIdx.x;
     if (slots) {
@@ -1825,8 +1853,8 @@ Status dense_begin(snnmap_hgraph* h, int32_t level)
     SNN_TRY(iota_i32(D.rowid, L.V, h->stream));
     SNN_TRY(fill_i32(D.fresh, 1, L.V, h->stream));
     if (L.V > 0) {
-        SNN_L k_dense_zero<<<grid_for((int64_t)L.V * 32, 256), 256, 0, h->stream>>>(L.V, D.fresh, D.rowid,
-                                                                            D.tab, D.M);
+        enqueue(k_dense_zero, grid_for((int64_t)L.V * 32, 256), 256, 0, h->stream, L.V, D.fresh,
+                D.rowid, D.tab, D.M);
         SNN_CUDA(cudaGetLastError());
     }
     D.level = level;
@@ -1847,8 +1875,8 @@ Status dense_descend(snnmap_hgraph* h, int32_t level)
         SNN_TRY(scan_run<int32_t>(UpperMember{L.pr}, RowIds{L.pr, L.cid, D.rowid, Vc, D.rowid2, D.fresh}, L.V,
                                   (int32_t*)nullptr, ar, s));
         std::swap(D.rowid, D.rowid2);
-        SNN_L k_dense_zero<<<grid_for((int64_t)L.V * 32, 256), 256, 0, s>>>(L.V, D.fresh, D.rowid, D.tab,
-                                                                     D.M);
+        enqueue(k_dense_zero, grid_for((int64_t)L.V * 32, 256), 256, 0, s, L.V, D.fresh, D.rowid,
+                D.tab, D.M);
         SNN_CUDA(cudaGetLastError());
     }
     D.level = level;
@@ -1864,7 +1892,7 @@ static Status pin_counts_into(snnmap_hgraph* h, Level& L, LevelExtra& X, int32_t
     cudaStream_t s = h->stream;
     Arena& ar = h->scratch;
     if (L.V > 0) {
-        SNN_L k_pstate_vertices<<<grid_for(L.V, 256), 256, 0, s>>>(L, rho, ps);
+        enqueue(k_pstate_vertices, grid_for(L.V, 256), 256, 0, s, L, rho, ps);
         SNN_CUDA(cudaGetLastError());
     }
     PinCountJob job{L.hoff, L.hpins, L.hsd, L.hk, L.hw, rho, pc, ps.pincnt, slots};
@@ -1896,7 +1924,7 @@ Status level_cost(snnmap_hgraph* h, int32_t level, int32_t K, const int32_t* rho
     cv.assign(base);
     SNN_CUDA(cudaMemsetAsync(base, 0, cv.total, h->stream));
     SNN_TRY(pin_counts_into(h, L, X, K, rho, pc, ps, slots));
-    SNN_L k_cost_slots<<<1, 256, 0, h->stream>>>(slots, h->d_scal + RS_COST);
+    enqueue(k_cost_slots, 1, 256, 0, h->stream, slots, h->d_scal + RS_COST);
     SNN_CUDA(cudaGetLastError());
     SNN_TRY(read_scalars(h));
     h->scratch.reset();
@@ -1921,6 +1949,7 @@ __global__ void __launch_bounds__(256)
                     const int32_t* __restrict__ rho, PState ps, int64_t* savev, int64_t* costv,
                     HedgeList hl)
 {
+    after_previous();
     int64_t istar = scal[RS_BEST] > 0 ? scal[RS_ISTAR] : -1;
     if (istar < 0) return;   // nothing is marked (the marks are cleared every round)
     int lane = threadIdx.x & 31;
@@ -1985,6 +2014,7 @@ __global__ void __launch_bounds__(256)
     k_prefix_saves(Level L, PinCounts pc, const int32_t* __restrict__ rho, int64_t* savev,
                    int32_t* hmark, int32_t* hdirty, HedgeList hl)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -2010,6 +2040,7 @@ __global__ void __launch_bounds__(256)
     k_prefix_recount(Level L, PinCountJob job, const int32_t* __restrict__ rho, int64_t* savev,
                      int32_t* hmark, int32_t* hdirty, HedgeList hl)
 {
+    after_previous();
     __shared__ __align__(16) uint32_t buf[8 * SEG_B1_CAP];
     const int lane = threadIdx.x & 31;
     uint32_t* s = buf + (threadIdx.x >> 5) * SEG_B1_CAP;
@@ -2048,6 +2079,7 @@ __global__ void __launch_bounds__(256)
 __global__ void k_apply(int32_t M, Moves mv, Level L, const int64_t* __restrict__ scal, PState ps,
                         int32_t* rho, int32_t* moveidx)
 {
+    after_previous();
     int64_t istar = scal[RS_BEST] > 0 ? scal[RS_ISTAR] : -1;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < M;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -2074,6 +2106,7 @@ __global__ void k_seg_filter(const int32_t* __restrict__ list, const int32_t* __
                              int32_t E, const int32_t* __restrict__ hdirty, int32_t* out,
                              int32_t* meta2)
 {
+    after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < E;
          i += (int64_t)gridDim.x * blockDim.x) {
         int32_t a = list[i];
@@ -2087,6 +2120,7 @@ __global__ void k_seg_filter(const int32_t* __restrict__ list, const int32_t* __
 
 __global__ void k_seg_meta_copy(const int32_t* __restrict__ meta, int32_t* meta2)
 {
+    after_previous();
     for (int b = threadIdx.x; b < SEG_NB; b += blockDim.x) meta2[b] = meta[b];
 }
 
@@ -2127,6 +2161,7 @@ __global__ void __launch_bounds__(256)
                    const int32_t* __restrict__ list, const int32_t* __restrict__ nlist, int64_t* savev,
                    int64_t* Wv)
 {
+    after_previous();
     __shared__ unsigned long long sum[2];
     const int32_t nl = *nlist;
     for (int32_t x = blockIdx.x; x < nl; x += gridDim.x) {
@@ -2187,9 +2222,9 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
         ProfScope prof(h, PS_PINCOUNT);
         if (!inc.ready) SNN_TRY(pin_counts_into(h, L, X, K, rho, pc, ps, inc.slots));
         host[HW_BAD] = 0;
-        SNN_L k_round_begin<<<inc.ready ? 1 : grid_for(K, 1024, 152), inc.ready ? 32 : 1024, 0, s>>>(h->d_scal, inc.costv,
-                                                                inc.ready ? nullptr : inc.slots, K, ps,
-                                                                prm.omega, prm.delta, prm.phi, host);
+        enqueue(k_round_begin, inc.ready ? 1 : grid_for(K, 1024, 152), inc.ready ? 32 : 1024, 0, s,
+                h->d_scal, inc.costv, inc.ready ? nullptr : inc.slots, K, ps, prm.omega, prm.delta,
+                prm.phi, host);
         SNN_CUDA(cudaGetLastError());
     }
     DenseRows& D = h->dense;
@@ -2208,15 +2243,15 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
         prof.reset(new ProfScope(h, PS_SAVE));
         if (inc.mlist) {
             if (inc.members > 0)
-                SNN_L k_save_members<<<dim3((unsigned)std::min<int64_t>(inc.members, 152 * 16), 4), 256, 0,
-                                       s>>>(L, pc, rho, inc.mlist, inc.mcnt, savev, Wv);
+                enqueue(k_save_members, dim3((unsigned)std::min<int64_t>(inc.members, 152 * 16), 4),
+                        256, 0, s, L, pc, rho, inc.mlist, inc.mcnt, savev, Wv);
             SNN_CUDA(cudaGetLastError());
         } else if (L.E > 0 && !h->wide && V <= SAVE_SMEM_V) {
             auto launch = [&](auto kern) -> Status {
                 SNN_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               SAVE_SMEM_V * 8));
-                SNN_L kern<<<grid_for(L.P, 4096, 152), SAVE_THREADS, (size_t)V * 8, s>>>(L, pc, rho,
-                                                                                        savev, Wv);
+                enqueue(kern, grid_for(L.P, 4096, 152), SAVE_THREADS, (size_t)V * 8, s, L, pc, rho,
+                        savev, Wv);
                 return Status{};
             };
             switch (hedge_lanes(L.P, L.E)) {
@@ -2234,9 +2269,9 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     prof.reset(new ProfScope(h, PS_GAINS));
     if (dense) {
         if (V > 0) {
-            SNN_L k_dense_best<<<grid_for((int64_t)V * 32, 256), 256, 0, s>>>(
-                L, rho, ps, savev, Wv, D.rowid, D.tab, D.M, D.cw, K, prm.omega, prm.delta,
-                prm.phi, prm.refine_nonpositive, pto, pgain, inc.dirty);
+            enqueue(k_dense_best, grid_for((int64_t)V * 32, 256), 256, 0, s, L, rho, ps, savev, Wv,
+                    D.rowid, D.tab, D.M, D.cw, K, prm.omega, prm.delta, prm.phi,
+                    prm.refine_nonpositive, pto, pgain, inc.dirty);
             SNN_CUDA(cudaGetLastError());
         }
     } else if (h->wide) {
@@ -2290,15 +2325,15 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     SNN_TRY(ar.alloc(&ev.dsize, ev.cap));
     SNN_TRY(ar.alloc(&ev.dinp, ev.cap));
     SNN_TRY(ar.alloc(&ev.dpc, ev.cap));
-    SNN_L k_moves<<<std::max(gm, gv), 256, 0, s>>>(M, vals, rho, pto, mv, moveidx, L, ev, gp, dv,
-                                                   inc.dirty, savev, inc.pst.save0);
+    enqueue(k_moves, std::max(gm, gv), 256, 0, s, M, vals, rho, pto, mv, moveidx, L, ev, gp, dv,
+            inc.dirty, savev, inc.pst.save0);
     SNN_CUDA(cudaGetLastError());
     // the hyperedges holding a proposed move
     int64_t nhl = std::max<int64_t>(1, std::min<int64_t>(L.E, deg));
     int32_t* hla;
     int32_t* hln = (int32_t*)(h->d_scal + RS_NHL);
     SNN_TRY(ar.alloc(&hla, nhl));
-    SNN_L k_prop_hedges<<<grid_for((int64_t)M * 32, 256), 256, 0, s>>>(M, mv, L, inc.hmark, hla, hln);
+    enqueue(k_prop_hedges, grid_for((int64_t)M * 32, 256), 256, 0, s, M, mv, L, inc.hmark, hla, hln);
     SNN_CUDA(cudaGetLastError());
     HedgeList hl{hla, hln};
     const int ghl = grid_for(nhl * 32, 256);
@@ -2312,18 +2347,19 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     SNN_TRY(ar.alloc(&hvc, L.E));
     const bool heavy = X.seg.n[SEG_BB1] + X.seg.n[SEG_BB2] + X.seg.n[SEG_BB3] > 0;
     if (L.E > 0) {
-        SNN_L k_replay_warp<<<ghl, 256, 0, s>>>(L, pc, moveidx, mv, mvbuf, gp, ev, 2 * (int64_t)M, hv,
-                                                hvc, h->d_scal, hl);
+        enqueue(k_replay_warp, ghl, 256, 0, s, L, pc, moveidx, mv, mvbuf, gp, ev, 2 * (int64_t)M, hv,
+                hvc, h->d_scal, hl);
         // only a hyperedge of more than REPLAY_WARP_MAX pins holds more moves
         if (heavy)
-            SNN_L k_replay_block<<<152 * 2, 256, 0, s>>>(L, pc, mv, mvbuf, gp, ev, 2 * (int64_t)M, hv, hvc,
-                                                   h->d_scal);
+            enqueue(k_replay_block, 152 * 2, 256, 0, s, L, pc, mv, mvbuf, gp, ev, 2 * (int64_t)M, hv,
+                    hvc, h->d_scal);
         SNN_CUDA(cudaGetLastError());
     }
     if (ev.cap <= TAIL_EVENTS) {
         // S10, S11
         prof.reset(new ProfScope(h, PS_VALIDITY));
-        SNN_L k_round_tail<<<1, SB_THREADS, 0, s>>>(M, ev, ps, prm.omega, prm.delta, prm.phi, gp, h->d_scal);
+        enqueue(k_round_tail, 1, SB_THREADS, 0, s, M, ev, ps, prm.omega, prm.delta, prm.phi, gp,
+                h->d_scal);
         SNN_CUDA(cudaGetLastError());
     } else {
         prof.reset();
@@ -2343,10 +2379,10 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
         SNN_TRY(ar.alloc(&pbeg, 2 * (int64_t)K));
         pend = pbeg + K;
         SNN_CUDA(cudaMemsetAsync(pbeg, 0, (size_t)K * 8, s));
-        SNN_L k_part_bounds<<<grid_for(T, 256), 256, 0, s>>>(T, ev.key, ev.ibits, pbeg, pend);
+        enqueue(k_part_bounds, grid_for(T, 256), 256, 0, s, T, ev.key, ev.ibits, pbeg, pend);
         SNN_CUDA(cudaGetLastError());
-        SNN_L k_part_validity<<<grid_for((int64_t)K * 32, 256), 256, 0, s>>>(K, pbeg, pend, ev, ps, prm.omega,
-                                                                      prm.delta, prm.phi, dv);
+        enqueue(k_part_validity, grid_for((int64_t)K * 32, 256), 256, 0, s, K, pbeg, pend, ev, ps,
+                prm.omega, prm.delta, prm.phi, dv);
         SNN_CUDA(cudaGetLastError());
 
         // S11
@@ -2355,24 +2391,24 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
         SNN_TRY(ar.alloc(&nviol, M));
         SNN_TRY(scan_inclusive_i64(gp, G, M, ar, s));
         SNN_TRY(scan_inclusive_i32(dv, nviol, M, ar, s));
-        SNN_L k_best1<<<gm, 256, 0, s>>>(M, G, nviol, h->d_scal);
-        SNN_L k_best2<<<gm, 256, 0, s>>>(M, G, nviol, h->d_scal);
+        enqueue(k_best1, gm, 256, 0, s, M, G, nviol, h->d_scal);
+        enqueue(k_best2, gm, 256, 0, s, M, G, nviol, h->d_scal);
     }
     prof.reset(new ProfScope(h, PS_APPLY));
     // P* of the enacted prefix; when it is short, the rows (k_ps_rows) or the
     // column update after the pin counts below decide the next round's
     // proposals, otherwise the flags of the three rules here do
-    SNN_L k_ps_slots<<<gm, 256, 0, s>>>(M, mv, h->d_scal, inc.pst, inc.dirty);
+    enqueue(k_ps_slots, gm, 256, 0, s, M, mv, h->d_scal, inc.pst, inc.dirty);
     SNN_CUDA(cudaGetLastError());
     if (!dense && (!inc.pst.colc || 2 * (int64_t)M > PSTAR_MAX)) {
         SNN_CUDA(cudaMemsetAsync(inc.pchg, 0, (size_t)(K > 0 ? K : 1), s));
         SNN_CUDA(cudaMemsetAsync(inc.prel, 0, (size_t)(K > 0 ? K : 1), s));
-        SNN_L k_inc_parts<<<gm, 256, 0, s>>>(M, mv, h->d_scal, ps, inc.vmax, prm.omega, prm.delta,
-                                             prm.phi, inc.pchg, inc.prel, inc.pst.cnt);
+        enqueue(k_inc_parts, gm, 256, 0, s, M, mv, h->d_scal, ps, inc.vmax, prm.omega, prm.delta,
+                prm.phi, inc.pchg, inc.prel, inc.pst.cnt);
         if (L.E > 0)
-            SNN_L k_inc_hedges<<<grid_for((int64_t)L.E * 32, 256), 256, 0, s>>>(
-                L, pc, moveidx, mv, h->d_scal, inc.prel, mvbuf, inc.dirty, inc.pst.cnt);
-        SNN_L k_inc_targets<<<gv, 256, 0, s>>>(V, pto, inc.pchg, inc.dirty, inc.pst.cnt);
+            enqueue(k_inc_hedges, grid_for((int64_t)L.E * 32, 256), 256, 0, s, L, pc, moveidx, mv,
+                    h->d_scal, inc.prel, mvbuf, inc.dirty, inc.pst.cnt);
+        enqueue(k_inc_targets, gv, 256, 0, s, V, pto, inc.pchg, inc.dirty, inc.pst.cnt);
         SNN_CUDA(cudaGetLastError());
     }
     // carried pin counts: take out the hyperedges the prefix touches (old
@@ -2380,22 +2416,22 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
     prof.reset(new ProfScope(h, PS_PINCOUNT));
     if (L.E > 0) {
         RowsRef R{dense ? D.rowid : nullptr, D.tab, D.M, D.cw};
-        SNN_L k_prefix_hedges<<<ghl, 256, 0, s>>>(L, pc, moveidx, mv, h->d_scal, R, mvbuf, inc.hdirty, rho,
-                                                  ps, savev, inc.costv, hl);
+        enqueue(k_prefix_hedges, ghl, 256, 0, s, L, pc, moveidx, mv, h->d_scal, R, mvbuf, inc.hdirty,
+                rho, ps, savev, inc.costv, hl);
         SNN_CUDA(cudaGetLastError());
     }
-    SNN_L k_apply<<<gm, 256, 0, s>>>(M, mv, L, h->d_scal, ps, rho, moveidx);
+    enqueue(k_apply, gm, 256, 0, s, M, mv, L, h->d_scal, ps, rho, moveidx);
     SNN_CUDA(cudaGetLastError());
     if (L.E > 0) {
         PinCountJob job{L.hoff, L.hpins, L.hsd, L.hk, L.hw, rho, pc, ps.pincnt, inc.costv};
         job.cost_mask = 0;
         if (nhl <= RECOUNT_MAX && X.seg.n[SEG_BB2] + X.seg.n[SEG_BB3] == 0) {
-            SNN_L k_prefix_recount<<<ghl, 256, 0, s>>>(L, job, rho, savev, inc.hmark, inc.hdirty, hl);
+            enqueue(k_prefix_recount, ghl, 256, 0, s, L, job, rho, savev, inc.hmark, inc.hdirty, hl);
         } else {
             SNN_CUDA(cudaMemsetAsync(inc.hmeta, 0, 2 * SEG_NB * sizeof(int32_t), s));
-            SNN_L k_seg_meta_copy<<<1, 32, 0, s>>>(X.seg.meta, inc.hmeta);
-            SNN_L k_seg_filter<<<grid_for(L.E, 256), 256, 0, s>>>(X.seg.list, X.seg.meta, L.E, inc.hdirty,
-                                                                 inc.hlist, inc.hmeta);
+            enqueue(k_seg_meta_copy, 1, 32, 0, s, X.seg.meta, inc.hmeta);
+            enqueue(k_seg_filter, grid_for(L.E, 256), 256, 0, s, X.seg.list, X.seg.meta, L.E,
+                    inc.hdirty, inc.hlist, inc.hmeta);
             SNN_CUDA(cudaGetLastError());
             SegBuckets db = X.seg;
             db.list = inc.hlist;
@@ -2406,8 +2442,8 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
             job.cost = slots;
             job.cost_mask = COST_SLOTS - 1;
             SNN_TRY(seg_run(job, db, L.E, ar, s));
-            SNN_L k_cost_slots<<<1, 256, 0, s>>>(slots, inc.costv);
-            SNN_L k_prefix_saves<<<ghl, 256, 0, s>>>(L, pc, rho, savev, inc.hmark, inc.hdirty, hl);
+            enqueue(k_cost_slots, 1, 256, 0, s, slots, inc.costv);
+            enqueue(k_prefix_saves, ghl, 256, 0, s, L, pc, rho, savev, inc.hmark, inc.hdirty, hl);
         }
         SNN_CUDA(cudaGetLastError());
     }
@@ -2418,22 +2454,20 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
                 SNN_HEDGE_LAUNCH(hedge_lanes(L.P, 2 * (int64_t)L.E), k_ps_mark_counts, L.E, s, L, pc,
                                  h->d_scal, inc.pst);
             } else {
-                SNN_L k_ps_mark<<<grid_for(V, 256), 256, 0, s>>>(L, rho, h->d_scal, inc.pst);
+                enqueue(k_ps_mark, grid_for(V, 256), 256, 0, s, L, rho, h->d_scal, inc.pst);
             }
-            SNN_L k_ps_cols<<<152 * 8, 256, 0, s>>>(L, pc, rho, h->d_scal, inc.pst);
-            SNN_L k_ps_combine<<<gv, 256, 0, s>>>(L, rho, h->d_scal, inc.pst, ps, savev, Wv, prm.omega,
-                                                  prm.delta, prm.phi, prm.refine_nonpositive, pto,
-                                                  pgain, inc.dirty);
+            enqueue(k_ps_cols, 152 * 8, 256, 0, s, L, pc, rho, h->d_scal, inc.pst);
+            enqueue(k_ps_combine, gv, 256, 0, s, L, rho, h->d_scal, inc.pst, ps, savev, Wv, prm.omega,
+                    prm.delta, prm.phi, prm.refine_nonpositive, pto, pgain, inc.dirty);
         }
-        SNN_L k_ps_reset<<<gm, 256, 0, s>>>(M, mv, h->d_scal, inc.pst, host);
+        enqueue(k_ps_reset, gm, 256, 0, s, M, mv, h->d_scal, inc.pst, host);
         SNN_CUDA(cudaGetLastError());
     } else {
         prof.reset(new ProfScope(h, PS_GAINS));
         if (V > 0)
-            SNN_L k_ps_rows<<<gv, 256, 0, s>>>(L, rho, h->d_scal, inc.pst, ps, savev, Wv, D.rowid, D.tab,
-                                               prm.omega, prm.delta, prm.phi,
-                                               prm.refine_nonpositive, pto, pgain, inc.dirty);
-        SNN_L k_ps_reset<<<gm, 256, 0, s>>>(M, mv, h->d_scal, inc.pst, host);
+            enqueue(k_ps_rows, gv, 256, 0, s, L, rho, h->d_scal, inc.pst, ps, savev, Wv, D.rowid,
+                    D.tab, prm.omega, prm.delta, prm.phi, prm.refine_nonpositive, pto, pgain, inc.dirty);
+        enqueue(k_ps_reset, gm, 256, 0, s, M, mv, h->d_scal, inc.pst, host);
         SNN_CUDA(cudaGetLastError());
     }
     prof.reset();
@@ -2450,6 +2484,7 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
 
 __global__ void k_check_rho(int32_t V, const int32_t* __restrict__ rho, int32_t K, int64_t* scal)
 {
+    after_previous();
     int bad = 0;
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x)
@@ -2462,7 +2497,7 @@ Status check_rho(snnmap_hgraph* h, int32_t level, int32_t K, const int32_t* rho)
     Level& L = h->levels[level];
     SNN_TRY(zero_scalars(h));
     if (L.V > 0) {
-        SNN_L k_check_rho<<<grid_for(L.V, 256), 256, 0, h->stream>>>(L.V, rho, K, h->d_scal);
+        enqueue(k_check_rho, grid_for(L.V, 256), 256, 0, h->stream, L.V, rho, K, h->d_scal);
         SNN_CUDA(cudaGetLastError());
     }
     SNN_TRY(read_scalars(h));
@@ -2479,6 +2514,7 @@ __global__ void k_carry(int32_t V, const int32_t* __restrict__ cid, const uint8_
                         const int32_t* __restrict__ dirty_c, int32_t* pto, int64_t* pgain,
                         int32_t* dirty)
 {
+    after_previous();
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
         int32_t c = cid[n];
@@ -2533,6 +2569,7 @@ struct SaveIn {
 __global__ void k_refine_init(int32_t V, int32_t K, int32_t* moveidx, int32_t* dirty, PStar ps,
                               int32_t base, SaveIn si)
 {
+    after_previous();
     int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     int64_t step = (int64_t)gridDim.x * blockDim.x;
     for (int64_t n = t0; n < V; n += step) {
@@ -2649,9 +2686,8 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
             }
             CA.slevel = -1;
             if (!dense_level && CA.level == level + 1 && L.V > 0) {
-                SNN_L k_carry<<<grid_for(L.V, 256), 256, 0, s>>>(L.V, L.cid, L.pr, CA.pto[CA.cur],
-                                                                CA.pgain[CA.cur], CA.dirty[CA.cur],
-                                                                inc.pto, inc.pgain, inc.dirty);
+                enqueue(k_carry, grid_for(L.V, 256), 256, 0, s, L.V, L.cid, L.pr, CA.pto[CA.cur],
+                        CA.pgain[CA.cur], CA.dirty[CA.cur], inc.pto, inc.pgain, inc.dirty);
                 SNN_CUDA(cudaGetLastError());
                 inherited = true;
             }
@@ -2659,9 +2695,10 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
             CA.level = -1;
         }
         // without the saves (and columns) the column update stays off
-        SNN_L k_refine_init<<<grid_for(std::max<int64_t>(V, K), 256), 256, 0, s>>>(
-            L.V, K, moveidx, inherited ? nullptr : inc.dirty, pst, cols ? 0 : (1 << 30), si);
-        if (!dense_level && L.V > 0) SNN_L k_level_max<<<grid_for(L.V, 256, 152 * 4), 256, 0, s>>>(L, inc.vmax);
+        enqueue(k_refine_init, grid_for(std::max<int64_t>(V, K), 256), 256, 0, s, L.V, K, moveidx,
+                inherited ? nullptr : inc.dirty, pst, cols ? 0 : (1 << 30), si);
+        if (!dense_level && L.V > 0) enqueue(k_level_max, grid_for(L.V, 256, 152 * 4), 256, 0, s, L,
+                                             inc.vmax);
         SNN_CUDA(cudaGetLastError());
         return Status{};
     };

@@ -72,6 +72,7 @@ template <typename T, class In, class Out>
 __global__ void __cluster_dims__(SCAN_CTAS, 1, 1) __launch_bounds__(SCAN_THREADS)
     k_scan_cluster(In in, Out out, int64_t n, T* total)
 {
+    after_previous();
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     __shared__ __align__(16) unsigned char raw[sizeof(T) * (2 * 32 + 2)];
@@ -161,6 +162,7 @@ __device__ __forceinline__ T block_prefix(T v, T* sh, T* block_total)
 template <typename T, class In>
 __global__ void __launch_bounds__(SCT_THREADS) k_scan_sums(In in, int64_t n, T* bsum)
 {
+    after_previous();
     __shared__ __align__(16) unsigned char raw[sizeof(T) * (SCT_THREADS / 32)];
     T acc = T();
     int64_t base = (int64_t)blockIdx.x * SCT_TILE;
@@ -178,6 +180,7 @@ template <typename T, class In, class Out>
 __global__ void __launch_bounds__(SCT_THREADS)
     k_scan_apply(In in, Out out, int64_t n, const T* boff, T* total)
 {
+    after_previous();
     __shared__ __align__(16) unsigned char raw[sizeof(T) * (SCT_THREADS / 32)];
     int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t w0 = (int64_t)blockIdx.x * SCT_TILE + (int64_t)warp * 32 * SCT_ITEMS;
@@ -260,17 +263,17 @@ Status scan_run(const In& in, const Out& out, int64_t n, T* total, Arena& ar, cu
         return Status{};
     }
     if (n <= SCAN_CLUSTER_MAX) {
-        SNN_L k_scan_cluster<T, In, Out><<<SCAN_CTAS, SCAN_THREADS, 0, s>>>(in, out, n, total);
+        enqueue(k_scan_cluster<T, In, Out>, SCAN_CTAS, SCAN_THREADS, 0, s, in, out, n, total);
         SNN_CUDA(cudaGetLastError());
         return Status{};
     }
     int64_t nb = ceil_div(n, SCT_TILE);
     T* bsum = nullptr;
     SNN_TRY(ar.alloc(&bsum, nb));
-    SNN_L k_scan_sums<T, In><<<(unsigned)nb, SCT_THREADS, 0, s>>>(in, n, bsum);
+    enqueue(k_scan_sums<T, In>, (unsigned)nb, SCT_THREADS, 0, s, in, n, bsum);
     SNN_CUDA(cudaGetLastError());
     SNN_TRY((scan_run<T>(ScanLoad<T, T>{bsum}, ScanStore<T, false>{bsum}, nb, (T*)nullptr, ar, s)));
-    SNN_L k_scan_apply<T, In, Out><<<(unsigned)nb, SCT_THREADS, 0, s>>>(in, out, n, bsum, total);
+    enqueue(k_scan_apply<T, In, Out>, (unsigned)nb, SCT_THREADS, 0, s, in, out, n, bsum, total);
     SNN_CUDA(cudaGetLastError());
     return Status{};
 }

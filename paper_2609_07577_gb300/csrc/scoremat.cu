@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(256)
                const int32_t* __restrict__ OVm, int64_t Vs, int32_t omega, int32_t delta,
                int32_t phi, int32_t* cand, int64_t* cscore, int32_t* cov)
 {
+    after_previous();
     int lane = threadIdx.x & 31;
     int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(256)
 __global__ void k_mat_reps(int32_t V, const int32_t* __restrict__ cid,
                            const int32_t* __restrict__ match, int32_t* repof, int32_t* fresh)
 {
+    after_previous();
     for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < V;
          n += (int64_t)gridDim.x * blockDim.x) {
         int32_t m = match[n];
@@ -165,6 +167,7 @@ __global__ void __launch_bounds__(256)
                  const int32_t* __restrict__ Sm,
                  const int32_t* __restrict__ OVm, int64_t Vs, int32_t* S2, int32_t* OV2, int64_t Vs2)
 {
+    after_previous();
     for (int64_t i = blockIdx.x; i < V2; i += gridDim.x) {
         int64_t src = (int64_t)repof[i] * Vs;
         int64_t dst = i * Vs2;
@@ -251,9 +254,8 @@ Status mat_affinity(snnmap_hgraph* h, int32_t level, bool* done)
         M.level = level;
     }
     if (L.V > 0) {
-        SNN_L k_mat_best<<<grid_for((int64_t)L.V * 32, 256), 256, 0, s>>>(
-            L, M.S, M.OV, M.Vs, h->prm.omega, h->prm.delta, h->prm.phi, h->cand, h->cscore,
-            h->cov);
+        enqueue(k_mat_best, grid_for((int64_t)L.V * 32, 256), 256, 0, s, L, M.S, M.OV, M.Vs,
+                h->prm.omega, h->prm.delta, h->prm.phi, h->cand, h->cscore, h->cov);
         SNN_CUDA(cudaGetLastError());
     }
     h->extra[level].n_block = 0;
@@ -282,12 +284,12 @@ Status mat_descend(snnmap_hgraph* h, int32_t src)
     SNN_TRY(ar.alloc(&repof, L.V));
     SNN_TRY(ar.alloc(&fresh, L.V));
     if (F.V > 0) {
-        SNN_L k_mat_reps<<<grid_for(F.V, 256), 256, 0, s>>>(F.V, F.cid, h->match, repof, fresh);
+        enqueue(k_mat_reps, grid_for(F.V, 256), 256, 0, s, F.V, F.cid, h->match, repof, fresh);
         SNN_CUDA(cudaGetLastError());
     }
     if (L.V > 0) {
-        SNN_L k_mat_gather<<<(int)std::min<int64_t>(L.V, 152 * 16), 256, 0, s>>>(
-            L.V, repof, fresh, M.S, M.OV, M.Vs, M.S2, M.OV2, Vs2);
+        enqueue(k_mat_gather, (int)std::min<int64_t>(L.V, 152 * 16), 256, 0, s, L.V, repof, fresh, M.S,
+                M.OV, M.Vs, M.S2, M.OV2, Vs2);
         SNN_CUDA(cudaGetLastError());
     }
     std::swap(M.S, M.S2);

@@ -205,6 +205,7 @@ template <class Job>
 __global__ void __launch_bounds__(256) k_seg_small(Job job, const int32_t* __restrict__ lists,
                                                    const int32_t* __restrict__ meta, int gt, int gb0)
 {
+    after_previous();
     extern __shared__ uint32_t seg_dyn[];
     if constexpr (seg_shared<Job>::value) {
         for (int i = threadIdx.x; i < job.shared_words(); i += 256) seg_dyn[i] = 0;
@@ -256,6 +257,7 @@ __global__ void k_seg_big(Job job, const int32_t* __restrict__ lists,
                           const int32_t* __restrict__ meta, int bucket, uint32_t* gscratch,
                           int64_t cap)
 {
+    after_previous();
     extern __shared__ uint32_t sbuf[];
     uint32_t* s = gscratch ? gscratch + (int64_t)blockIdx.x * cap : sbuf;
     const int32_t* list = lists + meta[bucket];
@@ -339,22 +341,22 @@ Status seg_run(const Job& job, const SegBuckets& b, int32_t E, Arena& ar, cudaSt
         if (dyn)
             SNN_CUDA(cudaFuncSetAttribute(k_seg_small<Job>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)dyn));
-        SNN_L k_seg_small<Job><<<gt + gb0 + gb1, 256, dyn, s>>>(job, b.list, b.meta, gt, gb0);
+        enqueue(k_seg_small<Job>, gt + gb0 + gb1, 256, dyn, s, job, b.list, b.meta, gt, gb0);
         SNN_CUDA(cudaGetLastError());
     }
     if (count(SEG_BB2) > 0) {
         size_t smem = SEG_B2_CAP * sizeof(uint32_t);
         SNN_CUDA(cudaFuncSetAttribute(k_seg_big<Job>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)smem));
-        SNN_L k_seg_big<Job><<<seg_grid_big(count(SEG_BB2)), SEG_B2_THREADS, smem, s>>>(
-            job, b.list, b.meta, SEG_BB2, nullptr, 0);
+        enqueue(k_seg_big<Job>, seg_grid_big(count(SEG_BB2)), SEG_B2_THREADS, smem, s, job, b.list,
+                b.meta, SEG_BB2, nullptr, 0);
         SNN_CUDA(cudaGetLastError());
     }
     if (b.b3_cap > 0 && count(SEG_BB3) > 0) {
         uint32_t* g = nullptr;
         SNN_TRY(ar.alloc(&g, (int64_t)SEG_B3_BLOCKS * b.b3_cap));
-        SNN_L k_seg_big<Job><<<SEG_B3_BLOCKS, SEG_B3_THREADS, 0, s>>>(job, b.list, b.meta, SEG_BB3,
-                                                                       g, b.b3_cap);
+        enqueue(k_seg_big<Job>, SEG_B3_BLOCKS, SEG_B3_THREADS, 0, s, job, b.list, b.meta, SEG_BB3, g,
+                b.b3_cap);
         SNN_CUDA(cudaGetLastError());
     }
     return Status{};
