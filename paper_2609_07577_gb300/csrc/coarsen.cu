@@ -127,10 +127,11 @@ struct AffPol {
     __device__ void consider(int32_t n, int32_t m, int64_t s, uint32_t o, const Acc&, int64_t& bs,
                              int32_t& bk, uint32_t& bo) const
     {
+        if (!better(s, m, bs, bk)) return;   // before the state's gather
         int4 a = vst[n], b = vst[m];
         bool valid = (int64_t)a.x + b.x <= omega && (int64_t)a.y + b.y <= phi &&
                      (int64_t)a.z + b.z - (int64_t)o <= delta;
-        if (valid && better(s, m, bs, bk)) {
+        if (valid) {
             bs = s;
             bk = m;
             bo = o;

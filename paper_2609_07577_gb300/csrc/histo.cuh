@@ -175,7 +175,7 @@ __device__ __forceinline__ Seg<S> rec_seg(const HRec& r, uint32_t inc)
 // bits: one shared-memory atomic an element instead of two. LIST: the slots
 // in use are listed, so the result of a large table costs a read per key
 // instead of one per slot.
-template <bool LIST>
+template <bool LIST, bool CLAIM = false>
 struct PackedTable {
     int32_t* key;
     uint32_t* val;
@@ -188,7 +188,7 @@ struct PackedTable {
     {
         uint32_t slot = table_slot(m, mask);
         for (uint32_t probe = 0; probe < probes; probe++) {
-            int32_t k = *(volatile int32_t*)&key[slot];
+            int32_t k = CLAIM ? -1 : *(volatile int32_t*)&key[slot];
             if (k == -1) {
                 int32_t prev = atomicCAS(&key[slot], -1, m);
                 k = prev == -1 ? m : prev;
@@ -766,10 +766,12 @@ __global__ void __launch_bounds__(T, CAP <= 2048 ? HT_BLOCKS : 1)
     using Acc = typename Pol::Acc;
     extern __shared__ __align__(16) unsigned char ht_dyn[];
     __shared__ int sfail;
-    __shared__ int64_t slong[HT_NLONG];
     __shared__ int32_t nlong;
     constexpr int FLAT = T / 4;   // most incidences of the flattened form
-    __shared__ __align__(16) unsigned char sseg_raw[sizeof(Seg<S>) * FLAT];
+    // a vertex is flattened or visited by groups: one of the two is in use
+    constexpr size_t SEG_BYTES = sizeof(Seg<S>) * FLAT, LONG_BYTES = sizeof(int64_t) * HT_NLONG;
+    __shared__ __align__(16) unsigned char sseg_raw[SEG_BYTES > LONG_BYTES ? SEG_BYTES : LONG_BYTES];
+    int64_t* slong = (int64_t*)sseg_raw;
     __shared__ int32_t spre[FLAT];
     __shared__ int32_t swarp[FLAT / 32];
     Seg<S>* sseg = (Seg<S>*)sseg_raw;
@@ -876,30 +878,30 @@ __global__ void __launch_bounds__(T, CAP <= 2048 ? HT_BLOCKS : 1)
             if (LIST && sb >= 0) listed = true;
             pt.sb = sb;
         }
-        auto visit = [&](const auto& tb) {
-            const typename Pol::Own own = pol.own(n);
+        const typename Pol::Own own = pol.own(n);
+        auto visit_flat = [&](const auto& tb) {
+            constexpr int U = 4;   // elements in flight per thread
             bool k = true;
-            if (flat) {
-                constexpr int U = 4;   // elements in flight per thread
-                int32_t lo = 0;
-                for (int32_t v0 = threadIdx.x; v0 < total && k; v0 += U * T) {
-                    typename Pol::Item it[U];
+            int32_t lo = 0;
+            for (int32_t v0 = threadIdx.x; v0 < total && k; v0 += U * T) {
+                typename Pol::Item it[U];
 #pragma unroll
-                    for (int u = 0; u < U; u++) {
-                        int32_t v = v0 + u * T;
-                        if (v < total) {
-                            lo = seg_find(spre, deg, lo, v);
-                            it[u] = pol.load(n, own, sseg[lo], v - spre[lo]);
-                        } else {
-                            it[u] = Pol::none();
-                        }
+                for (int u = 0; u < U; u++) {
+                    int32_t v = v0 + u * T;
+                    if (v < total) {
+                        lo = seg_find(spre, deg, lo, v);
+                        it[u] = pol.load(n, own, sseg[lo], v - spre[lo]);
+                    } else {
+                        it[u] = Pol::none();
                     }
-#pragma unroll
-                    for (int u = 0; u < U; u++) k = pol.put(n, it[u], tb, acc) && k;
                 }
-                return k;
+#pragma unroll
+                for (int u = 0; u < U; u++) k = pol.put(n, it[u], tb, acc) && k;
             }
-            k = group_visit<S, T, 2>(pol, n, vb, ve, glog, threadIdx.x, tb, acc, slong, &nlong);
+            return k;
+        };
+        auto visit_groups = [&](const auto& tb) {
+            bool k = group_visit<S, T, 1>(pol, n, vb, ve, glog, threadIdx.x, tb, acc, slong, &nlong);
             __syncthreads();
             const int nlg = nlong < HT_NLONG ? nlong : HT_NLONG;
             Acc other;   // the segments' own terms are in already
@@ -914,11 +916,11 @@ __global__ void __launch_bounds__(T, CAP <= 2048 ? HT_BLOCKS : 1)
             }
             return k;
         };
-        if constexpr (sizeof(S) == 4) {
-            if (sb >= 0) ok = visit(pt);
-            else ok = visit(t);
+        if (sizeof(S) == 4 && sb >= 0) {
+            if (flat) ok = visit_flat(PackedTable<LIST, !LIST>{pt.key, pt.val, pt.used, pt.nused, pt.mask, pt.probes, sb});
+            else ok = visit_groups(pt);
         } else {
-            ok = visit(t);
+            ok = flat ? visit_flat(t) : visit_groups(t);
         }
         if (!ok) sfail = 1;
         Acc wa = Pol::warp_reduce(acc);
@@ -937,15 +939,32 @@ __global__ void __launch_bounds__(T, CAP <= 2048 ? HT_BLOCKS : 1)
         uint32_t bo = 0;
         if (sb >= 0) {
             const uint32_t omask = (1u << sb) - 1;   // sb < 32: multiplicities sum below 2^31
-            const int nk = LIST ? nused : CAP;
-            for (int x = threadIdx.x; x < nk; x += T) {
-                int i = LIST ? pt.used[x] : x;
-                int32_t k = pt.key[i];
-                if (!LIST && k < 0) continue;
-                uint32_t v = pt.val[i];
-                pt.key[i] = -1;
-                pt.val[i] = 0;
-                pol.consider(n, k, (int64_t)(v >> sb), v & omask, tot, bs, bk, bo);
+            if (LIST) {
+                const int nk = nused;
+                for (int x = threadIdx.x; x < nk; x += T) {
+                    int i = pt.used[x];
+                    int32_t k = pt.key[i];
+                    uint32_t v = pt.val[i];
+                    pt.key[i] = -1;
+                    pt.val[i] = 0;
+                    pol.consider(n, k, (int64_t)(v >> sb), v & omask, tot, bs, bk, bo);
+                }
+            } else {
+                for (int i = 4 * threadIdx.x; i < CAP; i += 4 * T) {
+                    int4* kp = reinterpret_cast<int4*>(pt.key + i);
+                    uint4* vp = reinterpret_cast<uint4*>(pt.val + i);
+                    const int4 k4 = *kp;
+                    if ((k4.x & k4.y & k4.z & k4.w) == -1) continue;
+                    const uint4 v4 = *vp;
+                    *kp = make_int4(-1, -1, -1, -1);
+                    *vp = make_uint4(0, 0, 0, 0);
+                    const int32_t ks[4] = {k4.x, k4.y, k4.z, k4.w};
+                    const uint32_t vs[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+                    for (int u = 0; u < 4; u++)
+                        if (ks[u] >= 0)
+                            pol.consider(n, ks[u], (int64_t)(vs[u] >> sb), vs[u] & omask, tot, bs, bk, bo);
+                }
             }
         } else {
             scan_slots<S>(pol, n, t, threadIdx.x, CAP, T, tot, bs, bk, bo);

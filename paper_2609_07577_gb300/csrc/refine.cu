@@ -584,27 +584,30 @@ __global__ void __launch_bounds__(256)
         int32_t bk = -1;
         const int64_t nq = ((int64_t)K + 3) >> 2;
         unsigned long long msk = M[rw];   // the same word in every lane
-        // marked entries four loads at a time, in increasing order: row entry
-        // it of the marked ones, 32 int4 per step (cw >> 2 of them a chunk)
-        const int per = (cw >> 2) > 32 ? (cw >> 2) / 32 : 1;   // steps per chunk
-        int step = 0, c = -1;
-        while (msk || step > 0) {
-            constexpr int U = 4;
+        // Marked entries, two loads a lane at a time: a step reads 32 int4, a
+        // part of one chunk or (cq < 32) one lane group per chunk of 32 / cq
+        // consecutive marked ones (cw is a power of two of at least 32).
+        const int cq = cw >> 2;                                 // int4 a chunk
+        const int per = cq > 32 ? (cq + 31) / 32 : 1;           // steps a chunk
+        const int side = cq < 32 ? 32 / cq : 1;                 // chunks a step
+        const int grp = cq < 32 ? lane / cq : 0;
+        const int at = cq < 32 ? lane - grp * cq : lane;
+        for (int g = 0; g < grp; g++) msk &= msk - 1;           // this group's first chunk
+        int part = 0;
+        while (__any_sync(FULL, msk != 0)) {
+            constexpr int U = 2;
             int4 c4[U];
             int64_t qq[U];
 #pragma unroll
             for (int u = 0; u < U; u++) {
-                if (step == 0 && msk) {
-                    c = __ffsll((long long)msk) - 1;
-                    msk &= msk - 1;
-                    step = per;
-                }
                 qq[u] = nq;
-                if (step > 0) {
-                    int64_t q0 = (int64_t)c * (cw >> 2);
-                    int64_t q = q0 + (int64_t)(per - step) * 32 + lane;
-                    if (q < q0 + (cw >> 2)) qq[u] = q;
-                    step--;
+                if (msk) {
+                    int q = at + part * 32;
+                    if (q < cq) qq[u] = (int64_t)(__ffsll((long long)msk) - 1) * cq + q;
+                    if (++part == per) {
+                        part = 0;
+                        for (int g = 0; g < side; g++) msk &= msk - 1;
+                    }
                 }
                 c4[u] = qq[u] < nq ? row[qq[u]] : make_int4(0, 0, 0, 0);
             }

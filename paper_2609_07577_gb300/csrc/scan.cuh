@@ -16,12 +16,16 @@
 
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 namespace snn {
 
 constexpr int SCAN_CTAS = 8;            // portable cluster size
 constexpr int SCAN_THREADS = 1024;
 constexpr int SCAN_ROUNDS = 8;          // elements per thread and sweep, at most
 constexpr int64_t SCAN_CLUSTER_MAX = 1 << 17;
+constexpr int SCAN_BLOCK_ROUNDS = 4;    // elements per thread of the one-block form, at most
+constexpr int64_t SCAN_BLOCK_MAX = SCAN_BLOCK_ROUNDS * SCAN_THREADS;
 constexpr int SCT_THREADS = 256;        // three-launch form
 constexpr int SCT_ITEMS = 8;
 constexpr int SCT_TILE = SCT_THREADS * SCT_ITEMS;
@@ -134,6 +138,47 @@ __global__ void __cluster_dims__(SCAN_CTAS, 1, 1) __launch_bounds__(SCAN_THREADS
     }
     if (total && rank == 0 && threadIdx.x == 0) *total = carry;
     cl.sync();   // no block leaves while another reads its shared memory
+}
+
+// The same by one block, for the short scans of late levels: no cluster to
+// place and no cluster barriers.
+template <typename T, class In, class Out>
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_block(In in, Out out, int32_t n, T* total)
+{
+    after_previous();
+    __shared__ __align__(16) unsigned char raw[sizeof(T) * 33];
+    T* swarp = (T*)raw;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int rounds = (n + (int)blockDim.x - 1) / (int)blockDim.x;   // <= SCAN_BLOCK_ROUNDS
+    const int w0 = warp * 32 * rounds + lane;
+    T v[SCAN_BLOCK_ROUNDS], ex[SCAN_BLOCK_ROUNDS];
+#pragma unroll
+    for (int r = 0; r < SCAN_BLOCK_ROUNDS; r++) v[r] = r < rounds && w0 + r * 32 < n ? in(w0 + r * 32) : T();
+    T run = T();
+#pragma unroll
+    for (int r = 0; r < SCAN_BLOCK_ROUNDS; r++) {
+        if (r < rounds) {
+            T inc = warp_inclusive(v[r]);
+            T e = scan_shfl_up(inc, 1);
+            ex[r] = lane == 0 ? run : run + e;
+            run = run + scan_shfl(inc, 31);
+        }
+    }
+    if (lane == 0) swarp[warp] = run;
+    __syncthreads();
+    if (warp == 0) {
+        T inc = warp_inclusive(lane < nw ? swarp[lane] : T());
+        T e = scan_shfl_up(inc, 1);
+        __syncwarp();
+        swarp[lane] = lane == 0 ? T() : e;
+        if (lane == 31) swarp[32] = inc;
+    }
+    __syncthreads();
+    const T off = swarp[warp];
+#pragma unroll
+    for (int r = 0; r < SCAN_BLOCK_ROUNDS; r++)
+        if (r < rounds && w0 + r * 32 < n) out(w0 + r * 32, off + ex[r], v[r]);
+    if (total && threadIdx.x == 0) *total = swarp[32];
 }
 
 // exclusive prefix of each thread's value over the block of SCT_THREADS
@@ -260,6 +305,12 @@ Status scan_run(const In& in, const Out& out, int64_t n, T* total, Arena& ar, cu
 {
     if (n <= 0) {
         if (total) SNN_CUDA(cudaMemsetAsync(total, 0, sizeof(T), s));
+        return Status{};
+    }
+    if (n <= SCAN_BLOCK_MAX) {
+        enqueue(k_scan_block<T, In, Out>, 1, (int)std::min<int64_t>((n + 31) & ~(int64_t)31, SCAN_THREADS), 0,
+                s, in, out, (int32_t)n, total);
+        SNN_CUDA(cudaGetLastError());
         return Status{};
     }
     if (n <= SCAN_CLUSTER_MAX) {

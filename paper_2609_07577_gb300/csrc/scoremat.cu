@@ -95,7 +95,13 @@ struct ScorePol {
 
 // candidate of n: the valid neighbour with the largest score, ties to the
 // lower id (the rules of the histogram path; its skip of vertices that cannot
-// merge even with the smallest vertex finds nothing valid here either)
+// merge even with the smallest vertex finds nothing valid here either). A
+// warp per row. What bounds it on late levels (2,500 vertices, a matrix that
+// the L2 cache holds) is latency: MB_FLY loads a lane are in flight, and of
+// their entries one state is read, the largest's (testing each larger entry
+// as it came was a chain of gathers).
+constexpr int MB_FLY = 4;
+
 __global__ void __launch_bounds__(256)
     k_mat_best(Level L, const int32_t* __restrict__ Sm,
                const int32_t* __restrict__ OVm, int64_t Vs, int32_t omega, int32_t delta,
@@ -112,18 +118,44 @@ __global__ void __launch_bounds__(256)
         int32_t bk = -1;
         {
             const int4* row = reinterpret_cast<const int4*>(Sm + r0);
-            for (int64_t q = lane; 4 * q < L.V; q += 32) {
-                int4 c4 = row[q];
-                int cv[4] = {c4.x, c4.y, c4.z, c4.w};
+            for (int64_t q0 = lane; 4 * q0 < L.V; q0 += 32 * MB_FLY) {
+                int4 c4[MB_FLY];
 #pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    int32_t m = (int32_t)(4 * q + u);
-                    int64_t sc = cv[u];
-                    if (m < L.V && sc > bs && m != n && sz + L.vsize[m] <= omega &&
-                        ip + L.vinpins[m] <= phi &&
-                        ic + L.vincnt[m] - (int64_t)OVm[r0 + m] <= delta) {
-                        bs = sc;
+                for (int f = 0; f < MB_FLY; f++) {
+                    int64_t q = q0 + 32 * f;
+                    c4[f] = 4 * q < L.V ? row[q] : make_int4(0, 0, 0, 0);
+                }
+                for (;;) {
+                    // the largest entry above the best so far, the first of
+                    // equals, and only its state is read
+                    int32_t top = 0, m = -1;
+#pragma unroll
+                    for (int f = 0; f < MB_FLY; f++) {
+                        const int cv[4] = {c4[f].x, c4[f].y, c4[f].z, c4[f].w};
+#pragma unroll
+                        for (int u = 0; u < 4; u++) {
+                            int32_t mm = (int32_t)(4 * (q0 + 32 * f) + u);
+                            if (cv[u] > top && mm != n && mm < L.V) {
+                                top = cv[u];
+                                m = mm;
+                            }
+                        }
+                    }
+                    if (m < 0 || top <= bs) break;
+                    const int32_t ms = L.vsize[m], mp = L.vinpins[m], mc = L.vincnt[m], mo = OVm[r0 + m];
+                    if (sz + ms <= omega && ip + mp <= phi && ic + mc - (int64_t)mo <= delta) {
+                        bs = top;
                         bk = m;
+                        break;
+                    }
+                    // it cannot take n: the next one
+                    const int32_t e = m - (int32_t)(4 * q0);
+#pragma unroll
+                    for (int f = 0; f < MB_FLY; f++) {
+                        if (e == 128 * f) c4[f].x = 0;
+                        if (e == 128 * f + 1) c4[f].y = 0;
+                        if (e == 128 * f + 2) c4[f].z = 0;
+                        if (e == 128 * f + 3) c4[f].w = 0;
                     }
                 }
             }
@@ -172,17 +204,25 @@ __global__ void __launch_bounds__(256)
         int64_t src = (int64_t)repof[i] * Vs;
         int64_t dst = i * Vs2;
         if (fresh[i]) {
-            for (int64_t j = threadIdx.x; j < Vs2; j += blockDim.x) {
-                S2[dst + j] = 0;
-                OV2[dst + j] = 0;
+            for (int64_t j0 = 4 * threadIdx.x; j0 < Vs2; j0 += 4 * blockDim.x) {
+                *reinterpret_cast<int4*>(S2 + dst + j0) = make_int4(0, 0, 0, 0);
+                *reinterpret_cast<int4*>(OV2 + dst + j0) = make_int4(0, 0, 0, 0);
             }
             continue;
         }
-        for (int64_t j = threadIdx.x; j < V2; j += blockDim.x) {
-            int64_t c = repof[j];
-            bool f = fresh[j];
-            S2[dst + j] = f ? 0 : Sm[src + c];
-            OV2[dst + j] = f ? 0 : OVm[src + c];
+        // Vs2 is V2 up to a multiple of four: quads of entries, the gathers of
+        // one in flight together
+        for (int64_t j0 = 4 * threadIdx.x; j0 < Vs2; j0 += 4 * blockDim.x) {
+            int sv[4], ov[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                bool keep = j0 + u < V2 && !fresh[j0 + u];
+                int64_t c = keep ? src + repof[j0 + u] : src;
+                sv[u] = keep ? Sm[c] : 0;
+                ov[u] = keep ? OVm[c] : 0;
+            }
+            *reinterpret_cast<int4*>(S2 + dst + j0) = make_int4(sv[0], sv[1], sv[2], sv[3]);
+            *reinterpret_cast<int4*>(OV2 + dst + j0) = make_int4(ov[0], ov[1], ov[2], ov[3]);
         }
     }
 }
