@@ -14,7 +14,7 @@
 // Then one round of all active jobs:
 //   k_ip_best     one thread per (x, y) pair: the steepest swap, ties to
 //                 the lowest x then y, in two passes of integer atomics
-//   k_ip_update   one block per job: stop, or swap and bring G and the
+//   k_ip_update   one block or cluster per job: stop, or swap and bring G and the
 //                 matrix up to date through the hyperedges of x and y only
 //                 (G deltas, weight changes of pairs of non-moving pins,
 //                 and the rebuilt row and column of the two moved nodes)
@@ -25,6 +25,8 @@
 // the cores in Hilbert order (k_ip_hkeys and a radix sort).
 #include "internal.cuh"
 #include "initial_items.cuh"
+
+#include <cooperative_groups.h>
 
 #include <climits>
 #include <new>
@@ -228,9 +230,14 @@ struct ColAddAtomic {
     }
 };
 
-// One block per (job, start): stop when no swap lowers the cut, else swap
-// x and y and update G and the job's matrix incrementally.
-__global__ void k_ip_update(int32_t np, int64_t pairs, Jobs jb, int32_t* done, int32_t* it,
+// One cluster of C blocks per (job, start): stop when no swap lowers the cut,
+// else swap x and y and update G and the job's matrix incrementally. A thread
+// walks a hyperedge, so what bounds a round of few jobs is the number of
+// hyperedges a thread has in turn: the cluster's blocks share those of x and
+// y, with its barrier between the phases (256 nodes of about 2,000
+// hyperedges, 8 starts: one block of 512 threads 104 us a round).
+template <int C>
+__global__ void __cluster_dims__(C, 1, 1) k_ip_update(int32_t np, int64_t pairs, Jobs jb, int32_t* done, int32_t* it,
                             const int64_t* __restrict__ bd,
                             const unsigned long long* __restrict__ bxy, const int64_t* __restrict__ voff,
                             const int32_t* __restrict__ vinc, const int64_t* __restrict__ off,
@@ -239,20 +246,22 @@ __global__ void k_ip_update(int32_t np, int64_t pairs, Jobs jb, int32_t* done, i
 {
     snn::after_previous();
     __shared__ int s_mode;   // 0 skip, 1 swap then stop, 2 swap and go on
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    auto sync = [&] {
+        if (C > 1) cl.sync();
+        else __syncthreads();
+    };
     const int64_t s = blockIdx.y;
-    const int32_t k = blockIdx.x;
+    const int32_t k = blockIdx.x / C, rank = blockIdx.x % C;
     const int64_t t = s * jb.J + k;
-    if (threadIdx.x == 0) {
-        int mode = 0;
-        if (!done[t]) {
-            if (bd[t] <= 0) done[t] = 1;
-            else mode = it[t] + 1 >= jb.cap[k] ? 1 : 2;
-        }
-        s_mode = mode;
-    }
-    __syncthreads();
+    const int32_t tid = rank * blockDim.x + threadIdx.x, nt = C * blockDim.x;
+    if (threadIdx.x == 0) s_mode = done[t] ? 0 : bd[t] <= 0 ? -1 : it[t] + 1 >= jb.cap[k] ? 1 : 2;
+    sync();   // every block has read the job's state before it changes
     const int mode = s_mode;
-    if (mode == 0) return;
+    if (mode <= 0) {   // the same in the whole cluster
+        if (mode < 0 && tid == 0) done[t] = 1;
+        return;
+    }
     const int32_t lo = jb.lo[k], mid = jb.mid[k], hi = jb.hi[k], nr = hi - mid;
     const int32_t x = (int32_t)(bxy[t] >> 32), y = (int32_t)(uint32_t)bxy[t];
     int32_t* ps = pos + s * np;
@@ -264,15 +273,15 @@ __global__ void k_ip_update(int32_t np, int64_t pairs, Jobs jb, int32_t* done, i
         const int64_t nx = voff[x + 1] - voff[x], ny = voff[y + 1] - voff[y];
         GAddAtomic gadd{Gs};
         MAddAtomic madd{Mk, nr};
-        for (int64_t u = threadIdx.x; u < nx + ny; u += blockDim.x) {
+        for (int64_t u = tid; u < nx + ny; u += nt) {
             bool from_y = u >= nx;
             int32_t a = from_y ? vinc[voff[y] + (u - nx)] : vinc[voff[x] + u];
             ip::swap_hedge_update(pins, off[a], off[a + 1], ps, lo, mid, hi, x, y, eta[a], from_y,
                                   gadd, madd);
         }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    sync();
+    if (tid == 0) {
         int32_t* qs = seq + s * np;
         qs[px] = y;
         qs[py] = x;
@@ -283,15 +292,14 @@ __global__ void k_ip_update(int32_t np, int64_t pairs, Jobs jb, int32_t* done, i
         else atomicAdd(active, 1);
     }
     if (mode == 1) return;
-    __syncthreads();
     // the moved nodes' row (y now at px in L) and column (x now at py in R)
     int64_t* row = Mk + (int64_t)(px - lo) * nr;
     int64_t* col = Mk + (py - mid);
-    for (int32_t j = threadIdx.x; j < nr; j += blockDim.x) row[j] = 0;
-    for (int32_t i = threadIdx.x; i < mid - lo; i += blockDim.x) col[(int64_t)i * nr] = 0;
-    __syncthreads();
+    for (int32_t j = tid; j < nr; j += nt) row[j] = 0;
+    for (int32_t i = tid; i < mid - lo; i += nt) col[(int64_t)i * nr] = 0;
+    sync();
     const int64_t nyi = voff[y + 1] - voff[y], nxi = voff[x + 1] - voff[x];
-    for (int64_t u = threadIdx.x; u < nyi + nxi; u += blockDim.x) {
+    for (int64_t u = tid; u < nyi + nxi; u += nt) {
         if (u < nyi) {
             ip::corr_row(vinc, voff[y] + u, voff[y] + u + 1, off, pins, eta, ps, lo, mid, hi,
                          RowAddAtomic{row});
@@ -301,6 +309,10 @@ __global__ void k_ip_update(int32_t np, int64_t pairs, Jobs jb, int32_t* done, i
         }
     }
 }
+
+// jobs whose clusters of eight 256-thread blocks the GPU holds at once (152
+// SMs of eight such blocks)
+constexpr int64_t IP_SPREAD_JOBS = 152;
 
 struct Tree {
     const int32_t *lo, *hi, *par, *kid;
@@ -539,8 +551,9 @@ Status initial_impl(int32_t np, int32_t ne, const int64_t* off, const int32_t* p
     const bool warps = (int64_t)np * S >= 152 * 32;
     const int capn = 152 * 32 / S > 0 ? 152 * 32 / S : 1;
     const dim3 gnode((unsigned)grid_for(np, warps ? 8 : 1, capn), (unsigned)S);
-    // a swap's block takes one hyperedge of the two nodes per thread
-    const int updt = 2 * P / np >= 512 ? 512 : 128;
+    // a swap's threads take one hyperedge of the two nodes each: 128, 512, or a
+    // cluster of eight blocks of 256 while the jobs leave SMs idle
+    const int64_t inc2 = 2 * P / np;
     for (int32_t d = 0; d <= ht.maxd; d++) {
         const std::vector<int32_t>& js = jobs_at[d];
         if (js.empty()) continue;
@@ -584,12 +597,15 @@ Status initial_impl(int32_t np, int32_t ne, const int64_t* off, const int32_t* p
         snn::enqueue(gc, gnode, 256, 0, s, np, pairs, jb, done, voff, vinc, off, pins, eta, seq, pos,
                      G, M);
         SNN_CUDA(cudaGetLastError());
-        const dim3 gupd((unsigned)J, (unsigned)S);
+        const bool spread = inc2 >= 512 && (int64_t)J * S <= IP_SPREAD_JOBS;
+        const dim3 gupd((unsigned)(spread ? 8 * J : J), (unsigned)S);
+        const int updt = spread ? 256 : inc2 >= 512 ? 512 : 128;
+        auto update = spread ? k_ip_update<8> : k_ip_update<1>;
         for (;;) {
             snn::enqueue(k_ip_reset, gjob, 256, 0, s, S, J, done, bd, bxy, active);
             snn::enqueue(k_ip_best<0>, gpair, 256, 0, s, np, pairs, jb, done, seq, G, M, bd, bxy);
             snn::enqueue(k_ip_best<1>, gpair, 256, 0, s, np, pairs, jb, done, seq, G, M, bd, bxy);
-            snn::enqueue(k_ip_update, gupd, updt, 0, s, np, pairs, jb, done, it, bd, bxy, voff, vinc,
+            snn::enqueue(update, gupd, updt, 0, s, np, pairs, jb, done, it, bd, bxy, voff, vinc,
                          off, pins, eta, seq, pos, G, M, active);
             SNN_CUDA(cudaGetLastError());
             int32_t hact = 0;

@@ -2158,7 +2158,8 @@ struct IncState {
 };
 
 // saves and W of the listed vertices (cleared before) from their hyperedges;
-// the four blocks of a column share a vertex's incidences
+// the 4 to 64 blocks of a column share a vertex's incidences, so that the one
+// heavy pair of a tail level is not a chain of gathers on a few warps
 __global__ void __launch_bounds__(256)
     k_save_members(Level L, PinCounts pc, const int32_t* __restrict__ rho,
                    const int32_t* __restrict__ list, const int32_t* __restrict__ nlist, int64_t* savev,
@@ -2170,20 +2171,17 @@ __global__ void __launch_bounds__(256)
     for (int32_t x = blockIdx.x; x < nl; x += gridDim.x) {
         const int32_t n = list[x];
         const int64_t vb = L.voff[n], ve = L.voff[n + 1];
-        if (vb + (int64_t)blockIdx.y * 1024 >= ve) continue;   // the whole block
+        if (vb + (int64_t)blockIdx.y * 256 >= ve) continue;   // the whole block
         if (threadIdx.x < 2) sum[threadIdx.x] = 0;
         __syncthreads();
         const int32_t p = rho[n];
         int64_t W = 0, save = 0;
-        for (int64_t t = vb + (int64_t)blockIdx.y * 1024; t < ve; t += 4 * 1024) {
-            const int64_t te = t + 1024 < ve ? t + 1024 : ve;
-            for (int64_t i = t + threadIdx.x; i < te; i += 256) {
-                HRec r = pc.rec[(int32_t)((uint32_t)L.vinc[i] & ~SRC_BIT)];
-                W += r.w;
-                int32_t c, d;
-                lookup_count(pc, r.b, r.n(), p, c, d);
-                if (c == 1) save += r.w;
-            }
+        for (int64_t i = vb + (int64_t)blockIdx.y * 256 + threadIdx.x; i < ve; i += (int64_t)gridDim.y * 256) {
+            HRec r = pc.rec[(int32_t)((uint32_t)L.vinc[i] & ~SRC_BIT)];
+            W += r.w;
+            int32_t c, d;
+            lookup_count(pc, r.b, r.n(), p, c, d);
+            if (c == 1) save += r.w;
         }
         W = warp_sum(W);
         save = warp_sum(save);
@@ -2246,7 +2244,9 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
         prof.reset(new ProfScope(h, PS_SAVE));
         if (inc.mlist) {
             if (inc.members > 0)
-                enqueue(k_save_members, dim3((unsigned)std::min<int64_t>(inc.members, 152 * 16), 4),
+                enqueue(k_save_members,
+                        dim3((unsigned)std::min<int64_t>(inc.members, 152 * 16),
+                             (unsigned)std::min<int64_t>(std::max<int64_t>(152 * 8 / inc.members, 4), 64)),
                         256, 0, s, L, pc, rho, inc.mlist, inc.mcnt, savev, Wv);
             SNN_CUDA(cudaGetLastError());
         } else if (L.E > 0 && !h->wide && V <= SAVE_SMEM_V) {

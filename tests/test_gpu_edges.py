@@ -196,3 +196,30 @@ def test_equal_content_keys():
     hg = _net("equalkeys", V, [(0, [1]), (x, a + 1), (x, b + 1), (x, [y]), (y, [x])], [7, 3, 5, 2, 1],
               64, 64, 1)
     assert lockstep(hg, max_levels=1) == 1
+
+
+@pytest.mark.parametrize("starts", [1, 3, 40])
+@pytest.mark.parametrize("n, hedges", [(21, 5400), (21, 1600), (64, 1500)])
+def test_initial_placement_swaps(n, hedges, starts):
+    """Swaps of nodes with at least 512 hyperedges a pair: a cluster per job
+    while there are few jobs, a block with more (40 starts at the deeper
+    levels) or with fewer hyperedges."""
+    import paper_2609_07577_gb300 as P
+    rng = np.random.default_rng(n + hedges)
+    pins, off = [], [0]
+    for _ in range(hedges):
+        p = rng.choice(n, int(rng.integers(2, 5)), replace=False)
+        pins.append(p)
+        off.append(off[-1] + p.size)
+    off, pins = np.asarray(off, np.int64), np.concatenate(pins).astype(np.int32)
+    eta = rng.integers(1, 30, hedges).astype(np.int64)
+    width = height = 8
+    seq0 = np.stack([rng.permutation(n) for _ in range(starts)]).astype(np.int32)
+    gamma = torch.empty((starts, n), dtype=torch.int32, device="cuda")
+    P.snnmap_place_initial(n, hedges, torch.tensor(off).cuda(), torch.tensor(pins).cuda(),
+                           torch.tensor(eta).cuda(), width, height, starts,
+                           torch.tensor(seq0).cuda(), gamma)
+    torch.cuda.synchronize()
+    got = gamma.cpu().numpy()
+    for s in range(starts):
+        assert np.array_equal(got[s], oracle.initial_placement(n, off, pins, eta, width, height, seq0[s]))
