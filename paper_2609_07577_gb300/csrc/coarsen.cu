@@ -79,9 +79,13 @@ struct AffPol {
         if (rec) return rec[a].n();
         return L.hoff[a + 1] - L.hoff[a];
     }
-    __device__ Seg<S> seg(int64_t i, Acc&) const
+    __device__ uint32_t inc(int64_t i) const { return (uint32_t)L.vinc[i]; }
+    __device__ void fetch(uint32_t inc) const
     {
-        uint32_t inc = (uint32_t)L.vinc[i];
+        if (rec) prefetch_l1(rec + (inc & ~SRC_BIT));
+    }
+    __device__ Seg<S> seg(uint32_t inc, Acc&) const
+    {
         int32_t a = (int32_t)(inc & ~SRC_BIT);
         if (rec) return rec_seg<S>(rec[a], inc);
         Seg<S> g;
@@ -625,9 +629,10 @@ struct AffNewPol {
     {
         return rec[(int32_t)((uint32_t)L.vinc[i] & ~SRC_BIT)].n();
     }
-    __device__ Seg<S> seg(int64_t i, Acc&) const
+    __device__ uint32_t inc(int64_t i) const { return (uint32_t)L.vinc[i]; }
+    __device__ void fetch(uint32_t inc) const { prefetch_l1(rec + (inc & ~SRC_BIT)); }
+    __device__ Seg<S> seg(uint32_t inc, Acc&) const
     {
-        uint32_t inc = (uint32_t)L.vinc[i];
         return rec_seg<S>(rec[(int32_t)(inc & ~SRC_BIT)], inc);
     }
     struct Item {

@@ -34,7 +34,9 @@
 //                                                   written by write(n, 0, -1, 0, Acc()))
 //   __device__ int64_t seg_len(int64_t i)           segment length of incidence i
 //   __device__ int64_t vb(n), ve(n)                 incidence range of vertex n
-//   __device__ Seg<S> seg(int64_t i, Acc&)          segment of incidence i
+//   __device__ uint32_t inc(int64_t i)              incidence i's word (hyperedge, source bit)
+//   __device__ Seg<S> seg(uint32_t inc, Acc&)       its segment
+//   __device__ void fetch(uint32_t inc)             brings what seg reads into the L1 cache
 //   struct Own, Own own(n)                          what load reads of the visiting vertex
 //   struct Item, Item load(n, Own, const Seg<S>&, off)  one element's reads; none() an empty Item
 //   __device__ bool put(n, const Item&, table, Acc&)  its table update
@@ -106,6 +108,11 @@ struct Table {
         return false;
     }
 };
+
+__device__ __forceinline__ void prefetch_l1(const void* p)
+{
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+}
 
 template <typename S>
 __host__ __device__ constexpr size_t slot_bytes()
@@ -225,7 +232,7 @@ __device__ bool warp_visit(const Pol& pol, int32_t n, int64_t vb, int64_t ve, co
     for (int64_t ib = vb; ib < ve; ib += 32) {
         int64_t i = ib + lane;
         Seg<S> sg{};
-        if (i < ve) sg = pol.seg(i, acc);
+        if (i < ve) sg = pol.seg(pol.inc(i), acc);
         int32_t pre = sg.len;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -300,11 +307,14 @@ __device__ __forceinline__ int group_log(int64_t deg, int64_t work)
 // of their group are finished by its whole warp; those longer than T go to
 // slong (if any) for the whole block, which would otherwise wait for one of
 // its warps (a vertex of the 1,048,576-neuron power-law network meets 47
-// pins a hyperedge on average, but up to 16,384). Returns false in lanes
-// whose insert failed.
+// pins a hyperedge on average, but up to 16,384). AHEAD: the next pass's
+// records are brought into the L1 cache and the words of the one after it are
+// read while a pass runs, for blocks that have an SM to themselves, where a
+// pass is a chain of three gathers (word, record, element). Returns false in
+// lanes whose insert failed.
 constexpr int HT_NLONG = 256;
 
-template <typename S, int T, int U, class Pol, class Tb>
+template <typename S, int T, int U, bool AHEAD, class Pol, class Tb>
 __device__ __forceinline__ bool group_visit(const Pol& pol, int32_t n, int64_t vb, int64_t ve,
                                             int glog, int tid, const Tb& t,
                                             typename Pol::Acc& acc, int64_t* slong = nullptr,
@@ -312,9 +322,19 @@ __device__ __forceinline__ bool group_visit(const Pol& pol, int32_t n, int64_t v
 {
     const int lane = tid & 31, G = 1 << glog, gl = lane & (G - 1);
     const int grp = tid >> glog, ngrp = T >> glog;
+    const bool longs = pol.L.maxlen > 8 * G || pol.L.maxlen > T;   // else no segment needs others' lanes
     bool ok = true;
     const typename Pol::Own own = pol.own(n);
     typename Pol::Acc other;   // a segment's own terms count once, in its first lane
+    uint32_t wd[AHEAD ? U : 1], wd2[AHEAD ? U : 1];   // words of this pass and the next
+    if (AHEAD) {
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            int64_t i = vb + (int64_t)u * ngrp + grp;
+            wd[u] = i < ve ? pol.inc(i) : 0u;
+            wd2[u] = i + (int64_t)U * ngrp < ve ? pol.inc(i + (int64_t)U * ngrp) : 0u;
+        }
+    }
     for (int64_t base = vb; base < ve; base += (int64_t)U * ngrp) {
         Seg<S> g[U];
         typename Pol::Item it[U];
@@ -322,9 +342,19 @@ __device__ __forceinline__ bool group_visit(const Pol& pol, int32_t n, int64_t v
         for (int u = 0; u < U; u++) {
             int64_t i = base + (int64_t)u * ngrp + grp;
             g[u] = Seg<S>{};
-            if (i < ve) g[u] = pol.seg(i, gl == 0 ? acc : other);
+            if (i < ve) g[u] = pol.seg(AHEAD ? wd[u] : pol.inc(i), gl == 0 ? acc : other);
         }
-        if (slong) {
+        if (AHEAD) {
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                int64_t i = base + (int64_t)(U + u) * ngrp + grp;
+                wd[u] = wd2[u];
+                if (i < ve) pol.fetch(wd[u]);
+                i += (int64_t)U * ngrp;
+                wd2[u] = i < ve ? pol.inc(i) : 0u;
+            }
+        }
+        if (slong && longs) {
 #pragma unroll
             for (int u = 0; u < U; u++) {
                 bool lg = g[u].len > T;
@@ -345,7 +375,7 @@ __device__ __forceinline__ bool group_visit(const Pol& pol, int32_t n, int64_t v
         for (int u = 0; u < U; u++) ok = pol.put(n, it[u], t, acc) && ok;
 #pragma unroll
         for (int u = 0; u < U; u++) {
-            const bool lg = G < 32 && g[u].len > 8 * G;
+            const bool lg = longs && G < 32 && g[u].len > 8 * G;
             if (!lg) {
                 for (int32_t off = gl + G; off < g[u].len; off += 2 * G) {
                     typename Pol::Item a = pol.load(n, own, g[u], off);
@@ -355,7 +385,7 @@ __device__ __forceinline__ bool group_visit(const Pol& pol, int32_t n, int64_t v
                     ok = pol.put(n, b, t, acc) && ok;
                 }
             }
-            unsigned m = G < 32 ? __ballot_sync(FULL, lg && gl == 0) : 0u;
+            unsigned m = longs && G < 32 ? __ballot_sync(FULL, lg && gl == 0) : 0u;
             while (m) {
                 int src = __ffs(m) - 1;
                 m &= m - 1;
@@ -826,7 +856,7 @@ __global__ void __launch_bounds__(T, CAP <= 2048 ? HT_BLOCKS : 1)
         if (flat) {
             if (threadIdx.x < FLAT) {   // whole warps
                 Seg<S> g{};
-                if ((int)threadIdx.x < deg) g = pol.seg(vb + threadIdx.x, acc);
+                if ((int)threadIdx.x < deg) g = pol.seg(pol.inc(vb + threadIdx.x), acc);
                 sseg[threadIdx.x] = g;
                 wsum = g.w;
                 ksum = g.k;
@@ -842,7 +872,7 @@ __global__ void __launch_bounds__(T, CAP <= 2048 ? HT_BLOCKS : 1)
         } else if (sizeof(S) == 4) {
             Acc other;
             for (int64_t i = vb + threadIdx.x; i < ve; i += T) {
-                Seg<S> g = pol.seg(i, other);
+                Seg<S> g = pol.seg(pol.inc(i), other);
                 wsum += g.w;
                 ksum += g.k;
             }
@@ -901,12 +931,12 @@ __global__ void __launch_bounds__(T, CAP <= 2048 ? HT_BLOCKS : 1)
             return k;
         };
         auto visit_groups = [&](const auto& tb) {
-            bool k = group_visit<S, T, 1>(pol, n, vb, ve, glog, threadIdx.x, tb, acc, slong, &nlong);
+            bool k = group_visit<S, T, 1, false>(pol, n, vb, ve, glog, threadIdx.x, tb, acc, slong, &nlong);
             __syncthreads();
             const int nlg = nlong < HT_NLONG ? nlong : HT_NLONG;
             Acc other;   // the segments' own terms are in already
             for (int x = 0; x < nlg && k; x++) {
-                Seg<S> g = pol.seg(slong[x], other);
+                Seg<S> g = pol.seg(pol.inc(slong[x]), other);
                 for (int32_t off = threadIdx.x; off < g.len && k; off += 2 * T) {
                     typename Pol::Item a = pol.load(n, own, g, off);
                     typename Pol::Item b = off + T < g.len ? pol.load(n, own, g, off + T) : Pol::none();
@@ -1030,11 +1060,11 @@ __device__ __forceinline__ void dense_count(const Pol& pol, int32_t n, int64_t v
     using Acc = typename Pol::Acc;
     const typename Pol::Own own = pol.own(n);
     Acc acc, other;
-    group_visit<S, T, 4>(pol, n, vb, ve, glog, threadIdx.x, t, acc, slong, nlong);
+    group_visit<S, T, 2, true>(pol, n, vb, ve, glog, threadIdx.x, t, acc, slong, nlong);
     __syncthreads();
     const int nlg = *nlong < HT_NLONG ? *nlong : HT_NLONG;
     for (int x = 0; x < nlg; x++) {
-        Seg<S> g = pol.seg(slong[x], other);   // its own terms are in already
+        Seg<S> g = pol.seg(pol.inc(slong[x]), other);   // its own terms are in already
         for (int32_t off = threadIdx.x; off < g.len; off += T)
             pol.put(n, pol.load(n, own, g, off), t, acc);
     }
@@ -1381,11 +1411,11 @@ __global__ void __launch_bounds__(HT_WARPS * 32)
             Table<S> p = priv;
             p.mask = (uint32_t)(scap[j] - 1);
             p.probes = (uint32_t)scap[j];
-            ok = __all_sync(FULL, (group_visit<S, 32, 2>(pol, n, vb, ve, glog, lane, p, acc)));
+            ok = __all_sync(FULL, (group_visit<S, 32, 2, false>(pol, n, vb, ve, glog, lane, p, acc)));
             __syncwarp();
             ok = flush_private(p, scap[j], g) && ok;
         } else {
-            ok = __all_sync(FULL, (group_visit<S, 32, 2>(pol, n, vb, ve, glog, lane, g, acc)));
+            ok = __all_sync(FULL, (group_visit<S, 32, 2, false>(pol, n, vb, ve, glog, lane, g, acc)));
         }
         if (!ok && lane == 0) ovf[j] = 1;
         Acc wa = Pol::warp_reduce(acc);

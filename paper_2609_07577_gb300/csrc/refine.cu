@@ -388,9 +388,10 @@ struct GainPol {
     {
         return pc.lam[(int32_t)((uint32_t)L.vinc[i] & ~SRC_BIT)];
     }
-    __device__ Seg<S> seg(int64_t i, Acc& acc) const
+    __device__ uint32_t inc(int64_t i) const { return (uint32_t)L.vinc[i]; }
+    __device__ void fetch(uint32_t inc) const { prefetch_l1(pc.rec + (inc & ~SRC_BIT)); }
+    __device__ Seg<S> seg(uint32_t inc, Acc& acc) const
     {
-        uint32_t inc = (uint32_t)L.vinc[i];
         HRec r = pc.rec[(int32_t)(inc & ~SRC_BIT)];
         acc.W += r.w;
         return rec_seg<S>(r, inc);
@@ -509,9 +510,10 @@ struct RowPol {
     {
         return pc.lam[(int32_t)((uint32_t)L.vinc[i] & ~SRC_BIT)];
     }
-    __device__ Seg<S> seg(int64_t i, Acc&) const
+    __device__ uint32_t inc(int64_t i) const { return (uint32_t)L.vinc[i]; }
+    __device__ void fetch(uint32_t inc) const { prefetch_l1(pc.rec + (inc & ~SRC_BIT)); }
+    __device__ Seg<S> seg(uint32_t inc, Acc&) const
     {
-        uint32_t inc = (uint32_t)L.vinc[i];
         return rec_seg<S>(pc.rec[(int32_t)(inc & ~SRC_BIT)], inc);
     }
     struct Item {

@@ -49,9 +49,17 @@ struct ScorePol {
         int32_t a = (int32_t)((uint32_t)L.vinc[i] & ~SRC_BIT);
         return L.hoff[a + 1] - L.hoff[a];
     }
-    __device__ Seg<S> seg(int64_t i, Acc&) const
+    __device__ uint32_t inc(int64_t i) const { return (uint32_t)L.vinc[i]; }
+    __device__ void fetch(uint32_t inc) const
     {
-        uint32_t inc = (uint32_t)L.vinc[i];
+        int32_t a = (int32_t)(inc & ~SRC_BIT);
+        prefetch_l1(L.hoff + a);
+        prefetch_l1(L.hw + a);
+        prefetch_l1(L.hk + a);
+        prefetch_l1(L.hsd + a);
+    }
+    __device__ Seg<S> seg(uint32_t inc, Acc&) const
+    {
         int32_t a = (int32_t)(inc & ~SRC_BIT);
         Seg<S> g;
         g.sd = L.hsd[a];
