@@ -75,6 +75,7 @@ __device__ __forceinline__ uint32_t table_slot(int32_t m, uint32_t mask)
 // Open-addressing slots: key (-1 empty), summed weight, summed overlap.
 template <typename S>
 struct Table {
+    static constexpr bool kFills = true;   // an insert can fail
     int32_t* key;
     S* sc;
     uint32_t* ov;
@@ -182,8 +183,13 @@ __device__ __forceinline__ Seg<S> rec_seg(const HRec& r, uint32_t inc)
 // bits: one shared-memory atomic an element instead of two. LIST: the slots
 // in use are listed, so the result of a large table costs a read per key
 // instead of one per slot.
+// CLAIM: a slot is tried by compare-and-swap at once instead of being read
+// first, for vertices of few long incidences, whose keys are mostly new
+// (power-law level 0: 24.3 -> 23.0 ms; the conv network's, whose pins repeat,
+// 31.4 -> 32.7 ms that way).
 template <bool LIST, bool CLAIM = false>
 struct PackedTable {
+    static constexpr bool kFills = true;
     int32_t* key;
     uint32_t* val;
     uint16_t* used;    // LIST: slots in use, *nused of them
@@ -404,7 +410,7 @@ __device__ __forceinline__ bool group_visit(const Pol& pol, int32_t n, int64_t v
                     ok = pol.put(n, pol.load(n, own, w, off), t, acc) && ok;
             }
         }
-        if (!__all_sync(FULL, ok)) break;
+        if (Tb::kFills && !__all_sync(FULL, ok)) break;
     }
     return ok;
 }
@@ -784,6 +790,9 @@ __device__ __forceinline__ int32_t seg_find(const int32_t* spre, int32_t n, int3
 // Held to 32 registers so that eight blocks share an SM: at 6 blocks (40
 // registers) the two networks above take 36.8 and 20.1 ms, at 5 39.5 and
 // 21.5, at 8 31.9 and 19.2, a few spilled words included.
+// (Their scratch is shared so that it fits: with quads in the table's scan,
+// one segment a group in flight and no checks for long segments where the
+// level has none, 28.1 and 17.0 ms.)
 constexpr int HT_BLOCKS = 8;
 
 template <class Pol, int T, int CAP, int TIER, int NEXT>
@@ -1038,6 +1047,7 @@ constexpr int64_t HT_DENSE_BWORK = 8192;       // most elements a 256-thread blo
 
 template <typename S>
 struct DenseTable {
+    static constexpr bool kFills = false;
     S* sc;
     uint32_t* ov;
     __device__ __forceinline__ bool add(int32_t m, S w, uint32_t o) const

@@ -235,7 +235,8 @@ struct ColAddAtomic {
 // walks a hyperedge, so what bounds a round of few jobs is the number of
 // hyperedges a thread has in turn: the cluster's blocks share those of x and
 // y, with its barrier between the phases (256 nodes of about 2,000
-// hyperedges, 8 starts: one block of 512 threads 104 us a round).
+// hyperedges, 64 starts: 104 us a round by one block of 512 threads, 46 us by
+// a cluster of eight blocks of 256).
 template <int C>
 __global__ void __cluster_dims__(C, 1, 1) k_ip_update(int32_t np, int64_t pairs, Jobs jb, int32_t* done, int32_t* it,
                             const int64_t* __restrict__ bd,
@@ -311,7 +312,8 @@ __global__ void __cluster_dims__(C, 1, 1) k_ip_update(int32_t np, int64_t pairs,
 }
 
 // jobs whose clusters of eight 256-thread blocks the GPU holds at once (152
-// SMs of eight such blocks)
+// SMs of eight such blocks); with more, clusters and single blocks take the
+// same time (512 jobs: 143 us a round either way)
 constexpr int64_t IP_SPREAD_JOBS = 152;
 
 struct Tree {

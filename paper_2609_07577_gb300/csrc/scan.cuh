@@ -2,8 +2,8 @@
 // results consumed on the fly (Out), so that the kernels around a scan need
 // no flag, length or index array of their own.
 //
-// Up to SCAN_CLUSTER_MAX elements one cluster of 8 blocks does the whole
-// scan in one launch: a thread block cluster's barrier is a hardware one (no
+// Up to SCAN_BLOCK_MAX elements one block does the whole scan (k_scan_block),
+// up to SCAN_CLUSTER_MAX one cluster of 8 blocks in one launch: a thread block cluster's barrier is a hardware one (no
 // flag in memory to spin on or to clear) and the blocks' totals are
 // exchanged through distributed shared memory. What bounds a scan of a
 // level's arrays is not bandwidth but launches: the reduce/scan/tile form
@@ -141,7 +141,10 @@ __global__ void __cluster_dims__(SCAN_CTAS, 1, 1) __launch_bounds__(SCAN_THREADS
 }
 
 // The same by one block, for the short scans of late levels: no cluster to
-// place and no cluster barriers.
+// place and no cluster barriers. Four elements a thread is where the block's
+// own work has eaten that up (proposals' scan of the power-law networks'
+// levels of 50 to 4,000 vertices: 9.4 us by a cluster, 4.1 by a block; counts
+// of 6,000 take 10.9 by a cluster).
 template <typename T, class In, class Out>
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_block(In in, Out out, int32_t n, T* total)
 {

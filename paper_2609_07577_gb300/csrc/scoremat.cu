@@ -107,7 +107,8 @@ struct ScorePol {
 // warp per row. What bounds it on late levels (2,500 vertices, a matrix that
 // the L2 cache holds) is latency: MB_FLY loads a lane are in flight, and of
 // their entries one state is read, the largest's (testing each larger entry
-// as it came was a chain of gathers).
+// as it came was a chain of gathers: 28.0 us a level of the conv network of
+// 65,536 neurons, 13.2 so).
 constexpr int MB_FLY = 4;
 
 __global__ void __launch_bounds__(256)
