@@ -87,8 +87,6 @@ __device__ __forceinline__ unsigned lanemask_lt()
     return m;
 }
 
-__device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
-
 // 64-bit finalizer (splitmix64) used for hyperedge content hashes and
 // hash-table probing; only ever compared for equality, never for results.
 __host__ __device__ __forceinline__ uint64_t mix64(uint64_t x)

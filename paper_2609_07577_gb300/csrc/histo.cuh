@@ -465,7 +465,6 @@ constexpr int HT_WLOAD = HT_WCAP * 3 / 4;
 constexpr int HT_BTHREADS = 256;
 constexpr int HT_BCAP = 2048;           // block table slots
 constexpr int HT_GTHREADS = 512;        // big-block tier
-constexpr int64_t HT_CHUNK = 1024;      // incidences per split-tier work item
 enum : int { HT_TIER_WARP = 0, HT_TIER_BLOCK = 1, HT_TIER_BIG = 2, HT_TIER_SPLIT = 3, HT_NTIER = 4 };
 // counters of run_histogram: per-tier vertex counts, then the summed work and
 // the number of vertices given a histogram (not skipped)

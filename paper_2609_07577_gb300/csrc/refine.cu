@@ -126,6 +126,7 @@ struct PinCountJob {
     int32_t K = 0;     // words kept per block; 0: add to pincnt directly
     int32_t cost_mask = COST_SLOTS - 1;
     uint32_t* acc = nullptr;
+    static constexpr int kSharedWords = PC_SMEM_K;
     __host__ __device__ int shared_words() const { return K; }
     __device__ void attach(uint32_t* w) { acc = K > 0 ? w : nullptr; }
     __device__ void flush() const

@@ -19,8 +19,9 @@
 //                                                   (key i at s[i * st])
 //        the same, run by a single thread
 // and optionally kShared = true with
-//   int shared_words() const                     32-bit words of shared memory a block keeps
-//                                                for it (0: none), zero on entry
+//   static constexpr int kSharedWords            most 32-bit words of shared memory a block
+//                                                keeps for it, over all jobs of the type
+//   int shared_words() const                     those of this job (0: none), zero on entry
 //   __device__ void attach(uint32_t* words)      that memory, before any finish
 //   __device__ void flush() const                run by the whole block after its lists
 #pragma once
@@ -338,9 +339,11 @@ Status seg_run(const Job& job, const SegBuckets& b, int32_t E, Arena& ar, cudaSt
     int gb0 = count(SEG_BB0) > 0 ? grid_for(count(SEG_BB0), 8, cap) : 0;
     int gb1 = count(SEG_BB1) > 0 ? grid_for(count(SEG_BB1), 8, cap) : 0;
     if (gt + gb0 + gb1 > 0) {
-        if (dyn)
+        // the type's most, not this job's: the attribute is the kernel's, and a
+        // handle on another host thread may set it between here and the launch
+        if constexpr (seg_shared<Job>::value)
             SNN_CUDA(cudaFuncSetAttribute(k_seg_small<Job>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)dyn));
+                                          Job::kSharedWords * (int)sizeof(uint32_t)));
         enqueue(k_seg_small<Job>, gt + gb0 + gb1, 256, dyn, s, job, b.list, b.meta, gt, gb0);
         SNN_CUDA(cudaGetLastError());
     }

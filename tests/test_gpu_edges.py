@@ -223,3 +223,24 @@ def test_initial_placement_swaps(n, hedges, starts):
     got = gamma.cpu().numpy()
     for s in range(starts):
         assert np.array_equal(got[s], oracle.initial_placement(n, off, pins, eta, width, height, seq0[s]))
+
+
+def test_batch_of_uneven_partition_counts():
+    """Jobs at once whose kernels keep different amounts of shared memory a
+    block: each result equals the handle's own pass."""
+    import dataclasses
+    from paper_2609_07577_gb300 import HGraph, batch_partition
+    hgs = []
+    for name in ("cfg1", "cfg2s"):
+        hg = snngen.by_name(name)
+        for f in (1, 3, 8, 20, 40, 64):
+            hgs.append(dataclasses.replace(hg, omega=hg.omega * f, delta=hg.delta * f, phi=hg.phi * f))
+    rc, rs = batch_partition(hgs, slots=6)
+    assert rc == 0, [r.get("error") for r in rs]
+    for hg, r in zip(hgs, rs):
+        G = HGraph.from_hypergraph(hg)
+        rho, cost, _ = G.partition()
+        G.close()
+        assert r["cost"] == cost
+        assert np.array_equal(np.asarray(r["rho"].cpu() if hasattr(r["rho"], "cpu") else r["rho"]),
+                              rho.cpu().numpy())
