@@ -255,7 +255,8 @@ Status scan_inclusive_i32(const int32_t* in, int32_t* out, int64_t n, Arena& ar,
 Status scan_inclusive_max_i32(const int32_t* in, int32_t* out, int64_t n, Arena& ar,
                               cudaStream_t s);
 
-// Stable LSD radix sort of (key, value) pairs over key bits [0, end_bit).
+// Stable LSD radix sort of (key, value) pairs over key bits [0, end_bit):
+// higher bits take no part in the order and stay in their keys.
 // Sorted data ends in (keys, vals); the *_alt buffers are scratch of size n.
 Status radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t* vals_alt,
                         int64_t n, int end_bit, Arena& ar, cudaStream_t s);

@@ -279,8 +279,14 @@ constexpr int RS_WARPS = RS_THREADS / 32;
 constexpr int RS_ROUNDS = 16;
 constexpr int RS_TILE = RS_THREADS * RS_ROUNDS;
 
+// the bits of the digit at `shift` that lie below end_bit
+__host__ __device__ __forceinline__ uint32_t digit_mask(int shift, int end_bit)
+{
+    return end_bit - shift < 8 ? (1u << (end_bit - shift)) - 1 : 255u;
+}
+
 __global__ void __launch_bounds__(RS_THREADS)
-    k_rs_upsweep(const uint64_t* keys, int64_t n, int shift, uint32_t* counts, int nblk)
+    k_rs_upsweep(const uint64_t* keys, int64_t n, int shift, uint32_t dmask, uint32_t* counts, int nblk)
 {
     after_previous();
     __shared__ uint32_t hist[256];
@@ -289,7 +295,7 @@ __global__ void __launch_bounds__(RS_THREADS)
     int64_t base = (int64_t)blockIdx.x * RS_TILE;
     for (int i = threadIdx.x; i < RS_TILE; i += RS_THREADS) {
         int64_t j = base + i;
-        if (j < n) atomicAdd(&hist[(keys[j] >> shift) & 255], 1u);
+        if (j < n) atomicAdd(&hist[(keys[j] >> shift) & dmask], 1u);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < 256; i += RS_THREADS) counts[(int64_t)i * nblk + blockIdx.x] = hist[i];
@@ -297,7 +303,7 @@ __global__ void __launch_bounds__(RS_THREADS)
 
 __global__ void __launch_bounds__(RS_THREADS)
     k_rs_downsweep(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout,
-                   int64_t n, int shift, const uint32_t* offs, int nblk)
+                   int64_t n, int shift, uint32_t dmask, const uint32_t* offs, int nblk)
 {
     after_previous();
     __shared__ uint32_t wcnt[RS_WARPS][256];
@@ -316,7 +322,7 @@ __global__ void __launch_bounds__(RS_THREADS)
         int64_t j = base + r * 32 + lane;
         bool valid = j < n;
         k[r] = valid ? kin[j] : 0;
-        uint32_t d = valid ? (uint32_t)((k[r] >> shift) & 255) : 256u;
+        uint32_t d = valid ? (uint32_t)((k[r] >> shift) & dmask) : 256u;
         unsigned peers = __match_any_sync(FULL, d);
         int leader = __ffs(peers) - 1;
         if (lane == leader && valid) {
@@ -343,7 +349,7 @@ __global__ void __launch_bounds__(RS_THREADS)
     for (int r = 0; r < RS_ROUNDS; r++) {
         int64_t j = base + r * 32 + lane;
         if (j < n) {
-            uint32_t d = (uint32_t)((k[r] >> shift) & 255);
+            uint32_t d = (uint32_t)((k[r] >> shift) & dmask);
             uint32_t pos = wcnt[warp][d] + rank[r];
             kout[pos] = k[r];
             vout[pos] = vin[j];
@@ -366,7 +372,7 @@ constexpr int64_t RSC_MAX = (int64_t)RSC_CTAS * RSC_THREADS * RSC_ROUNDS;   // 9
 
 __global__ void __cluster_dims__(RSC_CTAS, 1, 1) __launch_bounds__(RSC_THREADS)
     k_rs_cluster(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t* vals_alt, int32_t n,
-                 int passes)
+                 int end_bit)
 {
     after_previous();
     namespace cg = cooperative_groups;
@@ -384,8 +390,8 @@ __global__ void __cluster_dims__(RSC_CTAS, 1, 1) __launch_bounds__(RSC_THREADS)
     const int w0 = (rank * RSC_THREADS + warp * 32) * rounds;
     uint64_t *ki = keys, *ko = keys_alt;
     uint32_t *vi = vals, *vo = vals_alt;
-    for (int p = 0; p < passes; p++) {
-        const int shift = 8 * p;
+    for (int shift = 0; shift < end_bit; shift += 8) {
+        const uint32_t dmask = digit_mask(shift, end_bit);
         for (int i = threadIdx.x; i < RSC_WARPS * 256; i += RSC_THREADS) (&wcnt[0][0])[i] = 0;
         if (threadIdx.x == 0) same = 0;
         uint64_t k[RSC_ROUNDS];
@@ -401,7 +407,7 @@ __global__ void __cluster_dims__(RSC_CTAS, 1, 1) __launch_bounds__(RSC_THREADS)
         for (int r = 0; r < RSC_ROUNDS; r++) {
             if (r >= rounds) continue;   // the same for the whole cluster
             bool valid = w0 + r * 32 + lane < n;
-            uint32_t d = valid ? (uint32_t)((k[r] >> shift) & 255) : 256u;
+            uint32_t d = valid ? (uint32_t)((k[r] >> shift) & dmask) : 256u;
             unsigned peers = __match_any_sync(FULL, d);
             int leader = __ffs(peers) - 1;
             if (lane == leader && valid) {
@@ -449,7 +455,7 @@ __global__ void __cluster_dims__(RSC_CTAS, 1, 1) __launch_bounds__(RSC_THREADS)
             for (int r = 0; r < RSC_ROUNDS; r++) {
                 int j = w0 + r * 32 + lane;
                 if (r < rounds && j < n) {
-                    uint32_t d = (uint32_t)((k[r] >> shift) & 255);
+                    uint32_t d = (uint32_t)((k[r] >> shift) & dmask);
                     uint32_t pos = goff[d] + wcnt[warp][d] + rk[r];
                     __stcg((unsigned long long*)&ko[pos], (unsigned long long)k[r]);
                     __stcg(&vo[pos], __ldcg(&vi[j]));
@@ -475,33 +481,38 @@ __global__ void __cluster_dims__(RSC_CTAS, 1, 1) __launch_bounds__(RSC_THREADS)
 }
 
 // Up to SB_MAX items one block sorts in shared memory: a bitonic network over
-// the words key << ibits | position, whose order is the stable order of the
-// keys. A refinement round sorts its moves and its events, mostly a few
+// the words key << ibits | position, the key cut to the bits that order it,
+// whose order is the stable order of the keys; whole keys and values then move
+// by position. A refinement round sorts its moves and its events, mostly a few
 // hundred to a few thousand of each, and there even one launch of the radix
 // passes is a chain of barriers: 1,000 keys of 20 bits take 24 us in the
 // cluster form.
 __global__ void __launch_bounds__(SB_THREADS)
-    k_sort_block(uint64_t* keys, uint32_t* vals, int32_t n, int N, int ibits)
+    k_sort_block(uint64_t* keys, uint32_t* vals, int32_t n, int N, int ibits, uint64_t kmask)
 {
     after_previous();
     __shared__ uint64_t w[SB_MAX];
+    uint64_t k[SB_MAX / SB_THREADS];
     uint32_t v[SB_MAX / SB_THREADS];
     const uint64_t imask = (1ull << ibits) - 1;
     for (int i = threadIdx.x; i < N; i += SB_THREADS)
-        w[i] = i < n ? (keys[i] << ibits) | (uint64_t)i : ~0ull;
+        w[i] = i < n ? (keys[i] & kmask) << ibits | (uint64_t)i : ~0ull;
     __syncthreads();
     block_sort_words(w, N);
 #pragma unroll
     for (int r = 0; r < SB_MAX / SB_THREADS; r++) {
         int i = r * SB_THREADS + threadIdx.x;
-        if (i < n) v[r] = vals[w[i] & imask];
+        if (i < n) {
+            k[r] = keys[w[i] & imask];
+            v[r] = vals[w[i] & imask];
+        }
     }
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < SB_MAX / SB_THREADS; r++) {
         int i = r * SB_THREADS + threadIdx.x;
         if (i < n) {
-            keys[i] = w[i] >> ibits;
+            keys[i] = k[r];
             vals[i] = v[r];
         }
     }
@@ -512,19 +523,19 @@ Status radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint
 {
     if (n <= 1 || end_bit <= 0) return Status{};
     if (n >= ((int64_t)1 << 32)) return Status{1, "radix sort: too many items"};
-    int passes = (end_bit + 7) / 8;
     if (n <= SB_MAX) {
         int N = 64, ib = bits_for((uint64_t)(n - 1));
         while (N < n) N <<= 1;
         if (end_bit + ib < 64) {   // the padding stays above every word
-            enqueue(k_sort_block, 1, SB_THREADS, 0, s, keys, vals, (int32_t)n, N, ib);
+            enqueue(k_sort_block, 1, SB_THREADS, 0, s, keys, vals, (int32_t)n, N, ib,
+                    ((uint64_t)1 << end_bit) - 1);
             SNN_CUDA(cudaGetLastError());
             return Status{};
         }
     }
     if (n <= RSC_MAX) {
         enqueue(k_rs_cluster, RSC_CTAS, RSC_THREADS, 0, s, keys, vals, keys_alt, vals_alt, (int32_t)n,
-                passes);
+                end_bit);
         SNN_CUDA(cudaGetLastError());
         return Status{};
     }
@@ -533,13 +544,14 @@ Status radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint
     SNN_TRY(ar.alloc(&counts, (int64_t)256 * nblk));
     uint64_t *ki = keys, *ko = keys_alt;
     uint32_t *vi = vals, *vo = vals_alt;
-    for (int p = 0; p < passes; p++) {
-        int shift = 8 * p;
-        enqueue(k_rs_upsweep, nblk, RS_THREADS, 0, s, ki, n, shift, counts, nblk);
+    for (int shift = 0; shift < end_bit; shift += 8) {
+        const uint32_t dmask = digit_mask(shift, end_bit);
+        enqueue(k_rs_upsweep, nblk, RS_THREADS, 0, s, ki, n, shift, dmask, counts, nblk);
         SNN_CUDA(cudaGetLastError());
         SNN_TRY((scan_plain<uint32_t, uint32_t, false>(counts, counts, (int64_t)256 * nblk,
                                                        (uint32_t*)nullptr, ar, s)));
-        enqueue(k_rs_downsweep, nblk, RS_THREADS, 0, s, ki, vi, ko, vo, n, shift, counts, nblk);
+        enqueue(k_rs_downsweep, nblk, RS_THREADS, 0, s, ki, vi, ko, vo, n, shift, dmask, counts,
+                nblk);
         SNN_CUDA(cudaGetLastError());
         uint64_t* tk = ki; ki = ko; ko = tk;
         uint32_t* tv = vi; vi = vo; vo = tv;
