@@ -103,9 +103,16 @@ __global__ void k_ip_reset(int32_t S, int32_t J, const int32_t* __restrict__ don
     }
 }
 
+struct RowAddAtomic {
+    int64_t* row;
+    __device__ void operator()(int32_t j, int64_t w) const
+    {
+        atomicAdd((unsigned long long*)&row[j], (unsigned long long)w);
+    }
+};
+
 // G of the node at each position of a depth's jobs and, for positions of L,
-// its row of the correction matrix (cleared before; ip::single_gain and
-// ip::corr_row, with the side counts of a hyperedge taken once for both). T
+// its row of the correction matrix (cleared before; ip::gain_corr_hedge). T
 // threads per position over the node's incidences: nodes of G_P are in
 // hundreds to thousands of hyperedges, so a thread per node walked a serial
 // chain (3.9 + 6.0 ms a depth for 64 starts of a 256-node G_P of 57,344
@@ -130,20 +137,11 @@ __global__ void __launch_bounds__(256)
         const int32_t lo = jb.lo[k], mid = jb.mid[k], hi = jb.hi[k];
         const int32_t x = seq[s * np + i];
         const int sd = ip::side_of((int32_t)i, lo, mid, hi);
-        unsigned long long* row = (unsigned long long*)M + s * pairs + jb.pairoff[k] +
-                                  (i - lo) * (int64_t)(hi - mid);
+        const RowAddAtomic add{M + s * pairs + jb.pairoff[k] + (i - lo) * (int64_t)(hi - mid)};
         int64_t g = 0;
         for (int64_t t = voff[x] + lane; t < voff[x + 1]; t += T) {
-            int32_t a = vinc[t], cL, cR;
-            int64_t b = off[a], e = off[a + 1], w = eta[a];
-            ip::side_counts(pins, b, e, ps, lo, mid, hi, &cL, &cR);
-            g += w * ip::move_delta(sd, cL, cR);
-            if (sd != 1 || cR == 0 || (cL != 1 && cR != 1)) continue;
-            if (cL == 1 && cR == 1) w *= 2;
-            for (int64_t j = b; j < e; j++) {
-                int32_t q = ps[pins[j]];
-                if (ip::side_of(q, lo, mid, hi) == 2) atomicAdd(&row[q - mid], (unsigned long long)w);
-            }
+            int32_t a = vinc[t];
+            g += ip::gain_corr_hedge(pins, off[a], off[a + 1], ps, sd, lo, mid, hi, eta[a], add);
         }
         g = warp_sum(g);
         if (T > 32) {
@@ -210,14 +208,6 @@ struct MAddAtomic {
     __device__ void operator()(int32_t i, int32_t j, int64_t d) const
     {
         atomicAdd((unsigned long long*)&M[(int64_t)i * nr + j], (unsigned long long)d);
-    }
-};
-
-struct RowAddAtomic {
-    int64_t* row;
-    __device__ void operator()(int32_t j, int64_t w) const
-    {
-        atomicAdd((unsigned long long*)&row[j], (unsigned long long)w);
     }
 };
 

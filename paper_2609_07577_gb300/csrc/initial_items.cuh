@@ -1,8 +1,8 @@
 // Per-item steps of the initial placement (Sec. 4.2, "Initial Placement")
 // of G_P: the Hilbert index of a core, the sides and cut changes of the
 // label propagation between two sibling sections, and the folding of the
-// bisection tree. The kernels of initial.cu run one item per thread; the
-// header uses no CUDA type, so the same steps also compile as plain host
+// bisection tree. The kernels of initial.cu call these steps for their items;
+// the header uses no CUDA type, so the same steps also compile as plain host
 // code and can be run one item at a time.
 //
 // Sections are intervals of a start's node sequence; pos[q] is the position
@@ -83,6 +83,26 @@ IP_HD int32_t move_delta(int sd, int32_t cL, int32_t cR)
     return 0;
 }
 
+// What one hyperedge (pins[b..e), weight w) adds to G(x) of a pin x on side
+// sd (returned) and, for x in L, to corr(x, .): add(j, w) as in corr_row. Its
+// side counts are taken once for both.
+template <typename Add>
+IP_HD int64_t gain_corr_hedge(const int32_t* pins, int64_t b, int64_t e, const int32_t* pos, int sd,
+                              int32_t lo, int32_t mid, int32_t hi, int64_t w, Add add)
+{
+    int32_t cL, cR;
+    side_counts(pins, b, e, pos, lo, mid, hi, &cL, &cR);
+    if (sd == 1 && cR != 0 && (cL == 1 || cR == 1)) {
+        int64_t c = cL == 1 && cR == 1 ? 2 * w : w;
+        for (int64_t j = b; j < e; j++) {
+            int32_t i = pos[pins[j]];
+            if (side_of(i, lo, mid, hi) == 2) add(i - mid, c);
+        }
+    }
+    return w * move_delta(sd, cL, cR);
+}
+
+// The same by definition, node by node (no kernel calls single_gain):
 // G(x) of node x on side sd: incidences inc[ib..ie) (hyperedge ids)
 IP_HD int64_t single_gain(const int32_t* inc, int64_t ib, int64_t ie, const int64_t* off,
                           const int32_t* pins, const int64_t* eta, const int32_t* pos, int sd,

@@ -185,15 +185,13 @@ __global__ void k_pl_init_stats(int32_t S, int64_t* st)
 }
 
 // lattice coordinates of every start's nodes
-__global__ void k_pl_xy(int64_t n, int32_t width, const int32_t* __restrict__ g, int2* xy)
+__global__ void k_pl_xy(int64_t n, int32_t width, const int32_t* __restrict__ g, place::Cell* xy)
 {
     snn::after_previous();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
-        xy[i] = make_int2(g[i] % width, g[i] / width);
+        xy[i] = place::cell_of(width, g[i]);
 }
-
-__device__ __forceinline__ int32_t xy_dist(int2 u, int2 v) { return abs(u.x - v.x) + abs(u.y - v.y); }
 
 // sum of v over the T threads (32 or the whole block of 256) of a node; the
 // result is valid in the first of them
@@ -211,56 +209,35 @@ __device__ __forceinline__ int64_t node_sum(int64_t v, unsigned long long* sh)
 }
 
 // Eq. force of every node towards its four neighbours, T threads per node
-// over its incidences, summed in registers. On a lattice the force towards a
-// neighbour only counts pins: moving one row up brings every pin above one
-// hop nearer and every other one hop farther away, and a pin on the
-// neighbour itself counts one less (the max(., 1) of Eq. force). So a pin
-// costs four comparisons and no distance; with a thread per pin entry, five
-// distances a pin (their coordinates by division) and four 64-bit atomics a
-// pin entry, a round took 1.05 ms for 64 starts of a 256-node G_P with
-// 57,344 hyperedges.
+// over its incidences (place::side_forces), summed in registers. With a
+// thread per pin entry, five distances a pin (their coordinates by division)
+// and four 64-bit atomics a pin entry, a round took 1.05 ms for 64 starts of
+// a 256-node G_P with 57,344 hyperedges.
 template <int T>
 __global__ void __launch_bounds__(256)
     k_pl_force(int32_t np, int32_t width, int32_t height, const int64_t* __restrict__ voff,
                const int32_t* __restrict__ vinc, const int64_t* __restrict__ off,
                const int32_t* __restrict__ pins, const int64_t* __restrict__ eta,
-               const int2* __restrict__ xy, const int32_t* __restrict__ act, int64_t* F)
+               const place::Cell* __restrict__ xy, const int32_t* __restrict__ act, int64_t* F)
 {
     snn::after_previous();
     __shared__ unsigned long long sh;
     int64_t s = blockIdx.y;
     if (!act[s]) return;
-    const int2* xs = xy + s * np;
+    const place::Cell* xs = xy + s * np;
     const int lane = threadIdx.x & (T - 1);
     for (int64_t p = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T; p < np;
          p += (int64_t)gridDim.x * (256 / T)) {
-        int2 c = xs[p];
+        const place::Cell c = xs[p];
         int64_t f[4] = {0, 0, 0, 0};
         for (int64_t t = voff[p] + lane; t < voff[p + 1]; t += T) {
             int32_t a = vinc[t];
-            int64_t e = off[a + 1];
-            int n = 0, l[4] = {0, 0, 0, 0};   // twice the pins beyond, less those on the neighbour
-            for (int64_t j = off[a]; j < e; j++) {
-                int32_t q = pins[j];
-                if (q == (int32_t)p) continue;
-                int2 d = xs[q];
-                int dx = d.x - c.x, dy = d.y - c.y;
-                n++;
-                l[0] += dy < 0 ? 2 : 0;
-                l[1] += dx < 0 ? 2 : 0;
-                l[2] += dx > 0 ? 2 : 0;
-                l[3] += dy > 0 ? 2 : 0;
-                if (abs(dx) + abs(dy) == 1) l[dy < 0 ? 0 : (dx < 0 ? 1 : (dx > 0 ? 2 : 3))]--;
-            }
-            int64_t w = eta[a];
-#pragma unroll
-            for (int d = 0; d < 4; d++) f[d] += w * (l[d] - n);
+            place::side_forces(pins, off[a], off[a + 1], xs, (int32_t)p, c, eta[a], f);
         }
-        bool in[4] = {c.y > 0, c.x > 0, c.x + 1 < width, c.y + 1 < height};
 #pragma unroll
         for (int d = 0; d < 4; d++) {
             int64_t v = node_sum<T>(f[d], &sh);
-            if (lane == 0) F[(s * np + p) * 4 + d] = in[d] ? v : 0;
+            if (lane == 0) F[(s * np + p) * 4 + d] = place::on_lattice(width, height, c, d) ? v : 0;
         }
     }
 }
@@ -359,14 +336,14 @@ __global__ void k_pl_rank(int64_t ns, int32_t nh, const uint32_t* __restrict__ v
 }
 
 // Re-evaluated tension: each swapping node's force towards its swap's other
-// core with every earlier swap of its start applied (place::core_before), T
+// core with every earlier swap of its start applied (place::reeval_cells), T
 // threads per node over its incidences; nodes outside swaps cost nothing.
 template <int T>
 __global__ void __launch_bounds__(256)
     k_pl_reeval(int32_t np, int32_t nh, int32_t width, const int64_t* __restrict__ voff,
                 const int32_t* __restrict__ vinc, const int64_t* __restrict__ off,
                 const int32_t* __restrict__ pins, const int64_t* __restrict__ eta,
-                const int32_t* __restrict__ g, const int2* __restrict__ cxy,
+                const int32_t* __restrict__ g, const place::Cell* __restrict__ cxy,
                 const int32_t* __restrict__ rank, const int32_t* __restrict__ mate,
                 const int32_t* __restrict__ segbeg, int64_t* Tn)
 {
@@ -382,19 +359,12 @@ __global__ void __launch_bounds__(256)
         int32_t h = gs[p];
         int32_t r = rs[h];
         if (r == NO_RANK) continue;   // the same for all T threads
-        int2 ch = cxy[h], ck = cxy[ms[h]];
+        const place::Cell ch = cxy[h], ck = cxy[ms[h]];
         int64_t v = 0;
         for (int64_t t = voff[p] + lane; t < voff[p + 1]; t += T) {
             int32_t a = vinc[t];
-            int64_t e = off[a + 1];
-            int64_t x = 0;
-            for (int64_t j = off[a]; j < e; j++) {
-                int32_t q = pins[j];
-                if (q == (int32_t)p) continue;
-                int2 c = cxy[place::core_before(rs, ms, gs[q], r)];
-                x += xy_dist(ch, c) - max(xy_dist(ck, c), 1);
-            }
-            v += eta[a] * x;
+            v += eta[a] * place::reeval_cells(pins, off[a], off[a + 1], gs, rs, ms, cxy, (int32_t)p, ch,
+                                              ck, r);
         }
         v = node_sum<T>(v, &sh);
         if (lane == 0 && v != 0)
@@ -457,20 +427,17 @@ __global__ void k_pl_apply(int64_t ns, int32_t nh, int32_t np, const uint32_t* _
 
 __global__ void k_pl_trd(int64_t P, int32_t np, const int32_t* __restrict__ hid,
                          const int64_t* __restrict__ off, const int32_t* __restrict__ pins,
-                         const int64_t* __restrict__ eta, const int2* __restrict__ xy,
+                         const int64_t* __restrict__ eta, const place::Cell* __restrict__ xy,
                          int64_t* acc)
 {
     snn::after_previous();
     int64_t s = blockIdx.y;
-    const int2* xs = xy + s * np;
+    const place::Cell* xs = xy + s * np;
     int64_t sum = 0;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P;
          j += (int64_t)gridDim.x * blockDim.x) {
         int32_t a = hid[j];
-        int64_t e = off[a + 1], x = 0;
-        int2 c = xs[pins[j]];
-        for (int64_t i = j + 1; i < e; i++) x += xy_dist(c, xs[pins[i]]);
-        sum += eta[a] * x;
+        sum += eta[a] * place::trd_cells(pins, j, off[a + 1], xs);
     }
     sum = warp_sum(sum);
     if ((threadIdx.x & 31) == 0 && sum != 0) atomicAdd((unsigned long long*)&acc[s], (unsigned long long)sum);
@@ -567,7 +534,7 @@ Status refine_impl(Input& in, int32_t* g, int32_t max_rounds, cudaStream_t s, in
     SNN_CUDA(cudaMemcpyAsync(act, h_act.data(), sizeof(int32_t) * S, cudaMemcpyHostToDevice, s));
     int64_t* voff;
     int32_t* vinc;
-    int2 *nxy, *cxy;
+    place::Cell *nxy, *cxy;
     SNN_TRY(gp_incidence(np, in.P, in.pins, hid, ar, s, &voff, &vinc));
     SNN_TRY(ar.alloc(&nxy, (int64_t)S * np));
     SNN_TRY(ar.alloc(&cxy, in.nh));
@@ -704,7 +671,7 @@ Status trd_impl(Input& in, const int32_t* g, cudaStream_t s, int64_t* trd_out)
     SNN_TRY(ar.alloc(&acc, in.S));
     SNN_CUDA(cudaMemsetAsync(acc, 0, sizeof(int64_t) * in.S, s));
     if (in.P > 0) {
-        int2* nxy;
+        place::Cell* nxy;
         const int64_t n = (int64_t)in.S * in.np;
         SNN_TRY(ar.alloc(&nxy, n));
         snn::enqueue(k_pl_xy, grid_for(n, 256), 256, 0, s, n, in.width, g, nxy);

@@ -1,8 +1,14 @@
 // Per-item steps of placement swap refinement (Sec. 4.2, "Swap Proposals"
 // and "Placement Refinement") on a width x height lattice of cores, core
-// h = y * width + x. The kernels of place.cu run one item per thread; the
-// header uses no CUDA type, so the same steps also compile as plain host
-// code and can be run one item at a time.
+// h = y * width + x. The header uses no CUDA type, so the same steps also
+// compile as plain host code and can be run one item at a time.
+//
+// The kernels of place.cu take their arithmetic from here: forces, their
+// re-evaluation and distances in the form over cells (side_forces,
+// reeval_cells, trd_cells; a warp or block per node, a hyperedge per lane),
+// proposals and tensions per core. force_terms, reeval_terms and trd_terms
+// are the same sums pin by pin from Eq. force and Eq. distance as written:
+// what the others have to equal.
 //
 // Per start, g[p] is the core of node p and pi[h] the node on core h (-1:
 // empty). Forces are kept four per node, one per direction d of the
@@ -132,6 +138,74 @@ PL_HD int64_t reeval_terms(const int32_t* pins, int64_t b, int64_t e, const int3
         int32_t dk = dist(width, k, c);
         s += dist(width, h, c) - (dk > 1 ? dk : 1);
     }
+    return s;
+}
+
+// a core's coordinates
+struct alignas(8) Cell {
+    int32_t x, y;
+};
+PL_HD Cell cell_of(int32_t width, int32_t h) { return Cell{h % width, h / width}; }
+
+PL_HD int32_t cell_dist(Cell u, Cell v)
+{
+    int32_t dx = u.x - v.x, dy = u.y - v.y;
+    return (dx < 0 ? -dx : dx) + (dy < 0 ? -dy : dy);
+}
+
+// force_terms by counting: moving one row up brings every pin above one hop
+// nearer and every other one hop farther away, and a pin on the neighbour
+// itself counts one less (the max(., 1) of Eq. force). So a pin costs four
+// comparisons and no distance. f[d] += w * the share, for all four directions
+// (those past the border mean nothing: on_lattice).
+PL_HD void side_forces(const int32_t* pins, int64_t b, int64_t e, const Cell* cell, int32_t p, Cell c,
+                       int64_t w, int64_t f[4])
+{
+    int32_t n = 0, l[4] = {0, 0, 0, 0};   // twice the pins beyond, less those on the neighbour
+    for (int64_t j = b; j < e; j++) {
+        int32_t q = pins[j];
+        if (q == p) continue;
+        Cell d = cell[q];
+        int32_t dx = d.x - c.x, dy = d.y - c.y;
+        n++;
+        l[0] += dy < 0 ? 2 : 0;
+        l[1] += dx < 0 ? 2 : 0;
+        l[2] += dx > 0 ? 2 : 0;
+        l[3] += dy > 0 ? 2 : 0;
+        if (cell_dist(d, c) == 1) l[dy < 0 ? 0 : (dx < 0 ? 1 : (dx > 0 ? 2 : 3))]--;
+    }
+    for (int d = 0; d < 4; d++) f[d] += w * (l[d] - n);
+}
+
+// whether the neighbour of c in direction d is on the lattice
+PL_HD bool on_lattice(int32_t width, int32_t height, Cell c, int d)
+{
+    return d == 0 ? c.y > 0 : d == 1 ? c.x > 0 : d == 2 ? c.x + 1 < width : c.y + 1 < height;
+}
+
+// reeval_terms with the cores' coordinates in hand: ch and ck those of p's
+// core and of the swap's other core
+PL_HD int64_t reeval_cells(const int32_t* pins, int64_t b, int64_t e, const int32_t* g,
+                           const int32_t* rank, const int32_t* mate, const Cell* core, int32_t p,
+                           Cell ch, Cell ck, int32_t r)
+{
+    int64_t s = 0;
+    for (int64_t j = b; j < e; j++) {
+        int32_t q = pins[j];
+        if (q == p) continue;
+        Cell c = core[core_before(rank, mate, g[q], r)];
+        int32_t dk = cell_dist(ck, c);
+        s += cell_dist(ch, c) - (dk > 1 ? dk : 1);
+    }
+    return s;
+}
+
+// trd_terms with the nodes' cells in hand
+PL_HD int64_t trd_cells(const int32_t* pins, int64_t j, int64_t e, const Cell* cell)
+{
+    int64_t s = 0;
+    Cell c = cell[pins[j]];
+    for (int64_t i = j + 1; i < e; i++) s += cell_dist(c, cell[pins[i]]);
     return s;
 }
 
