@@ -30,6 +30,7 @@
 //      enacted.
 #include "histo.cuh"
 #include "internal.cuh"
+#include "row_items.cuh"
 #include "scan.cuh"
 
 #include <algorithm>
@@ -586,34 +587,14 @@ __global__ void __launch_bounds__(256)
         int64_t bs = 0;
         int32_t bk = -1;
         const int64_t nq = ((int64_t)K + 3) >> 2;
-        unsigned long long msk = M[rw];   // the same word in every lane
-        // Marked entries, two loads a lane at a time: a step reads 32 int4, a
-        // part of one chunk or (cq < 32) one lane group per chunk of 32 / cq
-        // consecutive marked ones (cw is a power of two of at least 32). With
-        // one chunk a step, 8 of 32 lanes loaded at cw = 32 (conv network of
-        // 65,536 neurons: 11.7 us a round, 7.3 so).
-        const int cq = cw >> 2;                                 // int4 a chunk
-        const int per = cq > 32 ? (cq + 31) / 32 : 1;           // steps a chunk
-        const int side = cq < 32 ? 32 / cq : 1;                 // chunks a step
-        const int grp = cq < 32 ? lane / cq : 0;
-        const int at = cq < 32 ? lane - grp * cq : lane;
-        for (int g = 0; g < grp; g++) msk &= msk - 1;           // this group's first chunk
-        int part = 0;
-        while (__any_sync(FULL, msk != 0)) {
+        ChunkDeal deal(M[rw], cw, lane);   // two loads a lane at a time
+        while (__any_sync(FULL, deal.left())) {
             constexpr int U = 2;
             int4 c4[U];
             int64_t qq[U];
 #pragma unroll
             for (int u = 0; u < U; u++) {
-                qq[u] = nq;
-                if (msk) {
-                    int q = at + part * 32;
-                    if (q < cq) qq[u] = (int64_t)(__ffsll((long long)msk) - 1) * cq + q;
-                    if (++part == per) {
-                        part = 0;
-                        for (int g = 0; g < side; g++) msk &= msk - 1;
-                    }
-                }
+                qq[u] = deal.next(nq);
                 c4[u] = qq[u] < nq ? row[qq[u]] : make_int4(0, 0, 0, 0);
             }
 #pragma unroll
