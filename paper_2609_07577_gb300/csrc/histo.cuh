@@ -47,6 +47,7 @@
 #pragma once
 #include "common.cuh"
 #include "histo_tiers.cuh"
+#include "table_slot.cuh"
 
 #include <cooperative_groups.h>
 
@@ -62,14 +63,6 @@ __device__ __forceinline__ bool better(int64_t s1, int32_t m1, int64_t s2, int32
     if (m1 < 0) return false;
     if (m2 < 0) return true;
     return s1 > s2 || (s1 == s2 && m1 < m2);
-}
-
-// first slot probed for key m: the high bits of a multiplicative hash (the
-// golden ratio's), scaled to the table; runs of consecutive ids, which a
-// hyperedge's sorted pins often are, land spread over it
-__device__ __forceinline__ uint32_t table_slot(int32_t m, uint32_t mask)
-{
-    return __umulhi((uint32_t)m * 0x9e3779b1u, mask + 1);
 }
 
 // Open-addressing slots: key (-1 empty), summed weight, summed overlap.
