@@ -112,17 +112,17 @@ struct RowAddAtomic {
 };
 
 // G of the node at each position of a depth's jobs and, for positions of L,
-// its row of the correction matrix (cleared before; ip::gain_corr_hedge). T
-// threads per position over the node's incidences: nodes of G_P are in
+// its row of the correction matrix (both cleared before; ip::gain_corr_hedge).
+// T threads per piece of a node's incidences: nodes of G_P are in
 // hundreds to thousands of hyperedges, so a thread per node walked a serial
 // chain (3.9 + 6.0 ms a depth for 64 starts of a 256-node G_P of 57,344
 // hyperedges).
 template <int T>
 __global__ void __launch_bounds__(256)
-    k_ip_gain_corr(int32_t np, int64_t pairs, Jobs jb, const int32_t* __restrict__ done,
-                   const int64_t* __restrict__ voff, const int32_t* __restrict__ vinc,
-                   const int64_t* __restrict__ off, const int32_t* __restrict__ pins,
-                   const int64_t* __restrict__ eta, const int32_t* __restrict__ seq,
+    k_ip_gain_corr(int32_t np, snn::GpPieces pieces, int64_t pairs, Jobs jb,
+                   const int32_t* __restrict__ done, const int64_t* __restrict__ voff,
+                   const int32_t* __restrict__ vinc, const int64_t* __restrict__ off,
+                   const int32_t* __restrict__ pins, const int64_t* __restrict__ eta,
                    const int32_t* __restrict__ pos, int64_t* G, int64_t* M)
 {
     snn::after_previous();
@@ -130,16 +130,19 @@ __global__ void __launch_bounds__(256)
     int64_t s = blockIdx.y;
     const int32_t* ps = pos + s * np;
     const int lane = threadIdx.x & (T - 1);
-    for (int64_t i = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T; i < np;
-         i += (int64_t)gridDim.x * (256 / T)) {
-        int32_t k = jb.jobof[i];
-        if (k < 0 || done[s * jb.J + k]) continue;   // the same for all T threads
+    for (int64_t q = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T; q < pieces.n;
+         q += (int64_t)gridDim.x * (256 / T)) {
+        int64_t b, e;
+        bool whole;
+        const int32_t x = snn::gp_piece<T>(pieces, voff, q, &b, &e, &whole);
+        if (x < 0) continue;   // the same for all T threads, as below
+        const int32_t i = ps[x], k = jb.jobof[i];
+        if (k < 0 || done[s * jb.J + k]) continue;
         const int32_t lo = jb.lo[k], mid = jb.mid[k], hi = jb.hi[k];
-        const int32_t x = seq[s * np + i];
-        const int sd = ip::side_of((int32_t)i, lo, mid, hi);
+        const int sd = ip::side_of(i, lo, mid, hi);
         const RowAddAtomic add{M + s * pairs + jb.pairoff[k] + (i - lo) * (int64_t)(hi - mid)};
         int64_t g = 0;
-        for (int64_t t = voff[x] + lane; t < voff[x + 1]; t += T) {
+        for (int64_t t = b + lane; t < e; t += T) {
             int32_t a = vinc[t];
             g += ip::gain_corr_hedge(pins, off[a], off[a + 1], ps, sd, lo, mid, hi, eta[a], add);
         }
@@ -152,7 +155,9 @@ __global__ void __launch_bounds__(256)
             g = (int64_t)sh;
             __syncthreads();
         }
-        if (lane == 0) G[s * np + x] = g;
+        if (lane != 0) continue;
+        if (whole) G[s * np + x] = g;
+        else atomicAdd((unsigned long long*)&G[s * np + x], (unsigned long long)g);
     }
 }
 
@@ -542,7 +547,9 @@ Status initial_impl(int32_t np, int32_t ne, const int64_t* off, const int32_t* p
     // a block per node below that
     const bool warps = (int64_t)np * S >= 152 * 32;
     const int capn = 152 * 32 / S > 0 ? 152 * 32 / S : 1;
-    const dim3 gnode((unsigned)grid_for(np, warps ? 8 : 1, capn), (unsigned)S);
+    snn::GpPieces pieces;
+    SNN_TRY(gp_pieces(np, P, voff, warps ? 32 : 256, ar, s, &pieces));
+    const dim3 gnode((unsigned)grid_for(pieces.n, warps ? 8 : 1, capn), (unsigned)S);
     // a swap's threads take one hyperedge of the two nodes each: 128, 512, or a
     // cluster of eight blocks of 256 while the jobs leave SMs idle
     const int64_t inc2 = 2 * P / np;
@@ -585,8 +592,9 @@ Status initial_impl(int32_t np, int32_t ne, const int64_t* off, const int32_t* p
         const dim3 gpair = grid2(pairs, S);
         const int gjob = grid_for((int64_t)S * J, 256);
         SNN_CUDA(cudaMemsetAsync(M, 0, sizeof(int64_t) * S * pairs, s));
+        SNN_CUDA(cudaMemsetAsync(G, 0, sizeof(int64_t) * S * np, s));
         auto gc = warps ? k_ip_gain_corr<32> : k_ip_gain_corr<256>;
-        snn::enqueue(gc, gnode, 256, 0, s, np, pairs, jb, done, voff, vinc, off, pins, eta, seq, pos,
+        snn::enqueue(gc, gnode, 256, 0, s, np, pieces, pairs, jb, done, voff, vinc, off, pins, eta, pos,
                      G, M);
         SNN_CUDA(cudaGetLastError());
         const bool spread = inc2 >= 512 && (int64_t)J * S <= IP_SPREAD_JOBS;

@@ -239,6 +239,30 @@ Status gp_input(int32_t np, int32_t ne, const int64_t* off, const int32_t* pins,
 // q, one entry per pin entry, in any order
 Status gp_incidence(int32_t np, int64_t P, const int32_t* pins, const int32_t* hid, Arena& ar,
                     cudaStream_t s, int64_t** voff, int32_t** vinc);
+// Pieces of the nodes' incidence lists for kernels with T (32 or 256) threads
+// per node: a node of more than GP_PIECE T incidences is cut into several, so
+// that a hub's list does not hold up a launch; the sums of a cut node are
+// added up with atomics. node[i] (-1: none) and part[i], i < n.
+constexpr int GP_PIECE = 16;
+struct GpPieces {
+    int32_t* node = nullptr;
+    int32_t* part = nullptr;
+    int64_t n = 0;   // places for them (as many as there can be)
+};
+Status gp_pieces(int32_t np, int64_t P, const int64_t* voff, int T, Arena& ar, cudaStream_t s, GpPieces* out);
+// piece i's incidences [b, e) of node p (-1: none) and whether it is all of them
+template <int T>
+__device__ __forceinline__ int32_t gp_piece(const GpPieces& pc, const int64_t* __restrict__ voff, int64_t i,
+                                            int64_t* b, int64_t* e, bool* whole)
+{
+    const int32_t p = pc.node[i];
+    if (p < 0) return p;
+    const int64_t v0 = voff[p], v1 = voff[p + 1];
+    *b = v0 + (int64_t)pc.part[i] * (GP_PIECE * T);
+    *e = *b + GP_PIECE * T < v1 ? *b + GP_PIECE * T : v1;
+    *whole = v1 - v0 <= GP_PIECE * T;
+    return p;
+}
 // S3: next level from h->match
 Status contract_level(snnmap_hgraph* h);
 // after a contraction of `src`: candidates of src carried to src + 1

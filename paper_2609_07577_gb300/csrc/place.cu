@@ -23,6 +23,7 @@
 //   scan, k_pl_best, k_pl_first   the best positive prefix per start
 //   k_pl_apply    the prefix's swaps applied to gamma and pi
 #include "internal.cuh"
+#include "scan.cuh"
 
 #include <algorithm>
 #include <vector>
@@ -148,6 +149,37 @@ Status gp_incidence(int32_t np, int64_t P, const int32_t* pins, const int32_t* h
     return Status{};
 }
 
+// a node's number of pieces, and the pieces from a node's first place on
+struct GpPieceCount {
+    const int64_t* voff;
+    int64_t per;
+    __device__ int32_t operator()(int64_t p) const
+    {
+        const int64_t d = voff[p + 1] - voff[p];
+        return d > per ? (int32_t)((d + per - 1) / per) : 1;
+    }
+};
+struct GpPieceOut {
+    int32_t *node, *part;
+    __device__ void operator()(int64_t p, int32_t first, int32_t count) const
+    {
+        for (int32_t k = 0; k < count; k++) {
+            node[first + k] = (int32_t)p;
+            part[first + k] = k;
+        }
+    }
+};
+
+Status gp_pieces(int32_t np, int64_t P, const int64_t* voff, int T, Arena& ar, cudaStream_t s, GpPieces* out)
+{
+    const int64_t per = (int64_t)GP_PIECE * T;
+    out->n = np + P / per;
+    SNN_TRY(ar.alloc(&out->node, out->n));
+    SNN_TRY(ar.alloc(&out->part, out->n));
+    if (out->n > 0) SNN_CUDA(cudaMemsetAsync(out->node, 0xff, (size_t)out->n * sizeof(int32_t), s));
+    return scan_run<int32_t>(GpPieceCount{voff, per}, GpPieceOut{out->node, out->part}, np, (int32_t*)nullptr, ar, s);
+}
+
 }  // namespace snn
 
 namespace {
@@ -208,14 +240,17 @@ __device__ __forceinline__ int64_t node_sum(int64_t v, unsigned long long* sh)
     return (int64_t)*sh;
 }
 
-// Eq. force of every node towards its four neighbours, T threads per node
-// over its incidences (place::side_forces), summed in registers. With a
-// thread per pin entry, five distances a pin (their coordinates by division)
-// and four 64-bit atomics a pin entry, a round took 1.05 ms for 64 starts of
-// a 256-node G_P with 57,344 hyperedges.
+// Eq. force of every node towards its four neighbours (F cleared before), T
+// threads per piece of a node's incidences (place::side_forces), summed in
+// registers. With a thread per pin entry, five distances a pin (their
+// coordinates by division) and four 64-bit atomics a pin entry, a round took
+// 1.05 ms for 64 starts of a 256-node G_P with 57,344 hyperedges. With whole
+// nodes in place of pieces, 5,000 nodes of which four are in all 40,000
+// hyperedges took 4.5 s a placement (3.2 s pin by pin), 0.46 s in pieces; the
+// 256-node G_P 53.1 and 47.8 ms.
 template <int T>
 __global__ void __launch_bounds__(256)
-    k_pl_force(int32_t np, int32_t width, int32_t height, const int64_t* __restrict__ voff,
+    k_pl_force(int32_t np, GpPieces pieces, int32_t width, int32_t height, const int64_t* __restrict__ voff,
                const int32_t* __restrict__ vinc, const int64_t* __restrict__ off,
                const int32_t* __restrict__ pins, const int64_t* __restrict__ eta,
                const place::Cell* __restrict__ xy, const int32_t* __restrict__ act, int64_t* F)
@@ -226,18 +261,25 @@ __global__ void __launch_bounds__(256)
     if (!act[s]) return;
     const place::Cell* xs = xy + s * np;
     const int lane = threadIdx.x & (T - 1);
-    for (int64_t p = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T; p < np;
-         p += (int64_t)gridDim.x * (256 / T)) {
+    for (int64_t i = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T; i < pieces.n;
+         i += (int64_t)gridDim.x * (256 / T)) {
+        int64_t b, e;
+        bool whole;
+        const int32_t p = gp_piece<T>(pieces, voff, i, &b, &e, &whole);
+        if (p < 0) continue;   // the same for all T threads
         const place::Cell c = xs[p];
         int64_t f[4] = {0, 0, 0, 0};
-        for (int64_t t = voff[p] + lane; t < voff[p + 1]; t += T) {
+        for (int64_t t = b + lane; t < e; t += T) {
             int32_t a = vinc[t];
-            place::side_forces(pins, off[a], off[a + 1], xs, (int32_t)p, c, eta[a], f);
+            place::side_forces(pins, off[a], off[a + 1], xs, p, c, eta[a], f);
         }
 #pragma unroll
         for (int d = 0; d < 4; d++) {
             int64_t v = node_sum<T>(f[d], &sh);
-            if (lane == 0) F[(s * np + p) * 4 + d] = place::on_lattice(width, height, c, d) ? v : 0;
+            if (lane != 0 || !place::on_lattice(width, height, c, d)) continue;
+            int64_t* at = &F[(s * np + p) * 4 + d];
+            if (whole) *at = v;
+            else atomicAdd((unsigned long long*)at, (unsigned long long)v);
         }
     }
 }
@@ -337,10 +379,10 @@ __global__ void k_pl_rank(int64_t ns, int32_t nh, const uint32_t* __restrict__ v
 
 // Re-evaluated tension: each swapping node's force towards its swap's other
 // core with every earlier swap of its start applied (place::reeval_cells), T
-// threads per node over its incidences; nodes outside swaps cost nothing.
+// threads per piece of a node's incidences; nodes outside swaps cost nothing.
 template <int T>
 __global__ void __launch_bounds__(256)
-    k_pl_reeval(int32_t np, int32_t nh, int32_t width, const int64_t* __restrict__ voff,
+    k_pl_reeval(int32_t np, GpPieces pieces, int32_t nh, const int64_t* __restrict__ voff,
                 const int32_t* __restrict__ vinc, const int64_t* __restrict__ off,
                 const int32_t* __restrict__ pins, const int64_t* __restrict__ eta,
                 const int32_t* __restrict__ g, const place::Cell* __restrict__ cxy,
@@ -354,17 +396,20 @@ __global__ void __launch_bounds__(256)
     const int32_t* rs = rank + s * nh;
     const int32_t* ms = mate + s * nh;
     const int lane = threadIdx.x & (T - 1);
-    for (int64_t p = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T; p < np;
-         p += (int64_t)gridDim.x * (256 / T)) {
+    for (int64_t i = (int64_t)blockIdx.x * (256 / T) + threadIdx.x / T; i < pieces.n;
+         i += (int64_t)gridDim.x * (256 / T)) {
+        int64_t b, e;
+        bool whole;
+        const int32_t p = gp_piece<T>(pieces, voff, i, &b, &e, &whole);
+        if (p < 0) continue;
         int32_t h = gs[p];
         int32_t r = rs[h];
         if (r == NO_RANK) continue;   // the same for all T threads
         const place::Cell ch = cxy[h], ck = cxy[ms[h]];
         int64_t v = 0;
-        for (int64_t t = voff[p] + lane; t < voff[p + 1]; t += T) {
+        for (int64_t t = b + lane; t < e; t += T) {
             int32_t a = vinc[t];
-            v += eta[a] * place::reeval_cells(pins, off[a], off[a + 1], gs, rs, ms, cxy, (int32_t)p, ch,
-                                              ck, r);
+            v += eta[a] * place::reeval_cells(pins, off[a], off[a + 1], gs, rs, ms, cxy, p, ch, ck, r);
         }
         v = node_sum<T>(v, &sh);
         if (lane == 0 && v != 0)
@@ -454,10 +499,10 @@ dim3 grid2(int64_t n, int32_t S)
 // block per node below that
 inline bool warp_per_node(int64_t np, int32_t S) { return np * S >= 152 * 32; }
 
-dim3 node_grid(int64_t np, int32_t S)
+dim3 node_grid(int64_t pieces, bool warps, int32_t S)
 {
     int cap = 152 * 32 / S;
-    return dim3((unsigned)grid_for(np, warp_per_node(np, S) ? 8 : 1, cap > 0 ? cap : 1), (unsigned)S);
+    return dim3((unsigned)grid_for(pieces, warps ? 8 : 1, cap > 0 ? cap : 1), (unsigned)S);
 }
 
 struct Input {
@@ -548,9 +593,11 @@ Status refine_impl(Input& in, int32_t* g, int32_t max_rounds, cudaStream_t s, in
         ar.rewind(mk);
     }
     const bool warps = warp_per_node(np, S);
-    const dim3 gnode = node_grid(np, S);
+    GpPieces pieces;
+    SNN_TRY(gp_pieces(np, in.P, voff, warps ? 32 : 256, ar, s, &pieces));
+    const dim3 gnode = node_grid(pieces.n, warps, S);
     int32_t active = S;
-    const dim3 gn = grid2(in.P, S), gc = grid2(nh, S);
+    const dim3 gc = grid2(nh, S);
     for (int32_t round = 0; round < max_rounds && active > 0; round++) {
         Arena::Mark mk = ar.mark();
         SNN_CUDA(cudaMemsetAsync(F, 0, sizeof(int64_t) * S * (int64_t)np * 4, s));
@@ -559,8 +606,8 @@ Status refine_impl(Input& in, int32_t* g, int32_t max_rounds, cudaStream_t s, in
             snn::enqueue(k_pl_xy, grid_for((int64_t)S * np, 256), 256, 0, s, (int64_t)S * np, in.width,
                          g, nxy);
             auto force = warps ? k_pl_force<32> : k_pl_force<256>;
-            snn::enqueue(force, gnode, 256, 0, s, np, in.width, in.height, voff, vinc, in.off, in.pins,
-                         in.eta, nxy, act, F);
+            snn::enqueue(force, gnode, 256, 0, s, np, pieces, in.width, in.height, voff, vinc, in.off,
+                         in.pins, in.eta, nxy, act, F);
         }
         snn::enqueue(k_pl_propose, gc, 256, 0, s, nh, np, in.width, in.height, act, pi, F, cand,
                      cscore, st + (int64_t)PS_PROPS * S);
@@ -606,8 +653,8 @@ Status refine_impl(Input& in, int32_t* g, int32_t max_rounds, cudaStream_t s, in
             SNN_CUDA(cudaMemsetAsync(Tn, 0, sizeof(int64_t) * ns, s));
             if (in.P > 0) {
                 auto reeval = warps ? k_pl_reeval<32> : k_pl_reeval<256>;
-                snn::enqueue(reeval, gnode, 256, 0, s, np, nh, in.width, voff, vinc, in.off, in.pins,
-                             in.eta, g, cxy, rank, mate, segbeg, Tn);
+                snn::enqueue(reeval, gnode, 256, 0, s, np, pieces, nh, voff, vinc, in.off, in.pins, in.eta,
+                             g, cxy, rank, mate, segbeg, Tn);
             }
             SNN_CUDA(cudaGetLastError());
             SNN_TRY(scan_inclusive_i64(Tn, C, ns, ar, s));
