@@ -119,6 +119,18 @@ snn::Status count_nonempty(snnmap_hgraph* h, int32_t V, int32_t K, const int32_t
     return snn::Status{};
 }
 
+// Connection rows are optional: when memory for them ran out, st is cleared, the
+// rows are given back and the levels left take histograms. Any other failure
+// stays.
+bool rows_refused(snnmap_hgraph* h, snn::Status& st)
+{
+    if (st.code != SNNMAP_ERR_OOM) return false;
+    cudaGetLastError();
+    snn::dense_close(h);
+    st = snn::Status{};
+    return true;
+}
+
 }  // namespace
 
 namespace snn {
@@ -373,10 +385,10 @@ static int snnmap_partition_impl(snnmap_hgraph* h, void* stream, int32_t* d_rho_
         int64_t per = ((((int64_t)K + 3) & ~(int64_t)3) * 8 + 20);
         if (rb > 0 && !h->wide && !h->wzero && h->wsum <= INT32_MAX)
             for (int32_t l = nl - 1; l >= 0 && (int64_t)h->levels[l].V * per <= rb; l--) lb = l;
-        if (lb < nl && (!snn::dense_open(h, K, h->levels[lb].V).ok() || !snn::dense_grow(h, K).ok())) {
-            snn::dense_close(h);
-            cudaGetLastError();
-            lb = nl;
+        if (s2.ok() && lb < nl) {
+            s2 = snn::dense_open(h, K, h->levels[lb].V);
+            if (s2.ok()) s2 = snn::dense_grow(h, K);
+            if (rows_refused(h, s2)) lb = nl;
         }
     }
     if (s2.ok()) s2 = snn::carry_open(h, V0);
@@ -401,13 +413,12 @@ static int snnmap_partition_impl(snnmap_hgraph* h, void* stream, int32_t* d_rho_
                 int64_t fresh = 2 * (V - h->levels[l + 1].V);
                 bool keep = h->dense.level == l + 1;
                 if (keep ? 4 * fresh <= V || busy : busy) {
-                    if (snn::dense_grow(h, V).ok()) {
+                    s2 = snn::dense_grow(h, V);
+                    if (s2.ok()) {
                         s2 = keep ? snn::dense_descend(h, l) : snn::dense_begin(h, l);
                         rows_here = true;
-                    } else {
-                        cudaGetLastError();   // no room: histograms from here down
-                        snn::dense_close(h);
-                        lb = nl;
+                    } else if (rows_refused(h, s2)) {
+                        lb = nl;   // histograms from here down
                     }
                 }
             } else {

@@ -156,6 +156,10 @@ struct snnmap_hgraph {
     bool wzero = false;          // some kept hyperedge has omega 0: adjacency is not a
                                  // nonzero score, so no score matrix and no connection rows
     int64_t row_budget = -1;     // bytes for connection rows (-1: default, 0: none)
+    struct {                     // set by tests: dense_grow past `rows` rows fails with `code`
+        int64_t rows = INT64_MAX;
+        int code = SNNMAP_ERR_OOM;
+    } row_fault;
     snn::DenseRows dense;
     snn::ScoreMat mat;
     snn::GpOut gp;

@@ -1803,6 +1803,7 @@ Status dense_grow(snnmap_hgraph* h, int64_t rows)
 {
     DenseRows& D = h->dense;
     if (!D.rowid || rows > D.cap) return Status{SNNMAP_ERR_STATE, "connection rows: capacity"};
+    if (rows > h->row_fault.rows) return Status{h->row_fault.code, "connection rows: refused"};
     const int64_t per = (int64_t)1 << D.tab.shift;
     const size_t had = D.chunks.size(), need = (size_t)ceil_div(std::max<int64_t>(rows - D.rows, 0), per);
     std::vector<int32_t*> ptrs;
