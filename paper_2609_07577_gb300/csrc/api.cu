@@ -362,6 +362,7 @@ static int snnmap_partition_impl(snnmap_hgraph* h, void* stream, int32_t* d_rho_
     int32_t* tmp = nullptr;
     cudaError_t e = snn::dev_malloc(&tmp, (size_t)(V0 > 0 ? V0 : 1) * 4, h->stream);
     if (e != cudaSuccess) return fail(SNNMAP_ERR_OOM, cudaGetErrorString(e));
+    h->call_bytes = 4 * (int64_t)V0;
     // rho of the current level lives in `cur`; projection writes `oth`
     int32_t* cur = ((nl - 1) % 2 == 0) ? d_rho_out : tmp;
     int32_t* oth = cur == d_rho_out ? tmp : d_rho_out;
@@ -441,6 +442,7 @@ static int snnmap_partition_impl(snnmap_hgraph* h, void* stream, int32_t* d_rho_
         evals_above = h->levels[l].V > 0 ? act / h->levels[l].V : 0;
     }
     cudaFreeAsync(tmp, h->stream);
+    h->call_bytes = 0;
     snn::dense_close(h);
     snn::carry_close(h);
     if (!s2.ok()) return fail(s2);

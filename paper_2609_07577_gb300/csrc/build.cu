@@ -4,6 +4,8 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
+
 namespace snn {
 
 // ---------------------------------------------------------------------------
@@ -127,13 +129,18 @@ int64_t held_bytes(const snnmap_hgraph* h)
     int64_t t = (int64_t)h->scratch.held() + (int64_t)h->cap_v * 20;
     if (h->dense.rowid) t += h->dense.rows * h->dense.Kp * 8 + h->dense.cap * 20;
     if (h->mat.S) t += h->mat.cap * 16;
+    if (h->carry.pto[0]) t += h->carry.cap * CARRY_BYTES;
+    if (h->icar.cand) t += h->icar.cap * AFF_CARRY_BYTES;
+    if (h->gp.hoff) t += 8 * ((int64_t)h->gp.E + 1) + 4 * h->gp.P + 13 * (int64_t)h->gp.E;
     for (auto& L : h->levels) t += (int64_t)L.bytes + 5 * (int64_t)L.V;
-    return t;
+    return t + h->call_bytes;
 }
 
 void note_bytes(snnmap_hgraph* h)
 {
-    int64_t b = held_bytes(h);
+    const size_t now = h->scratch.held();
+    int64_t b = held_bytes(h) + (int64_t)(std::max(h->scratch.high, now) - now);
+    h->scratch.high = now;
     if (b > h->peak_bytes) h->peak_bytes = b;
 }
 

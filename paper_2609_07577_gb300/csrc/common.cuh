@@ -205,6 +205,8 @@ inline cudaError_t dev_malloc(T** p, size_t bytes, cudaStream_t s)
 // adds `delta` (+1 at handle creation, -1 at its release) to the count of
 // live handles and returns the new count; at 0 the pools are trimmed
 int pool_handles(int delta);
+// the most bytes that device dev's pool had in use at once since the last call
+cudaError_t pool_high(int dev, uint64_t* bytes);
 
 // Bump allocator for temporaries of one step. Memory stays reserved across
 // steps and grows (stream-ordered) when a step needs more.
@@ -214,6 +216,7 @@ struct Arena {
     size_t used = 0;      // in the last chunk
     size_t peak = 0;      // sum needed by the largest step
     size_t step_total = 0;
+    size_t high = 0;      // most held since note_bytes last looked
     cudaStream_t stream = 0;
 
     Status reserve(size_t bytes);

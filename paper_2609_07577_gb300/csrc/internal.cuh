@@ -97,6 +97,7 @@ struct Carry {
     int32_t level = -1;   // level whose final proposals buffers[cur] hold (-1: none)
     int32_t slevel = -1;  // level whose final saves save[cur] holds (-1: none)
 };
+constexpr int64_t CARRY_BYTES = 2 * (4 + 8 + 4 + 16);   // per vertex
 
 // Candidates carried through a contraction (coarsen.cu, aff_carry): for each
 // vertex of `level`, what its previous-level candidate says about it
@@ -110,6 +111,7 @@ struct AffCarry {
     int64_t cap = 0;
     int32_t level = -1;         // level the carry describes (-1: none)
 };
+constexpr int64_t AFF_CARRY_BYTES = 4 + 8 + 4 + 1 + 1;   // per vertex
 
 // The partition hypergraph G_P of the last snnmap_partition_graph call.
 struct GpOut {
@@ -149,6 +151,7 @@ struct snnmap_hgraph {
     int64_t level_budget = 0;    // bytes of intermediate levels kept resident
     int32_t keep_stride = 1;     // intermediate levels kept: multiples of this
     int64_t peak_bytes = 0;      // largest held_bytes() seen at a checkpoint
+    int64_t call_bytes = 0;      // device memory of the call in progress outside the arena
     bool have_matching = false;
     int32_t last_pairs = 0;
     bool wide = false;           // some neighbour score may reach 2^32
@@ -209,7 +212,9 @@ Status read_scalars(snnmap_hgraph* h);
 Status zero_scalars(snnmap_hgraph* h);
 
 // device bytes the handle holds now (levels, cid maps, scratch, per-vertex
-// arrays), and the running maximum of that figure
+// arrays, carried state, rows, score matrix, partition hypergraph, the buffers
+// of the call in progress), and the running maximum of that figure with the
+// most that the scratch held in between
 int64_t held_bytes(const snnmap_hgraph* h);
 void note_bytes(snnmap_hgraph* h);
 

@@ -80,6 +80,16 @@ int pool_handles(int delta)
     return g_live_handles;
 }
 
+cudaError_t pool_high(int dev, uint64_t* bytes)
+{
+    cudaMemPool_t pool = nullptr;
+    cudaError_t e = pool_of(dev, &pool);
+    if (e == cudaSuccess) e = cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemHigh, bytes);
+    uint64_t zero = 0;
+    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &zero);
+    return e;
+}
+
 // ---------------------------------------------------------------------------
 // Arena
 
@@ -108,6 +118,7 @@ Status Arena::take(size_t bytes, void** out)
         chunks.push_back(p);
         sizes.push_back(want);
         used = 0;
+        if (held() > high) high = held();
     }
     *out = (char*)chunks.back() + used;
     used += bytes;

@@ -2652,7 +2652,11 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
         cudaGetLastError();
         cols = nullptr;
     }
+    const int64_t mine = (int64_t)(cv.total + (cols ? co.total : 0));
+    h->call_bytes += mine;
     auto give_back = [&]() {
+        note_bytes(h);
+        h->call_bytes -= mine;
         cudaFreeAsync(block, s);
         if (cols) cudaFreeAsync(cols, s);
     };

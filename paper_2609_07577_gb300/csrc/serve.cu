@@ -28,24 +28,39 @@ namespace {
 using Clock = std::chrono::steady_clock;
 
 // Device bytes of one level as level_alloc lays it out (arrays rounded up
-// to 256 bytes) plus its cid map.
+// to 256 bytes) plus its cid map and pair bytes.
 int64_t level_bytes(int64_t V, int64_t E, int64_t P)
 {
     auto r = [](int64_t b) { return ((b > 0 ? b : 1) + 255) / 256 * 256; };
     return r(8 * (E + 1)) + 2 * r(4 * P) + r(8 * E) + 2 * r(4 * E) + r(E) + r(8 * (V + 1)) +
-           4 * r(4 * V) + r(4 * V) + 4096;
+           4 * r(4 * V) + r(5 * V) + 4096;
 }
 
 // Footprint model of one pass: level 0, the newest contracted level (at most
 // the size of level 0), the intermediate levels kept under a budget of one
-// level 0, the scratch arena (sort buffers, pin counts and the hash-table
-// pools, which the histogram engine bounds by max(64 MiB, 4 bytes per pin)),
-// the per-vertex matching arrays, a fixed allowance for the arena's 64 MiB
+// level 0; the arrays that live through the pass; refine_level's block at
+// level 0; the scratch arena (sort buffers, the contraction's tables, hyperedge
+// records and the hash-table pools, which the histogram engine bounds by
+// max(64 MiB, 4 bytes per pin)), a fixed allowance for the arena's 64 MiB
 // minimum chunk and the split tier's minimum pool, and the job's budget for
-// refinement connection rows and the coarsening score matrix.
+// refinement connection rows and the coarsening score matrix. The scratch is an
+// allowance, the other terms what is allocated. The library's pool had at most
+// 0.89 of it in use over 46 networks of 1,000 to 3,000,000 neurons (layered,
+// conv, power-law, and hyperedges of two pins), the most on power-law ones.
 constexpr int64_t kFootLevels = 3;
 constexpr int64_t kFootScratch = 3;
 constexpr int64_t kFootFixed = (int64_t)160 << 20;
+
+// through the pass: candidates, scores, overlaps and matching; the second copy
+// of rho; carried candidates; carried proposals and saves
+constexpr int64_t kFootVertex = 20 + 4 + snn::AFF_CARRY_BYTES + snn::CARRY_BYTES;
+// refine_level: move indices and the list of pairs' members, partition state
+// (at most one partition a vertex), pin counts, hyperedge marks and filtered
+// lists, their 32-byte records; the column update (16 slots of 12 B, a mask and the
+// round-start save a vertex; a mask and a list entry a hyperedge)
+constexpr int64_t kFootRefineV = 4 + 2 + 30 + 204;
+constexpr int64_t kFootRefineE = 16 + 32 + 8;
+constexpr int64_t kFootRefineP = 12;
 
 // connection rows / score matrix memory granted to a job (part of its
 // footprint)
@@ -59,11 +74,8 @@ int64_t input_bytes(int64_t V, int64_t E, int64_t P)
 int64_t footprint(int64_t V, int64_t E, int64_t P, bool on_host)
 {
     int64_t L0 = level_bytes(V, E, P);
-    // 20 B per vertex of candidate arrays, 17 B of carried candidates, and the
-    // refinement's column update of short prefixes (16 slots of 12 B, 16 B of
-    // flags and saves per vertex, 8 B per hyperedge)
-    int64_t f = (kFootLevels + kFootScratch) * L0 + (20 + 17 + 208) * V + 8 * E + kFootFixed +
-                job_row_budget(L0);
+    int64_t f = (kFootLevels + kFootScratch) * L0 + (kFootVertex + kFootRefineV) * V + kFootRefineE * E +
+                kFootRefineP * P + kFootFixed + job_row_budget(L0);
     if (on_host) f += input_bytes(V, E, P);
     return f;
 }
