@@ -2403,14 +2403,16 @@ static Status refine_round(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* 
         SNN_CUDA(cudaGetLastError());
     }
     // carried pin counts: take out the hyperedges the prefix touches (old
-    // counts, old rho), move, count them again, add them back
-    prof.reset(new ProfScope(h, PS_PINCOUNT));
+    // counts, old rho; on levels with rows the pass updates those as well, the
+    // stage "cross"), move, count them again, add them back
+    prof.reset(new ProfScope(h, dense ? PS_CROSS : PS_PINCOUNT));
     if (L.E > 0) {
         RowsRef R{dense ? D.rowid : nullptr, D.tab, D.M, D.cw};
         enqueue(k_prefix_hedges, ghl, 256, 0, s, L, pc, moveidx, mv, h->d_scal, R, mvbuf, inc.hdirty,
                 rho, ps, savev, inc.costv, hl);
         SNN_CUDA(cudaGetLastError());
     }
+    if (dense) prof.reset(new ProfScope(h, PS_PINCOUNT));
     enqueue(k_apply, gm, 256, 0, s, M, mv, L, h->d_scal, ps, rho, moveidx);
     SNN_CUDA(cudaGetLastError());
     if (L.E > 0) {
