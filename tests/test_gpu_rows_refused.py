@@ -28,12 +28,11 @@ def harness(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("nth", [0, 1, -1])
-@pytest.mark.parametrize("code", [OOM, CUDA])
-@pytest.mark.parametrize("name", ["cfg1s", "cfg2s"])
+@pytest.mark.parametrize("name, code, nth", [(n, c, k) for n in ("cfg1s", "cfg2s") for c in (OOM, CUDA)
+                                             for k in (0, 1, -1)] + [("cfg3s", OOM, -1)])
 def test_rows_refused(harness, tmp_path, name, code, nth):
     """Rows are refused from the coarsest, the next and the finest level that
-    has them on."""
+    has them on (cfg3s: after rounds on rows that enacted moves)."""
     hg = snngen.by_name(name)
     rho, cost, *_ = oracle.partition(hg, oracle.params_of(hg))
     net = str(tmp_path / "net")
