@@ -4,14 +4,11 @@
 //
 // Histogram. For vertex n, every pin m != n of every hyperedge a incident to
 // n adds omega(a) to score(n, m) and, when n and m are both destinations of a,
-// k(a) (original axons merged into a) to their shared inbound count. The
-// table is an open-addressing hash table keyed by m: one per warp in shared
-// memory for ordinary vertices; vertices whose distinct neighbours overflow
-// it are redone by a block with a larger shared table, and those overflowing
-// that by a block with a table in global scratch. Sums are integer atomics,
-// so the result does not depend on the order of updates. The pins of up to
-// 32 incident hyperedges are flattened into one virtual range so all 32
-// lanes load consecutive pins even when hyperedges are short.
+// k(a) (original axons merged into a) to their shared inbound count. The sums
+// are kept by the tiers of histo.cuh: open-addressing hash tables keyed by m
+// in shared memory (a warp's, a block's), arrays over the whole level where
+// its vertices fit one, tables in global scratch for the heaviest. They are
+// integer atomics, so the result does not depend on the order of updates.
 //
 // Candidate. Among neighbours m that keep the merged super-node within
 // Omega, Phi and Delta (merged inbound set = in_count(n) + in_count(m) -
@@ -375,7 +372,7 @@ static Status affinity(snnmap_hgraph* h, Level& L)
     int64_t* cnt;
     SNN_TRY(h->scratch.alloc(&cnt, HT_NCNT));
     if (L.V <= 0) SNN_CUDA(cudaMemsetAsync(cnt, 0, HT_NCNT * sizeof(int64_t), h->stream));
-    SNN_TRY(run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->d_scal, h->tiers, L.V,
+    SNN_TRY(run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->tiers, L.V,
                           !h->wzero));
     // the counters reach the level record after the matching's synchronization
     SNN_CUDA(cudaMemcpyAsync(h->h_tier, cnt, HT_NCNT * sizeof(int64_t), cudaMemcpyDeviceToHost,
@@ -811,7 +808,7 @@ static Status affinity_carried(snnmap_hgraph* h, Level& L, bool* done)
         pol.cand = h->cand;
         pol.cscore = h->cscore;
         pol.cov = h->cov;
-        SNN_TRY(run_histogram(pol, ar, s, cnt, h->h_scal + 12, h->d_scal, h->tiers, L.V, !h->wzero));
+        SNN_TRY(run_histogram(pol, ar, s, cnt, h->h_scal + 12, h->tiers, L.V, !h->wzero));
         SNN_CUDA(cudaMemcpyAsync(h->h_tier, cnt, HT_NCNT * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     }
     enqueue(k_ac_check, grid_for(L.V, 256), 256, 0, s, L, C, h->prm.omega, h->prm.delta, h->prm.phi);
@@ -831,7 +828,7 @@ static Status affinity_carried(snnmap_hgraph* h, Level& L, bool* done)
         pol.cand = h->cand;
         pol.cscore = h->cscore;
         pol.cov = h->cov;
-        SNN_TRY(run_histogram(pol, ar, s, cnt, h->h_scal + 12, h->d_scal, h->tiers, L.V, !h->wzero));
+        SNN_TRY(run_histogram(pol, ar, s, cnt, h->h_scal + 12, h->tiers, L.V, !h->wzero));
         SNN_CUDA(cudaMemcpyAsync(h->h_tier + TIER_SLOTS, cnt, HT_NCNT * sizeof(int64_t),
                                  cudaMemcpyDeviceToHost, s));
     }

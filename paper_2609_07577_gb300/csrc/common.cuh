@@ -266,7 +266,6 @@ Status radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint
 
 // Small fills.
 Status fill_i32(int32_t* p, int32_t v, int64_t n, cudaStream_t s);
-Status fill_i64(int64_t* p, int64_t v, int64_t n, cudaStream_t s);
 Status iota_i32(int32_t* p, int64_t n, cudaStream_t s);
 
 // Grid size for grid-stride loops over n items.

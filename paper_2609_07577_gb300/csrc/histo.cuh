@@ -1621,12 +1621,11 @@ Status split_cuts(const Pol& pol, Arena& ar, cudaStream_t s, const int32_t* sl, 
 
 // Host driver: work, classification and the warp, block and big-block tiers
 // run without host synchronization; the split tier follows reads of its
-// sizes. d_cnt: >= HT_NTIER device int64; h_cnt: a pinned host int64[>=3];
-// status: device word. d_cnt: >= HT_NCNT device int64 (per-tier counts, summed
-// work, vertices histogrammed).
+// sizes. d_cnt: >= HT_NCNT device int64 (per-tier counts, summed work, vertices
+// histogrammed); h_cnt: a pinned host int64[>=3].
 template <class Pol>
 Status run_histogram(const Pol& pol, Arena& ar, cudaStream_t s, int64_t* d_cnt, int64_t* h_cnt,
-                     int64_t* status, HtTiers tiers, int32_t key_space, bool positive)
+                     HtTiers tiers, int32_t key_space, bool positive)
 {
     using S = typename Pol::S;
     int32_t V = pol.V;

@@ -199,14 +199,6 @@ Status fill_i32(int32_t* p, int32_t v, int64_t n, cudaStream_t s)
     return Status{};
 }
 
-Status fill_i64(int64_t* p, int64_t v, int64_t n, cudaStream_t s)
-{
-    if (n <= 0) return Status{};
-    enqueue(k_fill<int64_t>, grid_for(n, 256), 256, 0, s, p, v, n);
-    SNN_CUDA(cudaGetLastError());
-    return Status{};
-}
-
 Status iota_i32(int32_t* p, int64_t n, cudaStream_t s)
 {
     if (n <= 0) return Status{};

@@ -477,7 +477,7 @@ struct HedgeList {
 // dcnt(p, e) > 0. A round then needs no histogram: the best move of n is a
 // scan of its row against the partition state. Rows change only when a
 // partition's count in a hyperedge crosses zero, which applied moves report
-// (k_dense_cross). Projection to the next finer level leaves the rows of
+// (rows_cross). Projection to the next finer level leaves the rows of
 // unmatched vertices exact (their hyperedges map one to one onto hyperedges
 // of the same omega, k, destination role and partition set); the two
 // members of each contracted pair get fresh rows (RowPol).
@@ -1104,7 +1104,7 @@ __global__ void k_ps_combine(Level L, const int32_t* __restrict__ rho,
 }
 
 // The same update on levels refined from connection rows: a vertex's
-// columns of P* are entries of its row (already updated by k_dense_cross;
+// columns of P* are entries of its row (already updated by k_prefix_hedges;
 // adjacency is a positive entry there, rows being used only when every
 // omega is positive). With more than PSTAR_MAX partitions in P*, every
 // vertex is flagged for a row scan.
@@ -1740,7 +1740,7 @@ static Status gains(snnmap_hgraph* h, Level& L, const PinCounts& pc, const int32
     pol.pgain = pgain;
     int64_t* cnt;
     SNN_TRY(h->scratch.alloc(&cnt, HT_NCNT));
-    return run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->d_scal, h->tiers, K,
+    return run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->tiers, K,
                          !h->wzero);
 }
 
@@ -1760,7 +1760,7 @@ static Status dense_fresh(snnmap_hgraph* h, Level& L, const PinCounts& pc)
     pol.cw = D.cw;
     int64_t* cnt;
     SNN_TRY(h->scratch.alloc(&cnt, HT_NCNT));
-    return run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->d_scal, h->tiers, D.K,
+    return run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->tiers, D.K,
                          !h->wzero);
 }
 
@@ -1886,6 +1886,10 @@ static Status pin_counts_into(snnmap_hgraph* h, Level& L, LevelExtra& X, int32_t
         SNN_CUDA(cudaGetLastError());
     }
     PinCountJob job{L.hoff, L.hpins, L.hsd, L.hk, L.hw, rho, pc, ps.pincnt, slots};
+    // with many hyperedges a partition, as every block clears and adds up K
+    // words; where the line lies is of no consequence (2 and 128 hyperedges a
+    // partition: within 0.5 % of this on eight passes of 4,096 to 1,048,576
+    // neurons)
     if (K <= PC_SMEM_K && L.E >= 16 * (int64_t)K) job.K = K;
     return seg_run(job, X.seg, L.E, ar, s);
 }
@@ -2602,6 +2606,9 @@ Status refine_level(snnmap_hgraph* h, int32_t level, int32_t K, int32_t* rho, in
     cv.add(&inc.ps.inpins, K);
     cv.add(&inc.ps.pincnt, K);
     cv.add(&inc.slots, COST_SLOTS);
+    // the members of pairs walk their incidence lists: while they are few. Pass
+    // of the 1,048,576-neuron conv network: 585 ms with at most a quarter of the
+    // vertices in pairs, 591 with all, 595 with a 32nd
     const bool inherit_save =
         use_carry && CA.slevel == level + 1 && 8 * (V - h->levels[level + 1].V) <= V;
     if (inherit_save) cv.add(&inc.mcnt, 1);

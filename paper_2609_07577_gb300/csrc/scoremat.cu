@@ -249,7 +249,7 @@ static Status mat_rows(snnmap_hgraph* h, const Level& L, const int32_t* fresh)
     pol.Vs = M.Vs;
     int64_t* cnt;
     SNN_TRY(h->scratch.alloc(&cnt, HT_NCNT));
-    return run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->d_scal, h->tiers, L.V,
+    return run_histogram(pol, h->scratch, h->stream, cnt, h->h_scal + 12, h->tiers, L.V,
                          !h->wzero);
 }
 

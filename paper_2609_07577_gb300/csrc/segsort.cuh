@@ -189,6 +189,11 @@ __device__ __forceinline__ void seg_thread_lists(const Job& job, const int32_t* 
     }
 }
 
+template <class J, class = void>
+struct seg_shared : std::false_type {};
+template <class J>
+struct seg_shared<J, std::enable_if_t<J::kShared>> : std::true_type {};
+
 // The three small buckets in one launch: blocks [0, gt) take T, the next gb0
 // blocks B0 and the rest B1, so a level pays one launch and one tail for
 // them (three launches of mostly few blocks before).
@@ -196,12 +201,7 @@ __device__ __forceinline__ void seg_thread_lists(const Job& job, const int32_t* 
 // B0 and B1 sort in registers. B1 held its keys in shared memory, one
 // compare-exchange a load pair, a store pair and a warp barrier: the
 // partition hypergraph of the 1,048,576-neuron conv network (917,504 lists
-// of 77 keys) took 2.14 ms there; see the measured figure at seg_run.
-template <class J, class = void>
-struct seg_shared : std::false_type {};
-template <class J>
-struct seg_shared<J, std::enable_if_t<J::kShared>> : std::true_type {};
-
+// of 77 keys) took 2.14 ms there and takes 1.0 ms here.
 template <class Job>
 __global__ void __launch_bounds__(256) k_seg_small(Job job, const int32_t* __restrict__ lists,
                                                    const int32_t* __restrict__ meta, int gt, int gb0)
