@@ -784,7 +784,8 @@ __device__ __forceinline__ int32_t seg_find(const int32_t* spre, int32_t n, int3
 // 21.5, at 8 31.9 and 19.2, a few spilled words included.
 // (Their scratch is shared so that it fits: with quads in the table's scan,
 // one segment a group in flight and no checks for long segments where the
-// level has none, 28.1 and 17.0 ms.)
+// level has none, 28.1 and 17.0 ms; 29.2 and 17.2 with ids folded into the
+// slots, table_slot.cuh.)
 constexpr int HT_BLOCKS = 8;
 
 template <class Pol, int T, int CAP, int TIER, int NEXT>

@@ -45,8 +45,9 @@ int64_t level_bytes(int64_t V, int64_t E, int64_t P)
 // minimum chunk and the split tier's minimum pool, and the job's budget for
 // refinement connection rows and the coarsening score matrix. The scratch is an
 // allowance, the other terms what is allocated. The library's pool had at most
-// 0.89 of it in use over 46 networks of 1,000 to 3,000,000 neurons (layered,
-// conv, power-law, and hyperedges of two pins), the most on power-law ones.
+// 0.89 of it in use over 48 networks of 1,000 to 3,000,000 neurons (layered,
+// conv, power-law, and hyperedges of two pins), 0.93 over 256 jobs of a batch
+// with a larger row budget each; the most on power-law networks.
 constexpr int64_t kFootLevels = 3;
 constexpr int64_t kFootScratch = 3;
 constexpr int64_t kFootFixed = (int64_t)160 << 20;
